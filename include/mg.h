@@ -427,7 +427,7 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *stats);
  * call builds the dense pseudo-inverse from scratch and applies it; it needs
  * no handle and calls no cudaMalloc, cudaFree or other allocating routine.
  * Working memory is one fixed array in this library's device image (about
- * 2.1 MB, held on every GPU that loads the library until the process exits),
+ * 2.4 MB, held on every GPU that loads the library until the process exits),
  * so nx*ny*nz must be at most MG_NOALLOC_MAX_CELLS (MG_ERR_ARG otherwise).
  * The first call on each device looks up that array's device address (with
  * that device current); make it before any stream capture.  Every call uses

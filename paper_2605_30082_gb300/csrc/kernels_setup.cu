@@ -1,6 +1,5 @@
 // Set-up kernels: density mixing (Eq. (5)), face coefficients, coarsening,
-// inverse diagonals, precision copies, CSF faces, RHS assembly and the dense
-// coarse-level inverse.  All FP64, one thread per cell (these run once per
+// inverse diagonals, precision copies, CSF faces and RHS assembly.  All FP64, one thread per cell (these run once per
 // density field, not inside the V-cycle).
 #include "mg_internal.cuh"
 
@@ -248,144 +247,6 @@ __global__ void k_rhs(Dims d, double ih, const double *b0, const double *__restr
     b[c] = v;
 }
 
-// ---- dense coarse inverse -----------------------------------------------------------
-// M (row-major nc x nc) = A_c; one thread per row
-__global__ void k_coarse_assemble(Dims d, double ih2, const double *__restrict__ fx,
-                                  const double *__restrict__ fy, const double *__restrict__ fz,
-                                  double *M) {
-    i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= d.n) return;
-    const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
-    int i = (int)(cu_ - ru_ * (unsigned)d.nx);
-    int j = (int)(ru_ % (unsigned)d.ny);
-    int k = (int)(ru_ / (unsigned)d.ny);
-    double *row = M + c * d.n;
-    for (i64 q = 0; q < d.n; ++q) row[q] = 0.0;
-    double diag = 0.0, v;
-    if (i > 0) { v = fx[c] * ih2; row[c - 1] -= v; diag += v; }
-    if (i < d.nx - 1) { v = fx[c + 1] * ih2; row[c + 1] -= v; diag += v; }
-    if (j > 0) { v = fy[c] * ih2; row[c - d.nx] -= v; diag += v; }
-    if (j < d.ny - 1) { v = fy[c + d.nx] * ih2; row[c + d.nx] -= v; diag += v; }
-    if (k > 0) { v = fz[c] * ih2; row[c - d.nxy] -= v; diag += v; }
-    if (k < d.nz - 1) { v = fz[c + d.nxy] * ih2; row[c + d.nxy] -= v; diag += v; }
-    row[c] = diag;
-}
-
-// scal[0] = c = mean(diag)/nc; adds c to every entry; scal[1] = 1/M[0][0]
-__global__ void k_coarse_shift(int nc, double *M, double *scal) {
-    __shared__ double red[1024];
-    double t = 0.0;
-    for (int q = threadIdx.x; q < nc; q += blockDim.x) t += M[(i64)q * nc + q];
-    red[threadIdx.x] = t;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    double cshift = red[0] / nc / nc;
-    __syncthreads();
-    for (i64 q = threadIdx.x; q < (i64)nc * nc; q += blockDim.x) M[q] += cshift;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        scal[0] = cshift;
-        scal[1] = 1.0 / M[0];
-    }
-}
-
-// ---- blocked Gauss-Jordan inversion in place (no pivoting: M is symmetric positive definite)
-// Block step on the pivot block K = [kb, kb + bs): P^-1 (one block), the row panel
-// M[K, J] <- P^-1 M[K, J], the trailing update M[I, J] <- M[I, J] - M[I, K] M[K, J], and the
-// column panel M[I, K] <- -M[I, K] P^-1, M[K, K] <- P^-1 (I, J outside K).  The same algebra as
-// the element-wise sweeps, BS pivots per step, so n / BS steps of four launches instead of n.
-constexpr int GJ_BS = kGjBlock;
-
-// P^-1 of the bs x bs pivot block by element-wise Gauss-Jordan in shared memory; Pinv (bs x bs,
-// row-major) written to global scratch.  One block of GJ_BS x GJ_BS threads.
-__global__ void k_gj_pivot_inv(int n, int kb, int bs, const double *__restrict__ M, double *Pinv) {
-    __shared__ double P[GJ_BS][GJ_BS + 1];
-    __shared__ double rps;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    if (tx < bs && ty < bs) P[ty][tx] = M[(i64)(kb + ty) * n + kb + tx];
-    __syncthreads();
-    for (int k = 0; k < bs; ++k) {
-        // one FP64 division per pivot (by one thread), not one per thread
-        if (tx == 0 && ty == 0) rps = 1.0 / P[k][k];
-        __syncthreads();
-        double v = 0.0;
-        if (tx < bs && ty < bs) {
-            const double rp = rps;
-            if (ty == k && tx == k) v = rp;
-            else if (ty == k) v = P[k][tx] * rp;
-            else if (tx == k) v = -P[ty][k] * rp;
-            else v = P[ty][tx] - P[ty][k] * (P[k][tx] * rp);
-        }
-        __syncthreads();
-        if (tx < bs && ty < bs) P[ty][tx] = v;
-        __syncthreads();
-    }
-    if (tx < bs && ty < bs) Pinv[ty * GJ_BS + tx] = P[ty][tx];
-}
-
-// row panel: for the 32-column tile blockIdx.x (skipping K's columns), M[K, J] <- P^-1 M[K, J]
-__global__ void k_gj_row_panel(int n, int kb, int bs, double *M, const double *__restrict__ Pinv) {
-    __shared__ double Pi[GJ_BS][GJ_BS + 1], R[GJ_BS][GJ_BS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int j = blockIdx.x * GJ_BS + tx;
-    const bool colok = j < n && (j < kb || j >= kb + bs);
-    if (ty < bs && tx < bs) Pi[ty][tx] = Pinv[ty * GJ_BS + tx];
-    if (ty < bs) R[ty][tx] = colok ? M[(i64)(kb + ty) * n + j] : 0.0;
-    __syncthreads();
-    if (ty < bs && colok) {
-        double acc = 0.0;
-        for (int t = 0; t < bs; ++t) acc = fma(Pi[ty][t], R[t][tx], acc);
-        M[(i64)(kb + ty) * n + j] = acc;
-    }
-}
-
-// trailing update of the 32 x 32 tile (blockIdx.y rows, blockIdx.x columns), rows and columns
-// outside K: M[i, j] -= sum_t M[i, kb + t] M[kb + t, j] (the row panel already updated)
-__global__ void k_gj_trailing(int n, int kb, int bs, double *M) {
-    __shared__ double C[GJ_BS][GJ_BS + 1], R[GJ_BS][GJ_BS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i = blockIdx.y * GJ_BS + ty, j = blockIdx.x * GJ_BS + tx;
-    const bool rowok = i < n && (i < kb || i >= kb + bs), colok = j < n && (j < kb || j >= kb + bs);
-    // C[ty][t] = M[i, kb + t], R[t][tx] = M[kb + t, j]
-    C[ty][tx] = (i < n && tx < bs) ? M[(i64)i * n + kb + tx] : 0.0;
-    R[ty][tx] = (ty < bs && j < n) ? M[(i64)(kb + ty) * n + j] : 0.0;
-    __syncthreads();
-    if (rowok && colok) {
-        double acc = M[(i64)i * n + j];
-        for (int t = 0; t < bs; ++t) acc = fma(-C[ty][t], R[t][tx], acc);
-        M[(i64)i * n + j] = acc;
-    }
-}
-
-// column panel: M[i, K] <- -M[i, K] P^-1 for rows i outside K; the block of rows holding K
-// writes M[K, K] = P^-1
-__global__ void k_gj_col_panel(int n, int kb, int bs, double *M, const double *__restrict__ Pinv) {
-    __shared__ double Pi[GJ_BS][GJ_BS + 1], C[GJ_BS][GJ_BS + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i = blockIdx.x * GJ_BS + ty;
-    if (ty < bs && tx < bs) Pi[ty][tx] = Pinv[ty * GJ_BS + tx];
-    C[ty][tx] = (i < n && tx < bs) ? M[(i64)i * n + kb + tx] : 0.0;
-    __syncthreads();
-    if (i < n && tx < bs) {
-        if (i >= kb && i < kb + bs) {
-            M[(i64)i * n + kb + tx] = Pi[i - kb][tx];
-        } else {
-            double acc = 0.0;
-            for (int t = 0; t < bs; ++t) acc = fma(C[ty][t], Pi[t][tx], acc);
-            M[(i64)i * n + kb + tx] = -acc;
-        }
-    }
-}
-
-__global__ void k_pinv_finish(int nc, double *M, const double *__restrict__ scal) {
-    i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (i64)nc * nc) return;
-    M[e] -= 1.0 / (scal[0] * (double)nc * (double)nc);
-}
-
 }  // namespace
 
 void launch_density(cudaStream_t s, i64 n, int nfrac, const double *const *frac,
@@ -460,32 +321,6 @@ void launch_rhs(cudaStream_t s, Dims d, double h, const double *b0, const double
     count_launch();
     k_rhs<<<blocks_for(d.n), kThreads, 0, s>>>(d, 1.0 / h, b0, ux, uy, uz, fx, fy, fz, csfx, csfy,
                                                csfz, sigma, b);
-}
-
-void launch_coarse_assemble(cudaStream_t s, Dims d, double ih2, const double *fx, const double *fy,
-                            const double *fz, double *M, double *scal) {
-    count_launch();
-    k_coarse_assemble<<<blocks_for(d.n), kThreads, 0, s>>>(d, ih2, fx, fy, fz, M);
-    count_launch();
-    k_coarse_shift<<<1, 1024, 0, s>>>((int)d.n, M, scal);
-}
-
-void launch_gj_blocked(cudaStream_t s, int nc, double *M, double *scratch) {
-    const dim3 blk(GJ_BS, GJ_BS);
-    const int nt = (nc + GJ_BS - 1) / GJ_BS;
-    for (int kb = 0; kb < nc; kb += GJ_BS) {
-        const int bs = nc - kb < GJ_BS ? nc - kb : GJ_BS;
-        count_launch(4);
-        k_gj_pivot_inv<<<1, blk, 0, s>>>(nc, kb, bs, M, scratch);
-        k_gj_row_panel<<<nt, blk, 0, s>>>(nc, kb, bs, M, scratch);
-        k_gj_trailing<<<dim3(nt, nt), blk, 0, s>>>(nc, kb, bs, M);
-        k_gj_col_panel<<<nt, blk, 0, s>>>(nc, kb, bs, M, scratch);
-    }
-}
-
-void launch_pinv_finish(cudaStream_t s, int nc, double *M, const double *scal) {
-    count_launch();
-    k_pinv_finish<<<blocks_for((i64)nc * nc), kThreads, 0, s>>>(nc, M, scal);
 }
 
 }  // namespace mg

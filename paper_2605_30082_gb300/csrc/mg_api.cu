@@ -50,7 +50,7 @@ struct mg_handle {
     int nlev;
     Level lv[MG_MAX_LEVELS];
     int nc;
-    double *pinv, *gj_tmp, *scal;
+    double *pinv, *pinv_tmp;
     double *bt;        // zero-mean fine RHS (scaled by h^2 in the mixed modes)
     float2 *bt2, *p2;  // MIXED_DF: the RHS and the solution as FP32 pairs
     double *partials;  // reduction partials
@@ -419,9 +419,7 @@ int finish_operator(mg_handle *h) {
     }
     // dense pseudo-inverse of the coarsest operator
     Level &C = h->lv[h->nlev - 1];
-    mg::launch_coarse_assemble(s, C.d, C.ih2, C.fx64, C.fy64, C.fz64, h->pinv, h->scal);
-    mg::launch_gj_blocked(s, h->nc, h->pinv, h->gj_tmp);  // in place, 32 pivots per step
-    mg::launch_pinv_finish(s, h->nc, h->pinv, h->scal);
+    mg::launch_coarse_pinv(s, C.d, C.ih2, C.fx64, C.fy64, C.fz64, h->pinv, h->pinv_tmp);
     prof_end(h);  // MG_PROF_SETUP, begun by the caller
     int st = check_launch(h, "operator set-up");
     if (st) return st;
@@ -812,8 +810,7 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
         }
     }
     add((void **)&h->pinv, 8 * (size_t)nc * nc);
-    add((void **)&h->gj_tmp, 8 * (size_t)mg::kGjBlock * mg::kGjBlock);
-    add((void **)&h->scal, 8 * 4);
+    add((void **)&h->pinv_tmp, 8 * mg::coarse_scratch_doubles(h->lv[nl - 1].d));
     add((void **)&h->bt, 8 * (size_t)h->lv[0].d.n);
     if (dfm) {
         add((void **)&h->bt2, 8 * (size_t)h->lv[0].d.n);

@@ -203,14 +203,12 @@ void launch_rhs(cudaStream_t s, Dims d, double h, const double *b0, const double
                 const double *uz, const double *fx, const double *fy, const double *fz,
                 const double *csfx, const double *csfy, const double *csfz, double sigma,
                 double *b);
-// dense coarse inverse (Gauss-Jordan on A_c + c 1 1^T, then minus 1/(c n^2))
-void launch_coarse_assemble(cudaStream_t s, Dims d, double ih2, const double *fx, const double *fy,
-                            const double *fz, double *M, double *scal);
-// Gauss-Jordan inversion in place by blocks of kGjBlock pivots (scratch: kGjBlock x kGjBlock
-// doubles, the inverse of the current pivot block)
-constexpr int kGjBlock = 32;
-void launch_gj_blocked(cudaStream_t s, int nc, double *M, double *scratch);
-void launch_pinv_finish(cudaStream_t s, int nc, double *M, const double *scal);
+// ---- dense coarse solve (kernels_coarse.cu) -----------------------------------------
+// M (n x n, row-major) = pseudo-inverse of the operator of a grid of n <= MG_MAX_COARSE cells,
+// n >= 2 (low faces fx, fy, fz); scratch: coarse_scratch_doubles(d) doubles
+size_t coarse_scratch_doubles(Dims d);
+void launch_coarse_pinv(cudaStream_t s, Dims d, double ih2, const double *fx, const double *fy, const double *fz,
+                        double *M, double *scratch);
 
 // ---- V-cycle kernels --------------------------------------------------------------
 // ---- FP32 colour-split level kernels (kernels_split.cu) ----

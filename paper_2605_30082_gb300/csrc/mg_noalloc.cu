@@ -22,11 +22,11 @@
 namespace {
 
 constexpr int kMaxCells = MG_NOALLOC_MAX_CELLS;
-constexpr size_t kPivotDoubles = (size_t)mg::kGjBlock * mg::kGjBlock;
-// layout in doubles: M [kMaxCells^2] | W [the inverse of one pivot block of the Gauss-Jordan
-// elimination] | fx, fy, fz [kMaxCells each] | scal [4] | error word.  About 2.1 MB in all.
-constexpr size_t kScratchDoubles =
-    (size_t)kMaxCells * kMaxCells + kPivotDoubles + 3 * (size_t)kMaxCells + 8;
+// plane inverses (n m doubles, m <= n^(2/3) = 64 cells per plane) and column means
+constexpr size_t kPinvDoubles = (size_t)kMaxCells * 64 + kMaxCells;
+// layout in doubles: M [kMaxCells^2] | W [scratch of launch_coarse_pinv] | fx, fy, fz
+// [kMaxCells each] | error word.  About 2.4 MB in all.
+constexpr size_t kScratchDoubles = (size_t)kMaxCells * kMaxCells + kPinvDoubles + 3 * (size_t)kMaxCells + 8;
 
 __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
 
@@ -69,11 +69,10 @@ extern "C" int mg_dense_solve_noalloc(int nx, int ny, int nz, double h, const do
     const int nc = (int)n;
     double *M = base;
     double *W = M + (size_t)kMaxCells * kMaxCells;
-    double *fx = W + kPivotDoubles;
+    double *fx = W + kPinvDoubles;
     double *fy = fx + kMaxCells;
     double *fz = fy + kMaxCells;
-    double *scal = fz + kMaxCells;
-    unsigned *err = reinterpret_cast<unsigned *>(scal + 4);
+    unsigned *err = reinterpret_cast<unsigned *>(fz + kMaxCells);
     mg::Dims d = mg::make_dims(nx, ny, nz);
 
     // the error word keeps the previous call's value: clear it first
@@ -82,10 +81,8 @@ extern "C" int mg_dense_solve_noalloc(int nx, int ny, int nz, double h, const do
         return MG_ERR_CUDA;
     }
     mg::launch_faces_from_api(s, d, bx, by, bz, fx, fy, fz, err);
-    // every entry of M, W and scal below is written before it is read
-    mg::launch_coarse_assemble(s, d, 1.0 / (h * h), fx, fy, fz, M, scal);
-    mg::launch_gj_blocked(s, nc, M, W);  // in place; W holds each pivot block's inverse
-    mg::launch_pinv_finish(s, nc, M, scal);
+    // every entry of M and W below is written before it is read
+    mg::launch_coarse_pinv(s, d, 1.0 / (h * h), fx, fy, fz, M, W);
     mg::launch_coarse_matvec<double>(s, nc, M, r, e);
     unsigned herr = 0;
     if (cudaGetLastError() != cudaSuccess ||
