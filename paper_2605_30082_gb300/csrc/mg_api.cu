@@ -76,6 +76,10 @@ struct mg_handle {
     // kernel by kernel
     cudaGraphExec_t tail_exec;
     long long tail_launches;
+    // the levels from tail_l (>= 1) down as one cluster launch (kernels_tail.cu); 0: none
+    int tail_l, tail_split;
+    mg::TailArgs tail;
+    void *tail_img;
     // optional per-class timing of level-0 kernels (events recorded around launches)
     int prof_on;
     cudaEvent_t *pev;
@@ -194,6 +198,20 @@ void replay_tail(mg_handle *h) {
     // a failed launch leaves its error for the solve's check_launch
 }
 
+// ---- the coarse levels in one cluster (kernels_tail.cu) ----------------------------------
+void run_tail(mg_handle *h) {
+    const bool f64 = h->o.precision == MG_FP64;
+    if (!h->tail_split) {
+        mg::launch_tail(h->s, h->tail, f64, mg::kTailAll);
+        return;
+    }
+    Level &C = h->lv[h->nlev - 1];
+    mg::launch_tail(h->s, h->tail, f64, mg::kTailDown);
+    if (f64) mg::launch_coarse_matvec<double>(h->s, h->nc, h->pinv, C.b64, C.x64);
+    else mg::launch_coarse_matvec32(h->s, C.lay, h->pinv, C.b32, C.x32);
+    mg::launch_tail(h->s, h->tail, f64, mg::kTailUp);
+}
+
 // ---- FP64 V-cycle: in-place per-colour half sweeps, standalone transfers --------------
 // (FP64 arithmetic, not bytes, bounds these kernels on GB300, so they do no
 // redundant work; see the fused FP32 passes below for the bandwidth-bound cycle)
@@ -236,6 +254,10 @@ void vcycle64(mg_handle *h, int l, const double *b, double *x, bool x_zero) {
         return;
     }
     Level &L = h->lv[l], &C = h->lv[l + 1];
+    if (l > 0 && l == h->tail_l && x_zero && b == L.b64 && x == L.x64) {
+        run_tail(h);
+        return;
+    }
     if (x_zero) cudaMemsetAsync(x, 0, sizeof(double) * (size_t)L.d.n, h->s);
     presmooth_restrict64(h, l, b, x, C.b64, h->o.pre);
     if (l == 0) prof_begin(h, MG_PROF_COARSE_LEVELS);
@@ -352,6 +374,10 @@ void vcycle32(mg_handle *h, int l, const float *b, float *x, const OuterUpdate *
         if (l == 0) prof_end(h);
         return;
     }
+    if (l > 0 && l == h->tail_l && from_zero && b == L.b32 && x == L.x32) {
+        run_tail(h);
+        return;
+    }
     Level &C = h->lv[l + 1];
     presmooth_restrict32(h, l, b, x, C.b32, h->o.pre, from_zero);
     if (l == 0) prof_begin(h, MG_PROF_COARSE_LEVELS);
@@ -359,6 +385,68 @@ void vcycle32(mg_handle *h, int l, const float *b, float *x, const OuterUpdate *
     else vcycle32(h, l + 1, C.b32, C.x32);
     if (l == 0) prof_end(h);
     prolong_postsmooth32(h, l, b, C.x32, x, h->o.post, up);
+}
+
+// Which levels run as one cluster launch: from the first level (below the finest) that fits the
+// threads and shared memory of 16 CTAs (8 where the device refuses 16): 32768 cells in FP32 and
+// 16384 in FP64, where 16 SMs update one colour in about 1 us, half of what a launch over the
+// whole device costs.  With more than 512 coarse cells the dense product (n^2 FP64 FMAs, 4 us
+// on 16 SMs at 512) goes to the whole device between two cluster launches.
+constexpr int kTailCoarse = 512;
+
+// before the arena is carved: which levels, and the bytes of their image
+void plan_tail(mg_handle *h) {
+    h->tail_l = h->tail_split = 0;
+    const bool f64 = h->o.precision == MG_FP64;
+    if (h->nlev < 3 || h->o.pre < 1 || h->o.post < 1 || h->o.prolong != MG_PROLONG_TRILINEAR) return;
+    for (int l = 1; l < h->nlev - 1; ++l) {
+        if (h->nlev - 1 - l > mg::kTailLevels) continue;
+        mg::TailArgs &a = h->tail;
+        std::memset(&a, 0, sizeof(a));
+        a.nl = h->nlev - 1 - l;
+        a.nc = h->nc;
+        a.pre = h->o.pre;
+        a.post = h->o.post;
+        for (int q = 0; q < a.nl; ++q) {
+            Level &L = h->lv[l + q];
+            mg::TailLevel &t = a.lv[q];
+            t.nx = L.d.nx;
+            t.ny = L.d.ny;
+            t.nz = L.d.nz;
+            t.half = L.lay.half;
+            t.h2 = L.h2;
+            t.ih2 = L.ih2;
+        }
+        if (mg::tail_layout(a, f64, 16) || mg::tail_layout(a, f64, 8)) {
+            h->tail_l = l;
+            h->tail_split = h->nc > kTailCoarse;
+            return;
+        }
+    }
+}
+
+// after the arena is carved: the arrays of the tail's levels
+void bind_tail(mg_handle *h) {
+    if (!h->tail_l) return;
+    const bool f64 = h->o.precision == MG_FP64;
+    mg::TailArgs &a = h->tail;
+    a.pinv = h->pinv;
+    a.img = h->tail_img;
+    Level &C = h->lv[h->nlev - 1];
+    a.bc = f64 ? (void *)C.b64 : (void *)C.b32;
+    a.xc = f64 ? (void *)C.x64 : (void *)C.x32;
+    a.half_c = C.lay.half;
+    for (int q = 0; q < a.nl; ++q) {
+        Level &L = h->lv[h->tail_l + q];
+        mg::TailLevel &t = a.lv[q];
+        t.fx = f64 ? (const void *)L.fx64 : (const void *)L.fx32;
+        t.fy = f64 ? (const void *)L.fy64 : (const void *)L.fy32;
+        t.fz = f64 ? (const void *)L.fz64 : (const void *)L.fz32;
+        t.invd = L.invd64;
+        t.diag = L.d64;
+        t.x = f64 ? (void *)L.x64 : (void *)L.x32;
+        t.b = f64 ? (void *)L.b64 : (void *)L.b32;
+    }
 }
 
 // Record levels 1 .. coarsest of one V-cycle (FP64 or FP32, as the handle's cycle) on a private
@@ -417,6 +505,7 @@ int finish_operator(mg_handle *h) {
         mg::launch_split(s, F.d.n, F.fz64, F.fz2);
         mg::launch_split(s, F.d.n, F.d64, F.d2);
     }
+    if (h->tail_l) mg::launch_tail_prepare(s, h->tail, !mixed);
     // dense pseudo-inverse of the coarsest operator
     Level &C = h->lv[h->nlev - 1];
     mg::launch_coarse_pinv(s, C.d, C.ih2, C.fx64, C.fy64, C.fz64, h->pinv, h->pinv_tmp);
@@ -809,6 +898,8 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
             add((void **)&L.b64, 8 * n);
         }
     }
+    plan_tail(h);
+    if (h->tail_l) add((void **)&h->tail_img, (size_t)h->tail.img_total);
     add((void **)&h->pinv, 8 * (size_t)nc * nc);
     add((void **)&h->pinv_tmp, 8 * mg::coarse_scratch_doubles(h->lv[nl - 1].d));
     add((void **)&h->bt, 8 * (size_t)h->lv[0].d.n);
@@ -861,6 +952,7 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
         mg_destroy(h);
         return MG_ERR_CUDA;
     }
+    bind_tail(h);
     build_tail_graph(h);
     h->msg[0] = 0;
     *out = h;

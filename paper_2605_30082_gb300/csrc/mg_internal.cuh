@@ -308,6 +308,43 @@ void launch_prolong(cudaStream_t s, Dims coarse, const T *ec, T *e, int kind, in
 template <typename T>
 void launch_coarse_matvec(cudaStream_t s, int nc, const double *pinv, const T *r, T *e);
 
+// ---- the coarse levels of a V-cycle in one cluster launch (kernels_tail.cu) -------------
+constexpr int kTailLevels = 6;
+constexpr int kTailCells32 = 2, kTailCells64 = 1;  // cells of a colour per thread
+constexpr int kTailMaxSmem = 227 * 1024;  // per CTA, dynamic
+enum { kTailAll = 0, kTailDown = 1, kTailUp = 2 };
+struct TailLevel {
+    int nx, ny, nz;
+    i64 half;              // colour stride of the FP32 arrays in memory (Lay.half)
+    double h2, ih2;
+    const void *fx, *fy, *fz, *invd, *diag;  // the level's arrays (FP32 in its Lay, FP64 natural)
+    void *x, *b;
+    // set by tail_layout
+    int hx, q4, nit, rs;   // nx / 2, row quads and cells of a colour per CTA, row stride of x
+    unsigned magic_nx, magic_hx;
+    int off_x, off_b, off_c, off_w, off_q;
+    int img_bytes;         // one CTA's contexts and tables, from off_c
+    i64 img;               // offset of the level's images in TailArgs::img
+};
+// nl smoothed levels and the dense coarse solve of nc cells below them
+struct TailArgs {
+    int nl, nc, pre, post;
+    TailLevel lv[kTailLevels];
+    const double *pinv;
+    void *bc, *xc;         // the coarsest level's b and x in memory (split runs), colour stride half_c
+    i64 half_c;
+    void *img;             // img_total bytes, written by launch_tail_prepare
+    i64 img_total;
+    int ncta, smem, off_rc, off_ec, off_cw;
+};
+// lays the levels (nx, ny, nz, nc set) out over ncta CTAs; false if they do not fit
+bool tail_layout(TailArgs &a, bool fp64, int ncta);
+// the cells' coefficients and addresses as the launches below read them, from the levels' arrays
+void launch_tail_prepare(cudaStream_t s, const TailArgs &a, bool fp64);
+// one V-cycle of those levels from x = 0 on lv[0].b into lv[0].x (mode kTailAll), or its descent
+// or ascent alone.  pre, post >= 1, trilinear prolongation, every level's nx, ny, nz even.
+void launch_tail(cudaStream_t s, const TailArgs &a, bool fp64, int mode);
+
 // ---- reductions, fine-level FP64 passes, adjoint -----------------------------------
 // partials: reduce_blocks(n) x 2 doubles; out: 2 doubles (deterministic order)
 // scalars for the host: a one-thread-per-value kernel stores n (<= 32) doubles, or one
