@@ -1,27 +1,19 @@
 // Set-up of the dense coarse solve: the pseudo-inverse A^+ of the coarsest operator (at most
-// 1024 cells), by block elimination along the longest axis.
+// 1024 cells), A^+ = (A + c 1 1^T)^-1 - 1 1^T / (c n^2), c = mean(diag) / n, by blocked
+// Gauss-Jordan in place without pivoting (the matrix is symmetric positive definite).
 //
-// Ordered in planes across its longest axis the operator is block tridiagonal: L planes of m
-// cells (m <= 101), the blocks between planes diagonal (one face per cell).  With Schur
-// complements taken from both ends towards the middle plane,
-//     W_k = (A_kk - F W_(k-1) F)^-1   from below,   W_k = (A_kk - F' W_(k+1) F')^-1   from above,
-// F the diagonal of face coefficients between the two planes, and in the middle
-//     W_mid = (A_mid - both terms + c 1 1^T)^-1,
-// which inverts A + c v v^T, v the indicator of the middle plane (the middle Schur complement
-// is singular, its null vector the constants; v v^T does not change A^+ r, because a zero-sum
-// right-hand side gives v . x = 0).  Each column of that inverse G is one elimination towards
-// the middle and one back-substitution outwards with the W_k, and A^+ = P G P with
-// P = I - 1 1^T / n, which is G minus its row and column means plus its mean.
+// A step takes 32 pivots K: P^-1 of the pivot block, the row panel M[K, J] <- P^-1 M[K, J], the
+// trailing update M[I, J] <- M[I, J] - M[I, K] M[K, J], and the column panel
+// M[I, K] <- -M[I, K] P^-1, M[K, K] <- P^-1 (I, J outside K).
 //
-// What bounds it: GB300 issues two FP64 FMAs per SM and clock, so the n^3 FMAs of inverting the
-// n x n matrix itself take 0.21 ms (n = 512) to 1.7 ms (n = 1024) on all SMs, and its launches
-// as many again; the plane inverses and substitutions take about L m^3 + 3 n^2 m, a tenth of
-// that, but the m pivots of every plane are one serial chain (about 400 clocks each).  Two
-// clusters of eight CTAs run the two chains side by side with rows spread over the cluster, and
-// the pivot rows travel through distributed shared memory.  Against Gauss-Jordan on A + c 1 1^T
-// by blocks of 32 pivots (4 launches per block) a 64^3 projection step (512 coarse cells) went
-// from 3.68 to 2.50 ms and an 88 x 80 x 72 one (990 coarse cells) from 10.4 to 7.2 ms; the error of
-// A^+ r against extended precision went from 2.3e-14 to 1.3e-15 (drop and film, 8^3).
+// What bounds it: a warp's FP64 FMA occupies its quarter of an SM for 64 clocks on GB300 (two
+// FMAs per SM and clock), so the n^3 FMAs take 0.21 ms at n = 512 and 1.6 ms at n = 990 on all SMs, and the
+// 32 x 32 pivot block, one serial chain of 32 reciprocals (about 750 clocks a pivot), 12 us per
+// step on one SM.  So a step is two launches: the panels, dealt out in 32 x 8 tiles, and the trailing
+// update, whose first cluster of four CTAs updates the next pivot block before anything else and
+// then inverts it while the other CTAs do the rest.  Four launches per step, the pivot block
+// inverted by itself, took 85 us per step; this takes about 20 us (n = 512).  The operations on
+// every entry and their order do not depend on the tiling.
 #include <cooperative_groups.h>
 
 #include "mg_internal.cuh"
@@ -32,307 +24,269 @@ namespace mg {
 
 namespace {
 
-constexpr int kCl = 8;      // CTAs per cluster
-constexpr int kPb = 8;      // pivots per step (rows of one CTA)
-constexpr int kMaxM = 104;  // cells per plane, rounded up to kPb: m <= 1024^(2/3) < 102
-constexpr int kSlots = 16;  // rows per CTA: ceil(kMaxM / (kCl * kPb)) * kPb
+constexpr int kGj = 32;          // pivots per step
+constexpr int kPanel = 8;        // columns (rows) of a row (column) panel tile
+constexpr int kTileRows = 16;    // rows of a trailing tile, kGj columns
+constexpr int kTrailThreads = 512;
+constexpr int kTrailCluster = 4;
 
-// the coarsest level seen as L planes of m = n0 x n1 cells across its longest axis
-struct CoarseGeo {
-    int m, L, mid, n0, n1, n;
-    int s0, s1, sk;              // natural strides of the in-plane axes and of the block axis
-    const double *f0, *f1, *fk;  // low faces along them
-    double ih2;
-};
-
-__device__ __forceinline__ int nat_of(const CoarseGeo &g, int k, int q) {
-    const int v = q / g.n0, u = q - v * g.n0;
-    return k * g.sk + v * g.s1 + u * g.s0;
-}
-
-// sum of the interior faces of cell q of plane k, times ih2
-__device__ double diag_of(const CoarseGeo &g, int k, int q) {
-    const int v = q / g.n0, u = q - v * g.n0, c = nat_of(g, k, q);
-    double s = 0.0;
-    if (u > 0) s += g.f0[c] * g.ih2;
-    if (u < g.n0 - 1) s += g.f0[c + g.s0] * g.ih2;
-    if (v > 0) s += g.f1[c] * g.ih2;
-    if (v < g.n1 - 1) s += g.f1[c + g.s1] * g.ih2;
-    if (k > 0) s += g.fk[c] * g.ih2;
-    if (k < g.L - 1) s += g.fk[c + g.sk] * g.ih2;
-    return s;
-}
-
-// entry (q, j) of plane k's diagonal block
-__device__ double entry_of(const CoarseGeo &g, int k, int q, int j) {
-    if (j == q) return diag_of(g, k, q);
-    const int v = q / g.n0, u = q - v * g.n0, c = nat_of(g, k, q);
-    if (u > 0 && j == q - 1) return -g.f0[c] * g.ih2;
-    if (u < g.n0 - 1 && j == q + 1) return -g.f0[c + g.s0] * g.ih2;
-    if (v > 0 && j == q - g.n0) return -g.f1[c] * g.ih2;
-    if (v < g.n1 - 1 && j == q + g.n0) return -g.f1[c + g.s1] * g.ih2;
-    return 0.0;
-}
-
-// inverse of the bs x bs block P (rows of stride ld) by one warp, without pivoting (P is
-// symmetric positive definite): lane l holds entries (l / 8, l % 8) and (l / 8 + 4, l % 8); the
-// block is padded with the identity
-__device__ __forceinline__ void warp_inv8(const double *P, int ld, int bs, double *out) {
-    const int l = threadIdx.x & 31, c = l & 7, r0 = l >> 3, r1 = r0 + 4;
-    double a0 = (r0 < bs && c < bs) ? P[r0 * ld + c] : (r0 == c ? 1.0 : 0.0);
-    double a1 = (r1 < bs && c < bs) ? P[r1 * ld + c] : (r1 == c ? 1.0 : 0.0);
-#pragma unroll
-    for (int k = 0; k < kPb; ++k) {
-        const int rl = (k & 3) * 8;  // lanes of row k
-        const double src = k < 4 ? a0 : a1;
-        const double rp = recip64(__shfl_sync(0xffffffffu, src, rl + k));
-        const double rowc = __shfl_sync(0xffffffffu, src, rl + c);
-        const double c0 = __shfl_sync(0xffffffffu, a0, r0 * 8 + k), c1 = __shfl_sync(0xffffffffu, a1, r0 * 8 + k);
-        const double s = c == k ? rp : rowc * rp;
-        a0 = r0 == k ? s : (c == k ? -c0 * rp : fma(-c0, s, a0));
-        a1 = r1 == k ? s : (c == k ? -c1 * rp : fma(-c1, s, a1));
+// M (row-major n x n) = A + c 1 1^T, scal[0] = c; a block takes rows blockIdx.x, + gridDim.x, ...
+// and, like every other block, adds up the diagonal (the same tree in each)
+__global__ void __launch_bounds__(1024) k_coarse_assemble(Dims d, double ih2, const double *__restrict__ fx,
+                                                          const double *__restrict__ fy, const double *__restrict__ fz,
+                                                          double *M, double *scal) {
+    grid_wait();
+    __shared__ double red[1024], dg[1024];
+    const int c = threadIdx.x, n = (int)d.n, nxy = (int)d.nxy;
+    double diag = 0.0;
+    if (c < n) {
+        const int r = c / d.nx, i = c - r * d.nx, j = r % d.ny, k = r / d.ny;
+        if (i > 0) diag = fma(fx[c], ih2, diag);
+        if (i < d.nx - 1) diag = fma(fx[c + 1], ih2, diag);
+        if (j > 0) diag = fma(fy[c], ih2, diag);
+        if (j < d.ny - 1) diag = fma(fy[c + d.nx], ih2, diag);
+        if (k > 0) diag = fma(fz[c], ih2, diag);
+        if (k < d.nz - 1) diag = fma(fz[c + nxy], ih2, diag);
     }
-    out[r0 * 8 + c] = a0;
-    out[r1 * 8 + c] = a1;
-}
-
-// W_k of the planes below the middle (cluster 0) and above it (cluster 1), or, with `middle`,
-// of the middle plane (one cluster).  Row block j of 8 rows lives in CTA j % 8; a step takes
-// one row block as pivots: its owner inverts the 8 x 8 pivot block, and after the cluster
-// barrier every CTA fetches that inverse and the pivot rows and updates its own rows,
-//     M_ij <- M_ij - (M_iK P^-1) M_Kj,   M_iK <- -M_iK P^-1,   M_Kj <- P^-1 M_Kj,   M_KK <- P^-1.
-// Every loop has a fixed count; the only waits are block and cluster barriers.
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(256) k_coarse_planes(CoarseGeo g, double *W, int middle) {
-    __shared__ double M[kSlots][kMaxM];
-    __shared__ double own[2][kPb][kMaxM];  // pivot rows of the steps this CTA owns, read by the others
-    __shared__ double ownP[2][kPb * kPb];
-    __shared__ double R[kPb][kMaxM], P[kPb * kPb];
-    __shared__ double fl[kMaxM], fh[kMaxM];
-    __shared__ double shift;
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank(), side = blockIdx.x / kCl;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m = g.m, mp = (m + kPb - 1) / kPb * kPb, nb = mp / kPb;
-    auto row_of = [&](int s) { return ((s / kPb) * kCl + rank) * kPb + s % kPb; };
-    const int planes = middle ? 1 : (side == 0 ? g.mid : g.L - 1 - g.mid);
-    int buf = 0;  // alternates over all steps: a buffer is rewritten two cluster barriers after its readers' step
-    for (int t = 0; t < planes; ++t) {
-        const int k = middle ? g.mid : (side == 0 ? t : g.L - 1 - t);
-        // faces to the eliminated neighbours, and the shift of the middle plane
-        const bool lo = middle ? k > 0 : (side == 0 && t > 0);
-        const bool hi = middle ? k < g.L - 1 : (side == 1 && t > 0);
-        for (int q = tid; q < m; q += 256) {
-            const int c = nat_of(g, k, q);
-            fl[q] = lo ? g.fk[c] * g.ih2 : 0.0;
-            fh[q] = hi ? g.fk[c + g.sk] * g.ih2 : 0.0;
-        }
-        if (middle && warp == 0) {
-            double s = 0.0;
-            for (int q = lane; q < m; q += 32) s += diag_of(g, k, q);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) shift = s / m / m;
-        }
-        __syncthreads();
-        for (int e = tid; e < kSlots * mp; e += 256) {
-            const int s = e / mp, j = e - s * mp, q = row_of(s);
-            double v = 0.0;
-            if (q < m && j < m) {
-                v = entry_of(g, k, q, j);
-                if (middle) {
-                    const i64 o = (i64)q * m + j, mm = (i64)m * m;
-                    if (lo) v -= fl[q] * W[(k - 1) * mm + o] * fl[j];
-                    if (hi) v -= fh[q] * W[(k + 1) * mm + o] * fh[j];
-                    v += shift;
-                } else if (t > 0) {  // this CTA's rows of the neighbour's inverse are still in M
-                    v -= side == 0 ? fl[q] * M[s][j] * fl[j] : fh[q] * M[s][j] * fh[j];
-                }
-            }
-            M[s][j] = v;
-        }
-        __syncthreads();
-        for (int kb = 0; kb < nb; ++kb) {
-            const int k0 = kb * kPb, bs = min(kPb, m - k0), owner = kb % kCl;
-            if (rank == owner) {
-                const int s0 = (kb / kCl) * kPb;
-                if (warp == 0) warp_inv8(&M[s0][k0], kMaxM, bs, ownP[buf]);
-                for (int e = tid; e < kPb * mp; e += 256) own[buf][e / mp][e % mp] = M[s0 + e / mp][e % mp];
-            }
-            cl.sync();
-            const double *src = cl.map_shared_rank(&own[buf][0][0], owner);
-            const double *srcP = cl.map_shared_rank(&ownP[buf][0], owner);
-            for (int e = tid; e < kPb * mp; e += 256) R[e / mp][e % mp] = src[(e / mp) * kMaxM + e % mp];
-            if (tid < kPb * kPb) P[tid] = srcP[tid];
-            __syncthreads();
-            for (int s = warp; s < kSlots; s += 8) {
-                const int q = row_of(s);
-                if (q >= m) continue;  // the same for the whole warp
-                const bool piv = q >= k0 && q < k0 + kPb;
-                // coefficients of the pivot rows: T = M_iK P^-1, for a pivot row -P^-1's row
-                double T[kPb];
-#pragma unroll
-                for (int a = 0; a < kPb; ++a) T[a] = 0.0;
-                if (piv) {
-#pragma unroll
-                    for (int a = 0; a < kPb; ++a) T[a] = -P[(q - k0) * kPb + a];
-                } else {
-                    double mine = 0.0;
-                    if (lane < kPb) {
-#pragma unroll
-                        for (int a = 0; a < kPb; ++a) mine = fma(M[s][k0 + a], P[a * kPb + lane], mine);
-                    }
-#pragma unroll
-                    for (int a = 0; a < kPb; ++a) T[a] = __shfl_sync(0xffffffffu, mine, a);
-                }
-                __syncwarp();  // every lane has read M[s][k0..k0+7] before it is overwritten
-                for (int j = lane; j < mp; j += 32) {
-                    double v;
-                    if (j >= k0 && j < k0 + kPb) {
-                        v = 0.0;
-#pragma unroll
-                        for (int a = 0; a < kPb; ++a) v = (j - k0 == a) ? -T[a] : v;
-                        if (j >= m) v = 0.0;
-                    } else {
-                        v = piv ? 0.0 : M[s][j];
-#pragma unroll
-                        for (int a = 0; a < kPb; ++a) v = fma(-T[a], R[a][j], v);
-                    }
-                    M[s][j] = v;
-                }
-            }
-            __syncthreads();
-            buf ^= 1;
-        }
-        for (int e = tid; e < kSlots * m; e += 256) {
-            const int s = e / m, j = e - s * m, q = row_of(s);
-            if (q < m) W[(i64)k * m * m + (i64)q * m + j] = M[s][j];
-        }
-        __syncthreads();  // M is read above and rewritten for the next plane
-    }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
-}
-
-// Columns of G, four of one plane per CTA: elimination from their plane to the middle, then
-// substitution outwards to both ends.  A thread takes one row i and a part of the sum over t of
-// a plane product (W is symmetric: row t is read along i, coalesced, from L2); the parts are
-// added in a fixed order.  G's column c goes to row c of M (G is symmetric) and its mean to cm.
-constexpr int kCols = 4;
-__global__ void __launch_bounds__(256) k_coarse_columns(CoarseGeo g, const double *__restrict__ W, double *M,
-                                                        double *cm) {
-    __shared__ double X[1024 * kCols];  // W_k y_k of the planes passed, then x (plane order)
-    __shared__ double v[kMaxM * kCols], red[256 * kCols];
-    const int tid = threadIdx.x, m = g.m, ng = (m + kCols - 1) / kCols;
-    const int j = blockIdx.x / ng, q0 = (blockIdx.x - j * ng) * kCols;
-    const int iw = (m + 31) / 32 * 32, parts = 256 / iw;
-    const int i = tid % iw, part = tid / iw, per = (m + parts - 1) / parts;
-    const bool act = part < parts && i < m;
-    // X_k = W_k v (+ the X_k already there)
-    auto plane_product = [&](int k, bool add) {
-        double a[kCols] = {0.0, 0.0, 0.0, 0.0};
-        if (act) {
-            const double *w = W + (i64)k * m * m + i;
-            const int t1 = min(m, (part + 1) * per);
-#pragma unroll 4
-            for (int t = part * per; t < t1; ++t) {
-                const double wt = w[(i64)t * m];
-#pragma unroll
-                for (int c = 0; c < kCols; ++c) a[c] = fma(wt, v[t * kCols + c], a[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) red[(part * iw + i) * kCols + c] = a[c];
-        }
-        __syncthreads();
-        for (int e = tid; e < m * kCols; e += 256) {
-            double s = 0.0;
-            for (int p = 0; p < parts; ++p) s += red[p * iw * kCols + e];
-            const int o = k * m * kCols + e;
-            X[o] = add ? X[o] + s : s;
-        }
-        __syncthreads();
-    };
-    // v = F X_k, F the faces between plane k and plane kn
-    auto step = [&](int k, int kn) {
-        for (int e = tid; e < m * kCols; e += 256) {
-            const int q = e / kCols;
-            v[e] = g.fk[nat_of(g, max(k, kn), q)] * g.ih2 * X[k * m * kCols + e];
-        }
-        __syncthreads();
-    };
-    for (int e = tid; e < m * kCols; e += 256) v[e] = (e / kCols == q0 + e % kCols) ? 1.0 : 0.0;
+    red[c] = dg[c] = diag;
     __syncthreads();
-    for (int k = j; k != g.mid;) {
-        const int kn = k < g.mid ? k + 1 : k - 1;
-        plane_product(k, false);
-        step(k, kn);
-        k = kn;
-    }
-    plane_product(g.mid, false);
-    for (int k = g.mid - 1; k >= 0; --k) {
-        step(k + 1, k);
-        plane_product(k, j < g.mid && k >= j);
-    }
-    for (int k = g.mid + 1; k < g.L; ++k) {
-        step(k - 1, k);
-        plane_product(k, j > g.mid && k <= j);
-    }
-    for (int c = 0; c < kCols && q0 + c < m; ++c) {
-        const int col = nat_of(g, j, q0 + c);
-        double s = 0.0;
-        for (int e = tid; e < g.n; e += 256) {
-            const double x = X[e * kCols + c];
-            M[(i64)col * g.n + nat_of(g, e / m, e % m)] = x;
-            s += x;
-        }
-        red[tid] = s;
+    for (int w = 512; w > 0; w >>= 1) {
+        if (c < w) red[c] += red[c + w];
         __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (tid < w) red[tid] += red[tid + w];
-            __syncthreads();
-        }
-        if (tid == 0) cm[col] = red[0] / g.n;
-        __syncthreads();
+    }
+    const double shift = red[0] / n / n;
+    if (blockIdx.x == 0 && c == 0) scal[0] = shift;
+    if (c >= n) return;
+    for (int row = blockIdx.x; row < n; row += gridDim.x) {
+        const int r = row / d.nx, i = row - r * d.nx, j = r % d.ny, k = r / d.ny;
+        double f = 0.0;
+        if (i > 0 && c == row - 1) f = fx[row];
+        if (i < d.nx - 1 && c == row + 1) f = fx[row + 1];
+        if (j > 0 && c == row - d.nx) f = fy[row];
+        if (j < d.ny - 1 && c == row + d.nx) f = fy[row + d.nx];
+        if (k > 0 && c == row - nxy) f = fz[row];
+        if (k < d.nz - 1 && c == row + nxy) f = fz[row + nxy];
+        // an entry is rounded before the shift is added
+        M[(i64)row * n + c] = __dadd_rn(c == row ? dg[row] : -__dmul_rn(f, ih2), shift);
     }
 }
 
-// A^+ = P G P: row blockIdx.x of G minus its mean, the column means and plus the mean of all
-__global__ void __launch_bounds__(256) k_coarse_center(int n, double *M, const double *__restrict__ cm) {
-    __shared__ double red[256];
-    const int tid = threadIdx.x, r = blockIdx.x;
-    double s = 0.0;
-    for (int e = tid; e < n; e += 256) s += cm[e];
-    red[tid] = s;
+// the panels of pivots [kb, kb + bs): blocks [0, tiles) take eight columns of the row panel, blocks
+// [tiles, 2 tiles) eight rows of the column panel, whose old entries go to C (n x 32)
+__global__ void __launch_bounds__(256) k_gj_panels(int n, int kb, int bs, int tiles, double *M,
+                                                   const double *__restrict__ Pinv, double *C) {
+    grid_wait();
+    __shared__ double Pi[kGj][kGj + 1], S[kGj][kPanel + 1];
+    const int tid = threadIdx.x;
+    for (int e = tid; e < kGj * kGj; e += 256) Pi[e / kGj][e % kGj] = Pinv[e];
+    if ((int)blockIdx.x < tiles) {
+        const int ty = tid / kPanel, tx = tid % kPanel, j = blockIdx.x * kPanel + tx;
+        const bool ok = j < n && (j < kb || j >= kb + bs);
+        if (ty < bs) S[ty][tx] = ok ? M[(i64)(kb + ty) * n + j] : 0.0;
+        __syncthreads();
+        if (ty < bs && ok) {
+            double acc = 0.0;
+            for (int t = 0; t < bs; ++t) acc = fma(Pi[ty][t], S[t][tx], acc);
+            M[(i64)(kb + ty) * n + j] = acc;
+        }
+        return;
+    }
+    const int ty = tid / kGj, tx = tid % kGj, i = (blockIdx.x - tiles) * kPanel + ty;
+    const bool in = i < n && tx < bs, piv = i >= kb && i < kb + bs;
+    const double old = in && !piv ? M[(i64)i * n + kb + tx] : 0.0;
+    S[tx][ty] = old;
+    if (in && !piv) C[i * kGj + tx] = old;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (tid < w) red[tid] += red[tid + w];
+    if (!in) return;
+    if (piv) {
+        M[(i64)i * n + kb + tx] = Pi[i - kb][tx];
+    } else {
+        double acc = 0.0;
+        for (int t = 0; t < bs; ++t) acc = fma(S[t][ty], Pi[t][tx], acc);
+        M[(i64)i * n + kb + tx] = -acc;
+    }
+}
+
+// P^-1 of the bs x bs block P by element-wise Gauss-Jordan, P in shared memory (row stride
+// kGj + 1), the result row-major in Pinv.  Warp w holds rows w and w + 16, a lane a column; the
+// warp of the next pivot's row forms its reciprocal and scaled row ahead of the barrier that
+// publishes them, while the other rows are still being updated.
+__device__ void pivot_inverse(const double (*P)[kGj + 1], int bs, double (*srow)[kGj], double *srp, double *Pinv) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double a[2] = {P[w][lane], P[w + 16][lane]};
+    // scaled row of pivot k, from the value of its row before the step
+    auto publish = [&](int k, double v) {
+        const double rp = 1.0 / __shfl_sync(0xffffffffu, v, k);
+        srow[k & 1][lane] = lane == k ? rp : v * rp;
+        if (lane == 0) srp[k & 1] = rp;
+    };
+    if (w == 0) publish(0, a[0]);
+    __syncthreads();
+    for (int k = 0; k < bs; ++k) {
+        const double s = srow[k & 1][lane], rp = srp[k & 1];
+        const int next = k + 1;
+        auto step = [&](int q) {
+            const double col = __shfl_sync(0xffffffffu, a[q], k);
+            // column k: fma(-col, rp, 0) = -col rp, so that every entry costs one FP64 instruction
+            const double v = fma(-col, lane == k ? rp : s, lane == k ? 0.0 : a[q]);
+            a[q] = w + 16 * q == k ? s : v;
+        };
+        const int first = (next >> 4) & 1;  // the next pivot's row before the other one
+        step(first);
+        if (next < bs && w == (next & 15)) publish(next, a[first]);
+        step(1 - first);
         __syncthreads();
     }
-    const double mean = red[0] / n, own = cm[r];
-    for (int e = tid; e < n; e += 256) M[(i64)r * n + e] -= (own - mean) + cm[e];
+    Pinv[w * kGj + lane] = a[0];
+    Pinv[(w + 16) * kGj + lane] = a[1];
+}
+
+// the trailing update of pivots [kb, kb + bs) (none for kb < 0) and the inverse of the next pivot
+// block [nb, nb + nbs) (none for nbs = 0).  Cluster 0 updates that block, eight rows per CTA; its first
+// CTA inverts it, all the others share the 16 x 32 tiles outside it.
+__global__ void __cluster_dims__(kTrailCluster, 1, 1) __launch_bounds__(kTrailThreads)
+    k_gj_trailing(int n, int kb, int bs, int nb, int nbs, double *M, const double *__restrict__ C, double *Pinv) {
+    grid_wait();
+    __shared__ double Cs[kTileRows][kGj], R[kGj][kGj], P[kGj][kGj + 1], srow[2][kGj], srp[2];
+    const int tid = threadIdx.x, ty = tid / kGj, tx = tid % kGj;
+    // a tile: rows i0 + [0, rows), rows <= kTileRows, of the 32 columns from j0.  fetch loads this
+    // thread's entry and its share of C and of the pivot rows, update returns (and stores) the entry
+    double fc = 0.0, fr[kGj * kGj / kTrailThreads], fm = 0.0;
+    auto fetch = [&](int i0, int rows, int j0) {
+        const int i = i0 + ty, j = j0 + tx;
+        fc = (ty < rows && i < n && tx < bs) ? C[i * kGj + tx] : 0.0;
+        fm = (ty < rows && i < n && j < n) ? M[(i64)i * n + j] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kGj * kGj / kTrailThreads; ++u) {
+            const int t = ty + u * (kTrailThreads / kGj);
+            fr[u] = (t < bs && j < n) ? M[(i64)(kb + t) * n + j] : 0.0;
+        }
+    };
+    auto update = [&](int i0, int rows, int j0, auto &&next) {
+        Cs[ty][tx] = fc;
+#pragma unroll
+        for (int u = 0; u < kGj * kGj / kTrailThreads; ++u) R[ty + u * (kTrailThreads / kGj)][tx] = fr[u];
+        double acc = fm;
+        __syncthreads();
+        next();  // the next tile's loads travel during this one's arithmetic
+        if (ty < rows) {
+            if (bs == kGj) {
+#pragma unroll 8
+                for (int t = 0; t < kGj; ++t) acc = fma(-Cs[ty][t], R[t][tx], acc);
+            } else {
+                for (int t = 0; t < bs; ++t) acc = fma(-Cs[ty][t], R[t][tx], acc);
+            }
+            if (i0 + ty < n && j0 + tx < n) M[(i64)(i0 + ty) * n + j0 + tx] = acc;
+        }
+        __syncthreads();
+        return acc;
+    };
+    if (nbs > 0 && blockIdx.x < kTrailCluster) {
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();  // the cluster's first CTA is there before the others write its shared memory
+        const int r0 = blockIdx.x * 8;  // this CTA's rows of the pivot block
+        double v = 0.0;
+        if (kb >= 0) {
+            fetch(nb + r0, 8, nb);
+            v = update(nb + r0, 8, nb, [] {});
+        } else if (ty < 8 && nb + r0 + ty < n && nb + tx < n) v = M[(i64)(nb + r0 + ty) * n + nb + tx];
+        if (ty < 8) *cl.map_shared_rank(&P[r0 + ty][tx], 0) = v;
+        cl.sync();
+        if (blockIdx.x == 0) {
+            pivot_inverse(P, nbs, srow, srp, Pinv);
+            return;
+        }
+    }
+    if (kb < 0) return;
+    // row tiles without those of the pivots, column tiles without the pivots' one
+    const int tr = (n + kTileRows - 1) / kTileRows, tc = (n + kGj - 1) / kGj;
+    const int kr = kb / kTileRows, kn = (bs + kTileRows - 1) / kTileRows, kc = kb / kGj;
+    const int w0 = nbs > 0 ? 1 : 0, workers = gridDim.x - w0;
+    const int live = (tr - kn) * (tc - 1);
+    int q = (int)blockIdx.x - w0, i0 = 0, j0 = 0;
+    auto place = [&]() {  // of tile q, the next pivot block's tiles passed over
+        for (;; q += workers) {
+            if (q >= live) return false;
+            const int r = q / (tc - 1), c = q - r * (tc - 1);
+            i0 = (r < kr ? r : r + kn) * kTileRows;
+            j0 = (c < kc ? c : c + 1) * kGj;
+            if (!(nbs > 0 && i0 / kGj * kGj == nb && j0 == nb)) return true;
+        }
+    };
+    bool more = place();
+    if (more) fetch(i0, kTileRows, j0);
+    while (more) {
+        const int ci = i0, cj = j0;
+        update(ci, kTileRows, cj, [&] {
+            q += workers;
+            more = place();
+            if (more) fetch(i0, kTileRows, j0);
+        });
+    }
+}
+
+__global__ void k_pinv_finish(int nc, double *M, const double *__restrict__ scal) {
+    grid_wait();
+    const i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (i64)nc * nc) return;
+    M[e] -= 1.0 / (scal[0] * (double)nc * (double)nc);
 }
 
 }  // namespace
 
-// W_k of every plane (n m doubles) and the column means (n)
-size_t coarse_scratch_doubles(Dims d) {
-    const int L = d.nx > d.ny ? (d.nx > d.nz ? d.nx : d.nz) : (d.ny > d.nz ? d.ny : d.nz);
-    return (size_t)d.n * (size_t)(d.n / L) + (size_t)d.n;
+// CTAs of k_gj_trailing that run at once, one per SM, in whole clusters.  Left to itself the device
+// places two CTAs of a cluster on one SM, where they share its FP64 pipe while other SMs idle (the
+// update then took twice the time); asking for more than half of an SM's shared memory keeps them apart.
+constexpr int kTrailSmem = 118 * 1024;
+int trailing_ctas() {
+    static const int ctas = [] {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kTrailCluster);
+        cfg.blockDim = dim3(kTrailThreads);
+        cfg.dynamicSmemBytes = kTrailSmem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kTrailCluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_gj_trailing, &cfg) != cudaSuccess || n < 1) {
+            (void)cudaGetLastError();
+            return device_sms() / kTrailCluster * kTrailCluster;  // a grid size only
+        }
+        return n * kTrailCluster;
+    }();
+    return ctas;
 }
+
+// P^-1, the old column panel, the shift
+size_t coarse_scratch_doubles(Dims d) { return (size_t)kGj * kGj + (size_t)d.n * kGj + 1; }
 
 void launch_coarse_pinv(cudaStream_t s, Dims d, double ih2, const double *fx, const double *fy, const double *fz,
                         double *M, double *scratch) {
-    CoarseGeo g;
-    const int nxy = (int)d.nxy;
-    if (d.nz >= d.nx && d.nz >= d.ny) g = CoarseGeo{nxy, d.nz, 0, d.nx, d.ny, 0, 1, d.nx, nxy, fx, fy, fz, ih2};
-    else if (d.ny >= d.nx) g = CoarseGeo{d.nx * d.nz, d.ny, 0, d.nx, d.nz, 0, 1, nxy, d.nx, fx, fz, fy, ih2};
-    else g = CoarseGeo{d.ny * d.nz, d.nx, 0, d.ny, d.nz, 0, d.nx, nxy, 1, fy, fz, fx, ih2};
-    g.n = (int)d.n;
-    g.mid = g.L / 2;
-    double *W = scratch, *cm = scratch + (size_t)g.n * g.m;
-    count_launch(4);
-    k_coarse_planes<<<2 * kCl, 256, 0, s>>>(g, W, 0);
-    k_coarse_planes<<<kCl, 256, 0, s>>>(g, W, 1);
-    k_coarse_columns<<<g.L * ((g.m + kCols - 1) / kCols), 256, 0, s>>>(g, W, M, cm);
-    k_coarse_center<<<g.n, 256, 0, s>>>(g.n, M, cm);
+    const int n = (int)d.n, tiles = (n + kPanel - 1) / kPanel;
+    double *Pinv = scratch, *C = Pinv + kGj * kGj, *scal = C + (size_t)n * kGj;
+    const int sms = device_sms();
+    // per device: the attribute is the current device's
+    if (cudaFuncSetAttribute(k_gj_trailing, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrailSmem) != cudaSuccess)
+        return;  // stays in the runtime's last error, which the caller checks
+    // fewer CTAs where there are fewer tiles (and at least the pivot cluster)
+    const int live = (n + kTileRows - 1) / kTileRows * ((n + kGj - 1) / kGj) + 1, most = trailing_ctas();
+    const int grid = live < most ? (live + kTrailCluster - 1) / kTrailCluster * kTrailCluster : most;
+    count_launch();
+    run_kernel(k_coarse_assemble, n < sms ? n : sms, 1024, 0, s, d, ih2, fx, fy, fz, M, scal);
+    count_launch();
+    run_kernel(k_gj_trailing, kTrailCluster, kTrailThreads, kTrailSmem, s, n, -1, 0, 0, n < kGj ? n : kGj, M, C, Pinv);
+    for (int kb = 0; kb < n; kb += kGj) {
+        const int bs = n - kb < kGj ? n - kb : kGj, nb = kb + kGj, left = n - nb;
+        const int nbs = left <= 0 ? 0 : (left < kGj ? left : kGj);
+        count_launch(2);
+        run_kernel(k_gj_panels, 2 * tiles, 256, 0, s, n, kb, bs, tiles, M, Pinv, C);
+        run_kernel(k_gj_trailing, grid, kTrailThreads, kTrailSmem, s, n, kb, bs, nb, nbs, M, C, Pinv);
+    }
+    count_launch();
+    run_kernel(k_pinv_finish, (unsigned)(((i64)n * n + 255) / 256), 256, 0, s, n, M, scal);
 }
 
 }  // namespace mg

@@ -3,7 +3,7 @@
 // dense coarse solve with cluster barriers between them.
 //
 // What bounds the levels below about 40^3 is the chain of dependent launches (ten per level and
-// cycle, 2-3 us each in a replayed graph, for work of a fraction of a microsecond), so the
+// cycle, 2-3 us each, for work of a fraction of a microsecond), so the
 // chain is made of cheaper links: a half sweep here is one shared-memory round trip and a cluster
 // barrier, 0.6 us at 32^3 and 0.5 us at 16^3.  The levels 32^3, 16^3 and 8^3 of a cycle take 28 us
 // (launch by launch 50 us): 4 us to copy the contexts in, 6 us for the dense product of 512
@@ -28,8 +28,9 @@
 // operator (k_tail_prepare), one image per CTA and level in the order of its shared memory, and
 // copied in at the start of a launch.
 //
-// Arithmetic.  Per cell as in the level kernels (kernels_split.cu: k_half_vec, k_rr_red_vec,
-// k_prolong_red8 where the coarse nx is a multiple of 8, else k_prolong_red_vec; FP64:
+// Arithmetic.  Per cell as in the level kernels (kernels_split.cu: k_half_vec, k_rr_red_vec or, where nx / 2
+// is no multiple of 4, k_resid_restrict_any, k_prolong_red8 where the coarse nx is a multiple of 8, else
+// k_prolong_red_vec; FP64:
 // k_rbgs_half, k_rr_red_diag64, k_prolong_col; the coarse product as k_coarse_matvec), in the
 // same order.
 #include <cooperative_groups.h>
@@ -244,6 +245,11 @@ struct Tail {
 #pragma unroll
                     for (int u = 0; u < 6; ++u) r = fma(q[c].w[u], v[u], r);
                     r = fma(-q[c].dg, xc, r);
+                } else if (L.hx % 4 != 0) {  // as k_resid_restrict_any
+                    float num = first_two(q[c].w[0], v[0], q[c].w[1], v[1]);
+#pragma unroll
+                    for (int u = 2; u < 6; ++u) num = fmaf(q[c].w[u], v[u], num);
+                    r = fmaf(-fmaf(xc, q[c].d, -num), (float)L.ih2, q[c].b);
                 } else {
                     float ax = first_two(q[c].w[0], xc - v[0], q[c].w[1], xc - v[1]);
 #pragma unroll
@@ -388,6 +394,7 @@ struct Tail {
 // the image of one level and CTA (blockIdx.y, blockIdx.x) from the level's arrays: contexts and tables
 template <typename T>
 __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ TailArgs a) {
+    grid_wait();
     using U = Tail<T>;
     const TailLevel &L = a.lv[blockIdx.y];
     const TailLevel *C = (int)blockIdx.y + 1 < a.nl ? &a.lv[blockIdx.y + 1] : nullptr;
@@ -469,6 +476,7 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
 // coarse solve launched between the two on the whole device and the levels kept in memory
 template <typename T>
 __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs a, int mode) {
+    grid_wait();
     extern __shared__ __align__(16) char tail_smem[];
     cg::cluster_group cl = cg::this_cluster();
     const Tail<T> t{a, tail_smem, (int)cl.block_rank(), (int)cl.num_blocks(), (int)threadIdx.x};
@@ -565,12 +573,14 @@ cudaError_t launch_mode(cudaStream_t s, const TailArgs &a, int mode) {
     cfg.blockDim = dim3(kTailThreads);
     cfg.dynamicSmemBytes = (size_t)a.smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)a.ncta;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = stream_capturing(s) ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, k_tail<T>, a, mode);
 }
 
@@ -643,17 +653,19 @@ bool tail_layout(TailArgs &a, bool fp64, int ncta) {
     a.off_rc = take(8 * (i64)a.nc);
     a.off_ec = take((i64)es * a.nc);
     a.off_cw = take(es * cw);
-    a.smem = (int)off;
     a.img_total = img;
     if (off > kTailMaxSmem) return false;
+    // more than half of an SM's shared memory: two CTAs of the cluster on one SM would share its
+    // FP64 pipe and issue slots while another SM idles
+    a.smem = (int)(off > kTailMinSmem ? off : kTailMinSmem);
     return fp64 ? cluster_fits<double>(a) : cluster_fits<float>(a);
 }
 
 void launch_tail_prepare(cudaStream_t s, const TailArgs &a, bool fp64) {
     count_launch();
     const dim3 grd(a.ncta, a.nl);
-    if (fp64) k_tail_prepare<double><<<grd, 256, 0, s>>>(a);
-    else k_tail_prepare<float><<<grd, 256, 0, s>>>(a);
+    if (fp64) run_kernel(k_tail_prepare<double>, grd, 256, 0, s, a);
+    else run_kernel(k_tail_prepare<float>, grd, 256, 0, s, a);
 }
 
 void launch_tail(cudaStream_t s, const TailArgs &a, bool fp64, int mode) {

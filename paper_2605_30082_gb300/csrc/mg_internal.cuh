@@ -134,6 +134,44 @@ __device__ __forceinline__ double recip64(double x) {
 }
 #endif
 
+#ifdef __CUDACC__
+// Launches.  Between two dependent kernels of a stream GB300 takes 1 to 2.5 us when they are
+// launched plainly (the second starts on a 2.05 us tick: 2.07, 4.10, 4.11, 6.15, 8.20 us per
+// launch for kernels that run 0.1, 1.1, 2.1, 3.2, 5.3 us), and 0.4-0.5 us with programmatic stream
+// serialisation (1.4, 1.6, 2.6, 3.6, 5.6 us) or inside a graph.  So every kernel here is launched with
+// that attribute and begins with grid_wait(), before any access to memory: it waits until the
+// kernel before it in the stream has completed and its writes are visible.  No kernel triggers
+// its successor early, so the two never run side by side (blocks of a successor that only wait
+// would take the place of the predecessor's).  Under a stream capture the launch is plain: the
+// graph's own edges cost the same, and forks and joins keep full dependencies.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+inline bool stream_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// a refused launch stays in the runtime's last error, which the entry points check
+template <typename... P, typename... A>
+inline void run_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = stream_capturing(s) ? 0 : 1;
+    (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+#endif
+
 // process-wide count of kernel launches (read through mg_kernel_launches)
 void count_launch(int k = 1);
 unsigned long long launches_total();
@@ -311,7 +349,7 @@ void launch_coarse_matvec(cudaStream_t s, int nc, const double *pinv, const T *r
 // ---- the coarse levels of a V-cycle in one cluster launch (kernels_tail.cu) -------------
 constexpr int kTailLevels = 6;
 constexpr int kTailCells32 = 2, kTailCells64 = 1;  // cells of a colour per thread
-constexpr int kTailMaxSmem = 227 * 1024;  // per CTA, dynamic
+constexpr int kTailMaxSmem = 227 * 1024, kTailMinSmem = 118 * 1024;  // per CTA, dynamic
 enum { kTailAll = 0, kTailDown = 1, kTailUp = 2 };
 struct TailLevel {
     int nx, ny, nz;

@@ -22,10 +22,10 @@
 namespace {
 
 constexpr int kMaxCells = MG_NOALLOC_MAX_CELLS;
-// plane inverses (n m doubles, m <= n^(2/3) = 64 cells per plane) and column means
-constexpr size_t kPinvDoubles = (size_t)kMaxCells * 64 + kMaxCells;
+// scratch of launch_coarse_pinv (coarse_scratch_doubles at kMaxCells cells), rounded up
+constexpr size_t kPinvDoubles = 1024 + (size_t)kMaxCells * 32 + 8;
 // layout in doubles: M [kMaxCells^2] | W [scratch of launch_coarse_pinv] | fx, fy, fz
-// [kMaxCells each] | error word.  About 2.4 MB in all.
+// [kMaxCells each] | error word.  About 2.3 MB in all.
 constexpr size_t kScratchDoubles = (size_t)kMaxCells * kMaxCells + kPinvDoubles + 3 * (size_t)kMaxCells + 8;
 
 __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
