@@ -143,10 +143,9 @@ void mg_default_opts(mg_opts *opts);
  * handle will use (hierarchy, scratch, coarse inverse) and a small mapped
  * pinned host buffer (cudaHostAllocMapped) into which kernels store the
  * scalars the host waits for, so that those waits never queue behind copies
- * other streams run on the copy engines: nothing is allocated later.  It also records the levels below the finest of one V-cycle as a
- * CUDA graph (on a private stream; nothing runs), which every cycle replays;
- * where recording is refused the cycles launch those kernels one by one.  On failure *out is NULL and the code says why (MG_ERR_ARG: opts;
- * MG_ERR_OOM; MG_ERR_CUDA). */
+ * other streams run on the copy engines: nothing is allocated later.  On
+ * failure *out is NULL and the code says why (MG_ERR_ARG: opts; MG_ERR_OOM;
+ * MG_ERR_CUDA). */
 int mg_create(const mg_opts *opts, void *stream, mg_handle **out);
 
 /* Free the handle and all its device memory (synchronises its stream). NULL is a no-op. */
@@ -306,7 +305,7 @@ enum {
     MG_PROF_PROJECT = 7,        /* velocity correction (mg_project) */
     MG_PROF_DENSITY_GRAD = 8,   /* density adjoint (mg_density_grads) */
     MG_PROF_COARSE_LEVELS = 9,  /* the V-cycle below the finest level: one interval per V-cycle
-                                   (the replayed graph of its launches, or the launches) */
+                                   (its launches) */
     MG_PROF_SETUP = 10,         /* operator set-up: one interval per mg_set_density /
                                    mg_set_face_coeffs (faces, coarsening, packs, coarse inverse) */
     MG_PROF_RHS = 11,           /* right-hand side (mg_rhs) */
@@ -427,7 +426,7 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *stats);
  * call builds the dense pseudo-inverse from scratch and applies it; it needs
  * no handle and calls no cudaMalloc, cudaFree or other allocating routine.
  * Working memory is one fixed array in this library's device image (about
- * 2.4 MB, held on every GPU that loads the library until the process exits),
+ * 2.3 MB, held on every GPU that loads the library until the process exits),
  * so nx*ny*nz must be at most MG_NOALLOC_MAX_CELLS (MG_ERR_ARG otherwise).
  * The first call on each device looks up that array's device address (with
  * that device current); make it before any stream capture.  Every call uses

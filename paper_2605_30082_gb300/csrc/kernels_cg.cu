@@ -49,6 +49,7 @@ __device__ __forceinline__ void block_sum_pair(double a, double b, double *parti
 
 // sc[slot_a] = sum of partials[2 q], sc[slot_b] = sum of partials[2 q + 1] (slot_b < 0: unused)
 __global__ void k_cg_final(const double *__restrict__ partials, int nb, double *sc, int slot_a, int slot_b) {
+    grid_wait();
     __shared__ double sa[256], sb[256];
     double a = 0.0, b = 0.0;
     for (int q = threadIdx.x; q < nb; q += blockDim.x) {
@@ -83,6 +84,7 @@ struct Coef32c {
 // same row and k in the rows y +- 1, z +- 1.
 template <bool SFORM>
 __global__ void k_cg_apply32(Lay L, float ih2, Coef32c cf, const float *__restrict__ d, float *q, double *partials) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const i64 rows = (i64)L.ny * L.nz;
     const i64 per_col = rows * kv;
@@ -179,6 +181,7 @@ __global__ void k_cg_apply32(Lay L, float ih2, Coef32c cf, const float *__restri
 // partial sums of (r . z, z . q), 4 floats per thread step
 __global__ void k_cg_dots32(i64 n4, const float4 *__restrict__ r, const float4 *__restrict__ z,
                             const float4 *__restrict__ q, double *partials) {
+    grid_wait();
     double a = 0.0, b = 0.0;
     for (i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x; m < n4; m += (i64)gridDim.x * blockDim.x) {
         const float4 rv = r[m], zv = z[m], qv = q[m];
@@ -191,6 +194,7 @@ __global__ void k_cg_dots32(i64 n4, const float4 *__restrict__ r, const float4 *
 // d = z + beta d with beta = -alpha (z . q_prev) / (r_prev . z_prev); first: d = z
 __global__ void k_cg_dir32(i64 n4, const float4 *__restrict__ z, float4 *dv, const double *__restrict__ sc,
                            int first, int rz_prev) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n4) return;
     const float4 zv = z[m];
@@ -210,6 +214,7 @@ __global__ void k_cg_dir32(i64 n4, const float4 *__restrict__ z, float4 *dv, con
 // alpha = (r . z) / (d . A d); x += alpha d, r -= alpha A d; the first thread records alpha
 __global__ void k_cg_update32(i64 n4, float4 *x, float4 *r, const float4 *__restrict__ dv,
                               const float4 *__restrict__ q, double *sc, int rz_cur) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const double alpha_d = sc[rz_cur] / sc[CG_PQ];
     if (m == 0) sc[CG_ALPHA] = alpha_d;
@@ -234,6 +239,7 @@ __global__ void k_cg_update32(i64 n4, float4 *x, float4 *r, const float4 *__rest
 __global__ void k_cg_apply64(Dims dm, double ih2, const double *__restrict__ fx, const double *__restrict__ fy,
                              const double *__restrict__ fz, const double *__restrict__ dg,
                              const double *__restrict__ d, double *q, double *partials) {
+    grid_wait();
     double acc = 0.0;
     const int nx = dm.nx, ny = dm.ny, nz = dm.nz;
     const i64 nxy = dm.nxy, rows = (i64)ny * nz;
@@ -258,6 +264,7 @@ __global__ void k_cg_apply64(Dims dm, double ih2, const double *__restrict__ fx,
 
 __global__ void k_cg_dots64(i64 n, const double *__restrict__ r, const double *__restrict__ z,
                             const double *__restrict__ q, double *partials) {
+    grid_wait();
     double a = 0.0, b = 0.0;
     for (i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (i64)gridDim.x * blockDim.x) {
         const double zv = z[m];
@@ -269,6 +276,7 @@ __global__ void k_cg_dots64(i64 n, const double *__restrict__ r, const double *_
 
 __global__ void k_cg_dir64(i64 n, const double *__restrict__ z, double *dv, const double *__restrict__ sc,
                            int first, int rz_prev) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     if (first) {
@@ -282,6 +290,7 @@ __global__ void k_cg_dir64(i64 n, const double *__restrict__ z, double *dv, cons
 // alpha = (r . z) / (d . A d); x += alpha d, r -= alpha A d; partials of |r|^2 (and of sum x)
 __global__ void k_cg_update64(i64 n, double *x, double *r, const double *__restrict__ dv,
                               const double *__restrict__ q, double *sc, int rz_cur, double *partials) {
+    grid_wait();
     const double alpha = sc[rz_cur] / sc[CG_PQ];
     if (blockIdx.x == 0 && threadIdx.x == 0) sc[CG_ALPHA] = alpha;
     double rr = 0.0, sx = 0.0;
@@ -307,9 +316,9 @@ void launch_cg_apply32(cudaStream_t s, Lay L, double ih2, const float *sinv, con
     static const int wave_n = wave_blocks((const void *)k_cg_apply32<false>, kThreads);
     const int nb = fill_blocks(reduce_blocks(L.n / 4), sinv ? wave_s : wave_n);
     count_launch(2);
-    if (sinv) k_cg_apply32<true><<<nb, kThreads, 0, s>>>(L, (float)ih2, cf, d, q, partials);
-    else k_cg_apply32<false><<<nb, kThreads, 0, s>>>(L, (float)ih2, cf, d, q, partials);
-    k_cg_final<<<1, 256, 0, s>>>(partials, nb, sc, CG_PQ, -1);
+    if (sinv) run_kernel(k_cg_apply32<true>, nb, kThreads, 0, s, L, (float)ih2, cf, d, q, partials);
+    else run_kernel(k_cg_apply32<false>, nb, kThreads, 0, s, L, (float)ih2, cf, d, q, partials);
+    run_kernel(k_cg_final, 1, 256, 0, s, partials, nb, sc, CG_PQ, -1);
 }
 
 void launch_cg_dots32(cudaStream_t s, i64 n, const float *r, const float *z, const float *q, double *partials,
@@ -317,22 +326,22 @@ void launch_cg_dots32(cudaStream_t s, i64 n, const float *r, const float *z, con
     static const int wave = wave_blocks((const void *)k_cg_dots32, kThreads);
     const int nb = fill_blocks(reduce_blocks(n / 4), wave);
     count_launch(2);
-    k_cg_dots32<<<nb, kThreads, 0, s>>>(n / 4, reinterpret_cast<const float4 *>(r),
+    run_kernel(k_cg_dots32, nb, kThreads, 0, s, n / 4, reinterpret_cast<const float4 *>(r),
                                         reinterpret_cast<const float4 *>(z), reinterpret_cast<const float4 *>(q),
                                         partials);
-    k_cg_final<<<1, 256, 0, s>>>(partials, nb, sc, rz_slot, CG_ZQ);
+    run_kernel(k_cg_final, 1, 256, 0, s, partials, nb, sc, rz_slot, CG_ZQ);
 }
 
 void launch_cg_dir32(cudaStream_t s, i64 n, const float *z, float *d, const double *sc, bool first, int rz_prev) {
     count_launch();
-    k_cg_dir32<<<blocks_for(n / 4), kThreads, 0, s>>>(n / 4, reinterpret_cast<const float4 *>(z),
+    run_kernel(k_cg_dir32, blocks_for(n / 4), kThreads, 0, s, n / 4, reinterpret_cast<const float4 *>(z),
                                                       reinterpret_cast<float4 *>(d), sc, first ? 1 : 0, rz_prev);
 }
 
 void launch_cg_update32(cudaStream_t s, i64 n, float *x, float *r, const float *d, const float *q, double *sc,
                         int rz_cur) {
     count_launch();
-    k_cg_update32<<<blocks_for(n / 4), kThreads, 0, s>>>(n / 4, reinterpret_cast<float4 *>(x),
+    run_kernel(k_cg_update32, blocks_for(n / 4), kThreads, 0, s, n / 4, reinterpret_cast<float4 *>(x),
                                                          reinterpret_cast<float4 *>(r),
                                                          reinterpret_cast<const float4 *>(d),
                                                          reinterpret_cast<const float4 *>(q), sc, rz_cur);
@@ -345,21 +354,21 @@ void launch_cg_apply64(cudaStream_t s, Dims d, double ih2, const double *fx, con
     int nb = fill_blocks(reduce_blocks(d.n), wave);
     if (nb > rows) nb = (int)rows;
     count_launch(2);
-    k_cg_apply64<<<nb, kThreads, 0, s>>>(d, ih2, fx, fy, fz, dg, dv, q, partials);
-    k_cg_final<<<1, 256, 0, s>>>(partials, nb, sc, CG_PQ, -1);
+    run_kernel(k_cg_apply64, nb, kThreads, 0, s, d, ih2, fx, fy, fz, dg, dv, q, partials);
+    run_kernel(k_cg_final, 1, 256, 0, s, partials, nb, sc, CG_PQ, -1);
 }
 
 void launch_cg_dots64(cudaStream_t s, i64 n, const double *r, const double *z, const double *q, double *partials,
                       double *sc, int rz_slot) {
     const int nb = reduce_blocks(n);
     count_launch(2);
-    k_cg_dots64<<<nb, kThreads, 0, s>>>(n, r, z, q, partials);
-    k_cg_final<<<1, 256, 0, s>>>(partials, nb, sc, rz_slot, CG_ZQ);
+    run_kernel(k_cg_dots64, nb, kThreads, 0, s, n, r, z, q, partials);
+    run_kernel(k_cg_final, 1, 256, 0, s, partials, nb, sc, rz_slot, CG_ZQ);
 }
 
 void launch_cg_dir64(cudaStream_t s, i64 n, const double *z, double *d, const double *sc, bool first, int rz_prev) {
     count_launch();
-    k_cg_dir64<<<blocks_for(n), kThreads, 0, s>>>(n, z, d, sc, first ? 1 : 0, rz_prev);
+    run_kernel(k_cg_dir64, blocks_for(n), kThreads, 0, s, n, z, d, sc, first ? 1 : 0, rz_prev);
 }
 
 void launch_cg_update64(cudaStream_t s, i64 n, double *x, double *r, const double *d, const double *q, double *sc,
@@ -367,8 +376,8 @@ void launch_cg_update64(cudaStream_t s, i64 n, double *x, double *r, const doubl
     static const int wave = wave_blocks((const void *)k_cg_update64, kThreads);
     const int nb = fill_blocks(reduce_blocks(n), wave);
     count_launch(2);
-    k_cg_update64<<<nb, kThreads, 0, s>>>(n, x, r, d, q, sc, rz_cur, partials);
-    k_cg_final<<<1, 256, 0, s>>>(partials, nb, sc, CG_RR, CG_SX);
+    run_kernel(k_cg_update64, nb, kThreads, 0, s, n, x, r, d, q, sc, rz_cur, partials);
+    run_kernel(k_cg_final, 1, 256, 0, s, partials, nb, sc, CG_RR, CG_SX);
 }
 
 }  // namespace mg

@@ -62,6 +62,7 @@ __device__ __forceinline__ T flux_sum(const Dims &d, int i, int j, int k, i64 c,
 // FP64 arithmetic rather than bytes, so it keeps zero redundant work
 template <typename T>
 __global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T *x, int colour) {
+    grid_wait();
     const int half = (d.nx + 1) >> 1;
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 rows = (i64)d.ny * d.nz;
@@ -79,6 +80,7 @@ __global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T
 
 template <typename T>
 __global__ void k_apply(Dims d, T ih2, Coef<T> cf, const T *__restrict__ x, T *y) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     int i, j, k;
@@ -89,6 +91,7 @@ __global__ void k_apply(Dims d, T ih2, Coef<T> cf, const T *__restrict__ x, T *y
 template <typename T>
 __global__ void k_residual(Dims d, T ih2, Coef<T> cf, const T *__restrict__ b,
                            const T *__restrict__ x, T *r) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     int i, j, k;
@@ -101,6 +104,7 @@ __global__ void k_residual(Dims d, T ih2, Coef<T> cf, const T *__restrict__ b,
 template <typename T>
 __global__ void k_resid_restrict(Dims f, Dims cd, T ih2, Coef<T> cf, const T *__restrict__ b,
                                  const T *__restrict__ x, T *bc, int red_only) {
+    grid_wait();
     i64 C = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (C >= cd.n) return;
     int I, J, K;
@@ -120,6 +124,7 @@ __global__ void k_resid_restrict(Dims f, Dims cd, T ih2, Coef<T> cf, const T *__
 // e += P ec on the cells of colour only_col (0 red, 1 black) or on all cells (-1)
 template <typename T>
 __global__ void k_prolong(Dims cd, Dims f, const T *__restrict__ ec, T *e, int kind, int only_col) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= f.n) return;
     int i, j, k;
@@ -158,6 +163,7 @@ __global__ void k_prolong(Dims cd, Dims f, const T *__restrict__ ec, T *e, int k
 __global__ void k_rr_red_diag64(Dims f, Dims cd, double h2, double ih2_8, Coef<double> cf,
                                 const double *__restrict__ dg, const double *__restrict__ b,
                                 const double *__restrict__ x, double *bc) {
+    grid_wait();
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= cd.nx) return;
     const i64 crows = (i64)cd.ny * cd.nz;
@@ -186,6 +192,7 @@ __global__ void k_rr_red_diag64(Dims f, Dims cd, double h2, double ih2_8, Coef<d
 // (grid x), blocks strided rows (grid y)
 template <typename T>
 __global__ void k_prolong_col(Dims cd, Dims f, const T *__restrict__ ec, T *e, int kind, int col) {
+    grid_wait();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const i64 rows = (i64)f.ny * f.nz;
     for (i64 row = blockIdx.y; row < rows; row += gridDim.y) {
@@ -221,6 +228,7 @@ __global__ void k_prolong_col(Dims cd, Dims f, const T *__restrict__ ec, T *e, i
 template <typename T>
 __global__ void k_coarse_matvec(int nc, const double *__restrict__ pinv, const T *__restrict__ r,
                                 T *e) {
+    grid_wait();
     int row = (int)(((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     int lane = threadIdx.x & 31;
     if (row >= nc) return;
@@ -238,19 +246,19 @@ void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const
                         int colour) {
     const i64 work = (i64)d.ny * d.nz * ((d.nx + 1) / 2);
     count_launch();
-    k_rbgs_half<double><<<blocks_for(work), kThreads, 0, s>>>(d, h2, c, b, p, colour);
+    run_kernel(k_rbgs_half<double>, blocks_for(work), kThreads, 0, s, d, h2, c, b, p, colour);
 }
 
 template <typename T>
 void launch_apply(cudaStream_t s, Dims d, double ih2, Coef<T> c, const T *x, T *y) {
     count_launch();
-    k_apply<T><<<blocks_for(d.n), kThreads, 0, s>>>(d, (T)ih2, c, x, y);
+    run_kernel(k_apply<T>, blocks_for(d.n), kThreads, 0, s, d, (T)ih2, c, x, y);
 }
 
 template <typename T>
 void launch_residual(cudaStream_t s, Dims d, double ih2, Coef<T> c, const T *b, const T *x, T *r) {
     count_launch();
-    k_residual<T><<<blocks_for(d.n), kThreads, 0, s>>>(d, (T)ih2, c, b, x, r);
+    run_kernel(k_residual<T>, blocks_for(d.n), kThreads, 0, s, d, (T)ih2, c, b, x, r);
 }
 
 template <typename T>
@@ -258,7 +266,7 @@ void launch_resid_restrict(cudaStream_t s, Dims fine, double ih2, Coef<T> c, con
                            const T *x, T *bc, bool red_only) {
     Dims cd = make_dims(fine.nx / 2, fine.ny / 2, fine.nz / 2);
     count_launch();
-    k_resid_restrict<T><<<blocks_for(cd.n), kThreads, 0, s>>>(fine, cd, (T)ih2, c, b, x, bc, red_only ? 1 : 0);
+    run_kernel(k_resid_restrict<T>, blocks_for(cd.n), kThreads, 0, s, fine, cd, (T)ih2, c, b, x, bc, red_only ? 1 : 0);
 }
 
 template <typename T>
@@ -269,10 +277,10 @@ void launch_prolong(cudaStream_t s, Dims coarse, const T *ec, T *e, int kind, in
         const unsigned gx = (unsigned)(((f.nx + 1) / 2 + 127) / 128);
         const i64 rows = (i64)f.ny * f.nz;
         const unsigned gy = (unsigned)(rows < 65535 ? rows : 65535);
-        k_prolong_col<T><<<dim3(gx, gy), 128, 0, s>>>(coarse, f, ec, e, kind, only_col);
+        run_kernel(k_prolong_col<T>, dim3(gx, gy), 128, 0, s, coarse, f, ec, e, kind, only_col);
         return;
     }
-    k_prolong<T><<<blocks_for(f.n), kThreads, 0, s>>>(coarse, f, ec, e, kind, only_col);
+    run_kernel(k_prolong<T>, blocks_for(f.n), kThreads, 0, s, coarse, f, ec, e, kind, only_col);
 }
 
 void launch_rr_red_diag64(cudaStream_t s, Dims fine, double h2, Coef<double> c, const double *dg,
@@ -282,14 +290,14 @@ void launch_rr_red_diag64(cudaStream_t s, Dims fine, double h2, Coef<double> c, 
     const unsigned gx = (unsigned)((cd.nx + 127) / 128);
     const i64 crows = (i64)cd.ny * cd.nz;
     const unsigned gy = (unsigned)(crows < 65535 ? crows : 65535);
-    k_rr_red_diag64<<<dim3(gx, gy), 128, 0, s>>>(fine, cd, h2, 1.0 / (8.0 * h2), c, dg, b, x, bc);
+    run_kernel(k_rr_red_diag64, dim3(gx, gy), 128, 0, s, fine, cd, h2, 1.0 / (8.0 * h2), c, dg, b, x, bc);
 }
 
 template <typename T>
 void launch_coarse_matvec(cudaStream_t s, int nc, const double *pinv, const T *r, T *e) {
     i64 threads = (i64)nc * 32;
     count_launch();
-    k_coarse_matvec<T><<<blocks_for(threads), kThreads, 0, s>>>(nc, pinv, r, e);
+    run_kernel(k_coarse_matvec<T>, blocks_for(threads), kThreads, 0, s, nc, pinv, r, e);
 }
 
 #define MG_INSTANTIATE(T)                                                                        \

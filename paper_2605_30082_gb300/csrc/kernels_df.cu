@@ -40,6 +40,7 @@ __device__ __forceinline__ void df_fma(float &ah, float &al, float xh, float xl,
 __device__ __forceinline__ float df_value(float h, float l) { return h + l; }
 
 __global__ void k_split(i64 n, const double *__restrict__ src, float2 *dst) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     const double v = src[m];
@@ -48,6 +49,7 @@ __global__ void k_split(i64 n, const double *__restrict__ src, float2 *dst) {
 }
 
 __global__ void k_join(i64 n, const float2 *__restrict__ src, double *dst) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     const float2 v = src[m];
@@ -61,6 +63,7 @@ __global__ void k_resid_df(Dims d, Lay L, const float2 *__restrict__ fx, const f
                            const float2 *__restrict__ fz, const float2 *__restrict__ dg,
                            const float2 *__restrict__ b, const float2 *__restrict__ p, float *r32, float s32,
                            double *partials) {
+    grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz, hx = nx >> 1;
     const int nxy = nx * ny;
@@ -152,6 +155,7 @@ __global__ void k_resid_df(Dims d, Lay L, const float2 *__restrict__ fx, const f
 }
 
 __global__ void k_final_df(const double *__restrict__ partials, int nb, double *out) {
+    grid_wait();
     __shared__ double sa[256], sb[256];
     double a = 0.0, b = 0.0;
     for (int q = threadIdx.x; q < nb; q += blockDim.x) {
@@ -217,6 +221,7 @@ constexpr int kDfsThreads = 128;
 __global__ void __launch_bounds__(kDfsThreads, 6)
     k_resid_dfs(Dims d, Lay L, const float2 *__restrict__ s2, const float2 *__restrict__ b, const float2 *__restrict__ p,
                 float *r32, float s32, double *partials, int tiles_x, int tiles_y, i64 ntiles) {
+    grid_wait();
     const int nx = d.nx, ny = d.ny, nz = d.nz, hx = nx >> 1;
     const i64 nxy = d.nxy;
     const int vb = blockDim.x, lane = threadIdx.x & 31;
@@ -356,6 +361,7 @@ __device__ __forceinline__ i64 sto(const Lay &L, int x, int y, int z) {
 
 // p = p + (alpha e - shift) in double-float (e in the level-0 FP32 layout)
 __global__ void k_update_df(Dims d, Lay L, float2 *p, const float *__restrict__ e, float alpha, float shift) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= d.n) return;
     const int i = (int)(m % d.nx);
@@ -373,12 +379,12 @@ __global__ void k_update_df(Dims d, Lay L, float2 *p, const float *__restrict__ 
 
 void launch_split(cudaStream_t s, i64 n, const double *src, float2 *dst) {
     count_launch();
-    k_split<<<blocks_for(n), kThreads, 0, s>>>(n, src, dst);
+    run_kernel(k_split, blocks_for(n), kThreads, 0, s, n, src, dst);
 }
 
 void launch_join(cudaStream_t s, i64 n, const float2 *src, double *dst) {
     count_launch();
-    k_join<<<blocks_for(n), kThreads, 0, s>>>(n, src, dst);
+    run_kernel(k_join, blocks_for(n), kThreads, 0, s, n, src, dst);
 }
 
 void launch_resid_df(cudaStream_t s, Dims d, Lay L, const float2 *fx, const float2 *fy, const float2 *fz,
@@ -387,9 +393,9 @@ void launch_resid_df(cudaStream_t s, Dims d, Lay L, const float2 *fx, const floa
     static const int wave = wave_blocks((const void *)k_resid_df, kReduceThreads);
     const int nb = fill_blocks(reduce_blocks(d.n / 2), wave);
     count_launch();
-    k_resid_df<<<nb, kReduceThreads, 0, s>>>(d, L, fx, fy, fz, diag, b, p, r32, s32, partials);
+    run_kernel(k_resid_df, nb, kReduceThreads, 0, s, d, L, fx, fy, fz, diag, b, p, r32, s32, partials);
     count_launch();
-    k_final_df<<<1, 256, 0, s>>>(partials, nb, out);
+    run_kernel(k_final_df, 1, 256, 0, s, partials, nb, out);
 }
 
 void launch_resid_dfs(cudaStream_t s, Dims d, Lay L, const float2 *s2, const float2 *b, const float2 *p,
@@ -403,14 +409,14 @@ void launch_resid_dfs(cudaStream_t s, Dims d, Lay L, const float2 *s2, const flo
     if (nb > ntiles) nb = ntiles;
     if (nb > reduce_blocks(d.n)) nb = reduce_blocks(d.n);  // the partials buffer holds reduce_blocks(n) pairs
     count_launch();
-    k_resid_dfs<<<(unsigned)nb, blk, 0, s>>>(d, L, s2, b, p, r32, s32, partials, tiles_x, tiles_y, ntiles);
+    run_kernel(k_resid_dfs, (unsigned)nb, blk, 0, s, d, L, s2, b, p, r32, s32, partials, tiles_x, tiles_y, ntiles);
     count_launch();
-    k_final_df<<<1, 256, 0, s>>>(partials, (int)nb, out);
+    run_kernel(k_final_df, 1, 256, 0, s, partials, (int)nb, out);
 }
 
 void launch_update_df(cudaStream_t s, Dims d, Lay L, float2 *p, const float *e32, double alpha, double shift) {
     count_launch();
-    k_update_df<<<blocks_for(d.n), kThreads, 0, s>>>(d, L, p, e32, (float)alpha, (float)shift);
+    run_kernel(k_update_df, blocks_for(d.n), kThreads, 0, s, d, L, p, e32, (float)alpha, (float)shift);
 }
 
 }  // namespace mg

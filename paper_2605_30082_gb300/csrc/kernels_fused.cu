@@ -216,6 +216,7 @@ template <bool FROM_ZERO, bool UPDATE>
 __global__ void __launch_bounds__(kThreads, 3)
     k_sweep_fused(Geo g, float h2, const float *__restrict__ sv, const float *__restrict__ b, const float *X,
                   float *Y, int c1, FUpd up, unsigned *err, int skip_plane) {
+    grid_wait();
     extern __shared__ __align__(16) float sm[];
     float *stages = sm;
     float *c1n = sm + (size_t)kStages * STAGE;  // 3 planes of new c1 values
@@ -455,7 +456,7 @@ void run_fused(cudaStream_t s, dim3 grid, const Geo &g, float h2, const float *s
         cudaFuncSetAttribute(k_sweep_fused<FZ, UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (dev >= 0 && dev < 64) done |= 1ull << dev;
     }
-    k_sweep_fused<FZ, UPD><<<grid, kThreads, kSmemBytes, s>>>(g, h2, sinv, b, X, Y, c1, up, err, skip_plane);
+    run_kernel(k_sweep_fused<FZ, UPD>, grid, kThreads, kSmemBytes, s, g, h2, sinv, b, X, Y, c1, up, err, skip_plane);
 }
 
 void launch_sweep_fused(cudaStream_t s, Lay L, double h2, const float *sinv, const float *b, const float *X,

@@ -49,6 +49,7 @@ __global__ void k_project(Dims d, double ih, int log2ih, double sigma, const dou
                           const double *__restrict__ fz, const double *__restrict__ csx,
                           const double *__restrict__ csy, const double *__restrict__ csz, const double *ux,
                           const double *uy, const double *uz, double *ox, double *oy, double *oz) {
+    grid_wait();
     const int nx = d.nx, ny = d.ny, nz = d.nz;
     const int j = blockIdx.x;
     const i64 nxy = d.nxy;
@@ -129,6 +130,7 @@ struct FracOut {
 __global__ void k_density_grads(Dims d, const double *__restrict__ rho, const float *__restrict__ gx,
                                 const float *__restrict__ gy, const float *__restrict__ gz, double *drho,
                                 int nfrac, FracOut fo) {
+    grid_wait();
     const int nx = d.nx, ny = d.ny, nz = d.nz;
     const i64 nxy = d.nxy;
     const int j = blockIdx.x;  // grid (ny, nz) as for k_project
@@ -186,30 +188,30 @@ void launch_project(cudaStream_t s, Dims d, double h, const double *p, const dou
     count_launch();
     if (csfx) {
         if (copy && log2ih >= 0)
-            k_project<true, true, true><<<nb, nt, 0, s>>>(d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
+            run_kernel(k_project<true, true, true>, nb, nt, 0, s, d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
                                                           uy, uz, ox, oy, oz);
         else if (log2ih >= 0)
-            k_project<true, false, true><<<nb, nt, 0, s>>>(d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
+            run_kernel(k_project<true, false, true>, nb, nt, 0, s, d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
                                                            uy, uz, ox, oy, oz);
         else if (copy)
-            k_project<true, true, false><<<nb, nt, 0, s>>>(d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
+            run_kernel(k_project<true, true, false>, nb, nt, 0, s, d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
                                                            uy, uz, ox, oy, oz);
         else
-            k_project<true, false, false><<<nb, nt, 0, s>>>(d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
+            run_kernel(k_project<true, false, false>, nb, nt, 0, s, d, ih, log2ih, sigma, p, fx, fy, fz, csfx, csfy, csfz, ux,
                                                             uy, uz, ox, oy, oz);
     } else if (log2ih >= 0) {
         if (copy)
-            k_project<false, true, true><<<nb, nt, 0, s>>>(d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
+            run_kernel(k_project<false, true, true>, nb, nt, 0, s, d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
                                                            nullptr, ux, uy, uz, ox, oy, oz);
         else
-            k_project<false, false, true><<<nb, nt, 0, s>>>(d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
+            run_kernel(k_project<false, false, true>, nb, nt, 0, s, d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
                                                             nullptr, ux, uy, uz, ox, oy, oz);
     } else {
         if (copy)
-            k_project<false, true, false><<<nb, nt, 0, s>>>(d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
+            run_kernel(k_project<false, true, false>, nb, nt, 0, s, d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
                                                             nullptr, ux, uy, uz, ox, oy, oz);
         else
-            k_project<false, false, false><<<nb, nt, 0, s>>>(d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
+            run_kernel(k_project<false, false, false>, nb, nt, 0, s, d, ih, log2ih, 0.0, p, fx, fy, fz, nullptr, nullptr,
                                                              nullptr, ux, uy, uz, ox, oy, oz);
     }
 }
@@ -223,7 +225,7 @@ void launch_density_grads(cudaStream_t s, Dims d, const double *rho, const float
         fo.dr[q] = q < nfrac ? (float)(rho_phase[q] - rho_phase[nfrac]) : 0.f;
     }
     count_launch();
-    k_density_grads<<<row_grid(d), row_threads(d), 0, s>>>(d, rho, gx, gy, gz, drho, nfrac, fo);
+    run_kernel(k_density_grads, row_grid(d), row_threads(d), 0, s, d, rho, gx, gy, gz, drho, nfrac, fo);
 }
 
 }  // namespace mg

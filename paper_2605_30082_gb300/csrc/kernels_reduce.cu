@@ -103,6 +103,7 @@ __device__ __forceinline__ void block_sum2(double a, double b, double *out) {
 }
 
 __global__ void k_final(const double *__restrict__ partials, int nb, double *out) {
+    grid_wait();
     double a = 0.0, b = 0.0;
     for (int q = threadIdx.x; q < nb; q += blockDim.x) {
         a += partials[2 * q];
@@ -132,6 +133,7 @@ inline __device__ bool aligned16(const void *p) { return (reinterpret_cast<uintp
 // gauge sums, which need no squares, take one FP64 addition per element instead of two.
 template <typename T, bool SQ>
 __global__ void k_sum_sumsq(i64 n, const T *__restrict__ x, double *partials) {
+    grid_wait();
     using V = Vec16<T>;
     double a = 0.0, b = 0.0;
     const i64 tid = (i64)blockIdx.x * blockDim.x + threadIdx.x, nt = (i64)gridDim.x * blockDim.x;
@@ -189,6 +191,7 @@ __device__ __forceinline__ double mul_pow2(double v, int m, double s) {
 template <bool POW2>
 __global__ void k_sub_mean(i64 n, const double *__restrict__ b, const double *__restrict__ sum,
                            double scale, int m2, double *b64, double *partials) {
+    grid_wait();
     const double mean = sum[0] / (double)n;
     double q = 0.0;
     auto f = [&](double u) { return POW2 ? mul_pow2(u - mean, m2, scale) : (u - mean) * scale; };
@@ -243,6 +246,7 @@ __global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__rest
                                   const double *__restrict__ fy, const double *__restrict__ fz,
                                   const double *__restrict__ dg, const double *__restrict__ b,
                                   const double *__restrict__ p, float *r32, float s32, double *partials) {
+    grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz, hx = nx >> 1;
     const int nxy = nx * ny;
@@ -302,10 +306,19 @@ __global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__rest
     block_sum2((double)q, (double)sp, partials + 2 * blockIdx.x);
 }
 
+// n4 words, the first 4 nv of them as 16-byte stores
+__global__ void k_zero(float *p, i64 nv, i64 n4) {
+    const i64 t0 = (i64)blockIdx.x * blockDim.x + threadIdx.x, nt = (i64)gridDim.x * blockDim.x;
+    grid_wait();
+    for (i64 t = t0; t < nv; t += nt) reinterpret_cast<float4 *>(p)[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (i64 t = 4 * nv + t0; t < n4; t += nt) p[t] = 0.f;
+}
+
 // r32 = s32 * (the residual of p = 0) in the level layout, rounded as the residual kernels round
 // theirs: the residual of p = 0 is h^2 b~ itself, truncated to FP32, times s32.  A cold-started
 // solve takes its first inner right-hand side from here instead of an FP64 residual pass.
 __global__ void k_zero_resid32(Dims d, Lay L, const double *__restrict__ b, float s32, float *r32) {
+    grid_wait();
     const i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu = (unsigned)c, r = cu / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -319,6 +332,7 @@ __global__ void k_fine_resid_cell(Dims d, Lay L, double h2, const double *__rest
                                   const double *__restrict__ fy, const double *__restrict__ fz,
                                   const double *__restrict__ dg, const double *__restrict__ b,
                                   const double *__restrict__ p, float *r32, float s32, double *partials) {
+    grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz;
     const i64 nxy = d.nxy;
@@ -348,6 +362,7 @@ __global__ void k_fine_residual(Dims d, Lay L, double ih2, const double *__restr
                                 const double *__restrict__ fy, const double *__restrict__ fz,
                                 const double *__restrict__ b, const double *__restrict__ p,
                                 float *r32, double scale, double *partials) {
+    grid_wait();
     double q = 0.0, sp = 0.0;
     for (i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x; c < d.n; c += (i64)gridDim.x * blockDim.x) {
         int i = (int)(c % d.nx);
@@ -371,6 +386,7 @@ __global__ void k_fine_residual(Dims d, Lay L, double ih2, const double *__restr
 
 // p = (p - shift) + alpha e: 2 FP64 operations, the FP32 value widened exactly with integer operations
 __global__ void k_update(Dims d, Lay L, double *p, const float *__restrict__ e, float alpha, float shift) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= d.n) return;
     const int i = (int)(m % d.nx);
@@ -384,12 +400,14 @@ __global__ void k_update(Dims d, Lay L, double *p, const float *__restrict__ e, 
 // n (<= 32) doubles from src, and with esrc one unsigned, into mapped pinned host memory
 __global__ void k_readback(const double *__restrict__ src, double *dst, int n, const unsigned *esrc,
                            unsigned *edst) {
+    grid_wait();
     const int t = threadIdx.x;
     if (t < n) dst[t] = src[t];
     if (t == 0 && esrc) *edst = *esrc;
 }
 
 __global__ void k_add_const(i64 n, double *p, double c) {
+    grid_wait();
     i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m < n) p[m] += c;
 }
@@ -406,6 +424,7 @@ __global__ void k_adjoint_grad(Dims d, float ih, float ih2, double ihd, const do
                                const double *__restrict__ csx, const double *__restrict__ csy,
                                const double *__restrict__ csz, float sigma, float *gx, float *gy,
                                float *gz, double *partials) {
+    grid_wait();
     double ds = 0.0;
     const int nx = d.nx, ny = d.ny;
     const i64 nxy = d.nxy, rows = (i64)ny * d.nz;
@@ -499,6 +518,7 @@ constexpr int kGradRows = 8, kGradPlanes = 32;
 __global__ void __launch_bounds__(32 * kGradRows) k_adjoint_grad_split(
     int nx, int ny, int nz, float ih2, const double *__restrict__ lam, const double *__restrict__ p,
     float *__restrict__ gx, float *__restrict__ gy, float *__restrict__ gz) {
+    grid_wait();
     const int lane = threadIdx.x;
     const int x = blockIdx.x * 32 + lane;
     const int y = blockIdx.y * kGradRows + threadIdx.y;
@@ -594,6 +614,7 @@ struct GradTile {
 __global__ void __launch_bounds__(32 * kGrad2Rows) k_adjoint_grad_split2(
     int nx, int ny, int nz, float ih2, const double *__restrict__ lam, const double *__restrict__ p,
     float *__restrict__ gx, float *__restrict__ gy, float *__restrict__ gz) {
+    grid_wait();
     __shared__ GradTile T;
     const int lane = threadIdx.x, ty = threadIdx.y;
     const int x0 = blockIdx.x * 64, y0 = blockIdx.y * kGrad2Rows;
@@ -704,10 +725,10 @@ void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, doubl
     static const int wave_s = wave_blocks((const void *)k_sum_sumsq<T, false>, kReduceThreads);
     const int nb = fill_blocks(reduce_blocks(n), squares ? wave_q : wave_s);
     count_launch();
-    if (squares) k_sum_sumsq<T, true><<<nb, kReduceThreads, 0, s>>>(n, x, partials);
-    else k_sum_sumsq<T, false><<<nb, kReduceThreads, 0, s>>>(n, x, partials);
+    if (squares) run_kernel(k_sum_sumsq<T, true>, nb, kReduceThreads, 0, s, n, x, partials);
+    else run_kernel(k_sum_sumsq<T, false>, nb, kReduceThreads, 0, s, n, x, partials);
     count_launch();
-    k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 template void launch_sum_sumsq<double>(cudaStream_t, i64, const double *, double *, double *, bool);
 template void launch_sum_sumsq<float>(cudaStream_t, i64, const float *, double *, double *, bool);
@@ -720,10 +741,10 @@ void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, 
     const bool pow2 = std::frexp(scale, &e) == 0.5;  // scale = 2^(e - 1)
     const int nb = fill_blocks(reduce_blocks(n), pow2 ? wave_p : wave_m);
     count_launch();
-    if (pow2) k_sub_mean<true><<<nb, kReduceThreads, 0, s>>>(n, b, sum, scale, e - 1, b64, partials);
-    else k_sub_mean<false><<<nb, kReduceThreads, 0, s>>>(n, b, sum, scale, 0, b64, partials);
+    if (pow2) run_kernel(k_sub_mean<true>, nb, kReduceThreads, 0, s, n, b, sum, scale, e - 1, b64, partials);
+    else run_kernel(k_sub_mean<false>, nb, kReduceThreads, 0, s, n, b, sum, scale, 0, b64, partials);
     count_launch();
-    k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 
 void launch_fine_residual(cudaStream_t s, Dims d, Lay L, double ih2, const double *fx, const double *fy,
@@ -732,9 +753,9 @@ void launch_fine_residual(cudaStream_t s, Dims d, Lay L, double ih2, const doubl
     static const int wave = wave_blocks((const void *)k_fine_residual, kReduceThreads);
     const int nb = fill_blocks(reduce_blocks(d.n), wave);
     count_launch();
-    k_fine_residual<<<nb, kReduceThreads, 0, s>>>(d, L, ih2, fx, fy, fz, b, p, r32, scale, partials);
+    run_kernel(k_fine_residual, nb, kReduceThreads, 0, s, d, L, ih2, fx, fy, fz, b, p, r32, scale, partials);
     count_launch();
-    k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 
 void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *fx, const double *fy,
@@ -745,10 +766,10 @@ void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *
         static const int wave_cf = wave_blocks((const void *)k_fine_resid_cell<false>, kReduceThreads);
         const int nb = fill_blocks(reduce_blocks(d.n), b_scaled ? wave_ct : wave_cf);
         count_launch();
-        if (b_scaled) k_fine_resid_cell<true><<<nb, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
-        else k_fine_resid_cell<false><<<nb, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        if (b_scaled) run_kernel(k_fine_resid_cell<true>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        else run_kernel(k_fine_resid_cell<false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
         count_launch();
-        k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+        run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
         return;
     }
     static const int wave_pt = wave_blocks((const void *)k_fine_resid_pair<true, false>, kReduceThreads);
@@ -762,45 +783,53 @@ void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *
         static const int wave_gf = wave_blocks((const void *)k_fine_resid_pair<false, true>, kReduceThreads);
         const int ng = fill_blocks(reduce_blocks(d.n / 2), b_scaled ? wave_gt : wave_gf);
         if (b_scaled)
-            k_fine_resid_pair<true, true><<<ng, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+            run_kernel(k_fine_resid_pair<true, true>, ng, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
         else
-            k_fine_resid_pair<false, true><<<ng, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+            run_kernel(k_fine_resid_pair<false, true>, ng, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
         count_launch();
-        k_final<<<1, kReduceThreads, 0, s>>>(partials, ng, out);
+        run_kernel(k_final, 1, kReduceThreads, 0, s, partials, ng, out);
         return;
     }
     if (b_scaled) {
-        k_fine_resid_pair<true, false><<<nb, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        run_kernel(k_fine_resid_pair<true, false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
     } else {
-        k_fine_resid_pair<false, false><<<nb, kReduceThreads, 0, s>>>(d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        run_kernel(k_fine_resid_pair<false, false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
     }
     count_launch();
-    k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 
 void launch_zero_resid32(cudaStream_t s, Dims d, Lay L, const double *b, double scale32, float *r32) {
     count_launch();
-    k_zero_resid32<<<blocks_for(d.n), kThreads, 0, s>>>(d, L, b, (float)scale32, r32);
+    run_kernel(k_zero_resid32, blocks_for(d.n), kThreads, 0, s, d, L, b, (float)scale32, r32);
 }
 
 void launch_update(cudaStream_t s, Dims d, Lay L, double *p, const float *e32, double alpha, double shift) {
     count_launch();
-    k_update<<<blocks_for(d.n), kThreads, 0, s>>>(d, L, p, e32, (float)alpha, (float)shift);
+    run_kernel(k_update, blocks_for(d.n), kThreads, 0, s, d, L, p, e32, (float)alpha, (float)shift);
 }
 
 void launch_readback(cudaStream_t s, const double *src, double *dst_mapped, int n) {
     count_launch();
-    k_readback<<<1, 32, 0, s>>>(src, dst_mapped, n, nullptr, nullptr);
+    run_kernel(k_readback, 1, 32, 0, s, src, dst_mapped, n, nullptr, nullptr);
 }
 
 void launch_readback_u32(cudaStream_t s, const unsigned *src, unsigned *dst_mapped) {
     count_launch();
-    k_readback<<<1, 32, 0, s>>>(nullptr, nullptr, 0, src, dst_mapped);
+    run_kernel(k_readback, 1, 32, 0, s, nullptr, nullptr, 0, src, dst_mapped);
+}
+
+void launch_zero(cudaStream_t s, void *p, size_t bytes) {
+    count_launch();
+    const bool vec = (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    const i64 n4 = (i64)(bytes / 4), nv = vec ? n4 / 4 : 0, work = nv + (n4 - 4 * nv);
+    const i64 cap = (i64)device_sms() * 16, nb = (work + kThreads - 1) / kThreads;
+    run_kernel(k_zero, (unsigned)(nb < cap ? (nb > 0 ? nb : 1) : cap), kThreads, 0, s, reinterpret_cast<float *>(p), nv, n4);
 }
 
 void launch_add_const(cudaStream_t s, i64 n, double *p, double c) {
     count_launch();
-    k_add_const<<<blocks_for(n), kThreads, 0, s>>>(n, p, c);
+    run_kernel(k_add_const, blocks_for(n), kThreads, 0, s, n, p, c);
 }
 
 inline bool aligned16h(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
@@ -817,13 +846,13 @@ void launch_adjoint_grad(cudaStream_t s, Dims d, double h, const double *lam, co
         if (d.nx % 2 == 0 && aligned16h(lam) && aligned16h(p) && aligned8h(gy) && aligned8h(gz)) {
             const dim3 grid((d.nx / 2 + 31) / 32, (d.ny + kGrad2Rows - 1) / kGrad2Rows,
                             (d.nz + kGrad2Planes - 1) / kGrad2Planes);
-            k_adjoint_grad_split2<<<grid, dim3(32, kGrad2Rows), 0, s>>>(d.nx, d.ny, d.nz, (float)(1.0 / (h * h)),
+            run_kernel(k_adjoint_grad_split2, grid, dim3(32, kGrad2Rows), 0, s, d.nx, d.ny, d.nz, (float)(1.0 / (h * h)),
                                                                         lam, p, gx, gy, gz);
             return;
         }
         const dim3 grid((d.nx + 31) / 32, (d.ny + kGradRows - 1) / kGradRows,
                         (d.nz + kGradPlanes - 1) / kGradPlanes);
-        k_adjoint_grad_split<<<grid, dim3(32, kGradRows), 0, s>>>(d.nx, d.ny, d.nz, (float)(1.0 / (h * h)),
+        run_kernel(k_adjoint_grad_split, grid, dim3(32, kGradRows), 0, s, d.nx, d.ny, d.nz, (float)(1.0 / (h * h)),
                                                                   lam, p, gx, gy, gz);
         return;
     }
@@ -832,11 +861,11 @@ void launch_adjoint_grad(cudaStream_t s, Dims d, double h, const double *lam, co
     count_launch();
     const i64 rows = (i64)d.ny * d.nz;
     if (nb > rows) nb = (int)rows;
-    k_adjoint_grad<<<nb, kReduceThreads, 0, s>>>(d, (float)(1.0 / h), (float)(1.0 / (h * h)), 1.0 / h, lam, p,
+    run_kernel(k_adjoint_grad, nb, kReduceThreads, 0, s, d, (float)(1.0 / h), (float)(1.0 / (h * h)), 1.0 / h, lam, p,
                                                  fx, fy, fz, csfx, csfy, csfz, (float)sigma, gx, gy, gz,
                                                  partials);
     count_launch();
-    k_final<<<1, kReduceThreads, 0, s>>>(partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 
 }  // namespace mg

@@ -23,6 +23,7 @@ struct FracArgs {
 // bound this kernel by the FP64 pipe); equal in exact arithmetic, within a few units in the
 // last place in FP64
 __global__ void k_density(i64 n, FracArgs a, double *rho) {
+    grid_wait();
     i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     double r = a.rho_last;
@@ -48,6 +49,7 @@ __device__ __forceinline__ double half_of(double v) {
 
 // s = 1/rho per cell, validating rho (finite and > 0)
 __global__ void k_inv_rho(i64 n, const double *__restrict__ rho, double *sinv, unsigned *err) {
+    grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= n) return;
     const double r = rho[m];
@@ -62,6 +64,7 @@ __global__ void k_inv_rho(i64 n, const double *__restrict__ rho, double *sinv, u
 // beta on the low faces: 1 / harmonic mean of the two densities = (s_L + s_R) / 2; blocks take
 // rows (grid y, strided), threads the cells of a row
 __global__ void k_faces_from_s(Dims d, const double *__restrict__ sv, double *fx, double *fy, double *fz) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.nx) return;
     const i64 rows = (i64)d.ny * d.nz;
@@ -79,6 +82,7 @@ __global__ void k_faces_from_s(Dims d, const double *__restrict__ sv, double *fx
 // pair's first cell is one scalar load, from the line the neighbouring lane reads); the same
 // additions in the same order as k_faces_from_s, so bitwise the same faces
 __global__ void k_faces_from_s2(Dims d, const double *__restrict__ sv, double *fx, double *fy, double *fz) {
+    grid_wait();
     const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= d.nx) return;
     const i64 rows = (i64)d.ny * d.nz;
@@ -108,6 +112,7 @@ __global__ void k_faces_from_s2(Dims d, const double *__restrict__ sv, double *f
 __global__ void k_faces_from_api(Dims d, const double *__restrict__ bx, const double *__restrict__ by,
                                  const double *__restrict__ bz, double *fx, double *fy, double *fz,
                                  unsigned *err) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -128,6 +133,7 @@ __global__ void k_faces_from_api(Dims d, const double *__restrict__ bx, const do
 
 __global__ void k_faces_to_api(Dims d, const double *__restrict__ fx, const double *__restrict__ fy,
                                const double *__restrict__ fz, double *bx, double *by, double *bz) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -146,6 +152,7 @@ __global__ void k_faces_to_api(Dims d, const double *__restrict__ fx, const doub
 
 __global__ void k_invdiag(Dims d, const double *__restrict__ fx, const double *__restrict__ fy,
                           const double *__restrict__ fz, double *invd64, double *diag) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -167,6 +174,7 @@ __global__ void k_invdiag(Dims d, const double *__restrict__ fx, const double *_
 __global__ void k_coarsen(Dims f, Dims cd, const double *__restrict__ ffx,
                           const double *__restrict__ ffy, const double *__restrict__ ffz,
                           double *cfx, double *cfy, double *cfz) {
+    grid_wait();
     i64 C = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (C >= cd.n) return;
     int I = (int)(C % cd.nx);
@@ -186,12 +194,14 @@ __global__ void k_coarsen(Dims f, Dims cd, const double *__restrict__ ffx,
 }
 
 __global__ void k_to_f32(i64 n, const double *__restrict__ src, float *dst) {
+    grid_wait();
     i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m < n) dst[m] = (float)src[m];
 }
 
 __global__ void k_csf_faces(Dims d, double ih, const double *__restrict__ f,
                             const double *__restrict__ kap, double *cx, double *cy, double *cz) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -216,6 +226,7 @@ __global__ void k_rhs(Dims d, double ih, const double *b0, const double *__restr
                       const double *__restrict__ fz, const double *__restrict__ csx,
                       const double *__restrict__ csy, const double *__restrict__ csz, double sigma,
                       double *b) {
+    grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
     const unsigned cu_ = (unsigned)c, ru_ = cu_ / (unsigned)d.nx;  // c < 2^32: 32-bit divisions
@@ -259,59 +270,59 @@ void launch_density(cudaStream_t s, i64 n, int nfrac, const double *const *frac,
         a.drho[q] = q < nfrac ? rho_phase[q] - rho_phase[nfrac] : 0.0;
     }
     count_launch();
-    k_density<<<blocks_for(n), kThreads, 0, s>>>(n, a, rho);
+    run_kernel(k_density, blocks_for(n), kThreads, 0, s, n, a, rho);
 }
 
 void launch_faces_from_rho(cudaStream_t s, Dims d, const double *rho, double *sinv, double *fx, double *fy,
                            double *fz, unsigned *err) {
     count_launch(2);
-    k_inv_rho<<<blocks_for(d.n), kThreads, 0, s>>>(d.n, rho, sinv, err);
+    run_kernel(k_inv_rho, blocks_for(d.n), kThreads, 0, s, d.n, rho, sinv, err);
     const i64 rows = (i64)d.ny * d.nz;
     auto a16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
     if (d.nx % 2 == 0 && a16(sinv) && a16(fx) && a16(fy) && a16(fz)) {
         const dim3 grd((unsigned)((d.nx / 2 + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
-        k_faces_from_s2<<<grd, 128, 0, s>>>(d, sinv, fx, fy, fz);
+        run_kernel(k_faces_from_s2, grd, 128, 0, s, d, sinv, fx, fy, fz);
         return;
     }
     const dim3 grd((unsigned)((d.nx + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
-    k_faces_from_s<<<grd, 128, 0, s>>>(d, sinv, fx, fy, fz);
+    run_kernel(k_faces_from_s, grd, 128, 0, s, d, sinv, fx, fy, fz);
 }
 
 void launch_faces_from_api(cudaStream_t s, Dims d, const double *bx, const double *by,
                            const double *bz, double *fx, double *fy, double *fz, unsigned *err) {
     count_launch();
-    k_faces_from_api<<<blocks_for(d.n), kThreads, 0, s>>>(d, bx, by, bz, fx, fy, fz, err);
+    run_kernel(k_faces_from_api, blocks_for(d.n), kThreads, 0, s, d, bx, by, bz, fx, fy, fz, err);
 }
 
 void launch_faces_to_api(cudaStream_t s, Dims d, const double *fx, const double *fy,
                          const double *fz, double *bx, double *by, double *bz) {
     count_launch();
-    k_faces_to_api<<<blocks_for(d.n), kThreads, 0, s>>>(d, fx, fy, fz, bx, by, bz);
+    run_kernel(k_faces_to_api, blocks_for(d.n), kThreads, 0, s, d, fx, fy, fz, bx, by, bz);
 }
 
 void launch_invdiag(cudaStream_t s, Dims d, const double *fx, const double *fy, const double *fz,
                     double *invd64, double *diag) {
     if (!invd64 && !diag) return;
     count_launch();
-    k_invdiag<<<blocks_for(d.n), kThreads, 0, s>>>(d, fx, fy, fz, invd64, diag);
+    run_kernel(k_invdiag, blocks_for(d.n), kThreads, 0, s, d, fx, fy, fz, invd64, diag);
 }
 
 void launch_coarsen(cudaStream_t s, Dims fine, const double *ffx, const double *ffy,
                     const double *ffz, double *cfx, double *cfy, double *cfz) {
     Dims cd = make_dims(fine.nx / 2, fine.ny / 2, fine.nz / 2);
     count_launch();
-    k_coarsen<<<blocks_for(cd.n), kThreads, 0, s>>>(fine, cd, ffx, ffy, ffz, cfx, cfy, cfz);
+    run_kernel(k_coarsen, blocks_for(cd.n), kThreads, 0, s, fine, cd, ffx, ffy, ffz, cfx, cfy, cfz);
 }
 
 void launch_to_f32(cudaStream_t s, i64 n, const double *src, float *dst) {
     count_launch();
-    k_to_f32<<<blocks_for(n), kThreads, 0, s>>>(n, src, dst);
+    run_kernel(k_to_f32, blocks_for(n), kThreads, 0, s, n, src, dst);
 }
 
 void launch_csf_faces(cudaStream_t s, Dims d, double h, const double *f, const double *kappa,
                       double *cx, double *cy, double *cz) {
     count_launch();
-    k_csf_faces<<<blocks_for(d.n), kThreads, 0, s>>>(d, 1.0 / h, f, kappa, cx, cy, cz);
+    run_kernel(k_csf_faces, blocks_for(d.n), kThreads, 0, s, d, 1.0 / h, f, kappa, cx, cy, cz);
 }
 
 void launch_rhs(cudaStream_t s, Dims d, double h, const double *b0, const double *ux, const double *uy,
@@ -319,7 +330,7 @@ void launch_rhs(cudaStream_t s, Dims d, double h, const double *b0, const double
                 const double *csfx, const double *csfy, const double *csfz, double sigma,
                 double *b) {
     count_launch();
-    k_rhs<<<blocks_for(d.n), kThreads, 0, s>>>(d, 1.0 / h, b0, ux, uy, uz, fx, fy, fz, csfx, csfy,
+    run_kernel(k_rhs, blocks_for(d.n), kThreads, 0, s, d, 1.0 / h, b0, ux, uy, uz, fx, fy, fz, csfx, csfy,
                                                csfz, sigma, b);
 }
 

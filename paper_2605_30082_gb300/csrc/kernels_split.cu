@@ -83,6 +83,7 @@ __device__ __forceinline__ void stencil_any(const Lay &L, const Coef32 &cf, cons
 // half sweep of colour `col`, one thread per cell of that colour, any layout
 __global__ void k_half_any(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            int from_zero) {
+    grid_wait();
     const int halfw = (L.nx + 1) >> 1;
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 rows = (i64)L.ny * L.nz;
@@ -130,6 +131,7 @@ __device__ __forceinline__ void df_add(float &h, float &l, float t) {
 template <bool SFORM, bool FROM_ZERO, int UPDATE = 0, bool GHOST = false>
 __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            Upd up = Upd{}) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 rows = (i64)L.ny * L.nz;
@@ -273,6 +275,7 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
 template <bool SFORM, bool FROM_ZERO, int UPDATE, int ZC, bool GHOST = false>
 __global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, const float *__restrict__ b,
                                                     float *xv, int col, Upd up) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const int kvi = blockIdx.x * blockDim.x + threadIdx.x;
     const int yi = blockIdx.y * blockDim.y + threadIdx.y;
@@ -460,6 +463,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int ZC, int MINB, bool GHOST = false>
 __global__ void __launch_bounds__(64, MINB) k_half_zs(Lay L, float h2, const float *__restrict__ sv,
                                                        const float *__restrict__ b, float *xv, int col) {
+    grid_wait();
     extern __shared__ float4 stg[];  // [kZsStages][kZsFields][64 threads]
     constexpr int D = kZsStages;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -615,6 +619,7 @@ constexpr size_t kZfSmem = (size_t)kZfStages * kZfFields * 64 * sizeof(float4);
 template <int ZC, int MINB>
 __global__ void __launch_bounds__(64, MINB) k_half_zf(Lay L, float h2, Coef32 cf, const float *__restrict__ b,
                                                        float *xv, int col) {
+    grid_wait();
     extern __shared__ float4 stg[];  // [kZfStages][kZfFields][64 threads]
     constexpr int D = kZfStages;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -757,7 +762,7 @@ void run_half_z(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const 
             return true;
         }();
         (void)carveout;
-        k_half_zs<16, 11, GHOST><<<dim3(gx, gy, (L.nz + 15) / 16), blk, kZsSmem, s>>>(L, h2, cf.s, b, x, col);
+        run_kernel(k_half_zs<16, 11, GHOST>, dim3(gx, gy, (L.nz + 15) / 16), blk, kZsSmem, s, L, h2, cf.s, b, x, col);
         return;
     }
     // the face form's regular sweeps, staged, where the grid gives at least four waves of
@@ -771,13 +776,13 @@ void run_half_z(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const 
             return true;
         }();
         (void)carveout;
-        k_half_zf<4, 11><<<dim3(gx, gy, (L.nz + 3) / 4), blk, kZfSmem, s>>>(L, h2, cf, b, x, col);
+        run_kernel(k_half_zf<4, 11>, dim3(gx, gy, (L.nz + 3) / 4), blk, kZfSmem, s, L, h2, cf, b, x, col);
         return;
     }
     if ((i64)gx * gy * ((L.nz + 15) / 16) >= 4 * sms * 12)
-        k_half_z<SFORM, FROM_ZERO, UPDATE, 16, GHOST><<<dim3(gx, gy, (L.nz + 15) / 16), blk, 0, s>>>(L, h2, cf, b, x, col, up);
+        run_kernel(k_half_z<SFORM, FROM_ZERO, UPDATE, 16, GHOST>, dim3(gx, gy, (L.nz + 15) / 16), blk, 0, s, L, h2, cf, b, x, col, up);
     else
-        k_half_z<SFORM, FROM_ZERO, UPDATE, 4, GHOST><<<dim3(gx, gy, (L.nz + 3) / 4), blk, 0, s>>>(L, h2, cf, b, x, col, up);
+        run_kernel(k_half_z<SFORM, FROM_ZERO, UPDATE, 4, GHOST>, dim3(gx, gy, (L.nz + 3) / 4), blk, 0, s, L, h2, cf, b, x, col, up);
 }
 
 // ---- vectorised red-only residual + restriction (split fine level, hx % 4 == 0) ----------
@@ -790,6 +795,7 @@ constexpr int kRrThreads = 64;
 template <bool SFORM, bool GHOST = false>
 __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                              const float *__restrict__ xv, float *bc) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const i64 T = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 crows = (i64)Lc.ny * Lc.nz;
@@ -885,6 +891,7 @@ __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, fl
 // ---- vectorised red-only prolongation + correction (split fine level, hx % 4 == 0) -------
 // one thread adds P ec to 4 consecutive red cells of one fine row
 __global__ void k_prolong_red_vec(Lay L, Lay Lc, const float *__restrict__ ec, float *xv, int kind) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 rows = (i64)L.ny * L.nz;
@@ -958,6 +965,7 @@ constexpr int kProlThreads = 64;
 // where the whole grid would read them instead of the wall's mirror)
 template <bool GHOST = false>
 __global__ void __launch_bounds__(kProlThreads, 10) k_prolong_red8(Lay L, Lay Lc, const float *__restrict__ ec, float *xv) {
+    grid_wait();
     const int hx = L.hx, kv = hx >> 3;  // 8-cell groups per fine row
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 crows = (i64)Lc.ny * Lc.nz;
@@ -1043,6 +1051,7 @@ __device__ __forceinline__ float resid_any(const Lay &L, float ih2, const Coef32
 
 __global__ void k_residual_any(Lay L, float ih2, Coef32 cf, const float *__restrict__ b,
                                const float *__restrict__ xv, float *r, int apply_only) {
+    grid_wait();
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.n) return;
     const int x = (int)(t % L.nx);
@@ -1062,6 +1071,7 @@ __global__ void k_residual_any(Lay L, float ih2, Coef32 cf, const float *__restr
 // (exact after a black half sweep, which solves every black row)
 __global__ void k_resid_restrict_any(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                                      const float *__restrict__ xv, float *bc, int red_only) {
+    grid_wait();
     const i64 T = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (T >= Lc.n) return;
     const int I = (int)(T % Lc.nx);
@@ -1080,6 +1090,7 @@ __global__ void k_resid_restrict_any(Lay L, Lay Lc, float ih2, Coef32 cf, const 
 
 // x += P ec on cells of colour `only_col` (0 red, 1 black) or on all cells (-1)
 __global__ void k_prolong_any(Lay L, Lay Lc, const float *__restrict__ ec, float *xv, int kind, int only_col) {
+    grid_wait();
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.n) return;
     const int x = (int)(t % L.nx);
@@ -1112,6 +1123,7 @@ __global__ void k_prolong_any(Lay L, Lay Lc, const float *__restrict__ ec, float
 
 // e = pinv r on the coarsest level (FP64 accumulation), pinv in natural cell order
 __global__ void k_coarse_matvec_lay(Lay L, const double *__restrict__ pinv, const float *__restrict__ r, float *e) {
+    grid_wait();
     const int nc = (int)L.n;
     const int row = (int)(((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -1132,6 +1144,7 @@ __global__ void k_coarse_matvec_lay(Lay L, const double *__restrict__ pinv, cons
 
 // natural <-> level storage
 __global__ void k_pack(Lay L, const float *__restrict__ nat, float *st) {
+    grid_wait();
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.n) return;
     const int x = (int)(t % L.nx);
@@ -1139,6 +1152,7 @@ __global__ void k_pack(Lay L, const float *__restrict__ nat, float *st) {
     st[sto(L, x, (int)(row % L.ny), (int)(row / L.ny))] = nat[t];
 }
 __global__ void k_unpack(Lay L, const float *__restrict__ st, float *nat) {
+    grid_wait();
     const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.n) return;
     const int x = (int)(t % L.nx);
@@ -1147,6 +1161,7 @@ __global__ void k_unpack(Lay L, const float *__restrict__ st, float *nat) {
 }
 // FP64 natural -> FP32 level storage, rounded to nearest; blocks take rows (grid y, strided)
 __global__ void k_pack64(Lay L, const double *__restrict__ nat, float *st) {
+    grid_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= L.nx) return;
     const i64 rows = (i64)L.ny * L.nz;
@@ -1158,6 +1173,7 @@ __global__ void k_pack64(Lay L, const double *__restrict__ nat, float *st) {
 // s = 1/rho (FP64, natural): FP32 in the level's layout, and optionally as a pair (hi, lo) of
 // FP32 numbers with hi + lo = s to about 2^-48 (natural layout) for the double-float residual
 __global__ void k_pack_inv64(Lay L, const double *__restrict__ sinv, float *st, float2 *s2) {
+    grid_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= L.nx) return;
     const i64 rows = (i64)L.ny * L.nz;
@@ -1197,8 +1213,8 @@ void half32_slab(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const
         return;
     }
     const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
-    if (from_zero) k_half_vec<SFORM, true, 0, true><<<blocks_for(work), kThreads, 0, s>>>(L, h2, cf, b, x, col, Upd{});
-    else k_half_vec<SFORM, false, 0, true><<<blocks_for(work), kThreads, 0, s>>>(L, h2, cf, b, x, col, Upd{});
+    if (from_zero) run_kernel(k_half_vec<SFORM, true, 0, true>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
+    else run_kernel(k_half_vec<SFORM, false, 0, true>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
 }
 
 void launch_half32_slab(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col,
@@ -1226,15 +1242,15 @@ void launch_half32(cudaStream_t s, Lay L, double h2, const float *sinv, const fl
     } else if (L.split && L.hx % 4 == 0) {
         const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
         if (sinv) {
-            if (from_zero) k_half_vec<true, true><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, x, col);
-            else k_half_vec<true, false><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, x, col);
+            if (from_zero) run_kernel(k_half_vec<true, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
+            else run_kernel(k_half_vec<true, false>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
         } else {
-            if (from_zero) k_half_vec<false, true><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, x, col);
-            else k_half_vec<false, false><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, x, col);
+            if (from_zero) run_kernel(k_half_vec<false, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
+            else run_kernel(k_half_vec<false, false>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
         }
     } else {
         const i64 work = (i64)L.ny * L.nz * ((L.nx + 1) / 2);
-        k_half_any<<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, x, col, from_zero ? 1 : 0);
+        run_kernel(k_half_any, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, from_zero ? 1 : 0);
     }
 }
 
@@ -1250,7 +1266,7 @@ void launch_half32_update(cudaStream_t s, Lay L, double h2, const float *sinv, c
     float *xv = const_cast<float *>(x);  // read only in the UPDATE variants
     if (L.zlo || L.zhi) {  // a slab: s-form, FP64 solution (the decomposed mixed cycle)
         if (half_z_ok(L)) run_half_z<true, false, 1, true>(s, L, (float)h2, cf, b, xv, 0, up);
-        else k_half_vec<true, false, 1, true><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, xv, 0, up);
+        else run_kernel(k_half_vec<true, false, 1, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
         return;
     }
     if (half_z_ok(L)) {
@@ -1264,11 +1280,11 @@ void launch_half32_update(cudaStream_t s, Lay L, double h2, const float *sinv, c
         return;
     }
     if (p2) {
-        if (sinv) k_half_vec<true, false, 2><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, xv, 0, up);
-        else k_half_vec<false, false, 2><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, xv, 0, up);
+        if (sinv) run_kernel(k_half_vec<true, false, 2>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+        else run_kernel(k_half_vec<false, false, 2>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
     } else {
-        if (sinv) k_half_vec<true, false, 1><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, xv, 0, up);
-        else k_half_vec<false, false, 1><<<blocks_for(work), kThreads, 0, s>>>(L, (float)h2, cf, b, xv, 0, up);
+        if (sinv) run_kernel(k_half_vec<true, false, 1>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+        else run_kernel(k_half_vec<false, false, 1>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
     }
 }
 
@@ -1276,7 +1292,7 @@ void launch_residual32(cudaStream_t s, Lay L, double ih2, const float *sinv, con
                        const float *fz, const float *b, const float *x, float *r, bool apply_only) {
     Coef32 cf{sinv, fx, fy, fz};
     count_launch();
-    k_residual_any<<<blocks_for(L.n), kThreads, 0, s>>>(L, (float)ih2, cf, b, x, r, apply_only ? 1 : 0);
+    run_kernel(k_residual_any, blocks_for(L.n), kThreads, 0, s, L, (float)ih2, cf, b, x, r, apply_only ? 1 : 0);
 }
 
 void launch_resid_restrict32(cudaStream_t s, Lay L, Lay Lc, double ih2, const float *sinv, const float *fx,
@@ -1287,13 +1303,13 @@ void launch_resid_restrict32(cudaStream_t s, Lay L, Lay Lc, double ih2, const fl
     if (red_only && L.split && L.hx % 4 == 0) {
         const i64 work = (i64)Lc.ny * Lc.nz * (L.hx / 4);
         const unsigned nb = (unsigned)((work + kRrThreads - 1) / kRrThreads);
-        if ((L.zlo || L.zhi) && sinv) k_rr_red_vec<true, true><<<nb, kRrThreads, 0, s>>>(L, Lc, (float)ih2, cf, b, x, bc);
-        else if (L.zlo || L.zhi) k_rr_red_vec<false, true><<<nb, kRrThreads, 0, s>>>(L, Lc, (float)ih2, cf, b, x, bc);
-        else if (sinv) k_rr_red_vec<true><<<nb, kRrThreads, 0, s>>>(L, Lc, (float)ih2, cf, b, x, bc);
-        else k_rr_red_vec<false><<<nb, kRrThreads, 0, s>>>(L, Lc, (float)ih2, cf, b, x, bc);
+        if ((L.zlo || L.zhi) && sinv) run_kernel(k_rr_red_vec<true, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
+        else if (L.zlo || L.zhi) run_kernel(k_rr_red_vec<false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
+        else if (sinv) run_kernel(k_rr_red_vec<true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
+        else run_kernel(k_rr_red_vec<false>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         return;
     }
-    k_resid_restrict_any<<<blocks_for(Lc.n), kThreads, 0, s>>>(L, Lc, (float)ih2, cf, b, x, bc, red_only ? 1 : 0);
+    run_kernel(k_resid_restrict_any, blocks_for(Lc.n), kThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc, red_only ? 1 : 0);
 }
 
 void launch_prolong32(cudaStream_t s, Lay L, Lay Lc, const float *ec, float *x, int kind, int only_col) {
@@ -1302,42 +1318,42 @@ void launch_prolong32(cudaStream_t s, Lay L, Lay Lc, const float *ec, float *x, 
         2 * Lc.nx == L.nx && 2 * Lc.ny == L.ny && 2 * Lc.nz == L.nz) {
         const i64 work = (i64)Lc.ny * Lc.nz * (L.hx / 8);
         const unsigned nb = (unsigned)((work + kProlThreads - 1) / kProlThreads);
-        if (Lc.zlo || Lc.zhi) k_prolong_red8<true><<<nb, kProlThreads, 0, s>>>(L, Lc, ec, x);
-        else k_prolong_red8<<<nb, kProlThreads, 0, s>>>(L, Lc, ec, x);
+        if (Lc.zlo || Lc.zhi) run_kernel(k_prolong_red8<true>, nb, kProlThreads, 0, s, L, Lc, ec, x);
+        else run_kernel(k_prolong_red8<false>, nb, kProlThreads, 0, s, L, Lc, ec, x);
         return;
     }
     if (only_col == 0 && L.split && L.hx % 4 == 0) {
         const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
-        k_prolong_red_vec<<<blocks_for(work), kThreads, 0, s>>>(L, Lc, ec, x, kind);
+        run_kernel(k_prolong_red_vec, blocks_for(work), kThreads, 0, s, L, Lc, ec, x, kind);
         return;
     }
-    k_prolong_any<<<blocks_for(L.n), kThreads, 0, s>>>(L, Lc, ec, x, kind, only_col);
+    run_kernel(k_prolong_any, blocks_for(L.n), kThreads, 0, s, L, Lc, ec, x, kind, only_col);
 }
 
 void launch_coarse_matvec32(cudaStream_t s, Lay L, const double *pinv, const float *r, float *e) {
     count_launch();
-    k_coarse_matvec_lay<<<blocks_for(L.n * 32), kThreads, 0, s>>>(L, pinv, r, e);
+    run_kernel(k_coarse_matvec_lay, blocks_for(L.n * 32), kThreads, 0, s, L, pinv, r, e);
 }
 
 void launch_pack32(cudaStream_t s, Lay L, const float *nat, float *st) {
     count_launch();
-    k_pack<<<blocks_for(L.n), kThreads, 0, s>>>(L, nat, st);
+    run_kernel(k_pack, blocks_for(L.n), kThreads, 0, s, L, nat, st);
 }
 void launch_unpack32(cudaStream_t s, Lay L, const float *st, float *nat) {
     count_launch();
-    k_unpack<<<blocks_for(L.n), kThreads, 0, s>>>(L, st, nat);
+    run_kernel(k_unpack, blocks_for(L.n), kThreads, 0, s, L, st, nat);
 }
 void launch_pack64to32(cudaStream_t s, Lay L, const double *nat, float *st) {
     count_launch();
     const i64 rows = (i64)L.ny * L.nz;
     const dim3 grd((unsigned)((L.nx + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
-    k_pack64<<<grd, 128, 0, s>>>(L, nat, st);
+    run_kernel(k_pack64, grd, 128, 0, s, L, nat, st);
 }
 void launch_pack_inv_rho(cudaStream_t s, Lay L, const double *sinv, float *st, float2 *s2) {
     count_launch();
     const i64 rows = (i64)L.ny * L.nz;
     const dim3 grd((unsigned)((L.nx + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
-    k_pack_inv64<<<grd, 128, 0, s>>>(L, sinv, st, s2);
+    run_kernel(k_pack_inv64, grd, 128, 0, s, L, sinv, st, s2);
 }
 
 }  // namespace mg

@@ -71,11 +71,6 @@ struct mg_handle {
     int sform0;        // level-0 FP32 kernels use s = 1/rho (operator set from a density)
     int inject;        // pending one-shot test faults (MG_INJECT_* bits, mg_debug_inject)
     cudaEvent_t ev0, ev1;
-    // the V-cycle below the finest level, recorded once at mg_create as a CUDA graph (its
-    // launches use fixed buffers and parameters) and replayed by every cycle; null: launched
-    // kernel by kernel
-    cudaGraphExec_t tail_exec;
-    long long tail_launches;
     // the levels from tail_l (>= 1) down as one cluster launch (kernels_tail.cu); 0: none
     int tail_l, tail_split;
     mg::TailArgs tail;
@@ -175,12 +170,6 @@ void prof_collect(mg_handle *h) {
     h->pev_used = 0;
 }
 
-// ---- the V-cycle below the finest level as a CUDA graph ------------------------------
-// Levels 1 .. coarsest run many short launches (about 60 per cycle at 512^3, most of a few
-// microseconds); replaying them as one graph removes the per-launch host cost and most of the
-// gaps between them.  The graph is recorded once in mg_create (build_tail_graph) from the
-// same functions the cycle calls, so a replay launches the same kernels with the same
-// arguments in the same order.
 }  // namespace
 
 namespace mg {
@@ -192,11 +181,6 @@ cudaStream_t swap_handle_stream(mg_handle *h, cudaStream_t s) {
 }  // namespace mg
 
 namespace {
-
-void replay_tail(mg_handle *h) {
-    if (cudaGraphLaunch(h->tail_exec, h->s) == cudaSuccess) mg::count_launch((int)h->tail_launches);
-    // a failed launch leaves its error for the solve's check_launch
-}
 
 // ---- the coarse levels in one cluster (kernels_tail.cu) ----------------------------------
 void run_tail(mg_handle *h) {
@@ -258,11 +242,10 @@ void vcycle64(mg_handle *h, int l, const double *b, double *x, bool x_zero) {
         run_tail(h);
         return;
     }
-    if (x_zero) cudaMemsetAsync(x, 0, sizeof(double) * (size_t)L.d.n, h->s);
+    if (x_zero) mg::launch_zero(h->s, x, sizeof(double) * (size_t)L.d.n);
     presmooth_restrict64(h, l, b, x, C.b64, h->o.pre);
     if (l == 0) prof_begin(h, MG_PROF_COARSE_LEVELS);
-    if (l == 0 && h->tail_exec) replay_tail(h);
-    else vcycle64(h, l + 1, C.b64, C.x64, true);
+    vcycle64(h, l + 1, C.b64, C.x64, true);
     if (l == 0) prof_end(h);
     prolong_postsmooth64(h, l, b, C.x64, x, h->o.post);
 }
@@ -318,7 +301,7 @@ void smooth32(mg_handle *h, int l, const float *b, float *x, int sweeps, int ord
 // x <- pre-smoothing (from zero if from_zero), bc = R(b - A x)
 void presmooth_restrict32(mg_handle *h, int l, const float *b, float *x, float *bc, int sweeps, bool from_zero) {
     Level &L = h->lv[l], &C = h->lv[l + 1];
-    if (sweeps == 0 && from_zero) cudaMemsetAsync(x, 0, sizeof(float) * (size_t)L.d.n, h->s);
+    if (sweeps == 0 && from_zero) mg::launch_zero(h->s, x, sizeof(float) * (size_t)L.d.n);
     smooth32(h, l, b, x, sweeps, 0, from_zero);
     if (l == 0) prof_begin(h, MG_PROF_RESID_RESTRICT);
     // after a pre-smoothing sweep (black last) every black residual is zero
@@ -381,8 +364,7 @@ void vcycle32(mg_handle *h, int l, const float *b, float *x, const OuterUpdate *
     Level &C = h->lv[l + 1];
     presmooth_restrict32(h, l, b, x, C.b32, h->o.pre, from_zero);
     if (l == 0) prof_begin(h, MG_PROF_COARSE_LEVELS);
-    if (l == 0 && h->tail_exec) replay_tail(h);
-    else vcycle32(h, l + 1, C.b32, C.x32);
+    vcycle32(h, l + 1, C.b32, C.x32);
     if (l == 0) prof_end(h);
     prolong_postsmooth32(h, l, b, C.x32, x, h->o.post, up);
 }
@@ -449,38 +431,6 @@ void bind_tail(mg_handle *h) {
     }
 }
 
-// Record levels 1 .. coarsest of one V-cycle (FP64 or FP32, as the handle's cycle) on a private
-// stream under capture; nothing runs.  Without a graph (capture or instantiation refused) the
-// cycle launches the kernels itself.
-void build_tail_graph(mg_handle *h) {
-    h->tail_exec = nullptr;
-    h->tail_launches = 0;
-    if (h->nlev < 2) return;
-    cudaStream_t cap = nullptr;
-    if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    cudaStream_t saved = h->s;
-    h->s = cap;
-    const unsigned long long l0 = mg::launches_total();
-    cudaGraph_t g = nullptr;
-    bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    if (ok) {
-        if (h->o.precision == MG_FP64) vcycle64(h, 1, h->lv[1].b64, h->lv[1].x64, true);
-        else vcycle32(h, 1, h->lv[1].b32, h->lv[1].x32);
-        ok = cudaStreamEndCapture(cap, &g) == cudaSuccess && g != nullptr;
-    }
-    const long long n = (long long)(mg::launches_total() - l0);
-    mg::count_launch((int)-n);  // recorded, not run
-    h->s = saved;
-    if (ok && cudaGraphInstantiate(&h->tail_exec, g, 0) != cudaSuccess) h->tail_exec = nullptr;
-    if (g) cudaGraphDestroy(g);
-    cudaStreamDestroy(cap);
-    cudaGetLastError();
-    h->tail_launches = h->tail_exec ? n : 0;
-}
-
 // ---- set-up of the operator hierarchy -------------------------------------------------
 int finish_operator(mg_handle *h) {
     cudaStream_t s = h->s;
@@ -532,7 +482,7 @@ void inner_fcg32(mg_handle *h, int k) {
     Level &F = h->lv[0];
     cudaStream_t s = h->s;
     const i64 n = F.d.n;
-    cudaMemsetAsync(F.x32, 0, sizeof(float) * (size_t)n, s);
+    mg::launch_zero(s, F.x32, sizeof(float) * (size_t)n);
     for (int j = 0; j < k; ++j) {
         const int rz_cur = (j & 1) ? mg::CG_RZ1 : mg::CG_RZ0, rz_prev = (j & 1) ? mg::CG_RZ0 : mg::CG_RZ1;
         vcycle32(h, 0, F.b32, h->cg_z32);  // z = V(r)
@@ -599,7 +549,7 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
     const bool fcg = h->o.method == MG_METHOD_FCG;
     double rr = 0.0;
     if (nb == 0.0) {
-        MG_CUDA(h, cudaMemsetAsync(p, 0, sizeof(double) * (size_t)n, s));
+        mg::launch_zero(s, p, sizeof(double) * (size_t)n);
         hist[hist_n++] = 0.0;
     } else {
         if (warm) {
@@ -608,7 +558,7 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
             MG_CUDA(h, cudaStreamSynchronize(s));
             mg::launch_add_const(s, n, p, -h->hred[4] / (double)n);
         } else {
-            MG_CUDA(h, cudaMemsetAsync(p, 0, sizeof(double) * (size_t)n, s));
+            mg::launch_zero(s, p, sizeof(double) * (size_t)n);
         }
         double scale = 1.0 / nb;  // r32 = scale * r (scale = 1 / previous residual norm)
         const bool fuse = mixed && h->nlev > 1 && h->o.post >= 1 && mg::half32_update_ok(F.lay);
@@ -793,14 +743,7 @@ namespace mg {
 Lay handle_lay32(mg_handle *h, int l) { return h->lv[l].lay; }
 float *handle_b32(mg_handle *h, int l) { return h->lv[l].b32; }
 float *handle_x32(mg_handle *h, int l) { return h->lv[l].x32; }
-void handle_vcycle32(mg_handle *h, int l, bool recording) {
-    // under a stream capture the coarse levels are recorded launch by launch, not as a replay
-    // of the handle's own graph
-    cudaGraphExec_t tail = h->tail_exec;
-    if (recording) h->tail_exec = nullptr;
-    vcycle32(h, l, h->lv[l].b32, h->lv[l].x32);
-    h->tail_exec = tail;
-}
+void handle_vcycle32(mg_handle *h, int l) { vcycle32(h, l, h->lv[l].b32, h->lv[l].x32); }
 int handle_first_inner() { return kFirstAdaptive; }
 int handle_next_inner(double rr_prev, double rr, int k, double rtol) { return next_inner(rr_prev, rr, k, rtol); }
 }  // namespace mg
@@ -953,7 +896,6 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
         return MG_ERR_CUDA;
     }
     bind_tail(h);
-    build_tail_graph(h);
     h->msg[0] = 0;
     *out = h;
     return MG_OK;
@@ -962,7 +904,6 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
 int mg_destroy(mg_handle *h) {
     if (!h) return MG_OK;
     cudaStreamSynchronize(h->s);
-    if (h->tail_exec) cudaGraphExecDestroy(h->tail_exec);
     if (h->pev) {
         for (int q = 0; q < kProfEvents; ++q) cudaEventDestroy(h->pev[q]);
         delete[] h->pev;
@@ -1007,7 +948,7 @@ int mg_set_density(mg_handle *h, const double *rho) {
     if (!rho) return fail(h, MG_ERR_ARG, "rho is NULL");
     h->have_op = 0;
     prof_begin(h, MG_PROF_SETUP);  // ended by finish_operator
-    MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->s));
+    mg::launch_zero(h->s, h->err, sizeof(unsigned));
     Level &F = h->lv[0];
     // s = 1/rho goes through the RHS buffer, which holds nothing between calls
     mg::launch_faces_from_rho(h->s, F.d, rho, h->bt, F.fx64, F.fy64, F.fz64, h->err);
@@ -1022,7 +963,7 @@ int mg_set_face_coeffs(mg_handle *h, const double *bx, const double *by, const d
     if (!bx || !by || !bz) return fail(h, MG_ERR_ARG, "face arrays must be non-null");
     h->have_op = 0;
     prof_begin(h, MG_PROF_SETUP);  // ended by finish_operator
-    MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->s));
+    mg::launch_zero(h->s, h->err, sizeof(unsigned));
     Level &F = h->lv[0];
     mg::launch_faces_from_api(h->s, F.d, bx, by, bz, F.fx64, F.fy64, F.fz64, h->err);
     h->sform0 = 0;

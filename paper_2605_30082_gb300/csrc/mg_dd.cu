@@ -61,6 +61,7 @@ struct Slab {
 // slab's planes and its ghost planes into the slab's colour-split layout, rounded to nearest as
 // the whole-grid pack rounds it; z0 is the slab's first whole-grid plane (even, so colours agree)
 __global__ void k_pack_slab_s32(mg::Lay L, int z0, int nz_total, const double *__restrict__ s_whole, float *s32) {
+    mg::grid_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= L.nx) return;
     const int rows = L.ny * (L.nz + 2);
@@ -77,6 +78,7 @@ __global__ void k_pack_slab_s32(mg::Lay L, int z0, int nz_total, const double *_
 // planes; for fz also the face to the ghost plane above, `planes` = nz + 1) into its colour-split
 // layout, rounded to nearest as the whole-grid pack rounds them
 __global__ void k_pack_slab_faces(mg::Lay L, int planes, const double *__restrict__ f, float *f32) {
+    mg::grid_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= L.nx) return;
     const int rows = L.ny * planes;
@@ -89,11 +91,13 @@ __global__ void k_pack_slab_faces(mg::Lay L, int planes, const double *__restric
 
 // out = (in - c) * scale, the mixed modes' scaled zero-mean right-hand side
 __global__ void k_sub_scalar_scale(mg::i64 n, const double *__restrict__ in, double c, double scale, double *out) {
+    mg::grid_wait();
     const mg::i64 m = (mg::i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m < n) out[m] = (in[m] - c) * scale;
 }
 
 __global__ void k_sub_scalar(mg::i64 n, const double *__restrict__ in, double c, double *out) {
+    mg::grid_wait();
     const mg::i64 m = (mg::i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (m < n) out[m] = in[m] - c;
 }
@@ -101,6 +105,7 @@ __global__ void k_sub_scalar(mg::i64 n, const double *__restrict__ in, double c,
 // the coarse low z faces of one plane from the 2 x 2 fine faces that tile them
 __global__ void k_coarsen_z_plane(mg::Dims f, mg::Dims c, const double *__restrict__ ffz_plane,
                                   double *cfz_plane) {
+    mg::grid_wait();
     const int C = blockIdx.x * blockDim.x + threadIdx.x;
     if (C >= c.nx * c.ny) return;
     const int I = C % c.nx, J = C / c.nx;
@@ -364,9 +369,8 @@ int half_mixed(mg_dd *dd, int l, int c, bool from_zero) {
 
 // One FP32 V-cycle from cut level l down, in the order of the whole-grid cycle: from x32 = 0
 // (from_zero) or from the slabs' x32; with alpha_shift (finest level), the last red half sweep
-// adds alpha x - shift to the slabs' FP64 p instead of storing x32.  `recording`: under a stream
-// capture (the whole-grid handle then records its levels launch by launch).
-int vcycle_mixed(mg_dd *dd, int l, bool from_zero, const double *alpha_shift, bool recording = false) {
+// adds alpha x - shift to the slabs' FP64 p instead of storing x32.
+int vcycle_mixed(mg_dd *dd, int l, bool from_zero, const double *alpha_shift) {
     std::vector<Slab> &R = dd->lv[l];
     const double h2 = h2_of(dd, l);
     int rc;
@@ -384,9 +388,9 @@ int vcycle_mixed(mg_dd *dd, int l, bool from_zero, const double *alpha_shift, bo
     });
     if (rc) return rc;
     if (l + 1 < dd->ndec) {
-        if ((rc = vcycle_mixed(dd, l + 1, true, nullptr, recording))) return rc;
+        if ((rc = vcycle_mixed(dd, l + 1, true, nullptr))) return rc;
     } else {
-        mg::handle_vcycle32(dd->ch, 0, recording);  // the switch level down, on the caller's stream
+        mg::handle_vcycle32(dd->ch, 0);  // the switch level down, on the caller's stream
     }
     // the prolongation back: the red cells of each slab from its coarse planes and those beside
     rc = per_rank(dd, [&](int r, cudaStream_t st) -> int {
@@ -462,7 +466,7 @@ void build_cycle_graph(mg_dd *dd) {
         return;
     }
     for (int k = 0; k < 2; ++k)
-        dd->mix_exec[k] = record_cycle(dd, [&] { return vcycle_mixed(dd, 0, k == 0, nullptr, true); }, &dd->mix_launches[k]);
+        dd->mix_exec[k] = record_cycle(dd, [&] { return vcycle_mixed(dd, 0, k == 0, nullptr); }, &dd->mix_launches[k]);
 }
 
 // one V-cycle of level 0 from the slabs' x: the recorded graph, or call by call
@@ -570,7 +574,7 @@ int solve_mixed(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     }
     for (Slab &S : R) {
         mg::count_launch();
-        k_sub_scalar_scale<<<blocks_for(S.d.n), kThreads, 0, s>>>(S.d.n, b + (size_t)S.z0 * S.d.nxy, sb / n, h2, S.b);
+        mg::run_kernel(k_sub_scalar_scale, blocks_for(S.d.n), kThreads, 0, s, S.d.n, b + (size_t)S.z0 * S.d.nxy, sb / n, h2, S.b);
         DD_CUDA(dd, cudaMemsetAsync(S.xe, 0, 8 * (size_t)(S.d.n + 2 * S.d.nxy), s));
     }
     double t, q0;
@@ -929,7 +933,7 @@ int mg_dd_set_density(mg_dd *dd, const double *rho) {
             const int rows = S.lay.ny * (S.lay.nz + 2);
             const dim3 grd((unsigned)((S.lay.nx + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
             mg::count_launch();
-            k_pack_slab_s32<<<grd, 128, 0, s>>>(S.lay, S.z0, dd->o.nz, dd->sinv, S.s32);
+            mg::run_kernel(k_pack_slab_s32, grd, 128, 0, s, S.lay, S.z0, dd->o.nz, dd->sinv, S.s32);
         }
     }
     // decomposed levels: diagonal, then the next level's faces slab by slab
@@ -940,9 +944,9 @@ int mg_dd_set_density(mg_dd *dd, const double *rho) {
             if (dd->mixed && l > 0) {  // the FP32 faces of a cut level below the finest
                 const dim3 grd((unsigned)((S.lay.nx + 127) / 128), (unsigned)std::min(S.lay.ny * (S.lay.nz + 1), 65535));
                 mg::count_launch(3);
-                k_pack_slab_faces<<<grd, 128, 0, s>>>(S.lay, S.lay.nz, S.fx, S.fx32);
-                k_pack_slab_faces<<<grd, 128, 0, s>>>(S.lay, S.lay.nz, S.fy, S.fy32);
-                k_pack_slab_faces<<<grd, 128, 0, s>>>(S.lay, S.lay.nz + 1, S.fze, S.fz32);
+                mg::run_kernel(k_pack_slab_faces, grd, 128, 0, s, S.lay, S.lay.nz, S.fx, S.fx32);
+                mg::run_kernel(k_pack_slab_faces, grd, 128, 0, s, S.lay, S.lay.nz, S.fy, S.fy32);
+                mg::run_kernel(k_pack_slab_faces, grd, 128, 0, s, S.lay, S.lay.nz + 1, S.fze, S.fz32);
             }
             mg::Dims cd = mg::make_dims(S.d.nx / 2, S.d.ny / 2, S.d.nz / 2);
             if (l + 1 < dd->ndec) {
@@ -950,7 +954,7 @@ int mg_dd_set_density(mg_dd *dd, const double *rho) {
                 mg::launch_coarsen(s, S.d, S.fx, S.fy, S.fze, C.fx, C.fy, C.fze);
                 // the face to the ghost above: from the fine faces to the fine ghost above
                 mg::count_launch();
-                k_coarsen_z_plane<<<blocks_for(cd.nxy), kThreads, 0, s>>>(S.d, cd, S.fze + S.d.n, C.fze + C.d.n);
+                mg::run_kernel(k_coarsen_z_plane, blocks_for(cd.nxy), kThreads, 0, s, S.d, cd, S.fze + S.d.n, C.fze + C.d.n);
             } else {
                 // the switch level is whole: the slabs' coarse planes side by side
                 const mg::i64 off = (mg::i64)(S.z0 / 2) * cd.nxy;
@@ -1021,7 +1025,7 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     }
     for (Slab &S : dd->lv[0]) {
         mg::count_launch();
-        k_sub_scalar<<<blocks_for(S.d.n), kThreads, 0, s>>>(S.d.n, b + (size_t)S.z0 * S.d.nxy, sb / n, S.b);
+        mg::run_kernel(k_sub_scalar, blocks_for(S.d.n), kThreads, 0, s, S.d.n, b + (size_t)S.z0 * S.d.nxy, sb / n, S.b);
         DD_CUDA(dd, cudaMemsetAsync(S.xe, 0, 8 * (size_t)(S.d.n + 2 * S.d.nxy), s));
     }
     double t, nb2;

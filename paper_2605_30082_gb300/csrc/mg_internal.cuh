@@ -184,12 +184,11 @@ cudaStream_t swap_handle_stream(mg_handle *h, cudaStream_t s);
 // A mixed-precision handle's FP32 level l, for the decomposed mixed cycle (mg_dd.cu), which
 // runs the levels from its switch level down on a whole-grid handle: the level's storage layout,
 // its right-hand side and iterate arrays, and one FP32 V-cycle of the handle from level l down
-// (from x = 0, on that level's b32, into its x32; the handle's options and recorded tail, or,
-// `recording` under a stream capture, the tail's launches one by one)
+// (from x = 0, on that level's b32, into its x32; the handle's options)
 Lay handle_lay32(mg_handle *h, int l);
 float *handle_b32(mg_handle *h, int l);
 float *handle_x32(mg_handle *h, int l);
-void handle_vcycle32(mg_handle *h, int l, bool recording = false);
+void handle_vcycle32(mg_handle *h, int l);
 // the adaptive inner-cycle count of the mixed outer loop: the first, and the next from the
 // contraction of the last outer iteration (k cycles from relres rr_prev to rr)
 int handle_first_inner();
@@ -416,6 +415,9 @@ void launch_zero_resid32(cudaStream_t s, Dims d, Lay L, const double *b, double 
 // p = p - shift + alpha * e32 (e32 in the level-0 FP32 layout L; shift a host scalar)
 void launch_update(cudaStream_t s, Dims d, Lay L, double *p, const float *e32, double alpha, double shift);
 void launch_add_const(cudaStream_t s, i64 n, double *p, double c);
+// zeroes `bytes` bytes (a multiple of 4) at p (4-byte aligned): a kernel, because a memset between two
+// kernels costs both of them the 2 us gap that run_kernel avoids
+void launch_zero(cudaStream_t s, void *p, size_t bytes);
 void launch_adjoint_grad(cudaStream_t s, Dims d, double h, const double *lam, const double *p,
                          const double *fx, const double *fy, const double *fz, const double *csfx,
                          const double *csfy, const double *csfz, double sigma, float *gx,
