@@ -58,7 +58,7 @@ FP64_NOMINAL_TFLOPS = 1.25
 # streaming kernels' traffic grows in proportion to the cells): `ncu --metrics
 # dram__bytes_read.sum,dram__bytes_write.sum` of paper_2605_30082_gb300/profile_case.py, the
 # summaries in profiles/.  A kernel changed since its capture has no entry (traffic null).
-NCU_DRAM_BYTES_PER_CELL = {"k_half_zs": 10.03, "k_half_z": 10.12, "k_fine_resid_pair": 54.3,
+NCU_DRAM_BYTES_PER_CELL = {"k_half_zr": 10.03, "k_fine_resid_pair": 54.3,
                            "k_resid_dfs": 28.1, "k_adjoint_grad_split2": 27.5}
 # Relative L2 distance to the exact discrete solution that the pressure must meet, and the
 # residual tolerance at which the headline (mixed) solve meets it on the 512^3 workload
@@ -556,10 +556,10 @@ def run_ours(args):
     gbs_sm = bytes_sm / (ms_sm * 1e-3) / 1e9
     roof_sm = {"bound": "hbm", "achieved": round(gbs_sm, 1), "peak": peak, "unit": "GB/s",
                "frac": round(gbs_sm / peak, 3),
-               "traffic": _traffic("k_half_zs", cells),
-               "kernel": "k_half_zs<16, 11> (finest-level FP32 red-black half sweep, z-marching, each plane's "
-                         "loads staged by cp.async two planes ahead; the one from-zero sweep per outer "
-                         "iteration is k_half_z)",
+               "traffic": _traffic("k_half_zr", cells),
+               "kernel": "k_half_zr (finest-level FP32 red-black half sweep, z-marching tiles of rows shared "
+                         "in shared memory, planes loaded by cp.async two ahead; the one from-zero sweep per "
+                         "outer iteration is k_half_z0)",
                "launch_ms": round(avg_sm, 4), "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
     n_fr, ms_fr = prof["fine_residual"]
     avg_fr = ms_fr / max(n_fr, 1)

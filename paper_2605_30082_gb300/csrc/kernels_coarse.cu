@@ -268,9 +268,8 @@ void launch_coarse_pinv(cudaStream_t s, Dims d, double ih2, const double *fx, co
     const int n = (int)d.n, tiles = (n + kPanel - 1) / kPanel;
     double *Pinv = scratch, *C = Pinv + kGj * kGj, *scal = C + (size_t)n * kGj;
     const int sms = device_sms();
-    // per device: the attribute is the current device's
-    if (cudaFuncSetAttribute(k_gj_trailing, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrailSmem) != cudaSuccess)
-        return;  // stays in the runtime's last error, which the caller checks
+    static std::atomic<unsigned long long> opted{0};
+    if (!opt_in_smem((const void *)k_gj_trailing, kTrailSmem, opted)) return;
     // fewer CTAs where there are fewer tiles (and at least the pivot cluster)
     const int live = (n + kTileRows - 1) / kTileRows * ((n + kGj - 1) / kGj) + 1, most = trailing_ctas();
     const int grid = live < most ? (live + kTrailCluster - 1) / kTrailCluster * kTrailCluster : most;

@@ -264,17 +264,15 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
     }
 }
 
-// ---- z-marching vectorised half sweep (split levels, hx % 4 == 0, hx / 4 >= 32) -----------
-// A warp covers 32 consecutive 4-cell vectors of one row.  Each thread walks ZC planes in z
-// and keeps the other colour's x (and s) of planes z-1, z and z+1 in registers, so each plane
-// of the other colour comes from memory once per sweep instead of three times (z-1, z, z+1).
-// The same-row window scalars (x at k0-1 and k0+4) come from the neighbouring lanes; the
-// lanes at a warp's edge load them.  Lanes past the end of a row, or rows past ny, compute on
-// clamped (in-bounds) indices and store nothing; all lanes of a warp share one row and one
-// z-range, so the shuffles are always converged.  Arithmetic per cell is that of k_half_vec.
-template <bool SFORM, bool FROM_ZERO, int UPDATE, int ZC, bool GHOST = false>
-__global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, const float *__restrict__ b,
-                                                    float *xv, int col, Upd up) {
+// ---- z-marching half sweep from zero (split levels, rows of a multiple of 32 vectors) --------
+// The first half sweep of a V-cycle from x = 0 reads no x: with num = 0 it is h^2 b over the sum of the
+// coefficients.  A warp covers 32 consecutive vectors of one row; a thread walks ZC planes and keeps
+// the other colour's s of planes z - 1, z and z + 1 in registers, so that each plane of it comes from
+// memory once; the window scalars come from the neighbouring lanes.  Lanes past the end of a row,
+// or rows past ny, compute on clamped (in-bounds) indices and store nothing.  512^3 166 us against 185 with
+// k_half_vec, 256^3 23.9 against 25.1, 256 x 128 x 128 5.0 against 5.6, below that the latter is faster.
+template <bool SFORM, int ZC, bool GHOST = false>
+__global__ void __launch_bounds__(64, 12) k_half_z0(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col) {
     grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     const int kvi = blockIdx.x * blockDim.x + threadIdx.x;
@@ -291,13 +289,8 @@ __global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, c
     i64 own = (i64)col * L.half + ((i64)z0 * L.ny + y) * hx + k0;
     const float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f);
     auto ld = [](const float *A, i64 off) { return *reinterpret_cast<const float4 *>(A + off); };
-    // planes z-1 and z of the other colour (x, and s in SFORM)
-    float4 xzm = f0, xzc = f0, szm = f0, szc = f0;
     const bool glo = GHOST && L.zlo, ghi = GHOST && L.zhi;  // a slab's ghost planes are neighbours
-    if (!FROM_ZERO) {
-        if (z0 > 0 || glo) xzm = ld(xv, opp - dz);
-        xzc = ld(xv, opp);
-    }
+    float4 szm = f0, szc = f0;
     if (SFORM) {
         if (z0 > 0 || glo) szm = ld(cf.s, opp - dz);
         szc = ld(cf.s, opp);
@@ -307,12 +300,6 @@ __global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, c
         const bool hz0 = z > 0 || glo, hz1 = z < L.nz - 1 || ghi;
         const int p = (col + y + z) & 1;  // x = 2k + p
         const bool xw0 = (p == 0 && !kl), xw1 = (p == 1 && !kr);
-        float4 xzp = f0, ym = f0, yp = f0;
-        if (!FROM_ZERO) {
-            if (hz1) xzp = ld(xv, opp + dz);
-            if (hy0) ym = ld(xv, opp - dy);
-            if (hy1) yp = ld(xv, opp + dy);
-        }
         float w0[4], w1[4], w2[4], w3[4], w4[4], w5[4];
         float4 szp = f0;
         if (SFORM) {
@@ -361,75 +348,12 @@ __global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, c
         const float4 b4 = ld(b, own);
         const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
         float out[4];
-        if (FROM_ZERO) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float den = ((w0[v] + w1[v]) + (w2[v] + w3[v])) + (w4[v] + w5[v]);
-                out[v] = __fdividef(hh * bv[v], den);
-            }
-        } else {
-            float xl = __shfl_up_sync(0xffffffffu, xzc.w, 1), xr = __shfl_down_sync(0xffffffffu, xzc.x, 1);
-            if (lane == 0) xl = kl ? xv[opp - 1] : 0.f;
-            if (lane == 31) xr = kr ? xv[opp + 4] : 0.f;
-            const float xo[4] = {xzc.x, xzc.y, xzc.z, xzc.w};
-            const float ymv[4] = {ym.x, ym.y, ym.z, ym.w}, ypv[4] = {yp.x, yp.y, yp.z, yp.w};
-            const float zmv[4] = {xzm.x, xzm.y, xzm.z, xzm.w}, zpv[4] = {xzp.x, xzp.y, xzp.z, xzp.w};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float xm = p ? xo[v] : (v ? xo[v - 1] : xl);
-                const float xp = (v == 3 && xw1) ? 0.f : (p ? (v < 3 ? xo[v + 1] : xr) : xo[v]);
-                float num = w0[v] * xm;
-                num += w1[v] * xp;
-                num += w2[v] * ymv[v];
-                num += w3[v] * ypv[v];
-                num += w4[v] * zmv[v];
-                num += w5[v] * zpv[v];
-                const float den = ((w0[v] + w1[v]) + (w2[v] + w3[v])) + (w4[v] + w5[v]);
-                out[v] = __fdividef(hh * bv[v] + num, den);
-            }
+        for (int v = 0; v < 4; ++v) {
+            const float den = ((w0[v] + w1[v]) + (w2[v] + w3[v])) + (w4[v] + w5[v]);
+            out[v] = __fdividef(hh * bv[v], den);
         }
-        if (active) {
-            if (UPDATE == 0) {
-                *reinterpret_cast<float4 *>(xv + own) = make_float4(out[0], out[1], out[2], out[3]);
-            } else {
-                // red at x = 2k + p, black at x = 2k + 1 - p; the black values are xzc
-                const float bk[4] = {xzc.x, xzc.y, xzc.z, xzc.w};
-                const i64 nat = ((i64)z * L.ny + y) * L.nx + 2 * k0;
-                if (UPDATE == 2) {
-                    const float al = up.alpha, sh = up.shift;
-                    float2 *pr = up.p2 + nat;
-                    // all loads before the first store: otherwise the four read-modify-writes
-                    // of the same row run one HBM round trip after another
-                    float4 pvs[4];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) pvs[v] = *reinterpret_cast<const float4 *>(pr + 2 * v);  // (h0, l0, h1, l1)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        float4 pv = pvs[v];
-                        const float e0 = p ? bk[v] : out[v], e1 = p ? out[v] : bk[v];
-                        df_add(pv.x, pv.y, fmaf(al, e0, -sh));
-                        df_add(pv.z, pv.w, fmaf(al, e1, -sh));
-                        *reinterpret_cast<float4 *>(pr + 2 * v) = pv;
-                    }
-                } else {
-                    // FP32 correction alpha e - shift, one FP64 addition per cell
-                    const float al = up.alpha, sh = up.shift;
-                    double *pr = up.p + nat;
-                    double2 pvs[4];  // all loads before the first store (see above)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) pvs[v] = *reinterpret_cast<const double2 *>(pr + 2 * v);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const double2 pv = pvs[v];
-                        const float e0 = p ? bk[v] : out[v], e1 = p ? out[v] : bk[v];
-                        *reinterpret_cast<double2 *>(pr + 2 * v) =
-                            make_double2(pv.x + f2d_exact(fmaf(al, e0, -sh)), pv.y + f2d_exact(fmaf(al, e1, -sh)));
-                    }
-                }
-            }
-        }
-        xzm = xzc;
-        xzc = xzp;
+        if (active) *reinterpret_cast<float4 *>(xv + own) = make_float4(out[0], out[1], out[2], out[3]);
         szm = szc;
         szc = szp;
         own += dz;
@@ -437,19 +361,56 @@ __global__ void __launch_bounds__(64, 12) k_half_z(Lay L, float h2, Coef32 cf, c
     }
 }
 
-// Staged form of k_half_z for the s-form regular sweep (the finest level's dominant kernel).
-// The per-plane loads of a thread (the other colour's rows y -+ 1 and their s, its own s and
-// b: six 16-byte vectors) travel by cp.async into a ring of kZsStages planes in shared memory,
-// issued kZsStages - 1 planes ahead of the plane being computed.  In flight they hold no
-// registers (121 registers for one plane held in registers, 80 here), so 11 blocks fit per SM
-// instead of 8, each with two planes of loads under way.  Every thread reads back only its
-// own copies: cp.async.wait_group is its only wait (no barrier, no spin), and a slot is
-// refilled only after the arithmetic that used it.  The other colour's row y (planes z -+ 1
-// and the window) still rolls through registers, the next plane's window scalars of the
-// warp's edge lanes too.  Arithmetic as k_half_z: bitwise the same results.
-constexpr int kZsStages = 3;
-constexpr int kZsFields = 6;  // ym, yp, s2 (= s at y - 1), s3 (y + 1), own s, own b
-constexpr size_t kZsSmem = (size_t)kZsStages * kZsFields * 64 * sizeof(float4);
+// Row-sharing half sweep for the s-form regular sweep (the finest level's dominant kernel).  A
+// block takes a tile of RY rows of W four-cell vectors (RY W <= kZrThreads, one vector per
+// thread) and marches ZC planes.  The other colour's x and s of the tile's rows and of the rows
+// above and below travel by cp.async into a ring of kZrStages planes in shared memory, two planes
+// ahead, with the cells' own s and b; every row is fetched once per block and read three times
+// (as y - 1, y and y + 1) from there.  A slot is refilled behind the block barrier that ends its plane.
+//
+// What bounded its predecessor (each thread fetching its own six vectors per plane) was the traffic between L2 and the SMs, 36 B per updated cell, and 87 instructions per cell: 215 us per 512^3
+// half sweep (6.24 TB/s of its 10 B per cell, 0.92 of the copy bandwidth) and, on grids that fit L2, no
+// more than 5.3 TB/s.  Sharing rows (28 B at W = 64, RY = 2; 24 B at W = 32, RY = 4), walls folded into
+// s (a missing neighbour's s is taken as -s, so that its weight is an exact 0) and packed FP32
+// pairs (f32x2) leave it bound by HBM: 194 us, 6.92 TB/s; 512 x 512 x 64 38.4 -> 28 us, x 32 19.8 -> 12.7 us.  More rows per block
+// (4 of 64 vectors) gave 202 us, one 206 us, three stages 219 us, five 197 us.
+//
+// Blocks of black sweeps take the planes from above, so that a sweep begins with the planes the one
+// before it left in L2 (512 x 512 x 64: 28.4 -> 25.8 us; nothing at 512^3).  Arithmetic as
+// k_half_vec: bitwise the same results.
+constexpr int kZrThreads = 128, kZrStages = 4, kZrBlocks = 4;  // blocks per SM
+constexpr int kZrMaxSmem = 56 * 1024;                            // per block
+constexpr int kZrMinVec = 4;                                     // vectors per row
+constexpr i64 kZrFullCells = 3500000, kZrCells = 7000000;        // see run_half_zr
+struct ZrTile {
+    int w, ry, zc;  // vectors per row, rows and planes of a tile
+    int pitch;      // row stride in shared memory: whole 128 B lines, as cp.async writes them
+    int slot;       // float4 of one plane's slot: ry + 2 rows of x and of s, own s and b, and (rows in
+                    // several tiles) the vectors beside the tile's rows
+};
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -459,159 +420,225 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// 64 threads per block (64 vectors of one row, or 32 of two rows), ZC planes per block
-template <int ZC, int MINB, bool GHOST = false>
-__global__ void __launch_bounds__(64, MINB) k_half_zs(Lay L, float h2, const float *__restrict__ sv,
-                                                       const float *__restrict__ b, float *xv, int col) {
+template <bool GHOST>
+__global__ void __launch_bounds__(kZrThreads, kZrBlocks) k_half_zr(Lay L, ZrTile T, float h2, const float *__restrict__ sv,
+                                                                   const float *__restrict__ b, float *xv, int col) {
+    extern __shared__ float4 ring[];
     grid_wait();
-    extern __shared__ float4 stg[];  // [kZsStages][kZsFields][64 threads]
-    constexpr int D = kZsStages;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int hx = L.hx, kv = hx >> 2;
-    const int kvi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int yi = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool active = kvi < kv && yi < L.ny;
-    const int k0 = min(kvi, kv - 1) << 2;
-    const int y = min(yi, L.ny - 1);
-    const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, L.nz);
-    const int lane = threadIdx.x & 31;
+    constexpr int D = kZrStages;
+    const int tid = threadIdx.x, lane = tid & 31, hx = L.hx, kv = hx >> 2, pitch = T.pitch;
+    const int r = min(tid / T.w, T.ry - 1), v = tid % T.w;  // row and vector in the tile
+    const int yb = blockIdx.y * T.ry, vb = blockIdx.x * T.w;
+    const bool act = tid < T.ry * T.w && yb + r < L.ny && vb + v < kv;
+    const int y = min(yb + r, L.ny - 1), k0 = min(vb + v, kv - 1) << 2;
+    const int zb = col ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
+    const int z0 = zb * T.zc, z1 = min(z0 + T.zc, L.nz);
     const i64 dy = hx, dz = (i64)L.ny * hx;
-    const bool hy0 = y > 0, hy1 = y < L.ny - 1;
-    const bool kl = k0 > 0, kr = k0 + 4 < hx;
-    const i64 row0 = ((i64)z0 * L.ny + y) * hx + k0;
-    const i64 opp0 = (i64)(1 - col) * L.half + row0;
-    const i64 own0 = (i64)col * L.half + row0;
+    const i64 row0 = (i64)y * hx + k0;
+    const i64 opp0 = (i64)(1 - col) * L.half + row0, own0 = (i64)col * L.half + row0;
+    const bool glo = GHOST && L.zlo, ghi = GHOST && L.zhi;  // a slab's ghost planes are neighbours
+    const int zend = L.nz + (ghi ? 1 : 0);                  // planes readable above
+    const bool hy0 = y > 0, hy1 = y < L.ny - 1, kl = k0 > 0, kr = k0 + 4 < hx;
+    // who fetches the rows and vectors beside the tile
+    const bool top = act && r == T.ry - 1 && hy1, bottom = act && r == 0 && hy0;
+    const bool left = act && v == 0 && kl, right = act && v == T.w - 1 && kr;
+    // whose x - 1 and x + 1 come from a neighbouring lane
+    const bool lsh = lane > 0 && v > 0, rsh = lane < 31 && v < T.w - 1;
     const float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto ld = [](const float *A, i64 off) { return *reinterpret_cast<const float4 *>(A + off); };
-    auto slot = [&](int st, int f) { return stg + (st * kZsFields + f) * 64 + tid; };
-    // plane z0 + t into stage t % D (rows outside the grid are not copied; their slots are
-    // never read)
-    auto issue = [&](int t) {
-        const i64 o = opp0 + (i64)t * dz, w = own0 + (i64)t * dz;
-        const int st = t % D;
-        if (hy0) {
-            cp_async16(slot(st, 0), xv + o - dy);
-            cp_async16(slot(st, 2), sv + o - dy);
-        }
-        if (hy1) {
-            cp_async16(slot(st, 1), xv + o + dy);
-            cp_async16(slot(st, 3), sv + o + dy);
-        }
-        cp_async16(slot(st, 4), sv + w);
-        cp_async16(slot(st, 5), b + w);
-    };
-    // the window scalars beyond the warp's edge lanes (lane 0: x - 1, lane 31: x + 4)
-    auto scalars = [&](i64 o, float &xl, float &sl, float &xr, float &sr) {
-        xl = sl = xr = sr = 0.f;
-        if (lane == 0 && kl) {
-            xl = xv[o - 1];
-            sl = sv[o - 1];
-        }
-        if (lane == 31 && kr) {
-            xr = xv[o + 4];
-            sr = sv[o + 4];
-        }
-    };
-    // other colour, row y: planes z-1, z, z+1 (rolling); a slab's ghost planes are neighbours
-    const bool glo = GHOST && L.zlo, ghi = GHOST && L.zhi;
-    const int zend = L.nz + (ghi ? 1 : 0);  // planes readable above: the ghost plane too
-    float4 xzm = (z0 > 0 || glo) ? ld(xv, opp0 - dz) : f0, xzc = ld(xv, opp0);
-    float4 szm = (z0 > 0 || glo) ? ld(sv, opp0 - dz) : f0, szc = ld(sv, opp0);
-    float4 xzp = z0 + 1 < zend ? ld(xv, opp0 + dz) : f0, szp = z0 + 1 < zend ? ld(sv, opp0 + dz) : f0;
-#pragma unroll
-    for (int t = 0; t < D - 1; ++t) {
-        if (z0 + t < z1) issue(t);
-        cp_async_commit();  // one group per plane, empty past the chunk: the counting stays uniform
-    }
-    float cxl, csl, cxr, csr;
-    scalars(opp0, cxl, csl, cxr, csr);
-    const float hh = 2.f * h2;
-    for (int z = z0; z < z1; ++z) {
-        const int t = z - z0;
-        if (z + D - 1 < z1) issue(t + D - 1);
-        cp_async_commit();
-        const i64 opp = opp0 + (i64)t * dz, own = own0 + (i64)t * dz;
-        float nxl = 0.f, nsl = 0.f, nxr = 0.f, nsr = 0.f;
-        float4 xzpp = f0, szpp = f0;
-        if (z + 1 < z1) {
-            scalars(opp + dz, nxl, nsl, nxr, nsr);
-            if (z + 2 < zend) {
-                xzpp = ld(xv, opp + 2 * dz);
-                szpp = ld(sv, opp + 2 * dz);
+    const int nrow = (T.ry + 2) * pitch;  // x rows, then s rows, own s, own b
+    float4 *const mine = ring + (r + 1) * pitch + v, *const own = ring + 2 * nrow + tid;
+    float4 *const beside = ring + 2 * nrow + 2 * kZrThreads + 4 * r;  // x and s left of the tile's row, right of it
+    // plane z into its slot: x and s for plane z1 too, which the last plane reads as z + 1 (what lies
+    // beside the grid is not fetched and not read)
+    auto issue = [&](int z) {
+        if (act && z < zend && z <= z1) {
+            float4 *x = mine + (z % D) * T.slot, *s = x + nrow;
+            const float *gx = xv + opp0 + (i64)z * dz, *gs = sv + opp0 + (i64)z * dz;
+            cp_async16(x, gx);
+            cp_async16(s, gs);
+            if (z < z1) {
+                const i64 w = own0 + (i64)z * dz;
+                cp_async16(own + (z % D) * T.slot, sv + w);
+                cp_async16(own + (z % D) * T.slot + kZrThreads, b + w);
+                if (bottom) {
+                    cp_async16(x - pitch, gx - dy);
+                    cp_async16(s - pitch, gs - dy);
+                }
+                if (top) {
+                    cp_async16(x + pitch, gx + dy);
+                    cp_async16(s + pitch, gs + dy);
+                }
+                if (left) {
+                    cp_async16(beside + (z % D) * T.slot, gx - 4);
+                    cp_async16(beside + (z % D) * T.slot + 1, gs - 4);
+                }
+                if (right) {
+                    cp_async16(beside + (z % D) * T.slot + 2, gx + 4);
+                    cp_async16(beside + (z % D) * T.slot + 3, gs + 4);
+                }
             }
         }
-        cp_async_wait<D - 1>();  // all but the D - 1 newest groups done: plane z has landed
-        const int st = t % D;
-        const float4 cym = hy0 ? *slot(st, 0) : f0, cyp = hy1 ? *slot(st, 1) : f0;
-        const float4 cs2 = hy0 ? *slot(st, 2) : f0, cs3 = hy1 ? *slot(st, 3) : f0;
-        const float4 csc = *slot(st, 4), cbb = *slot(st, 5);
-        const bool hz0 = z > 0 || glo, hz1 = z < L.nz - 1 || ghi;
-        const int p = (col + y + z) & 1;  // x = 2k + p
-        const bool xw0 = (p == 0 && !kl), xw1 = (p == 1 && !kr);
-        float sl = __shfl_up_sync(0xffffffffu, szc.w, 1), sr = __shfl_down_sync(0xffffffffu, szc.x, 1);
-        float xl = __shfl_up_sync(0xffffffffu, xzc.w, 1), xr = __shfl_down_sync(0xffffffffu, xzc.x, 1);
-        if (lane == 0) {
-            sl = csl;
-            xl = cxl;
-        }
-        if (lane == 31) {
-            sr = csr;
-            xr = cxr;
-        }
-        const float so[4] = {szc.x, szc.y, szc.z, szc.w}, sc[4] = {csc.x, csc.y, csc.z, csc.w};
-        const float s2v[4] = {cs2.x, cs2.y, cs2.z, cs2.w}, s3v[4] = {cs3.x, cs3.y, cs3.z, cs3.w};
-        const float s4v[4] = {szm.x, szm.y, szm.z, szm.w}, s5v[4] = {szp.x, szp.y, szp.z, szp.w};
-        const float xov[4] = {xzc.x, xzc.y, xzc.z, xzc.w};
-        const float ymv[4] = {cym.x, cym.y, cym.z, cym.w}, ypv[4] = {cyp.x, cyp.y, cyp.z, cyp.w};
-        const float zmv[4] = {xzm.x, xzm.y, xzm.z, xzm.w}, zpv[4] = {xzp.x, xzp.y, xzp.z, xzp.w};
-        const float bv[4] = {cbb.x, cbb.y, cbb.z, cbb.w};
-        float out[4];
+        cp_async_commit();  // one group per plane, empty past the chunk: the counting stays uniform
+    };
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float sm = p ? so[v] : (v ? so[v - 1] : sl);
-            const float sp = p ? (v < 3 ? so[v + 1] : sr) : so[v];
-            const float w0 = (v == 0 && xw0) ? 0.f : sc[v] + sm;
-            const float w1 = (v == 3 && xw1) ? 0.f : sc[v] + sp;
-            const float w2 = hy0 ? sc[v] + s2v[v] : 0.f;
-            const float w3 = hy1 ? sc[v] + s3v[v] : 0.f;
-            const float w4 = hz0 ? sc[v] + s4v[v] : 0.f;
-            const float w5 = hz1 ? sc[v] + s5v[v] : 0.f;
-            const float xm = p ? xov[v] : (v ? xov[v - 1] : xl);
-            const float xp = (v == 3 && xw1) ? 0.f : (p ? (v < 3 ? xov[v + 1] : xr) : xov[v]);
-            float num = w0 * xm;
-            num += w1 * xp;
-            num += w2 * ymv[v];
-            num += w3 * ypv[v];
-            num += w4 * zmv[v];
-            num += w5 * zpv[v];
-            const float den = ((w0 + w1) + (w2 + w3)) + (w4 + w5);
-            out[v] = __fdividef(hh * bv[v] + num, den);
+    for (int q = 0; q < D - 1; ++q) issue(z0 + q);
+    auto ld = [](const float *A, i64 off) { return *reinterpret_cast<const float4 *>(A + off); };
+    const bool below = z0 > 0 || glo;
+    float4 xzm = below ? ld(xv, opp0 + (i64)(z0 - 1) * dz) : f0, szm = below ? ld(sv, opp0 + (i64)(z0 - 1) * dz) : f0;
+    float4 xzc = f0, szc = f0;
+    const float hh = 2.f * h2;
+    for (int z = z0; z < z1; ++z) {
+        cp_async_wait<D - 3>();  // planes z and z + 1 have landed
+        __syncthreads();         // for every thread, and plane z - 1 has been read by all
+        issue(z + D - 1);        // into the slot of plane z - 1
+        const float4 *x = mine + (z % D) * T.slot, *s = x + nrow;
+        const float4 *xn = mine + ((z + 1) % D) * T.slot, *sn = xn + nrow;
+        if (z == z0) {
+            xzc = *x;
+            szc = *s;
         }
-        if (active) __stcs(reinterpret_cast<float4 *>(xv + own), make_float4(out[0], out[1], out[2], out[3]));  // streaming store
+        float4 xzp = f0, szp = f0, ym = f0, yp = f0;
+        const float4 sc = own[(z % D) * T.slot], bv = own[(z % D) * T.slot + kZrThreads];
+        // beyond a wall x = 0 and s = -s of the cell, so that the weight s + s is an exact 0
+        const float4 ns = make_float4(-sc.x, -sc.y, -sc.z, -sc.w);
+        float4 s2 = ns, s3 = ns, s4 = szm, s5 = ns;
+        if (z + 1 < zend) {
+            xzp = *xn;
+            szp = s5 = *sn;
+        }
+        if (hy0) {
+            ym = x[-pitch];
+            s2 = s[-pitch];
+        }
+        if (hy1) {
+            yp = x[pitch];
+            s3 = s[pitch];
+        }
+        if (z == 0 && !glo) s4 = ns;
+        // x - 1 and x + 1: the own vector shifted by one cell or not (x = 2k + p)
+        float4 xm = xzc, xp = xzc, sm = szc, sp = szc;
+        const bool p = (col + y + z) & 1;
+        // lanes of one warp may hold rows of both parities: both shuffles
+        float xr = __shfl_down_sync(0xffffffffu, xzc.x, 1), sr = __shfl_down_sync(0xffffffffu, szc.x, 1);
+        float xl = __shfl_up_sync(0xffffffffu, xzc.w, 1), sl = __shfl_up_sync(0xffffffffu, szc.w, 1);
+        if (p) {
+            if (!rsh && kr) {
+                const float4 *e = beside + (z % D) * T.slot + 2;
+                xr = v == T.w - 1 ? e[0].x : x[1].x;
+                sr = v == T.w - 1 ? e[1].x : s[1].x;
+            }
+            if (!kr) {
+                xr = 0.f;
+                sr = ns.w;
+            }
+            xp = make_float4(xzc.y, xzc.z, xzc.w, xr);
+            sp = make_float4(szc.y, szc.z, szc.w, sr);
+        } else {
+            if (!lsh && kl) {
+                const float4 *e = beside + (z % D) * T.slot;
+                xl = v == 0 ? e[0].w : x[-1].w;
+                sl = v == 0 ? e[1].w : s[-1].w;
+            }
+            if (!kl) {
+                xl = 0.f;
+                sl = ns.x;
+            }
+            xm = make_float4(xl, xzc.x, xzc.y, xzc.z);
+            sm = make_float4(sl, szc.x, szc.y, szc.z);
+        }
+        float4 out;
+        auto pair = [&](f32x2 c, f32x2 bq, f32x2 a0, f32x2 a1, f32x2 a2, f32x2 a3, f32x2 a4, f32x2 a5, f32x2 v0, f32x2 v1,
+                        f32x2 v2, f32x2 v3, f32x2 v4, f32x2 v5, float &o0, float &o1) {
+            const f32x2 w0 = add2(c, a0), w1 = add2(c, a1), w2 = add2(c, a2), w3 = add2(c, a3), w4 = add2(c, a4), w5 = add2(c, a5);
+            f32x2 num = fma2(w0, v0, mul2(w1, v1));
+            num = fma2(w2, v2, num);
+            num = fma2(w3, v3, num);
+            num = fma2(w4, v4, num);
+            num = fma2(w5, v5, num);
+            num = fma2(pack2(hh, hh), bq, num);
+            const f32x2 den = add2(add2(add2(w0, w1), add2(w2, w3)), add2(w4, w5));
+            float n0, n1, d0, d1;
+            unpack2(num, n0, n1);
+            unpack2(den, d0, d1);
+            o0 = __fdividef(n0, d0);
+            o1 = __fdividef(n1, d1);
+        };
+        auto lo = [](const float4 &q) { return pack2(q.x, q.y); };
+        auto up = [](const float4 &q) { return pack2(q.z, q.w); };
+        pair(lo(sc), lo(bv), lo(sm), lo(sp), lo(s2), lo(s3), lo(s4), lo(s5), lo(xm), lo(xp), lo(ym), lo(yp), lo(xzm), lo(xzp),
+             out.x, out.y);
+        pair(up(sc), up(bv), up(sm), up(sp), up(s2), up(s3), up(s4), up(s5), up(xm), up(xp), up(ym), up(yp), up(xzm), up(xzp),
+             out.z, out.w);
+        if (act) *reinterpret_cast<float4 *>(xv + own0 + (i64)z * dz) = out;
         xzm = xzc;
         xzc = xzp;
-        xzp = xzpp;
         szm = szc;
         szc = szp;
-        szp = szpp;
-        cxl = nxl;
-        csl = nsl;
-        cxr = nxr;
-        csr = nsr;
     }
-    cp_async_wait<0>();  // only empty groups can remain; leave none behind
+    cp_async_wait<0>();  // only copies that nothing reads can remain; leave none behind
 }
 
-// Staged form of k_half_z for the face-form regular sweep (the levels below the finest, whose
+// Tiles of k_half_zr.  A tile that uses all of a block's threads comes first, then one that holds whole
+// rows (no vectors beside it), then a wide one; widths other than the whole row are multiples of 128 B.
+// 384^3 (48 vectors per row) takes 89.8 us in tiles of 16 x 8, 94 in 24 x 5, 99 in 48 x 2; 576 x 512 x 448 (72) 213 us in
+// 24 x 5, 221 in 16 x 8, 228 in 36 x 3; 448^3 (56) 143 us in 32 x 4, 147 in 56 x 2, 155 in 16 x 8.
+// Planes: the most up to 16 (fewer re-read boundary planes) that still give 1.6 waves of blocks, at least 4.
+ZrTile zr_tile(const Lay &L) {
+    ZrTile T;
+    const int kv = L.hx / 4;
+    int best = 0, parts = 1;
+    T.w = 1;
+    for (int w = 64; w >= 8; w -= 8) {
+        for (int q = 0; q < 2; ++q) {  // whole rows of up to 64 vectors (tried once, at w = 64), then w
+            const int cand = q == 0 ? kv : w;
+            if (q == 0 ? (w != 64 || kv > 64) : (cand >= kv || cand < 16)) continue;
+            const int n = (kv + cand - 1) / cand;
+            // per mille of the threads in use, times 1.1 for whole rows
+            const int score = (q == 0 ? 1100 : 1000) * (kv * (kZrThreads / cand)) / (n * kZrThreads);
+            if (score > best) {
+                best = score;
+                T.w = cand;
+                parts = n;
+            }
+        }
+    }
+    T.ry = kZrThreads / T.w;
+    const i64 xy = (i64)parts * ((L.ny + T.ry - 1) / T.ry);
+    const i64 want = (i64)device_sms() * kZrBlocks * 8 / 5;
+    T.zc = 16;
+    while (T.zc > 4 && xy * ((L.nz + T.zc - 1) / T.zc) < want) T.zc /= 2;
+    T.pitch = (T.w + 7) & ~7;
+    T.slot = 2 * (T.ry + 2) * T.pitch + 2 * kZrThreads + (parts > 1 ? 4 * T.ry : 0);
+    return T;
+}
+
+// Whether the s-form regular sweep of L goes to k_half_zr (and its launch).  Below these sizes
+// the whole level sits in L2 and k_half_vec, which loads everything at once, is as fast or faster: rows of
+// 32 vectors (every thread in use) 256 x 128 x 64 4.9 us against 5.0, 256 x 128 x 128 8.1 against 7.6, x 192 11.9 against 11.0; rows of 20 to
+// 28 vectors 160^3 8.8 against 9.5, 192^3 14.6 against 14.4, 224^3 27.7 against 22.5.
+template <bool GHOST>
+bool run_half_zr(cudaStream_t s, const Lay &L, float h2, const float *sv, const float *b, float *x, int col) {
+    const int kv = L.hx / 4;
+    if (!L.split || L.hx % 4 != 0 || kv < kZrMinVec) return false;
+    const ZrTile T = zr_tile(L);
+    if (L.n < (T.w * T.ry == kZrThreads ? kZrFullCells : kZrCells)) return false;
+    static std::atomic<unsigned long long> opted{0};
+    if (!opt_in_smem((const void *)k_half_zr<GHOST>, kZrMaxSmem, opted)) return true;  // the caller checks the error
+    run_kernel(k_half_zr<GHOST>, dim3((kv + T.w - 1) / T.w, (L.ny + T.ry - 1) / T.ry, (L.nz + T.zc - 1) / T.zc), kZrThreads,
+               (size_t)kZrStages * T.slot * sizeof(float4), s, L, T, h2, sv, b, x, col);
+    return true;
+}
+
+// Staged z-marching half sweep for the face-form regular sweep (the levels below the finest, whose
 // coarsened faces are stored per face, and a finest level loaded from face coefficients).  A
 // thread's nine per-plane vectors -- the other colour's x in rows y -+ 1, the other colour's
 // low x faces (its cells' high x faces), its own low x, y and z faces, the other colour's low
 // y faces in row y + 1 and low z faces in plane z + 1 (its high y and z faces), its own b --
 // travel by cp.async into a ring of kZfStages planes in shared memory, one plane ahead of the
-// plane being computed, as in k_half_zs; the other colour's row y (planes z -+ 1) rolls
+// plane being computed, as in k_half_zr; the other colour's row y (planes z -+ 1) rolls
 // through registers, the window scalars of the warp's edge lanes are loaded one plane ahead.
 // Every thread reads back only its own copies after cp.async.wait_group (no barrier, no spin).
-// Arithmetic as k_half_z, in the same order: bitwise the same results.
+// Arithmetic as k_half_vec, in the same order: bitwise the same results.
 constexpr int kZfStages = 2;
 constexpr int kZfFields = 9;  // ym, yp, fo, own fx, fy, fz, fy at y + 1, fz at z + 1, own b
 constexpr size_t kZfSmem = (size_t)kZfStages * kZfFields * 64 * sizeof(float4);
@@ -738,51 +765,50 @@ __global__ void __launch_bounds__(64, MINB) k_half_zf(Lay L, float h2, Coef32 cf
     cp_async_wait<0>();  // only empty groups can remain; leave none behind
 }
 
-bool half_z_ok(const Lay &L) { return L.split && L.hx % 4 == 0 && L.hx / 4 >= 32; }
+// rows of whole warps of vectors
+bool full_rows(const Lay &L) { return L.split && L.hx % 128 == 0; }
 
-// 16 planes per thread where that still gives about 4 waves of 64-thread blocks (12 resident
-// per SM, on the device's SM count), else 4
-template <bool SFORM, bool FROM_ZERO, int UPDATE, bool GHOST = false>
-void run_half_z(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col,
-                const Upd &up) {
-    const int kv = L.hx / 4;
-    const int vb = (kv % 64 == 0) ? 64 : 32;  // lanes per row
-    const int ry = 64 / vb;                    // rows per block
-    const unsigned gx = (kv + vb - 1) / vb, gy = (L.ny + ry - 1) / ry;
-    const dim3 blk(vb, ry);
-    const i64 sms = device_sms();
-    // a slab's launch runs beside the other slabs' ones: it needs about one wave by itself
-    if (SFORM && !FROM_ZERO && UPDATE == 0 && (i64)gx * gy * ((L.nz + 15) / 16) >= (GHOST ? 1 : 4) * sms * 8) {
-        // 11 blocks x 18 KB of staging per SM: ask for the largest shared-memory carveout
-        static const bool carveout = [] {
-            // a preference only: the launch is valid either way
-            if (cudaFuncSetAttribute(k_half_zs<16, 11, GHOST>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-                (void)cudaGetLastError();
-            return true;
-        }();
-        (void)carveout;
-        run_kernel(k_half_zs<16, 11, GHOST>, dim3(gx, gy, (L.nz + 15) / 16), blk, kZsSmem, s, L, h2, cf.s, b, x, col);
-        return;
+// blocks of 64 threads over the vectors (x) and rows (y) of a level with full rows, zc planes each
+void row_grid(const Lay &L, int zc, dim3 &grid, dim3 &block) {
+    const int kv = L.hx / 4, vb = (kv % 64 == 0) ? 64 : 32, ry = 64 / vb;
+    block = dim3(vb, ry);
+    grid = dim3(kv / vb, (L.ny + ry - 1) / ry, (L.nz + zc - 1) / zc);
+}
+
+// The first half sweep from zero of a level with full rows and at least 4 M cells: k_half_z0, 16 planes per thread
+// where that still gives about 4 waves of 64-thread blocks (12 resident per SM), else 4.  False: not one of its levels.
+template <bool SFORM, bool GHOST>
+bool run_half_z0(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col) {
+    if (!full_rows(L) || L.n < 4000000) return false;
+    dim3 grid, block;
+    row_grid(L, 16, grid, block);
+    if ((i64)grid.x * grid.y * grid.z >= (i64)4 * device_sms() * 12) {
+        run_kernel(k_half_z0<SFORM, 16, GHOST>, grid, block, 0, s, L, h2, cf, b, x, col);
+    } else {
+        row_grid(L, 4, grid, block);
+        run_kernel(k_half_z0<SFORM, 4, GHOST>, grid, block, 0, s, L, h2, cf, b, x, col);
     }
-    // the face form's regular sweeps, staged, where the grid gives at least four waves of
-    // 4-plane blocks (11 blocks x 18 KB of staging per SM, as k_half_zs)
-    if (!SFORM && !FROM_ZERO && UPDATE == 0 && !GHOST && (i64)gx * gy * ((L.nz + 3) / 4) >= 4 * sms * 11) {
-        static const bool carveout = [] {
-            // a preference only: the launch is valid either way
-            if (cudaFuncSetAttribute(k_half_zf<4, 11>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-                (void)cudaGetLastError();
-            return true;
-        }();
-        (void)carveout;
-        run_kernel(k_half_zf<4, 11>, dim3(gx, gy, (L.nz + 3) / 4), blk, kZfSmem, s, L, h2, cf, b, x, col);
-        return;
-    }
-    if ((i64)gx * gy * ((L.nz + 15) / 16) >= 4 * sms * 12)
-        run_kernel(k_half_z<SFORM, FROM_ZERO, UPDATE, 16, GHOST>, dim3(gx, gy, (L.nz + 15) / 16), blk, 0, s, L, h2, cf, b, x, col, up);
-    else
-        run_kernel(k_half_z<SFORM, FROM_ZERO, UPDATE, 4, GHOST>, dim3(gx, gy, (L.nz + 3) / 4), blk, 0, s, L, h2, cf, b, x, col, up);
+    return true;
+}
+
+// The face form's regular sweeps, staged, on levels with full rows that give at least four waves of 4-plane
+// blocks (11 blocks x 18 KB of staging per SM): 256^3 43.6 us against 52 with k_half_vec, 384^3 145 against 169;
+// 256 x 128 x 128 has too few blocks (8.6 against 8.8), and rows that leave lanes idle are slower (288^3 103 against 73).
+bool run_half_zf(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col) {
+    if (!full_rows(L)) return false;
+    dim3 grid, block;
+    row_grid(L, 4, grid, block);
+    if ((i64)grid.x * grid.y * grid.z < (i64)4 * device_sms() * 11) return false;
+    static const bool carveout = [] {
+        // a preference only: the launch is valid either way
+        if (cudaFuncSetAttribute(k_half_zf<4, 11>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            (void)cudaGetLastError();
+        return true;
+    }();
+    (void)carveout;
+    run_kernel(k_half_zf<4, 11>, grid, block, kZfSmem, s, L, h2, cf, b, x, col);
+    return true;
 }
 
 // ---- vectorised red-only residual + restriction (split fine level, hx % 4 == 0) ----------
@@ -1202,25 +1228,19 @@ Lay make_lay(Dims d) {
     return L;
 }
 
-// a slab (L.zlo / L.zhi): split layout with hx % 4 == 0 (the decomposed mixed cycle); s-form
-// (the finest level) or face form (the face arrays with their ghost plane above)
-template <bool SFORM>
-void half32_slab(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col,
-                 bool from_zero) {
-    if (half_z_ok(L)) {
-        if (from_zero) run_half_z<SFORM, true, 0, true>(s, L, h2, cf, b, x, col, Upd{});
-        else run_half_z<SFORM, false, 0, true>(s, L, h2, cf, b, x, col, Upd{});
+// one half sweep of a split level with hx % 4 == 0.  GHOST: a slab (L.zlo / L.zhi) of the decomposed
+// mixed cycle, its ghost planes as z neighbours (the face arrays with their ghost plane above)
+template <bool SFORM, bool GHOST>
+void half32_vec(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col, bool from_zero) {
+    const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
+    if (from_zero) {
+        if (!run_half_z0<SFORM, GHOST>(s, L, h2, cf, b, x, col))
+            run_kernel(k_half_vec<SFORM, true, 0, GHOST>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
         return;
     }
-    const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
-    if (from_zero) run_kernel(k_half_vec<SFORM, true, 0, true>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
-    else run_kernel(k_half_vec<SFORM, false, 0, true>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
-}
-
-void launch_half32_slab(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col,
-                        bool from_zero) {
-    if (cf.s) half32_slab<true>(s, L, h2, cf, b, x, col, from_zero);
-    else half32_slab<false>(s, L, h2, cf, b, x, col, from_zero);
+    if (SFORM && run_half_zr<GHOST>(s, L, h2, cf.s, b, x, col)) return;
+    if (!SFORM && !GHOST && run_half_zf(s, L, h2, cf, b, x, col)) return;
+    run_kernel(k_half_vec<SFORM, false, 0, GHOST>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
 }
 
 void launch_half32(cudaStream_t s, Lay L, double h2, const float *sinv, const float *fx, const float *fy,
@@ -1228,26 +1248,11 @@ void launch_half32(cudaStream_t s, Lay L, double h2, const float *sinv, const fl
     Coef32 cf{sinv, fx, fy, fz};
     count_launch();
     if (L.zlo || L.zhi) {
-        launch_half32_slab(s, L, (float)h2, cf, b, x, col, from_zero);
-        return;
-    }
-    if (half_z_ok(L)) {
-        if (sinv) {
-            if (from_zero) run_half_z<true, true, 0>(s, L, (float)h2, cf, b, x, col, Upd{});
-            else run_half_z<true, false, 0>(s, L, (float)h2, cf, b, x, col, Upd{});
-        } else {
-            if (from_zero) run_half_z<false, true, 0>(s, L, (float)h2, cf, b, x, col, Upd{});
-            else run_half_z<false, false, 0>(s, L, (float)h2, cf, b, x, col, Upd{});
-        }
+        if (sinv) half32_vec<true, true>(s, L, (float)h2, cf, b, x, col, from_zero);
+        else half32_vec<false, true>(s, L, (float)h2, cf, b, x, col, from_zero);
     } else if (L.split && L.hx % 4 == 0) {
-        const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
-        if (sinv) {
-            if (from_zero) run_kernel(k_half_vec<true, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
-            else run_kernel(k_half_vec<true, false>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
-        } else {
-            if (from_zero) run_kernel(k_half_vec<false, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
-            else run_kernel(k_half_vec<false, false>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, Upd{});
-        }
+        if (sinv) half32_vec<true, false>(s, L, (float)h2, cf, b, x, col, from_zero);
+        else half32_vec<false, false>(s, L, (float)h2, cf, b, x, col, from_zero);
     } else {
         const i64 work = (i64)L.ny * L.nz * ((L.nx + 1) / 2);
         run_kernel(k_half_any, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, x, col, from_zero ? 1 : 0);
@@ -1256,36 +1261,22 @@ void launch_half32(cudaStream_t s, Lay L, double h2, const float *sinv, const fl
 
 bool half32_update_ok(Lay L) { return L.split && L.hx % 4 == 0; }
 
+// k_half_vec at every size: its update sweep moves 26 B per cell at 6.46 TB/s (512^3 540 us; a z-marching
+// form took 567, at 256^3 79 against 71, at 288^3 163 against 102)
 void launch_half32_update(cudaStream_t s, Lay L, double h2, const float *sinv, const float *fx, const float *fy,
                           const float *fz, const float *b, const float *x, double *p, float2 *p2, double alpha,
                           double shift) {
     Coef32 cf{sinv, fx, fy, fz};
     Upd up{p, p2, (float)alpha, (float)shift};
     count_launch();
-    const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
+    const unsigned nb = blocks_for((i64)L.ny * L.nz * (L.hx / 4));
     float *xv = const_cast<float *>(x);  // read only in the UPDATE variants
-    if (L.zlo || L.zhi) {  // a slab: s-form, FP64 solution (the decomposed mixed cycle)
-        if (half_z_ok(L)) run_half_z<true, false, 1, true>(s, L, (float)h2, cf, b, xv, 0, up);
-        else run_kernel(k_half_vec<true, false, 1, true>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
-        return;
-    }
-    if (half_z_ok(L)) {
-        if (p2) {
-            if (sinv) run_half_z<true, false, 2>(s, L, (float)h2, cf, b, xv, 0, up);
-            else run_half_z<false, false, 2>(s, L, (float)h2, cf, b, xv, 0, up);
-        } else {
-            if (sinv) run_half_z<true, false, 1>(s, L, (float)h2, cf, b, xv, 0, up);
-            else run_half_z<false, false, 1>(s, L, (float)h2, cf, b, xv, 0, up);
-        }
-        return;
-    }
-    if (p2) {
-        if (sinv) run_kernel(k_half_vec<true, false, 2>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
-        else run_kernel(k_half_vec<false, false, 2>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
-    } else {
-        if (sinv) run_kernel(k_half_vec<true, false, 1>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
-        else run_kernel(k_half_vec<false, false, 1>, blocks_for(work), kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
-    }
+    if (L.zlo || L.zhi)  // a slab: s-form, FP64 solution (the decomposed mixed cycle)
+        run_kernel(k_half_vec<true, false, 1, true>, nb, kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+    else if (p2 && sinv) run_kernel(k_half_vec<true, false, 2>, nb, kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+    else if (p2) run_kernel(k_half_vec<false, false, 2>, nb, kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+    else if (sinv) run_kernel(k_half_vec<true, false, 1>, nb, kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
+    else run_kernel(k_half_vec<false, false, 1>, nb, kThreads, 0, s, L, (float)h2, cf, b, xv, 0, up);
 }
 
 void launch_residual32(cudaStream_t s, Lay L, double ih2, const float *sinv, const float *fx, const float *fy,

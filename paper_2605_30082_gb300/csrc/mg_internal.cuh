@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/mg.h"
 
 namespace mg {
@@ -171,6 +173,11 @@ inline void run_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
     (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 #endif
+
+// Opts `kernel` into `bytes` of dynamic shared memory (and the largest carveout) on the current
+// device, once per device: `done` is the kernel's own mask.  False: refused, and the reason stays
+// in the runtime's last error.
+bool opt_in_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done);
 
 // process-wide count of kernel launches (read through mg_kernel_launches)
 void count_launch(int k = 1);
