@@ -154,7 +154,7 @@ __global__ void k_resid_df(Dims d, Lay L, const float2 *__restrict__ fx, const f
     }
 }
 
-__global__ void k_final_df(const double *__restrict__ partials, int nb, double *out) {
+__global__ void k_final_df(const double *__restrict__ partials, int nb, ReduceOut ro) {
     grid_wait();
     __shared__ double sa[256], sb[256];
     double a = 0.0, b = 0.0;
@@ -173,8 +173,9 @@ __global__ void k_final_df(const double *__restrict__ partials, int nb, double *
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        out[0] = sa[0];
-        out[1] = sb[0];
+        ro.out[0] = sa[0];
+        ro.out[1] = sb[0];
+        to_host(ro);
     }
 }
 
@@ -389,17 +390,17 @@ void launch_join(cudaStream_t s, i64 n, const float2 *src, double *dst) {
 
 void launch_resid_df(cudaStream_t s, Dims d, Lay L, const float2 *fx, const float2 *fy, const float2 *fz,
                      const float2 *diag, const float2 *b, const float2 *p, float *r32, float s32,
-                     double *partials, double *out) {
+                     double *partials, ReduceOut ro) {
     static const int wave = wave_blocks((const void *)k_resid_df, kReduceThreads);
     const int nb = fill_blocks(reduce_blocks(d.n / 2), wave);
     count_launch();
     run_kernel(k_resid_df, nb, kReduceThreads, 0, s, d, L, fx, fy, fz, diag, b, p, r32, s32, partials);
     count_launch();
-    run_kernel(k_final_df, 1, 256, 0, s, partials, nb, out);
+    run_kernel(k_final_df, 1, 256, 0, s, partials, nb, ro);
 }
 
 void launch_resid_dfs(cudaStream_t s, Dims d, Lay L, const float2 *s2, const float2 *b, const float2 *p,
-                      float *r32, float s32, double *partials, double *out) {
+                      float *r32, float s32, double *partials, ReduceOut ro) {
     const int hx = d.nx / 2;
     const int vb = (hx % 64 == 0) ? 64 : 32;
     const dim3 blk(vb, kDfsThreads / vb);
@@ -411,7 +412,7 @@ void launch_resid_dfs(cudaStream_t s, Dims d, Lay L, const float2 *s2, const flo
     count_launch();
     run_kernel(k_resid_dfs, (unsigned)nb, blk, 0, s, d, L, s2, b, p, r32, s32, partials, tiles_x, tiles_y, ntiles);
     count_launch();
-    run_kernel(k_final_df, 1, 256, 0, s, partials, (int)nb, out);
+    run_kernel(k_final_df, 1, 256, 0, s, partials, (int)nb, ro);
 }
 
 void launch_update_df(cudaStream_t s, Dims d, Lay L, float2 *p, const float *e32, double alpha, double shift) {

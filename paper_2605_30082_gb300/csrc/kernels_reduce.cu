@@ -125,6 +125,31 @@ __global__ void k_final(const double *__restrict__ partials, int nb, double *out
     block_sum2(a, b, out);
 }
 
+// End of a reduction whose blocks have written their partials (block_sum2): the block that finishes
+// last adds them up in index order, as k_final does, and hands the two sums to the host, so that a
+// result the host waits for costs no further launch
+__device__ __forceinline__ void finish_reduction(const double *partials, const ReduceOut &o) {
+    if (!o.count) return;  // k_final follows
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(o.count, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double a = 0.0, b = 0.0;
+    for (int q = threadIdx.x; q < (int)gridDim.x; q += blockDim.x) {
+        a += __ldcg(partials + 2 * q);
+        b += __ldcg(partials + 2 * q + 1);
+    }
+    block_sum2(a, b, o.out);
+    if (threadIdx.x == 0) {
+        *o.count = 0;
+        to_host(o);
+    }
+}
+
 template <typename T> struct Vec16;
 template <> struct Vec16<double> {
     using type = double2;
@@ -145,7 +170,7 @@ inline __device__ bool aligned16(const void *p) { return (reinterpret_cast<uintp
 // scalar loop.  GB300 issues FP64 additions at a small fraction of its FP32 rate, so the
 // gauge sums, which need no squares, take one FP64 addition per element instead of two.
 template <typename T, bool SQ>
-__global__ void k_sum_sumsq(i64 n, const T *__restrict__ x, double *partials) {
+__global__ void k_sum_sumsq(i64 n, const T *__restrict__ x, double *partials, ReduceOut ro) {
     grid_wait();
     using V = Vec16<T>;
     double a = 0.0, b = 0.0;
@@ -183,6 +208,7 @@ __global__ void k_sum_sumsq(i64 n, const T *__restrict__ x, double *partials) {
         if (SQ) b += v * v;
     }
     block_sum2(a, b, partials + 2 * blockIdx.x);
+    finish_reduction(partials, ro);
 }
 
 // v * 2^m by an integer addition to the IEEE-754 exponent field (binary64: 11 exponent bits
@@ -202,8 +228,8 @@ __device__ __forceinline__ double mul_pow2(double v, int m, double s) {
 // (scale = 2^m: 1 in the FP64 mode, h^2 in the mixed modes when h is a power of two) the
 // scaling is an exponent addition: two FP64 operations per element instead of three.
 template <bool POW2>
-__global__ void k_sub_mean(i64 n, const double *__restrict__ b, const double *__restrict__ sum,
-                           double scale, int m2, double *b64, double *partials) {
+__global__ void __launch_bounds__(kReduceThreads, 5) k_sub_mean(i64 n, const double *__restrict__ b, const double *__restrict__ sum,
+                           double scale, int m2, double *b64, double *partials, ReduceOut ro) {
     grid_wait();
     const double mean = sum[0] / (double)n;
     double q = 0.0;
@@ -238,6 +264,7 @@ __global__ void k_sub_mean(i64 n, const double *__restrict__ b, const double *__
         q += v * v;
     }
     block_sum2(q, 0.0, partials + 2 * blockIdx.x);
+    finish_reduction(partials, ro);
 }
 
 __device__ __forceinline__ i64 sto(const Lay &L, int x, int y, int z) {
@@ -253,12 +280,13 @@ __device__ __forceinline__ i64 sto(const Lay &L, int x, int y, int z) {
 // One thread handles the cell pair x = 2k, 2k+1 of a row (even nx): aligned double2 loads,
 // and the pair's red and black r32 values land at index k of the two colour halves.
 // GHOST: a slab of a decomposed grid (d.zlo / d.zhi): its ghost planes count as interior
-// neighbours; whole-grid levels compile without the two extra tests
+// neighbours; whole-grid levels compile without the two extra tests.  Five blocks per SM: the grid is one
+// wave, and the end of the reduction must not cost the marching loop a resident block
 template <bool SCALED, bool GHOST>
-__global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
+__global__ void __launch_bounds__(kReduceThreads, 5) k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
                                   const double *__restrict__ fy, const double *__restrict__ fz,
                                   const double *__restrict__ dg, const double *__restrict__ b,
-                                  const double *__restrict__ p, float *r32, float s32, double *partials) {
+                                  const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
     grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz, hx = nx >> 1;
@@ -317,6 +345,7 @@ __global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__rest
         sp += d2f_trunc(pc.x) + d2f_trunc(pc.y);
     }
     block_sum2((double)q, (double)sp, partials + 2 * blockIdx.x);
+    finish_reduction(partials, ro);
 }
 
 // n4 words, the first 4 nv of them as 16-byte stores
@@ -344,7 +373,7 @@ template <bool SCALED>
 __global__ void k_fine_resid_cell(Dims d, Lay L, double h2, const double *__restrict__ fx,
                                   const double *__restrict__ fy, const double *__restrict__ fz,
                                   const double *__restrict__ dg, const double *__restrict__ b,
-                                  const double *__restrict__ p, float *r32, float s32, double *partials) {
+                                  const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
     grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz;
@@ -368,33 +397,7 @@ __global__ void k_fine_resid_cell(Dims d, Lay L, double h2, const double *__rest
         sp += d2f_trunc(pc);
     }
     block_sum2((double)q, (double)sp, partials + 2 * blockIdx.x);
-}
-
-// r = b - ih2 * sum_f beta_f (p_c - p_nb); partials: (sum r^2, sum p)
-__global__ void k_fine_residual(Dims d, Lay L, double ih2, const double *__restrict__ fx,
-                                const double *__restrict__ fy, const double *__restrict__ fz,
-                                const double *__restrict__ b, const double *__restrict__ p,
-                                float *r32, double scale, double *partials) {
-    grid_wait();
-    double q = 0.0, sp = 0.0;
-    for (i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x; c < d.n; c += (i64)gridDim.x * blockDim.x) {
-        int i = (int)(c % d.nx);
-        i64 row = c / d.nx;
-        int j = (int)(row % d.ny), k = (int)(row / d.ny);
-        double pc = p[c];
-        double s = 0.0;
-        if (i > 0) s += fx[c] * (pc - p[c - 1]);
-        if (i < d.nx - 1) s += fx[c + 1] * (pc - p[c + 1]);
-        if (j > 0) s += fy[c] * (pc - p[c - d.nx]);
-        if (j < d.ny - 1) s += fy[c + d.nx] * (pc - p[c + d.nx]);
-        if (k > 0) s += fz[c] * (pc - p[c - d.nxy]);
-        if (k < d.nz - 1) s += fz[c + d.nxy] * (pc - p[c + d.nxy]);
-        double r = b[c] - s * ih2;
-        if (r32) r32[sto(L, i, j, k)] = (float)(r * scale);
-        q += r * r;
-        sp += pc;
-    }
-    block_sum2(q, sp, partials + 2 * blockIdx.x);
+    finish_reduction(partials, ro);
 }
 
 // p = (p - shift) + alpha e: 2 FP64 operations, the FP32 value widened exactly with integer operations
@@ -419,10 +422,29 @@ __global__ void k_readback(const double *__restrict__ src, double *dst, int n, c
     if (t == 0 && esrc) *edst = *esrc;
 }
 
-__global__ void k_add_const(i64 n, double *p, double c) {
+// p += c, or with `sum` p -= sum[0] / n; two 16-byte accesses per thread and step where p is aligned
+__global__ void k_add_const(i64 n, double *p, double c0, const double *__restrict__ sum) {
     grid_wait();
-    i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < n) p[m] += c;
+    __shared__ double cs;
+    if (threadIdx.x == 0) cs = sum ? -sum[0] / (double)n : c0;  // one division per block
+    __syncthreads();
+    const double c = cs;
+    const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x, nt = (i64)gridDim.x * blockDim.x;
+    i64 m0 = 0;
+    if (aligned16(p)) {
+        double2 *pv = reinterpret_cast<double2 *>(p);
+        const i64 nv = n / 2;
+        for (i64 m = t; m < nv; m += 2 * nt) {
+            double2 u = pv[m];
+            const bool two = m + nt < nv;
+            double2 w = u;
+            if (two) w = pv[m + nt];
+            pv[m] = make_double2(u.x + c, u.y + c);
+            if (two) pv[m + nt] = make_double2(w.x + c, w.y + c);
+        }
+        m0 = nv * 2;
+    }
+    for (i64 m = m0 + t; m < n; m += nt) p[m] += c;
 }
 
 // dL/dbeta_f = -(lam_L - lam_R)(p_L - p_R) ih2 + sigma csf_f (lam_L - lam_R) ih on the low
@@ -732,84 +754,64 @@ __global__ void __launch_bounds__(32 * kGrad2Rows) k_adjoint_grad_split2(
 
 }  // namespace
 
+// the sums of nb partials: by the reduction's last block (ro.count), or by a launch of its own
+static void final_sums(cudaStream_t s, const double *partials, int nb, const ReduceOut &ro) {
+    if (ro.count) return;
+    count_launch();
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, ro.out);
+}
+
 template <typename T>
-void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, double *out, bool squares) {
+void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, ReduceOut ro, bool squares) {
     static const int wave_q = wave_blocks((const void *)k_sum_sumsq<T, true>, kReduceThreads);
     static const int wave_s = wave_blocks((const void *)k_sum_sumsq<T, false>, kReduceThreads);
     const int nb = fill_blocks(reduce_blocks(n), squares ? wave_q : wave_s);
     count_launch();
-    if (squares) run_kernel(k_sum_sumsq<T, true>, nb, kReduceThreads, 0, s, n, x, partials);
-    else run_kernel(k_sum_sumsq<T, false>, nb, kReduceThreads, 0, s, n, x, partials);
-    count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
+    if (squares) run_kernel(k_sum_sumsq<T, true>, nb, kReduceThreads, 0, s, n, x, partials, ro);
+    else run_kernel(k_sum_sumsq<T, false>, nb, kReduceThreads, 0, s, n, x, partials, ro);
+    final_sums(s, partials, nb, ro);
 }
-template void launch_sum_sumsq<double>(cudaStream_t, i64, const double *, double *, double *, bool);
-template void launch_sum_sumsq<float>(cudaStream_t, i64, const float *, double *, double *, bool);
+template void launch_sum_sumsq<double>(cudaStream_t, i64, const double *, double *, ReduceOut, bool);
+template void launch_sum_sumsq<float>(cudaStream_t, i64, const float *, double *, ReduceOut, bool);
 
 void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, double scale, double *b64,
-                     double *partials, double *out) {
+                     double *partials, ReduceOut ro) {
     static const int wave_p = wave_blocks((const void *)k_sub_mean<true>, kReduceThreads);
     static const int wave_m = wave_blocks((const void *)k_sub_mean<false>, kReduceThreads);
     int e = 0;
     const bool pow2 = std::frexp(scale, &e) == 0.5;  // scale = 2^(e - 1)
     const int nb = fill_blocks(reduce_blocks(n), pow2 ? wave_p : wave_m);
     count_launch();
-    if (pow2) run_kernel(k_sub_mean<true>, nb, kReduceThreads, 0, s, n, b, sum, scale, e - 1, b64, partials);
-    else run_kernel(k_sub_mean<false>, nb, kReduceThreads, 0, s, n, b, sum, scale, 0, b64, partials);
-    count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
-}
-
-void launch_fine_residual(cudaStream_t s, Dims d, Lay L, double ih2, const double *fx, const double *fy,
-                          const double *fz, const double *b, const double *p, float *r32,
-                          double scale, double *partials, double *out) {
-    static const int wave = wave_blocks((const void *)k_fine_residual, kReduceThreads);
-    const int nb = fill_blocks(reduce_blocks(d.n), wave);
-    count_launch();
-    run_kernel(k_fine_residual, nb, kReduceThreads, 0, s, d, L, ih2, fx, fy, fz, b, p, r32, scale, partials);
-    count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
+    if (pow2) run_kernel(k_sub_mean<true>, nb, kReduceThreads, 0, s, n, b, sum, scale, e - 1, b64, partials, ro);
+    else run_kernel(k_sub_mean<false>, nb, kReduceThreads, 0, s, n, b, sum, scale, 0, b64, partials, ro);
+    final_sums(s, partials, nb, ro);
 }
 
 void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *fx, const double *fy,
                         const double *fz, const double *diag, const double *b, bool b_scaled, const double *p,
-                        float *r32, float s32, double *partials, double *out) {
+                        float *r32, float s32, double *partials, ReduceOut ro) {
+    // each kernel its own wave: the ghost tests take more registers, one resident block fewer per SM
+    auto run = [&](auto kernel, int nb) {
+        count_launch();
+        run_kernel(kernel, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials, ro);
+        final_sums(s, partials, nb, ro);
+    };
     if (d.nx & 1) {
         static const int wave_ct = wave_blocks((const void *)k_fine_resid_cell<true>, kReduceThreads);
         static const int wave_cf = wave_blocks((const void *)k_fine_resid_cell<false>, kReduceThreads);
-        const int nb = fill_blocks(reduce_blocks(d.n), b_scaled ? wave_ct : wave_cf);
-        count_launch();
-        if (b_scaled) run_kernel(k_fine_resid_cell<true>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
-        else run_kernel(k_fine_resid_cell<false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
-        count_launch();
-        run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
-        return;
-    }
-    static const int wave_pt = wave_blocks((const void *)k_fine_resid_pair<true, false>, kReduceThreads);
-    static const int wave_pf = wave_blocks((const void *)k_fine_resid_pair<false, false>, kReduceThreads);
-    const int nb = fill_blocks(reduce_blocks(d.n / 2), b_scaled ? wave_pt : wave_pf);
-    count_launch();
-    if (d.zlo || d.zhi) {
-        // a slab; its own wave: the ghost tests take more registers, one resident block fewer
-        // per SM
+        if (b_scaled) run(k_fine_resid_cell<true>, fill_blocks(reduce_blocks(d.n), wave_ct));
+        else run(k_fine_resid_cell<false>, fill_blocks(reduce_blocks(d.n), wave_cf));
+    } else if (d.zlo || d.zhi) {
         static const int wave_gt = wave_blocks((const void *)k_fine_resid_pair<true, true>, kReduceThreads);
         static const int wave_gf = wave_blocks((const void *)k_fine_resid_pair<false, true>, kReduceThreads);
-        const int ng = fill_blocks(reduce_blocks(d.n / 2), b_scaled ? wave_gt : wave_gf);
-        if (b_scaled)
-            run_kernel(k_fine_resid_pair<true, true>, ng, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
-        else
-            run_kernel(k_fine_resid_pair<false, true>, ng, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
-        count_launch();
-        run_kernel(k_final, 1, kReduceThreads, 0, s, partials, ng, out);
-        return;
-    }
-    if (b_scaled) {
-        run_kernel(k_fine_resid_pair<true, false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        if (b_scaled) run(k_fine_resid_pair<true, true>, fill_blocks(reduce_blocks(d.n / 2), wave_gt));
+        else run(k_fine_resid_pair<false, true>, fill_blocks(reduce_blocks(d.n / 2), wave_gf));
     } else {
-        run_kernel(k_fine_resid_pair<false, false>, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials);
+        static const int wave_pt = wave_blocks((const void *)k_fine_resid_pair<true, false>, kReduceThreads);
+        static const int wave_pf = wave_blocks((const void *)k_fine_resid_pair<false, false>, kReduceThreads);
+        if (b_scaled) run(k_fine_resid_pair<true, false>, fill_blocks(reduce_blocks(d.n / 2), wave_pt));
+        else run(k_fine_resid_pair<false, false>, fill_blocks(reduce_blocks(d.n / 2), wave_pf));
     }
-    count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
 }
 
 void launch_zero_resid32(cudaStream_t s, Dims d, Lay L, const double *b, double scale32, float *r32) {
@@ -840,10 +842,13 @@ void launch_zero(cudaStream_t s, void *p, size_t bytes) {
     run_kernel(k_zero, (unsigned)(nb < cap ? (nb > 0 ? nb : 1) : cap), kThreads, 0, s, reinterpret_cast<float *>(p), nv, n4);
 }
 
-void launch_add_const(cudaStream_t s, i64 n, double *p, double c) {
+static void add_const(cudaStream_t s, i64 n, double *p, double c, const double *sum) {
+    const i64 nb = (n / 2 + kThreads - 1) / kThreads, cap = (i64)device_sms() * 16;
     count_launch();
-    run_kernel(k_add_const, blocks_for(n), kThreads, 0, s, n, p, c);
+    run_kernel(k_add_const, (unsigned)(nb < 1 ? 1 : (nb < cap ? nb : cap)), kThreads, 0, s, n, p, c, sum);
 }
+void launch_add_const(cudaStream_t s, i64 n, double *p, double c) { add_const(s, n, p, c, nullptr); }
+void launch_sub_sum(cudaStream_t s, i64 n, double *p, const double *sum) { add_const(s, n, p, 0.0, sum); }
 
 inline bool aligned16h(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
 inline bool aligned8h(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 7) == 0; }

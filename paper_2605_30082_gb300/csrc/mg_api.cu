@@ -5,6 +5,7 @@
 // Memory: every device buffer of a handle is carved out of one cudaMalloc made
 // in mg_create (a pool in the sense of the paper's §4.2: allocation happens
 // once, never inside a solve).
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -64,7 +65,8 @@ struct mg_handle {
                        // scalars), then the error word as an unsigned
     double *hred_dev;  // the device-side address of hred
     unsigned *herr;    // = (unsigned *)(hred + 16), host side
-    unsigned *err;     // device error word
+    unsigned long long seq;  // scalars requested so far; hred + 17 holds the last one delivered
+    unsigned *err;     // device error word; err + 32: the reductions' block counter
     void *arena;
     size_t arena_bytes;
     int have_op;
@@ -117,6 +119,29 @@ int fail(mg_handle *h, int code, const char *fmt, ...) {
             return fail((h), MG_ERR_CUDA, "%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_), \
                         __FILE__, __LINE__);                                                    \
     } while (0)
+
+// two sums of a reduction into red[k], red[k + 1] and hred[k], hred[k + 1]; wait_scalars() waits for them
+mg::ReduceOut sums_for_host(mg_handle *h, int k) {
+    return mg::ReduceOut{h->red + k, h->err + 32, h->hred_dev + k,
+                         reinterpret_cast<unsigned long long *>(h->hred_dev + 17), ++h->seq};
+}
+mg::ReduceOut sums_on_device(mg_handle *h, int k) {
+    return mg::ReduceOut{h->red + k, h->err + 32, nullptr, nullptr, 0};
+}
+int wait_scalars(mg_handle *h) {
+    const volatile unsigned long long *q = reinterpret_cast<const unsigned long long *>(h->hred + 17);
+    for (unsigned n = 1;; ++n) {
+        if (*q == h->seq) break;
+        if (n % 1024) continue;
+        // the stream ends with the sums delivered, or with an error
+        const cudaError_t e = cudaStreamQuery(h->s);
+        if (e == cudaErrorNotReady) continue;
+        if (*q == h->seq && e == cudaSuccess) break;
+        return fail(h, MG_ERR_CUDA, "waiting for a reduction failed: %s", cudaGetErrorString(e));
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return MG_OK;
+}
 
 int check_launch(mg_handle *h, const char *where) {
     cudaError_t e = cudaGetLastError();
@@ -531,11 +556,11 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
     const bool mixed = h->o.precision != MG_FP64;
     const bool df = h->o.precision == MG_MIXED_DF;
     const double bscale = mixed ? F.h2 : 1.0;
-    mg::launch_sum_sumsq<double>(s, n, b, h->partials, h->red, false);
-    mg::launch_sub_mean(s, n, b, h->red, bscale, h->bt, h->partials, h->red + 2);
-    MG_READBACK(h, s, h->hred, h->red, 4);
-    MG_CUDA(h, cudaStreamSynchronize(s));
+    mg::launch_sum_sumsq<double>(s, n, b, h->partials, sums_on_device(h, 0), false);
+    mg::launch_sub_mean(s, n, b, h->red, bscale, h->bt, h->partials, sums_for_host(h, 2));
     int rc = check_launch(h, "rhs preparation");
+    if (rc) return rc;
+    rc = wait_scalars(h);
     if (rc) return rc;
     const double nb = std::sqrt(h->hred[2]) / bscale;
     if (!std::isfinite(nb)) return fail(h, MG_ERR_ARG, "right-hand side is not finite");
@@ -553,10 +578,8 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
         hist[hist_n++] = 0.0;
     } else {
         if (warm) {
-            mg::launch_sum_sumsq<double>(s, n, p, h->partials, h->red + 4, false);
-            MG_READBACK(h, s, h->hred + 4, h->red + 4, 1);
-            MG_CUDA(h, cudaStreamSynchronize(s));
-            mg::launch_add_const(s, n, p, -h->hred[4] / (double)n);
+            mg::launch_sum_sumsq<double>(s, n, p, h->partials, sums_on_device(h, 4), false);
+            mg::launch_sub_sum(s, n, p, h->red + 4);
         } else {
             mg::launch_zero(s, p, sizeof(double) * (size_t)n);
         }
@@ -570,18 +593,21 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
             prof_begin(h, MG_PROF_FINE_RESIDUAL);
             if (df && h->sform0)
                 mg::launch_resid_dfs(s, F.d, F.lay, F.s2, h->bt2, h->p2, write32 ? F.b32 : nullptr,
-                                     (float)(F.ih2 * scale), h->partials, h->red + 6);
+                                     (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6));
             else if (df)
                 mg::launch_resid_df(s, F.d, F.lay, F.fx2, F.fy2, F.fz2, F.d2, h->bt2, h->p2,
-                                    write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, h->red + 6);
+                                    write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6));
             else
                 mg::launch_fine_resid2(s, F.d, F.lay, F.h2, F.fx64, F.fy64, F.fz64, F.d64, h->bt, mixed, p,
-                                       write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, h->red + 6);
+                                       write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6));
             prof_end(h);
-            MG_READBACK(h, s, h->hred + 6, h->red + 6, 2);
-            MG_CUDA(h, cudaStreamSynchronize(s));
-            prof_collect(h);
-            return check_launch(h, "fine residual");
+            const int bad = check_launch(h, "fine residual");
+            if (bad) return bad;
+            if (h->prof_on) {  // the recorded events have to be over before they are read
+                MG_CUDA(h, cudaStreamSynchronize(s));
+                prof_collect(h);
+            }
+            return wait_scalars(h);
         };
         double rn, mu;
         if (!warm && !df) {
@@ -683,10 +709,8 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
         }
         if (df) mg::launch_join(s, n, h->p2, p);
         // exact zero-mean gauge at exit (the per-iteration shifts use an FP32 sum)
-        mg::launch_sum_sumsq<double>(s, n, p, h->partials, h->red + 12, false);
-        MG_READBACK(h, s, h->hred + 12, h->red + 12, 1);
-        MG_CUDA(h, cudaStreamSynchronize(s));
-        mg::launch_add_const(s, n, p, -h->hred[12] / (double)n);
+        mg::launch_sum_sumsq<double>(s, n, p, h->partials, sums_on_device(h, 12), false);
+        mg::launch_sub_sum(s, n, p, h->red + 12);
         (void)mu;
     }
     MG_CUDA(h, cudaEventRecord(h->ev1, s));
@@ -881,7 +905,7 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
         *slots[q].p = cur;
         cur += slots[q].bytes;
     }
-    if (cudaHostAlloc((void **)&h->hred, 17 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+    if (cudaHostAlloc((void **)&h->hred, 18 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&h->hred_dev, h->hred, 0) != cudaSuccess ||
         cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess) {
         cudaGetLastError();
@@ -891,6 +915,7 @@ int mg_create(const mg_opts *o, void *stream, mg_handle **out) {
         return MG_ERR_CUDA;
     }
     h->herr = reinterpret_cast<unsigned *>(h->hred + 16);
+    std::memset(h->hred, 0, 18 * sizeof(double));
     if (cudaMemsetAsync(h->err, 0, 256, h->s) != cudaSuccess) {
         mg_destroy(h);
         return MG_ERR_CUDA;
@@ -1181,14 +1206,14 @@ int mg_residual(mg_handle *h, int level, int dtype, const void *x, const void *b
     Level &L = h->lv[level];
     if (dtype == MG_F64) {
         mg::launch_residual<double>(h->s, L.d, L.ih2, coef<double>(L), (const double *)b, (const double *)x, (double *)r);
-        if (norm2) mg::launch_sum_sumsq<double>(h->s, L.d.n, (const double *)r, h->partials, h->red + 10, true);
+        if (norm2) mg::launch_sum_sumsq<double>(h->s, L.d.n, (const double *)r, h->partials, mg::sums_to(h->red + 10), true);
     } else {
         mg::launch_pack32(h->s, L.lay, (const float *)x, L.s1_32);
         mg::launch_pack32(h->s, L.lay, (const float *)b, L.s2_32);
         mg::launch_residual32(h->s, L.lay, L.ih2, sinv32(h, level), L.fx32, L.fy32, L.fz32, L.s2_32, L.s1_32,
                               L.x32, false);
         mg::launch_unpack32(h->s, L.lay, L.x32, (float *)r);
-        if (norm2) mg::launch_sum_sumsq<float>(h->s, L.d.n, (const float *)r, h->partials, h->red + 10, true);
+        if (norm2) mg::launch_sum_sumsq<float>(h->s, L.d.n, (const float *)r, h->partials, mg::sums_to(h->red + 10), true);
     }
     rc = check_launch(h, "mg_residual");
     if (rc) return rc;

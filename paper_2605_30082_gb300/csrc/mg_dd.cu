@@ -488,7 +488,7 @@ int slab_residual_norms(mg_dd *dd, double *rn2_h4, double *sp) {
     for (int r = 0; r < P; ++r) {
         Slab &S = dd->lv[0][r];
         mg::launch_fine_resid2(dd->s, S.d, mg::make_lay(S.d), h2, S.fx, S.fy, S.fze, S.dg, S.b, false, S.x,
-                               nullptr, 0.f, dd->partials, dd->red + 2 * r);
+                               nullptr, 0.f, dd->partials, mg::sums_to(dd->red + 2 * r));
     }
     std::vector<double> h(2 * (size_t)P);
     DD_CUDA(dd, cudaMemcpyAsync(h.data(), dd->red, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, dd->s));
@@ -508,7 +508,7 @@ int slab_sum_x(mg_dd *dd, double *sum) {
     const int P = dd->P;
     for (int r = 0; r < P; ++r) {
         Slab &S = dd->lv[0][r];
-        mg::launch_sum_sumsq<double>(dd->s, S.d.n, S.x, dd->partials, dd->red + 2 * r, false);
+        mg::launch_sum_sumsq<double>(dd->s, S.d.n, S.x, dd->partials, mg::sums_to(dd->red + 2 * r), false);
     }
     std::vector<double> h(2 * (size_t)P);
     DD_CUDA(dd, cudaMemcpyAsync(h.data(), dd->red, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, dd->s));
@@ -524,7 +524,7 @@ int slab_sums_b(mg_dd *dd, double *sum, double *sumsq) {
     const int P = dd->P;
     for (int r = 0; r < P; ++r) {
         Slab &S = dd->lv[0][r];
-        mg::launch_sum_sumsq<double>(dd->s, S.d.n, S.b, dd->partials, dd->red + 2 * r, true);
+        mg::launch_sum_sumsq<double>(dd->s, S.d.n, S.b, dd->partials, mg::sums_to(dd->red + 2 * r), true);
     }
     std::vector<double> h(2 * (size_t)P);
     DD_CUDA(dd, cudaMemcpyAsync(h.data(), dd->red, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, dd->s));
@@ -566,7 +566,7 @@ int solve_mixed(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     std::vector<Slab> &R = dd->lv[0];
     double sb = 0.0;
     for (Slab &S : R) {
-        mg::launch_sum_sumsq<double>(s, S.d.n, b + (size_t)S.z0 * S.d.nxy, dd->partials, dd->red, false);
+        mg::launch_sum_sumsq<double>(s, S.d.n, b + (size_t)S.z0 * S.d.nxy, dd->partials, mg::sums_to(dd->red), false);
         double hb[2];
         DD_CUDA(dd, cudaMemcpyAsync(hb, dd->red, sizeof(hb), cudaMemcpyDeviceToHost, s));
         DD_CUDA(dd, cudaStreamSynchronize(s));
@@ -610,7 +610,7 @@ int solve_mixed(mg_dd *dd, const double *b, double *p, mg_stats *st) {
         for (int r = 0; r < dd->P; ++r) {
             Slab &S = R[r];
             mg::launch_fine_resid2(s, S.d, S.lay, h2, S.fx, S.fy, S.fze, S.dg, S.b, true, S.x, S.b32, (float)(ih2 * scale),
-                                   dd->partials, dd->red + 2 * r);
+                                   dd->partials, mg::sums_to(dd->red + 2 * r));
         }
         std::vector<double> hs(2 * (size_t)dd->P);
         DD_CUDA(dd, cudaMemcpyAsync(hs.data(), dd->red, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s));
@@ -1017,7 +1017,7 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     // b~ = b - mean(b) slab by slab (the mean from the slabs' partial sums)
     double sb = 0.0;
     for (Slab &S : dd->lv[0]) {
-        mg::launch_sum_sumsq<double>(s, S.d.n, b + (size_t)S.z0 * S.d.nxy, dd->partials, dd->red, false);
+        mg::launch_sum_sumsq<double>(s, S.d.n, b + (size_t)S.z0 * S.d.nxy, dd->partials, mg::sums_to(dd->red), false);
         double h[2];
         DD_CUDA(dd, cudaMemcpyAsync(h, dd->red, sizeof(h), cudaMemcpyDeviceToHost, s));
         DD_CUDA(dd, cudaStreamSynchronize(s));

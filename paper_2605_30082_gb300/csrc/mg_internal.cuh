@@ -224,6 +224,30 @@ int wave_blocks(const void *kernel, int threads);
 // min(nb, wave): the grid of a grid-stride reduction that needs nb <= reduce_blocks(n) blocks
 int fill_blocks(int nb, int wave);
 
+// Where a reduction's two sums go: device memory (out[0], out[1]), and with `host` also mapped
+// pinned host memory, followed by the sequence number `want` in *seq, which the host polls
+// (a stream synchronisation after a read-back launch takes about 10 us longer).  `count` (zero at
+// rest) lets the reduction's last block add up the partials; without it k_final does.
+struct ReduceOut {
+    double *out;
+    unsigned *count;
+    double *host;
+    unsigned long long *seq, want;
+};
+#ifdef __CUDACC__
+// the two sums into mapped host memory, then the sequence number the host polls
+__device__ __forceinline__ void to_host(const ReduceOut &o) {
+    if (!o.host) return;
+    volatile double *h = o.host;
+    h[0] = o.out[0];
+    h[1] = o.out[1];
+    __threadfence_system();
+    *(volatile unsigned long long *)o.seq = o.want;
+}
+#endif
+// sums into device memory only, by a launch of k_final
+inline ReduceOut sums_to(double *out) { return ReduceOut{out, nullptr, nullptr, nullptr, 0}; }
+
 // ---- setup kernels (FP64) -------------------------------------------------------
 void launch_density(cudaStream_t s, i64 n, int nfrac, const double *const *frac,
                     const double *rho_phase, double *rho);
@@ -293,10 +317,10 @@ void launch_join(cudaStream_t s, i64 n, const float2 *src, double *dst);    // v
 // optional r32 = s32 * h^2 r in the split level-0 layout.  Needs even nx.
 void launch_resid_df(cudaStream_t s, Dims d, Lay L, const float2 *fx, const float2 *fy, const float2 *fz,
                      const float2 *diag, const float2 *b, const float2 *p, float *r32, float s32,
-                     double *partials, double *out);
+                     double *partials, ReduceOut ro);
 // s-form double-float residual: s2 = 1/rho as FP32 pairs (natural layout), otherwise as launch_resid_df
 void launch_resid_dfs(cudaStream_t s, Dims d, Lay L, const float2 *s2, const float2 *b, const float2 *p,
-                      float *r32, float s32, double *partials, double *out);
+                      float *r32, float s32, double *partials, ReduceOut ro);
 // ---- flexible CG (kernels_cg.cu) --------------------------------------------------------
 // slots of the device scalar array: r . z of the current and of the previous iteration
 // alternate between CG_RZ0 and CG_RZ1
@@ -399,15 +423,10 @@ void launch_readback(cudaStream_t s, const double *src, double *dst_mapped, int 
 void launch_readback_u32(cudaStream_t s, const unsigned *src, unsigned *dst_mapped);
 // out[0] = sum x, out[1] = sum x^2 (0 unless `squares`)
 template <typename T>
-void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, double *out, bool squares);
+void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, ReduceOut ro, bool squares);
 // b64 = (b - sum[0]/n) * scale, with the sum of squares of b64 into out[0]
 void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, double scale, double *b64,
-                     double *partials, double *out);
-// fine FP64 residual r = b - A p: out[0] = sum r^2, out[1] = sum p; optional r32 = scale * r
-// stored in the level-0 FP32 layout L
-void launch_fine_residual(cudaStream_t s, Dims d, Lay L, double ih2, const double *fx, const double *fy,
-                          const double *fz, const double *b, const double *p, float *r32,
-                          double scale, double *partials, double *out);
+                     double *partials, ReduceOut ro);
 // fine FP64 residual in diagonal form, h^2 r = h^2 b - (diag p_c - sum_f beta_f p_nb):
 // out[0] = sum (h^2 r)^2, out[1] = sum p; optional r32 = s32 * h^2 r in the level-0 layout L.
 // On a slab of a decomposed grid (d.zlo or d.zhi, even nx; p with its ghost planes beside the
@@ -415,13 +434,15 @@ void launch_fine_residual(cudaStream_t s, Dims d, Lay L, double ih2, const doubl
 // and r32 is stored in the slab's layout L (L.half the colour stride)
 void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *fx, const double *fy,
                         const double *fz, const double *diag, const double *b, bool b_scaled, const double *p,
-                        float *r32, float s32, double *partials, double *out);
+                        float *r32, float s32, double *partials, ReduceOut ro);
 // r32 = (float)(ih2 scale) * trunc_fp32(b): the scaled FP32 residual of p = 0, as the outer
 // residual kernels would write it (b = h^2 b~ in the mixed modes)
 void launch_zero_resid32(cudaStream_t s, Dims d, Lay L, const double *b, double scale32, float *r32);
 // p = p - shift + alpha * e32 (e32 in the level-0 FP32 layout L; shift a host scalar)
 void launch_update(cudaStream_t s, Dims d, Lay L, double *p, const float *e32, double alpha, double shift);
 void launch_add_const(cudaStream_t s, i64 n, double *p, double c);
+// p -= sum[0] / n (sum on the device)
+void launch_sub_sum(cudaStream_t s, i64 n, double *p, const double *sum);
 // zeroes `bytes` bytes (a multiple of 4) at p (4-byte aligned): a kernel, because a memset between two
 // kernels costs both of them the 2 us gap that run_kernel avoids
 void launch_zero(cudaStream_t s, void *p, size_t bytes);
