@@ -38,6 +38,18 @@ bool opt_in_smem(const void *kernel, int bytes, std::atomic<unsigned long long> 
     return true;
 }
 
+bool prefer_smem(const void *kernel, std::atomic<unsigned long long> &done) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+    if (bit & done.load(std::memory_order_relaxed)) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared) !=
+        cudaSuccess)
+        return false;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return true;
+}
+
 int device_sms() {
     constexpr int kMaxDev = 64;
     static std::atomic<int> cache[kMaxDev];

@@ -818,10 +818,12 @@ constexpr int kRrThreads = 64;
 
 // GHOST: the fine level is a slab (L.zlo / L.zhi) and Lc a view of the whole coarse level
 // (its arrays at the slab's first coarse plane, an even one)
-template <bool SFORM, bool GHOST = false>
+// TAIL: the coarse levels' cluster launch follows, which may come in and copy its contexts meanwhile
+template <bool SFORM, bool GHOST = false, bool TAIL = false>
 __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                              const float *__restrict__ xv, float *bc) {
     grid_wait();
+    if (TAIL) trigger_next();
     const int hx = L.hx, kv = hx >> 2;
     const i64 T = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 crows = (i64)Lc.ny * Lc.nz;
@@ -1288,14 +1290,23 @@ void launch_residual32(cudaStream_t s, Lay L, double ih2, const float *sinv, con
 
 void launch_resid_restrict32(cudaStream_t s, Lay L, Lay Lc, double ih2, const float *sinv, const float *fx,
                              const float *fy, const float *fz, const float *b, const float *x, float *bc,
-                             bool red_only) {
+                             bool red_only, bool tail) {
     Coef32 cf{sinv, fx, fy, fz};
     count_launch();
     if (red_only && L.split && L.hx % 4 == 0) {
+        if (tail) {
+            // the cluster's CTAs want most of an SM's shared memory, which has to be set aside already
+            static std::atomic<unsigned long long> carved[2];
+            if (!prefer_smem((const void *)k_rr_red_vec<true, false, true>, carved[0]) ||
+                !prefer_smem((const void *)k_rr_red_vec<false, false, true>, carved[1]))
+                (void)cudaGetLastError();  // a preference only
+        }
         const i64 work = (i64)Lc.ny * Lc.nz * (L.hx / 4);
         const unsigned nb = (unsigned)((work + kRrThreads - 1) / kRrThreads);
         if ((L.zlo || L.zhi) && sinv) run_kernel(k_rr_red_vec<true, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else if (L.zlo || L.zhi) run_kernel(k_rr_red_vec<false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
+        else if (tail && sinv) run_kernel(k_rr_red_vec<true, false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
+        else if (tail) run_kernel(k_rr_red_vec<false, false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else if (sinv) run_kernel(k_rr_red_vec<true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else run_kernel(k_rr_red_vec<false>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         return;

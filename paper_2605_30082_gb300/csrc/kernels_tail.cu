@@ -476,7 +476,6 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
 // coarse solve launched between the two on the whole device and the levels kept in memory
 template <typename T>
 __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs a, int mode) {
-    grid_wait();
     extern __shared__ __align__(16) char tail_smem[];
     cg::cluster_group cl = cg::this_cluster();
     const Tail<T> t{a, tail_smem, (int)cl.block_rank(), (int)cl.num_blocks(), (int)threadIdx.x};
@@ -502,6 +501,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
         float4 *x4 = reinterpret_cast<float4 *>(t.x(L));  // rows and ghosts from zero
         for (int e = t.tid; e < (L.off_b - L.off_x) / 16; e += kTailThreads) x4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    grid_wait();  // the contexts were written long before (set-up ends with a synchronisation); b was not
     __syncthreads();
     t.load_b(a.lv[0]);
     if (from_mem) {

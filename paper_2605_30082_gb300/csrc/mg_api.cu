@@ -331,7 +331,7 @@ void presmooth_restrict32(mg_handle *h, int l, const float *b, float *x, float *
     if (l == 0) prof_begin(h, MG_PROF_RESID_RESTRICT);
     // after a pre-smoothing sweep (black last) every black residual is zero
     mg::launch_resid_restrict32(h->s, L.lay, C.lay, L.ih2, sinv32(h, l), L.fx32, L.fy32, L.fz32, b, x, bc,
-                                sweeps > 0);
+                                sweeps > 0, h->tail_l == l + 1 && bc == C.b32);
     if (l == 0) prof_end(h);
 }
 

@@ -142,11 +142,15 @@ __device__ __forceinline__ double recip64(double x) {
 // launch for kernels that run 0.1, 1.1, 2.1, 3.2, 5.3 us), and 0.4-0.5 us with programmatic stream
 // serialisation (1.4, 1.6, 2.6, 3.6, 5.6 us) or inside a graph.  So every kernel here is launched with
 // that attribute and begins with grid_wait(), before any access to memory: it waits until the
-// kernel before it in the stream has completed and its writes are visible.  No kernel triggers
-// its successor early, so the two never run side by side (blocks of a successor that only wait
-// would take the place of the predecessor's).  Under a stream capture the launch is plain: the
+// kernel before it in the stream has completed and its writes are visible.  No kernel but the
+// restriction into the coarse levels' cluster triggers its successor early, so two kernels do not
+// run side by side (blocks of a successor that only wait would take the place of the predecessor's).  Under a stream capture the launch is plain: the
 // graph's own edges cost the same, and forks and joins keep full dependencies.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// lets the next kernel's blocks come in beside this one's, up to their grid_wait(); only where that kernel
+// has work to do before it (k_tail)
+__device__ __forceinline__ void trigger_next() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 inline bool stream_capturing(cudaStream_t s) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -178,6 +182,8 @@ inline void run_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
 // device, once per device: `done` is the kernel's own mask.  False: refused, and the reason stays
 // in the runtime's last error.
 bool opt_in_smem(const void *kernel, int bytes, std::atomic<unsigned long long> &done);
+// the largest shared-memory carveout as a preference, once per device
+bool prefer_smem(const void *kernel, std::atomic<unsigned long long> &done);
 
 // process-wide count of kernel launches (read through mg_kernel_launches)
 void count_launch(int k = 1);
@@ -344,10 +350,11 @@ void launch_update_df(cudaStream_t s, Dims d, Lay L, float2 *p, const float *e32
 // r = b - A x (or r = A x when apply_only)
 void launch_residual32(cudaStream_t s, Lay L, double ih2, const float *sinv, const float *fx, const float *fy,
                        const float *fz, const float *b, const float *x, float *r, bool apply_only);
-// bc = mean of the 8 children's residuals (red_only: black children count as 0)
+// bc = mean of the 8 children's residuals (red_only: black children count as 0); tail: launch_tail
+// follows on the stream
 void launch_resid_restrict32(cudaStream_t s, Lay L, Lay Lc, double ih2, const float *sinv, const float *fx,
                              const float *fy, const float *fz, const float *b, const float *x, float *bc,
-                             bool red_only);
+                             bool red_only, bool tail = false);
 // x += P ec on the cells of colour only_col (0 red, 1 black) or all cells (-1)
 void launch_prolong32(cudaStream_t s, Lay L, Lay Lc, const float *ec, float *x, int kind, int only_col);
 void launch_coarse_matvec32(cudaStream_t s, Lay L, const double *pinv, const float *r, float *e);
