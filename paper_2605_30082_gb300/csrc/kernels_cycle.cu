@@ -64,7 +64,8 @@ template <typename T>
 __global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T *x, int colour) {
     grid_wait();
     const int half = (d.nx + 1) >> 1;
-    const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    // black sweeps run from the last plane down: they begin with what the red one left in L2
+    const i64 t = (i64)(colour ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
     const i64 rows = (i64)d.ny * d.nz;
     if (t >= rows * half) return;
     const unsigned tu = (unsigned)t, rowu = tu / (unsigned)half;  // t < 2^31: 32-bit divisions

@@ -94,6 +94,7 @@ int fill_blocks(int nb, int wave) {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr i64 kLastCells = 2000000;  // see k_fine_resid_pair
 
 inline unsigned blocks_for(i64 n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
@@ -127,14 +128,15 @@ __device__ __forceinline__ void block_sum2(double a, double b, double *out) {
     }
 }
 
-__global__ void k_final(const double *__restrict__ partials, int nb, double *out) {
+__global__ void k_final(const double *__restrict__ partials, int nb, ReduceOut ro) {
     grid_wait();
     double a = 0.0, b = 0.0;
     for (int q = threadIdx.x; q < nb; q += blockDim.x) {
         a += partials[2 * q];
         b += partials[2 * q + 1];
     }
-    block_sum2(a, b, out);
+    block_sum2(a, b, ro.out);
+    if (threadIdx.x == 0) to_host(ro);
 }
 
 // End of a reduction whose blocks have written their partials (block_sum2): the block that finishes
@@ -292,10 +294,11 @@ __device__ __forceinline__ i64 sto(const Lay &L, int x, int y, int z) {
 // One thread handles the cell pair x = 2k, 2k+1 of a row (even nx): aligned double2 loads,
 // and the pair's red and black r32 values land at index k of the two colour halves.
 // GHOST: a slab of a decomposed grid (d.zlo / d.zhi): its ghost planes count as interior
-// neighbours; whole-grid levels compile without the two extra tests.  Five blocks per SM: the grid is one
-// wave, and the end of the reduction must not cost the marching loop a resident block
-template <bool SCALED, bool GHOST>
-__global__ void __launch_bounds__(kReduceThreads, 5) k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
+// neighbours; whole-grid levels compile without the two extra tests.  LAST: the last block adds up
+// the partials (finish_reduction); its registers cost the loop about a tenth (256^3 206 -> 226 us), so only
+// grids of up to kLastCells cells, where a launch of k_final costs more, take that variant
+template <bool SCALED, bool GHOST, bool LAST>
+__global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
                                   const double *__restrict__ fy, const double *__restrict__ fz,
                                   const double *__restrict__ dg, const double *__restrict__ b,
                                   const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(kReduceThreads, 5) k_fine_resid_pair(Dims d, L
         sp += d2f_trunc(pc.x) + d2f_trunc(pc.y);
     }
     block_sum2((double)q, (double)sp, partials + 2 * blockIdx.x);
-    finish_reduction(partials, ro);
+    if (LAST) finish_reduction(partials, ro);
 }
 
 // n4 words, the first 4 nv of them as 16-byte stores
@@ -770,7 +773,7 @@ __global__ void __launch_bounds__(32 * kGrad2Rows) k_adjoint_grad_split2(
 static void final_sums(cudaStream_t s, const double *partials, int nb, const ReduceOut &ro) {
     if (ro.count) return;
     count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, ro.out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, ro);
 }
 
 template <typename T>
@@ -803,26 +806,34 @@ void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *
                         const double *fz, const double *diag, const double *b, bool b_scaled, const double *p,
                         float *r32, float s32, double *partials, ReduceOut ro) {
     // each kernel its own wave: the ghost tests take more registers, one resident block fewer per SM
-    auto run = [&](auto kernel, int nb) {
+    auto run = [&](auto kernel, int nb, bool last) {
+        ReduceOut o = ro;
+        if (!last) o.count = nullptr;
         count_launch();
-        run_kernel(kernel, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials, ro);
-        final_sums(s, partials, nb, ro);
+        run_kernel(kernel, nb, kReduceThreads, 0, s, d, L, h2, fx, fy, fz, diag, b, p, r32, s32, partials, o);
+        final_sums(s, partials, nb, o);
     };
+    const int cells = reduce_blocks(d.n), pairs = reduce_blocks(d.n / 2);
     if (d.nx & 1) {
         static const int wave_ct = wave_blocks((const void *)k_fine_resid_cell<true>, kReduceThreads);
         static const int wave_cf = wave_blocks((const void *)k_fine_resid_cell<false>, kReduceThreads);
-        if (b_scaled) run(k_fine_resid_cell<true>, fill_blocks(reduce_blocks(d.n), wave_ct));
-        else run(k_fine_resid_cell<false>, fill_blocks(reduce_blocks(d.n), wave_cf));
+        if (b_scaled) run(k_fine_resid_cell<true>, fill_blocks(cells, wave_ct), true);
+        else run(k_fine_resid_cell<false>, fill_blocks(cells, wave_cf), true);
     } else if (d.zlo || d.zhi) {
-        static const int wave_gt = wave_blocks((const void *)k_fine_resid_pair<true, true>, kReduceThreads);
-        static const int wave_gf = wave_blocks((const void *)k_fine_resid_pair<false, true>, kReduceThreads);
-        if (b_scaled) run(k_fine_resid_pair<true, true>, fill_blocks(reduce_blocks(d.n / 2), wave_gt));
-        else run(k_fine_resid_pair<false, true>, fill_blocks(reduce_blocks(d.n / 2), wave_gf));
+        static const int wave_gt = wave_blocks((const void *)k_fine_resid_pair<true, true, false>, kReduceThreads);
+        static const int wave_gf = wave_blocks((const void *)k_fine_resid_pair<false, true, false>, kReduceThreads);
+        if (b_scaled) run(k_fine_resid_pair<true, true, false>, fill_blocks(pairs, wave_gt), false);
+        else run(k_fine_resid_pair<false, true, false>, fill_blocks(pairs, wave_gf), false);
     } else {
-        static const int wave_pt = wave_blocks((const void *)k_fine_resid_pair<true, false>, kReduceThreads);
-        static const int wave_pf = wave_blocks((const void *)k_fine_resid_pair<false, false>, kReduceThreads);
-        if (b_scaled) run(k_fine_resid_pair<true, false>, fill_blocks(reduce_blocks(d.n / 2), wave_pt));
-        else run(k_fine_resid_pair<false, false>, fill_blocks(reduce_blocks(d.n / 2), wave_pf));
+        // both variants on the same grid: the partial sums do not depend on the variant
+        static const int wave_pt = wave_blocks((const void *)k_fine_resid_pair<true, false, false>, kReduceThreads);
+        static const int wave_pf = wave_blocks((const void *)k_fine_resid_pair<false, false, false>, kReduceThreads);
+        const int nb = fill_blocks(pairs, b_scaled ? wave_pt : wave_pf);
+        const bool last = ro.count && d.n <= kLastCells;
+        if (b_scaled && last) run(k_fine_resid_pair<true, false, true>, nb, true);
+        else if (b_scaled) run(k_fine_resid_pair<true, false, false>, nb, false);
+        else if (last) run(k_fine_resid_pair<false, false, true>, nb, true);
+        else run(k_fine_resid_pair<false, false, false>, nb, false);
     }
 }
 
@@ -895,7 +906,7 @@ void launch_adjoint_grad(cudaStream_t s, Dims d, double h, const double *lam, co
                                                  fx, fy, fz, csfx, csfy, csfz, (float)sigma, gx, gy, gz,
                                                  partials);
     count_launch();
-    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, out);
+    run_kernel(k_final, 1, kReduceThreads, 0, s, partials, nb, sums_to(out));
 }
 
 }  // namespace mg

@@ -133,7 +133,8 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
                            Upd up = Upd{}) {
     grid_wait();
     const int hx = L.hx, kv = hx >> 2;
-    const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    // black sweeps run from the last plane down: they begin with what the red one left in L2
+    const i64 t = (i64)(col ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
     const i64 rows = (i64)L.ny * L.nz;
     if (t >= rows * kv) return;
     // thread and row indices stay below 2^31 (at most 2e9 cells): 32-bit divisions, several
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(64, MINB) k_half_zf(Lay L, float h2, Coef32 cf
     const bool active = kvi < kv && yi < L.ny;
     const int k0 = min(kvi, kv - 1) << 2;
     const int y = min(yi, L.ny - 1);
-    const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, L.nz);
+    const int z0 = (col ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * ZC, z1 = min(z0 + ZC, L.nz);
     const int lane = threadIdx.x & 31;
     const i64 dy = hx, dz = (i64)L.ny * hx;
     const bool hy0 = y > 0, hy1 = y < L.ny - 1;
