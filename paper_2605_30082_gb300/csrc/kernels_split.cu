@@ -819,12 +819,10 @@ constexpr int kRrThreads = 64;
 
 // GHOST: the fine level is a slab (L.zlo / L.zhi) and Lc a view of the whole coarse level
 // (its arrays at the slab's first coarse plane, an even one)
-// TAIL: the coarse levels' cluster launch follows, which may come in and copy its contexts meanwhile
-template <bool SFORM, bool GHOST = false, bool TAIL = false>
+template <bool SFORM, bool GHOST = false>
 __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                              const float *__restrict__ xv, float *bc) {
     grid_wait();
-    if (TAIL) trigger_next();
     const int hx = L.hx, kv = hx >> 2;
     const i64 T = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     const i64 crows = (i64)Lc.ny * Lc.nz;
@@ -913,6 +911,108 @@ __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, fl
             acc[v] += bb[v] - ax * ih2;
         }
     }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) bc[sto(Lc, k0 + v, J, K)] = acc[v] * 0.125f;
+}
+
+// The same with one fine row per thread: lanes v, v + 8, v + 16, v + 24 of a warp take the four fine rows of
+// the same four coarse cells, and the first adds the four residuals up in their order.  Levels of up to
+// kRrRowCells cells have too few coarse cells to fill the device with k_rr_red_vec, whose threads then
+// wait for four rounds of loads: 64^3 2.8 -> 2.1 us (s-form) and 3.2 -> 2.0 us (faces), 96^3 3.4 -> 3.1 and 3.6 -> 2.9;
+// 128^3 4.5 against 6.0 us and 512^3 238 against 425 us, where it loads more lines than it uses.
+// TAIL: the coarse levels' cluster launch follows, which may come in and copy its contexts meanwhile.
+constexpr i64 kRrRowCells = 1000000;
+constexpr int kRrRowThreads = 128;
+template <bool SFORM, bool TAIL>
+__global__ void __launch_bounds__(kRrRowThreads, 6) k_rr_red_row(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
+                                                                 const float *__restrict__ xv, float *bc) {
+    grid_wait();
+    if (TAIL) trigger_next();
+    const int hx = L.hx, kv = hx >> 2;
+    const unsigned T = blockIdx.x * blockDim.x + threadIdx.x, lane = T & 31, total = (unsigned)Lc.ny * Lc.nz * kv;
+    const unsigned vi = (T >> 5) * 8 + (lane & 7), vc = min(vi, total - 1);  // 4-cell vector of the coarse level
+    const int ch = lane >> 3;
+    const unsigned crow = vc / (unsigned)kv;
+    const int k0 = (int)(vc - crow * (unsigned)kv) << 2;
+    const int J = (int)(crow % (unsigned)Lc.ny), K = (int)(crow / (unsigned)Lc.ny);
+    const i64 dy = hx, dz = (i64)L.ny * hx;
+    const int y = 2 * J + (ch & 1), z = 2 * K + (ch >> 1);
+    const int p = (y + z) & 1;  // red cells of this row sit at x = 2k + p
+    const i64 row = (i64)z * L.ny + y;
+    const i64 own = row * hx + k0, opp = L.half + row * hx + k0;
+    const bool hy0 = y > 0, hy1 = y < L.ny - 1, hz0 = z > 0, hz1 = z < L.nz - 1;
+    const bool xw0 = (p == 0 && k0 == 0), xw1 = (p == 1 && k0 + 4 == hx);
+    auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
+        const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
+        if (p) {
+            const float e = (k0 + 4 < hx) ? O[opp + 4] : 0.f;
+            m[0] = c4.x; m[1] = c4.y; m[2] = c4.z; m[3] = c4.w;
+            q[0] = c4.y; q[1] = c4.z; q[2] = c4.w; q[3] = e;
+        } else {
+            const float e = (k0 > 0) ? O[opp - 1] : 0.f;
+            m[0] = e; m[1] = c4.x; m[2] = c4.y; m[3] = c4.z;
+            q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
+        }
+    };
+    auto ld4 = [&](const float *A, i64 off, bool ok, float (&v)[4]) {
+        if (ok) {
+            const float4 c4 = *reinterpret_cast<const float4 *>(A + off);
+            v[0] = c4.x; v[1] = c4.y; v[2] = c4.z; v[3] = c4.w;
+        } else {
+            v[0] = v[1] = v[2] = v[3] = 0.f;
+        }
+    };
+    float xc[4], xm[4], xp[4], ym[4], yp[4], zm[4], zp[4], bb[4];
+    ld4(xv, own, true, xc);
+    window(xv, xm, xp);
+    ld4(xv, opp - dy, hy0, ym);
+    ld4(xv, opp + dy, hy1, yp);
+    ld4(xv, opp - dz, hz0, zm);
+    ld4(xv, opp + dz, hz1, zp);
+    ld4(b, own, true, bb);
+    float w0[4], w1[4], w2[4], w3[4], w4[4], w5[4];
+    if (SFORM) {
+        float sc[4], sm_[4], sp_[4], s2[4], s3[4], s4[4], s5[4];
+        ld4(cf.s, own, true, sc);
+        window(cf.s, sm_, sp_);
+        ld4(cf.s, opp - dy, hy0, s2);
+        ld4(cf.s, opp + dy, hy1, s3);
+        ld4(cf.s, opp - dz, hz0, s4);
+        ld4(cf.s, opp + dz, hz1, s5);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            w0[v] = (v == 0 && xw0) ? 0.f : 0.5f * (sc[v] + sm_[v]);
+            w1[v] = (v == 3 && xw1) ? 0.f : 0.5f * (sc[v] + sp_[v]);
+            w2[v] = hy0 ? 0.5f * (sc[v] + s2[v]) : 0.f;
+            w3[v] = hy1 ? 0.5f * (sc[v] + s3[v]) : 0.f;
+            w4[v] = hz0 ? 0.5f * (sc[v] + s4[v]) : 0.f;
+            w5[v] = hz1 ? 0.5f * (sc[v] + s5[v]) : 0.f;
+        }
+    } else {
+        float d0[4];
+        ld4(cf.fx, own, true, w0);
+        window(cf.fx, d0, w1);
+        if (xw1) w1[3] = 0.f;
+        ld4(cf.fy, own, true, w2);
+        ld4(cf.fy, opp + dy, hy1, w3);
+        ld4(cf.fz, own, true, w4);
+        ld4(cf.fz, opp + dz, hz1, w5);
+    }
+    float acc[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        // the sum of products in the order k_rr_red_vec forms it
+        float ax = fmaf(w0[v], xc[v] - xm[v], w1[v] * (xc[v] - xp[v]));
+        ax = fmaf(w2[v], xc[v] - ym[v], ax);
+        ax = fmaf(w3[v], xc[v] - yp[v], ax);
+        ax = fmaf(w4[v], xc[v] - zm[v], ax);
+        ax = fmaf(w5[v], xc[v] - zp[v], ax);
+        const float r = fmaf(-ax, ih2, bb[v]);
+        const float r1 = __shfl_down_sync(0xffffffffu, r, 8), r2 = __shfl_down_sync(0xffffffffu, r, 16);
+        const float r3 = __shfl_down_sync(0xffffffffu, r, 24);
+        acc[v] = ((r + r1) + r2) + r3;
+    }
+    if (vi >= total || ch) return;
 #pragma unroll
     for (int v = 0; v < 4; ++v) bc[sto(Lc, k0 + v, J, K)] = acc[v] * 0.125f;
 }
@@ -1065,6 +1165,55 @@ __global__ void __launch_bounds__(kProlThreads, 10) k_prolong_red8(Lay L, Lay Lc
             *reinterpret_cast<float4 *>(xr + 4) = make_float4(o[4], o[5], o[6], o[7]);
         }
     }
+}
+
+// The same with one fine row per thread (four coarse rows each, the sums in the same order): four times the
+// threads on levels of up to kProlRowCells cells, 64^3 2.6 -> 1.6 us, 96^3 3.4 -> 2.2, 192^3 7.9 -> 7.2; 256^3 12.2 against
+// 14.3 us, where the coarse rows read again cost more.
+constexpr i64 kProlRowCells = 8000000;
+constexpr int kProlRowThreads = 128;
+__global__ void __launch_bounds__(kProlRowThreads, 8) k_prolong_red_row(Lay L, Lay Lc, const float *__restrict__ ec, float *xv) {
+    grid_wait();
+    const int hx = L.hx, kv = hx >> 3;  // 8-cell groups per fine row
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = t / (unsigned)kv;
+    if (row >= (unsigned)L.ny * L.nz) return;
+    const int k0 = (int)(t - row * (unsigned)kv) << 3;
+    const int y = (int)(row % (unsigned)L.ny), z = (int)(row / (unsigned)L.ny);
+    const int d = y & 1, e = z & 1, J = y >> 1, K = z >> 1, hxc = Lc.hx;
+    const int J2 = d ? min(J + 1, Lc.ny - 1) : max(J - 1, 0), K2 = e ? min(K + 1, Lc.nz - 1) : max(K - 1, 0);
+    float *xr = xv + (i64)row * hx + k0;
+    const float4 a4 = *reinterpret_cast<const float4 *>(xr), b4 = *reinterpret_cast<const float4 *>(xr + 4);
+    float R[10];
+#pragma unroll
+    for (int u = 0; u < 10; ++u) R[u] = 0.f;
+    // coarse rows in the order J - 1, J, J + 1 and, in each, K - 1, K, K + 1
+#pragma unroll
+    for (int ja = 0; ja < 2; ++ja) {
+#pragma unroll
+        for (int ka = 0; ka < 2; ++ka) {
+            const bool jn = ja == d, kn = ka == e;  // the neighbour row comes first for d = 0, last for d = 1
+            const int JJ = jn ? J2 : J, KK = kn ? K2 : K, q = (JJ + KK) & 1;
+            const i64 rowc = (i64)KK * Lc.ny + JJ;
+            const float *ev = ec + (i64)q * Lc.half + rowc * hxc;        // even I, position I / 2
+            const float *od = ec + (i64)(1 - q) * Lc.half + rowc * hxc;  // odd I
+            const float4 e4 = *reinterpret_cast<const float4 *>(ev + (k0 >> 1));
+            const float4 o4 = *reinterpret_cast<const float4 *>(od + (k0 >> 1));
+            float v[10];
+            v[1] = e4.x; v[2] = o4.x; v[3] = e4.y; v[4] = o4.y;
+            v[5] = e4.z; v[6] = o4.z; v[7] = e4.w; v[8] = o4.w;
+            v[0] = k0 > 0 ? od[(k0 >> 1) - 1] : v[1];
+            v[9] = k0 + 8 < Lc.nx ? ev[(k0 >> 1) + 4] : v[8];
+            const float w = (jn ? 0.25f : 0.75f) * (kn ? 0.25f : 0.75f);
+#pragma unroll
+            for (int u = 0; u < 10; ++u) R[u] = fmaf(w, v[u], R[u]);
+        }
+    }
+    const int p = (d + e) & 1;  // red x = 2k + p
+    float o[8] = {a4.x, a4.y, a4.z, a4.w, b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+    for (int v = 0; v < 8; ++v) o[v] += fmaf(0.75f, R[v + 1], 0.25f * (p ? R[v + 2] : R[v]));
+    *reinterpret_cast<float4 *>(xr) = make_float4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<float4 *>(xr + 4) = make_float4(o[4], o[5], o[6], o[7]);
 }
 
 // ---- residual (generic) ------------------------------------------------------------------
@@ -1295,19 +1444,24 @@ void launch_resid_restrict32(cudaStream_t s, Lay L, Lay Lc, double ih2, const fl
     Coef32 cf{sinv, fx, fy, fz};
     count_launch();
     if (red_only && L.split && L.hx % 4 == 0) {
-        if (tail) {
-            // the cluster's CTAs want most of an SM's shared memory, which has to be set aside already
-            static std::atomic<unsigned long long> carved[2];
-            if (!prefer_smem((const void *)k_rr_red_vec<true, false, true>, carved[0]) ||
-                !prefer_smem((const void *)k_rr_red_vec<false, false, true>, carved[1]))
-                (void)cudaGetLastError();  // a preference only
-        }
         const i64 work = (i64)Lc.ny * Lc.nz * (L.hx / 4);
+        if (!(L.zlo || L.zhi) && L.n <= kRrRowCells) {
+            if (tail) {
+                // the cluster's CTAs want most of an SM's shared memory, which has to be set aside already
+                static std::atomic<unsigned long long> carved[2];
+                if (!prefer_smem((const void *)k_rr_red_row<true, true>, carved[0]) ||
+                    !prefer_smem((const void *)k_rr_red_row<false, true>, carved[1]))
+                    (void)cudaGetLastError();  // a preference only
+            }
+            auto kernel = sinv ? (tail ? k_rr_red_row<true, true> : k_rr_red_row<true, false>)
+                               : (tail ? k_rr_red_row<false, true> : k_rr_red_row<false, false>);
+            run_kernel(kernel, (unsigned)((4 * ((work + 7) / 8 * 8) + kRrRowThreads - 1) / kRrRowThreads), kRrRowThreads, 0, s, L, Lc,
+                       (float)ih2, cf, b, x, bc);
+            return;
+        }
         const unsigned nb = (unsigned)((work + kRrThreads - 1) / kRrThreads);
         if ((L.zlo || L.zhi) && sinv) run_kernel(k_rr_red_vec<true, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else if (L.zlo || L.zhi) run_kernel(k_rr_red_vec<false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
-        else if (tail && sinv) run_kernel(k_rr_red_vec<true, false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
-        else if (tail) run_kernel(k_rr_red_vec<false, false, true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else if (sinv) run_kernel(k_rr_red_vec<true>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         else run_kernel(k_rr_red_vec<false>, nb, kRrThreads, 0, s, L, Lc, (float)ih2, cf, b, x, bc);
         return;
@@ -1320,6 +1474,10 @@ void launch_prolong32(cudaStream_t s, Lay L, Lay Lc, const float *ec, float *x, 
     if (only_col == 0 && kind == MG_PROLONG_TRILINEAR && L.split && Lc.split && Lc.nx % 8 == 0 &&
         2 * Lc.nx == L.nx && 2 * Lc.ny == L.ny && 2 * Lc.nz == L.nz) {
         const i64 work = (i64)Lc.ny * Lc.nz * (L.hx / 8);
+        if (!(Lc.zlo || Lc.zhi) && L.n <= kProlRowCells) {
+            run_kernel(k_prolong_red_row, (unsigned)((4 * work + kProlRowThreads - 1) / kProlRowThreads), kProlRowThreads, 0, s, L, Lc, ec, x);
+            return;
+        }
         const unsigned nb = (unsigned)((work + kProlThreads - 1) / kProlThreads);
         if (Lc.zlo || Lc.zhi) run_kernel(k_prolong_red8<true>, nb, kProlThreads, 0, s, L, Lc, ec, x);
         else run_kernel(k_prolong_red8<false>, nb, kProlThreads, 0, s, L, Lc, ec, x);
