@@ -58,9 +58,12 @@ __device__ __forceinline__ T flux_sum(const Dims &d, int i, int j, int k, i64 c,
 
 // red-black Gauss-Seidel half sweep of colour q ((i+j+k) % 2 == q), in place:
 //   x_c = (h2 b_c + sum_f beta_f x_nb) * invd_c   (invd = 1 / sum_f beta_f)
-// one thread per cell of the colour; used by the FP64 V-cycle, whose cost is
-// FP64 arithmetic rather than bytes, so it keeps zero redundant work
-template <typename T>
+// one thread per cell of the colour; used by the FP64 V-cycle.  Eight FP64 operations a cell (110 us for a
+// half sweep of 256^3) against 48 bytes per cell of the grid: the faces, of which a half sweep needs all, x in
+// natural order (all of its lines read, all written), and half of b and invd where these lie colour by colour as in
+// Lay (BSPLIT, DSPLIT; even nx; b then times h2): 56 bytes in natural order took 137 us, 122 us in colour order.
+// ZERO (red, x = 0 on entry): x = h2 b invd, no neighbour is read
+template <bool BSPLIT, bool DSPLIT, bool ZERO, typename T>
 __global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T *x, int colour) {
     grid_wait();
     const int half = (d.nx + 1) >> 1;
@@ -75,8 +78,9 @@ __global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T
     const int i = 2 * m + ((colour + j + k) & 1);
     if (i >= d.nx) return;
     const i64 c = row * d.nx + i;
-    const T num = nb_sum(d, i, j, k, c, cf, x);
-    x[c] = (h2 * b[c] + num) * cf.invd[c];
+    const i64 cs = colour * (d.n >> 1) + t;  // its place in colour order
+    const T num = ZERO ? T(0) : nb_sum(d, i, j, k, c, cf, x);
+    x[c] = (BSPLIT ? b[cs] + num : h2 * b[c] + num) * cf.invd[DSPLIT ? cs : c];
 }
 
 template <typename T>
@@ -160,7 +164,9 @@ __global__ void k_prolong(Dims cd, Dims f, const T *__restrict__ ec, T *e, int k
 // Red-only residual + restriction in diagonal form on a level with the diagonal d = sum beta:
 //   h^2 r_c = h^2 b_c + sum_f beta_f x_nb - d_c x_c   (7 FMA and one multiply per red child),
 // coarse b = ih2/8 * (sum over the 4 red children).  Blocks take coarse rows (grid y, strided),
-// threads coarse I: no 64-bit division per cell.
+// threads coarse I: no 64-bit division per cell.  BSPLIT: h2 b colour by
+// colour as in Lay (even nx): 256^3 165 -> 133 us
+template <bool BSPLIT>
 __global__ void k_rr_red_diag64(Dims f, Dims cd, double h2, double ih2_8, Coef<double> cf,
                                 const double *__restrict__ dg, const double *__restrict__ b,
                                 const double *__restrict__ x, double *bc) {
@@ -176,7 +182,7 @@ __global__ void k_rr_red_diag64(Dims f, Dims cd, double h2, double ih2_8, Coef<d
             const int j = 2 * J + (q & 1), k = 2 * K + (q >> 1);
             const int i = 2 * I + ((j + k) & 1);  // the red child in this fine row
             const i64 c = ((i64)k * f.ny + j) * f.nx + i;
-            double a = h2 * b[c];
+            double a = BSPLIT ? b[((i64)k * f.ny + j) * (f.nx >> 1) + I] : h2 * b[c];
             if (i > 0) a = fma(cf.fx[c], x[c - 1], a);
             if (i < f.nx - 1) a = fma(cf.fx[c + 1], x[c + 1], a);
             if (j > 0) a = fma(cf.fy[c], x[c - f.nx], a);
@@ -226,6 +232,55 @@ __global__ void k_prolong_col(Dims cd, Dims f, const T *__restrict__ ec, T *e, i
     }
 }
 
+// k_prolong_col for the red cells, FP64, trilinear: a thread takes one coarse cell and its four red children.
+// The weights 3/4 and 1/4 per axis become 3 and 1 with 1/64 in the last multiply-add, y and z are summed before x
+// and shared between the children, and the neighbour's sums in x come from shared memory:
+// 18 FP64 operations per four children against 36 with the eight products written out; these still bound it: 62 of
+// 78 us into 256^3 (42 us of bytes), which took 148 us.
+// A block takes kProlOut consecutive coarse cells; its first and last thread only form their sums.
+constexpr int kProl64 = 256, kProlOut = kProl64 - 2;
+__global__ void __launch_bounds__(kProl64) k_prolong_red64(Dims cd, const double *__restrict__ ec, double *x) {
+    grid_wait();
+    __shared__ double S[4][kProl64];
+    const int t = threadIdx.x;
+    const i64 C = (i64)blockIdx.x * kProlOut + t - 1;
+    const unsigned cu = (unsigned)(C < 0 ? 0 : (C < cd.n ? C : cd.n - 1)), row = cu / (unsigned)cd.nx;
+    const int I = (int)(cu - row * (unsigned)cd.nx), J = (int)(row % (unsigned)cd.ny), K = (int)(row / (unsigned)cd.ny);
+    const double *e0 = ec + cu;
+    const i64 ym = J > 0 ? -cd.nx : 0, yp = J + 1 < cd.ny ? cd.nx : 0;  // at a wall the cell itself
+    const i64 zm = K > 0 || cd.zlo ? -cd.nxy : 0, zp = K + 1 < cd.nz || cd.zhi ? cd.nxy : 0;
+    double A[2][3];  // per y child, in the planes K - 1, K, K + 1
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double *e = e0 + (q == 0 ? zm : q == 2 ? zp : 0);
+        const double c = e[0];
+        A[0][q] = fma(3.0, c, e[ym]);
+        A[1][q] = fma(3.0, c, e[yp]);
+    }
+    double s[2][2];  // per y and z child
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        s[d][0] = fma(3.0, A[d][1], A[d][0]);
+        s[d][1] = fma(3.0, A[d][1], A[d][2]);
+        S[2 * d][t] = s[d][0];
+        S[2 * d + 1][t] = s[d][1];
+    }
+    __syncthreads();
+    if (t == 0 || t == kProl64 - 1 || C >= cd.n) return;
+    const int nx = 2 * cd.nx, ny = 2 * cd.ny;
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int p = d ^ e;  // the red child sits at x = 2I + p
+            const bool in = p ? I + 1 < cd.nx : I > 0;
+            const double v = fma(3.0, s[d][e], S[2 * d + e][in ? (p ? t + 1 : t - 1) : t]);
+            double *xc = x + ((i64)(2 * K + e) * ny + 2 * J + d) * nx + 2 * I + p;
+            *xc = fma(v, 0.015625, *xc);
+        }
+    }
+}
+
 template <typename T>
 __global__ void k_coarse_matvec(int nc, const double *__restrict__ pinv, const T *__restrict__ r,
                                 T *e) {
@@ -243,11 +298,14 @@ __global__ void k_coarse_matvec(int nc, const double *__restrict__ pinv, const T
 
 }  // namespace
 
-void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const double *b, double *p,
-                        int colour) {
+void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const double *b, double *p, int colour,
+                        bool b_split, bool invd_split, bool from_zero) {
     const i64 work = (i64)d.ny * d.nz * ((d.nx + 1) / 2);
     count_launch();
-    run_kernel(k_rbgs_half<double>, blocks_for(work), kThreads, 0, s, d, h2, c, b, p, colour);
+    auto kernel = !invd_split ? (from_zero ? k_rbgs_half<false, false, true, double> : k_rbgs_half<false, false, false, double>)
+                  : !b_split  ? (from_zero ? k_rbgs_half<false, true, true, double> : k_rbgs_half<false, true, false, double>)
+                              : k_rbgs_half<true, true, false, double>;
+    run_kernel(kernel, blocks_for(work), kThreads, 0, s, d, h2, c, b, p, colour);
 }
 
 template <typename T>
@@ -274,6 +332,12 @@ template <typename T>
 void launch_prolong(cudaStream_t s, Dims coarse, const T *ec, T *e, int kind, int only_col) {
     Dims f = make_dims(coarse.nx * 2, coarse.ny * 2, coarse.nz * 2);
     count_launch();
+    if constexpr (std::is_same<T, double>::value) {
+        if (only_col == 0 && kind == MG_PROLONG_TRILINEAR) {
+            run_kernel(k_prolong_red64, (unsigned)((coarse.n + kProlOut - 1) / kProlOut), kProl64, 0, s, coarse, ec, e);
+            return;
+        }
+    }
     if (only_col >= 0) {
         const unsigned gx = (unsigned)(((f.nx + 1) / 2 + 127) / 128);
         const i64 rows = (i64)f.ny * f.nz;
@@ -285,13 +349,14 @@ void launch_prolong(cudaStream_t s, Dims coarse, const T *ec, T *e, int kind, in
 }
 
 void launch_rr_red_diag64(cudaStream_t s, Dims fine, double h2, Coef<double> c, const double *dg,
-                          const double *b, const double *x, double *bc) {
+                          const double *b, const double *x, double *bc, bool b_split) {
     Dims cd = make_dims(fine.nx / 2, fine.ny / 2, fine.nz / 2);
     count_launch();
     const unsigned gx = (unsigned)((cd.nx + 127) / 128);
     const i64 crows = (i64)cd.ny * cd.nz;
     const unsigned gy = (unsigned)(crows < 65535 ? crows : 65535);
-    run_kernel(k_rr_red_diag64, dim3(gx, gy), 128, 0, s, fine, cd, h2, 1.0 / (8.0 * h2), c, dg, b, x, bc);
+    run_kernel(b_split ? k_rr_red_diag64<true> : k_rr_red_diag64<false>, dim3(gx, gy), 128, 0, s, fine, cd, h2, 1.0 / (8.0 * h2), c, dg,
+               b, x, bc);
 }
 
 template <typename T>

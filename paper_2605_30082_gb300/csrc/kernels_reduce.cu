@@ -241,18 +241,32 @@ __device__ __forceinline__ double mul_pow2(double v, int m, double s) {
 // thread and iteration, where b and b64 are 16-byte aligned (as k_sum_sumsq).  With POW2
 // (scale = 2^m: 1 in the FP64 mode, h^2 in the mixed modes when h is a power of two) the
 // scaling is an exponent addition: two FP64 operations per element instead of three.
-template <bool POW2>
+// SPLIT: b64 colour by colour as in Lay (d: the grid, even nx)
+template <bool POW2, bool SPLIT>
 __global__ void __launch_bounds__(kReduceThreads, 5) k_sub_mean(i64 n, const double *__restrict__ b, const double *__restrict__ sum,
-                           double scale, int m2, double *b64, double *partials, ReduceOut ro) {
+                           double scale, int m2, double *b64, double *partials, ReduceOut ro, Dims d) {
     grid_wait();
     const double mean = sum[0] / (double)n;
     double q = 0.0;
     auto f = [&](double u) { return POW2 ? mul_pow2(u - mean, m2, scale) : (u - mean) * scale; };
     const i64 tid = (i64)blockIdx.x * blockDim.x + threadIdx.x, nt = (i64)gridDim.x * blockDim.x;
+    // cells 2m and 2m + 1 of a row lie at m in the two colours' halves
+    auto red_first = [&](i64 m) {
+        const unsigned row = (unsigned)m / (unsigned)(d.nx >> 1);
+        return ((row % (unsigned)d.ny + row / (unsigned)d.ny) & 1) == 0;
+    };
+    auto put = [&](i64 m, double2 w) {
+        if (SPLIT) {
+            const bool r = red_first(m);
+            b64[m] = r ? w.x : w.y;
+            b64[(n >> 1) + m] = r ? w.y : w.x;
+        } else {
+            reinterpret_cast<double2 *>(b64)[m] = w;
+        }
+    };
     i64 m0 = 0;
     if (aligned16(b) && aligned16(b64)) {
         const double2 *bv = reinterpret_cast<const double2 *>(b);
-        double2 *ov = reinterpret_cast<double2 *>(b64);
         const i64 nv = n / 2;
         for (i64 m = tid; m < nv; m += 2 * nt) {
             const double2 u0 = bv[m];
@@ -260,12 +274,12 @@ __global__ void __launch_bounds__(kReduceThreads, 5) k_sub_mean(i64 n, const dou
             double2 u1 = u0;
             if (two) u1 = bv[m + nt];
             const double2 w0 = make_double2(f(u0.x), f(u0.y));
-            ov[m] = w0;
+            put(m, w0);
             q += w0.x * w0.x;
             q += w0.y * w0.y;
             if (two) {
                 const double2 w1 = make_double2(f(u1.x), f(u1.y));
-                ov[m + nt] = w1;
+                put(m + nt, w1);
                 q += w1.x * w1.x;
                 q += w1.y * w1.y;
             }
@@ -274,7 +288,7 @@ __global__ void __launch_bounds__(kReduceThreads, 5) k_sub_mean(i64 n, const dou
     }
     for (i64 m = m0 + tid; m < n; m += nt) {
         const double v = f(b[m]);
-        b64[m] = v;
+        b64[SPLIT ? (red_first(m >> 1) == ((m & 1) == 0) ? 0 : (n >> 1)) + (m >> 1) : m] = v;
         q += v * v;
     }
     block_sum2(q, 0.0, partials + 2 * blockIdx.x);
@@ -296,12 +310,14 @@ __device__ __forceinline__ i64 sto(const Lay &L, int x, int y, int z) {
 // GHOST: a slab of a decomposed grid (d.zlo / d.zhi): its ghost planes count as interior
 // neighbours; whole-grid levels compile without the two extra tests.  LAST: the last block adds up
 // the partials (finish_reduction); its registers cost the loop about a tenth (256^3 206 -> 226 us), so only
-// grids of up to kLastCells cells, where a launch of k_final costs more, take that variant
-template <bool SCALED, bool GHOST, bool LAST>
-__global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
-                                  const double *__restrict__ fy, const double *__restrict__ fz,
-                                  const double *__restrict__ dg, const double *__restrict__ b,
-                                  const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
+// grids of up to kLastCells cells, where a launch of k_final costs more, take that variant.  BSPLIT: b colour by
+// colour as in Lay
+template <bool SCALED, bool GHOST, bool LAST, bool BSPLIT>
+__device__ __forceinline__ void fine_resid_pair(const Dims &d, const Lay &L, double h2, const double *__restrict__ fx,
+                                                const double *__restrict__ fy, const double *__restrict__ fz,
+                                                const double *__restrict__ dg, const double *__restrict__ b,
+                                                const double *__restrict__ p, float *r32, float s32, double *partials,
+                                                const ReduceOut &ro) {
     grid_wait();
     float q = 0.f, sp = 0.f;
     const int nx = d.nx, ny = d.ny, nz = d.nz, hx = nx >> 1;
@@ -312,7 +328,14 @@ __global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__rest
         const int j = row % ny, z = row / ny;
         const int c = row * nx + 2 * k;  // cells c (x = 2k) and c + 1
         const double2 pc = *reinterpret_cast<const double2 *>(p + c);
-        const double2 bb = *reinterpret_cast<const double2 *>(b + c);
+        double2 bb;
+        if (BSPLIT) {
+            const bool red_first = ((j + z) & 1) == 0;
+            const double r = b[t], q = b[npairs + t];
+            bb = make_double2(red_first ? r : q, red_first ? q : r);
+        } else {
+            bb = *reinterpret_cast<const double2 *>(b + c);
+        }
         const double2 fxa = *reinterpret_cast<const double2 *>(fx + c);   // low x faces of both cells
         const double2 fya = *reinterpret_cast<const double2 *>(fy + c);
         const double2 fza = *reinterpret_cast<const double2 *>(fz + c);
@@ -361,6 +384,24 @@ __global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__rest
     }
     block_sum2((double)q, (double)sp, partials + 2 * blockIdx.x);
     if (LAST) finish_reduction(partials, ro);
+}
+
+template <bool SCALED, bool GHOST, bool LAST>
+__global__ void k_fine_resid_pair(Dims d, Lay L, double h2, const double *__restrict__ fx,
+                                  const double *__restrict__ fy, const double *__restrict__ fz,
+                                  const double *__restrict__ dg, const double *__restrict__ b,
+                                  const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
+    fine_resid_pair<SCALED, GHOST, LAST, false>(d, L, h2, fx, fy, fz, dg, b, p, r32, s32, partials, ro);
+}
+
+// the FP64 V-cycle iteration's, h2 b colour by colour: 256^3 264 us with b unscaled in natural order, 210 us; the
+// select between the two colours would take a sixth of the resident blocks without the bound
+template <bool LAST>
+__global__ void __launch_bounds__(kReduceThreads, 5)
+    k_fine_resid_pair_bs(Dims d, Lay L, double h2, const double *__restrict__ fx, const double *__restrict__ fy,
+                         const double *__restrict__ fz, const double *__restrict__ dg, const double *__restrict__ b,
+                         const double *__restrict__ p, float *r32, float s32, double *partials, ReduceOut ro) {
+    fine_resid_pair<true, false, LAST, true>(d, L, h2, fx, fy, fz, dg, b, p, r32, s32, partials, ro);
 }
 
 // n4 words, the first 4 nv of them as 16-byte stores
@@ -790,21 +831,22 @@ template void launch_sum_sumsq<double>(cudaStream_t, i64, const double *, double
 template void launch_sum_sumsq<float>(cudaStream_t, i64, const float *, double *, ReduceOut, bool);
 
 void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, double scale, double *b64,
-                     double *partials, ReduceOut ro) {
-    static const int wave_p = wave_blocks((const void *)k_sub_mean<true>, kReduceThreads);
-    static const int wave_m = wave_blocks((const void *)k_sub_mean<false>, kReduceThreads);
+                     double *partials, ReduceOut ro, const Dims *split) {
+    static const int wave_p = wave_blocks((const void *)k_sub_mean<true, false>, kReduceThreads);
+    static const int wave_m = wave_blocks((const void *)k_sub_mean<false, false>, kReduceThreads);
     int e = 0;
     const bool pow2 = std::frexp(scale, &e) == 0.5;  // scale = 2^(e - 1)
     const int nb = fill_blocks(reduce_blocks(n), pow2 ? wave_p : wave_m);
     count_launch();
-    if (pow2) run_kernel(k_sub_mean<true>, nb, kReduceThreads, 0, s, n, b, sum, scale, e - 1, b64, partials, ro);
-    else run_kernel(k_sub_mean<false>, nb, kReduceThreads, 0, s, n, b, sum, scale, 0, b64, partials, ro);
+    auto kernel = pow2 ? (split ? k_sub_mean<true, true> : k_sub_mean<true, false>)
+                       : (split ? k_sub_mean<false, true> : k_sub_mean<false, false>);
+    run_kernel(kernel, nb, kReduceThreads, 0, s, n, b, sum, scale, pow2 ? e - 1 : 0, b64, partials, ro, split ? *split : Dims{});
     final_sums(s, partials, nb, ro);
 }
 
 void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *fx, const double *fy,
                         const double *fz, const double *diag, const double *b, bool b_scaled, const double *p,
-                        float *r32, float s32, double *partials, ReduceOut ro) {
+                        float *r32, float s32, double *partials, ReduceOut ro, bool b_split) {
     // each kernel its own wave: the ghost tests take more registers, one resident block fewer per SM
     auto run = [&](auto kernel, int nb, bool last) {
         ReduceOut o = ro;
@@ -830,7 +872,9 @@ void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *
         static const int wave_pf = wave_blocks((const void *)k_fine_resid_pair<false, false, false>, kReduceThreads);
         const int nb = fill_blocks(pairs, b_scaled ? wave_pt : wave_pf);
         const bool last = ro.count && d.n <= kLastCells;
-        if (b_scaled && last) run(k_fine_resid_pair<true, false, true>, nb, true);
+        if (b_split && last) run(k_fine_resid_pair_bs<true>, nb, true);
+        else if (b_split) run(k_fine_resid_pair_bs<false>, nb, false);
+        else if (b_scaled && last) run(k_fine_resid_pair<true, false, true>, nb, true);
         else if (b_scaled) run(k_fine_resid_pair<true, false, false>, nb, false);
         else if (last) run(k_fine_resid_pair<false, false, true>, nb, true);
         else run(k_fine_resid_pair<false, false, false>, nb, false);

@@ -151,7 +151,7 @@ __global__ void k_faces_to_api(Dims d, const double *__restrict__ fx, const doub
 }
 
 __global__ void k_invdiag(Dims d, const double *__restrict__ fx, const double *__restrict__ fy,
-                          const double *__restrict__ fz, double *invd64, double *diag) {
+                          const double *__restrict__ fz, double *invd64, i64 invd_half, double *diag) {
     grid_wait();
     i64 c = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d.n) return;
@@ -166,7 +166,8 @@ __global__ void k_invdiag(Dims d, const double *__restrict__ fx, const double *_
     if (j < d.ny - 1) s += fy[c + d.nx];
     s += fz[c];
     if (k < d.nz - 1 || d.zhi) s += fz[c + d.nxy];  // a slab's face to its ghost plane counts
-    if (invd64) invd64[c] = recip64(s);
+    // colour by colour (invd_half = n / 2, even nx) or, with invd_half 0, in natural order
+    if (invd64) invd64[invd_half ? ((i + j + k) & 1) * invd_half + (c >> 1) : c] = recip64(s);
     if (diag) diag[c] = s;
 }
 
@@ -301,10 +302,10 @@ void launch_faces_to_api(cudaStream_t s, Dims d, const double *fx, const double 
 }
 
 void launch_invdiag(cudaStream_t s, Dims d, const double *fx, const double *fy, const double *fz,
-                    double *invd64, double *diag) {
+                    double *invd64, i64 invd_half, double *diag) {
     if (!invd64 && !diag) return;
     count_launch();
-    run_kernel(k_invdiag, blocks_for(d.n), kThreads, 0, s, d, fx, fy, fz, invd64, diag);
+    run_kernel(k_invdiag, blocks_for(d.n), kThreads, 0, s, d, fx, fy, fz, invd64, invd_half, diag);
 }
 
 void launch_coarsen(cudaStream_t s, Dims fine, const double *ffx, const double *ffy,

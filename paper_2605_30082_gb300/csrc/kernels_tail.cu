@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
             f[4] = fz[g];
             if (z < L.nz - 1) f[5] = fz[U::gidx(L, 1 - col, k, y, z + 1)];
             if constexpr (U::f64) {
-                f[6] = reinterpret_cast<const T *>(L.invd)[g];
+                f[6] = reinterpret_cast<const T *>(L.invd)[col * L.half + ((i64)z * L.ny + y) * L.hx + k];
                 f[7] = reinterpret_cast<const T *>(L.diag)[g];
             } else {
                 f[6] = ((f[0] + f[1]) + (f[2] + f[3])) + (f[4] + f[5]);

@@ -52,7 +52,7 @@ struct mg_handle {
     Level lv[MG_MAX_LEVELS];
     int nc;
     double *pinv, *pinv_tmp;
-    double *bt;        // zero-mean fine RHS (scaled by h^2 in the mixed modes)
+    double *bt;        // zero-mean fine RHS (scaled by h^2 but in the FP64 CG; FP64 V-cycle: colour by colour)
     float2 *bt2, *p2;  // MIXED_DF: the RHS and the solution as FP32 pairs
     double *partials;  // reduction partials
     // flexible CG (MG_METHOD_FCG): FP32 finest-level vectors (mixed; r and x are the level's
@@ -222,40 +222,42 @@ void run_tail(mg_handle *h) {
 }
 
 // ---- FP64 V-cycle: in-place per-colour half sweeps, standalone transfers --------------
-// (FP64 arithmetic, not bytes, bounds these kernels on GB300, so they do no
-// redundant work; see the fused FP32 passes below for the bandwidth-bound cycle)
-void smooth64(mg_handle *h, int l, double *x, const double *b, int sweeps, int order) {
+// (FP64 arithmetic and the face arrays bound these kernels on GB300 about equally; the
+// reciprocal diagonal lies colour by colour, and with bs so does b, times h^2).  zero: x = 0, not yet written
+void smooth64(mg_handle *h, int l, double *x, const double *b, int sweeps, int order, bool bs = false, bool zero = false) {
     Level &L = h->lv[l];
     for (int sw = 0; sw < sweeps; ++sw)
         for (int half = 0; half < 2; ++half) {
             if (l == 0) prof_begin(h, MG_PROF_SMOOTH);
-            mg::launch_rbgs_half64(h->s, L.d, L.h2, coef<double>(L), b, x, order ? 1 - half : half);
+            mg::launch_rbgs_half64(h->s, L.d, L.h2, coef<double>(L), b, x, order ? 1 - half : half, bs, L.lay.split,
+                                   zero && sw == 0 && half == 0);
             if (l == 0) prof_end(h);
         }
 }
 
-void presmooth_restrict64(mg_handle *h, int l, const double *b, double *x, double *bc, int sweeps) {
+void presmooth_restrict64(mg_handle *h, int l, const double *b, double *x, double *bc, int sweeps, bool bs = false, bool zero = false) {
     Level &L = h->lv[l];
-    smooth64(h, l, x, b, sweeps, 0);
+    if (zero && sweeps == 0) mg::launch_zero(h->s, x, sizeof(double) * (size_t)L.d.n);
+    smooth64(h, l, x, b, sweeps, 0, bs, zero);
     if (l == 0) prof_begin(h, MG_PROF_RESID_RESTRICT);
     // after a pre-smoothing sweep (black last) every black residual is zero
     if (sweeps > 0 && L.d64)
-        mg::launch_rr_red_diag64(h->s, L.d, L.h2, coef<double>(L), L.d64, b, x, bc);
+        mg::launch_rr_red_diag64(h->s, L.d, L.h2, coef<double>(L), L.d64, b, x, bc, bs);
     else
         mg::launch_resid_restrict<double>(h->s, L.d, L.ih2, coef<double>(L), b, x, bc, sweeps > 0);
     if (l == 0) prof_end(h);
 }
 
-void prolong_postsmooth64(mg_handle *h, int l, const double *b, const double *ec, double *x, int sweeps) {
+void prolong_postsmooth64(mg_handle *h, int l, const double *b, const double *ec, double *x, int sweeps, bool bs = false) {
     if (l == 0) prof_begin(h, MG_PROF_PROLONG);
     // the first post sweep (black first) overwrites every black cell: correct the red ones only
     mg::launch_prolong<double>(h->s, h->lv[l + 1].d, ec, x, h->o.prolong, sweeps > 0 ? 0 : -1);
     if (l == 0) prof_end(h);
-    smooth64(h, l, x, b, sweeps, 1);
+    smooth64(h, l, x, b, sweeps, 1, bs);
 }
 
-// one V-cycle on level l for A x = b, x in place (x_zero: x starts at zero)
-void vcycle64(mg_handle *h, int l, const double *b, double *x, bool x_zero) {
+// one V-cycle on level l for A x = b, x in place (x_zero: x starts at zero; bs: h^2 b colour by colour)
+void vcycle64(mg_handle *h, int l, const double *b, double *x, bool x_zero, bool bs = false) {
     if (l == h->nlev - 1) {
         if (l == 0) prof_begin(h, MG_PROF_COARSE);
         mg::launch_coarse_matvec<double>(h->s, h->nc, h->pinv, b, x);
@@ -267,12 +269,11 @@ void vcycle64(mg_handle *h, int l, const double *b, double *x, bool x_zero) {
         run_tail(h);
         return;
     }
-    if (x_zero) mg::launch_zero(h->s, x, sizeof(double) * (size_t)L.d.n);
-    presmooth_restrict64(h, l, b, x, C.b64, h->o.pre);
+    presmooth_restrict64(h, l, b, x, C.b64, h->o.pre, bs, x_zero);
     if (l == 0) prof_begin(h, MG_PROF_COARSE_LEVELS);
     vcycle64(h, l + 1, C.b64, C.x64, true);
     if (l == 0) prof_end(h);
-    prolong_postsmooth64(h, l, b, C.x64, x, h->o.post);
+    prolong_postsmooth64(h, l, b, C.x64, x, h->o.post, bs);
 }
 
 // ---- FP32 V-cycle on colour-split levels ------------------------------------------------
@@ -466,7 +467,7 @@ int finish_operator(mg_handle *h) {
     bool mixed = h->o.precision != MG_FP64;
     for (int l = 0; l < h->nlev; ++l) {
         Level &L = h->lv[l];
-        mg::launch_invdiag(s, L.d, L.fx64, L.fy64, L.fz64, L.invd64, L.d64);
+        mg::launch_invdiag(s, L.d, L.fx64, L.fy64, L.fz64, L.invd64, L.lay.split ? L.lay.half : 0, L.d64);
         if (mixed && !(l == 0 && h->sform0)) {  // the s-form finest level has no FP32 faces
             mg::launch_pack64to32(s, L.lay, L.fx64, L.fx32);
             mg::launch_pack64to32(s, L.lay, L.fy64, L.fy32);
@@ -555,9 +556,11 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
     // the mixed modes keep b~ scaled by h^2 (what their outer residual kernels consume)
     const bool mixed = h->o.precision != MG_FP64;
     const bool df = h->o.precision == MG_MIXED_DF;
-    const double bscale = mixed ? F.h2 : 1.0;
+    // the FP64 V-cycle iteration keeps b~ scaled too, and colour by colour, as its half sweeps read it
+    const bool bs = !mixed && h->o.method == MG_METHOD_VCYCLE && h->nlev > 1 && h->o.pre > 0 && F.lay.split;
+    const double bscale = mixed || bs ? F.h2 : 1.0;
     mg::launch_sum_sumsq<double>(s, n, b, h->partials, sums_on_device(h, 0), false);
-    mg::launch_sub_mean(s, n, b, h->red, bscale, h->bt, h->partials, sums_for_host(h, 2));
+    mg::launch_sub_mean(s, n, b, h->red, bscale, h->bt, h->partials, sums_for_host(h, 2), bs ? &F.d : nullptr);
     int rc = check_launch(h, "rhs preparation");
     if (rc) return rc;
     rc = wait_scalars(h);
@@ -598,8 +601,8 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
                 mg::launch_resid_df(s, F.d, F.lay, F.fx2, F.fy2, F.fz2, F.d2, h->bt2, h->p2,
                                     write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6));
             else
-                mg::launch_fine_resid2(s, F.d, F.lay, F.h2, F.fx64, F.fy64, F.fz64, F.d64, h->bt, mixed, p,
-                                       write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6));
+                mg::launch_fine_resid2(s, F.d, F.lay, F.h2, F.fx64, F.fy64, F.fz64, F.d64, h->bt, mixed || bs, p,
+                                       write32 ? F.b32 : nullptr, (float)(F.ih2 * scale), h->partials, sums_for_host(h, 6), bs);
             prof_end(h);
             const int bad = check_launch(h, "fine residual");
             if (bad) return bad;
@@ -683,7 +686,7 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
                 }
                 scale = 1.0 / rn;
             } else {
-                vcycle64(h, 0, h->bt, p, false);
+                vcycle64(h, 0, h->bt, p, false, bs);
             }
             rc = residual(mixed);
             if (rc) return rc;
@@ -692,9 +695,9 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
                 h->inject &= ~MG_INJECT_DIVERGE;
                 rn = HUGE_VAL;
             }
-            double mu_new = h->hred[7] / (double)n;
-            if (!mixed) mg::launch_add_const(s, n, p, -mu_new);  // FP64 path: zero mean each cycle
-            mu = mixed ? mu_new : 0.0;
+            // the next update takes the mean off; the FP64 cycle, which a constant in p does not change, leaves it
+            // to the exit
+            mu = mixed ? h->hred[7] / (double)n : 0.0;
             const double rr_prev = rr;
             rr = rn / nb;
             cycles += inner;
@@ -1166,8 +1169,7 @@ int mg_presmooth_restrict(mg_handle *h, int level, int dtype, void *x, const voi
     if (!x || !b || !bc || sweeps < 0) return fail(h, MG_ERR_ARG, "mg_presmooth_restrict: bad argument");
     Level &L = h->lv[level], &C = h->lv[level + 1];
     if (dtype == MG_F64) {
-        if (x_is_zero) MG_CUDA(h, cudaMemsetAsync(x, 0, 8 * (size_t)L.d.n, h->s));
-        presmooth_restrict64(h, level, (const double *)b, (double *)x, (double *)bc, sweeps);
+        presmooth_restrict64(h, level, (const double *)b, (double *)x, (double *)bc, sweeps, false, x_is_zero != 0);
     } else {
         mg::launch_pack32(h->s, L.lay, (const float *)b, L.s2_32);
         if (!x_is_zero) mg::launch_pack32(h->s, L.lay, (const float *)x, L.s1_32);

@@ -940,7 +940,7 @@ int mg_dd_set_density(mg_dd *dd, const double *rho) {
     for (int l = 0; l < dd->ndec; ++l) {
         for (int r = 0; r < dd->P; ++r) {
             Slab &S = dd->lv[l][r];
-            mg::launch_invdiag(s, S.d, S.fx, S.fy, S.fze, S.invd, S.dg);
+            mg::launch_invdiag(s, S.d, S.fx, S.fy, S.fze, S.invd, 0, S.dg);
             if (dd->mixed && l > 0) {  // the FP32 faces of a cut level below the finest
                 const dim3 grd((unsigned)((S.lay.nx + 127) / 128), (unsigned)std::min(S.lay.ny * (S.lay.nz + 1), 65535));
                 mg::count_launch(3);

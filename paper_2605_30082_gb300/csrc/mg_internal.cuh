@@ -266,7 +266,7 @@ void launch_faces_to_api(cudaStream_t s, Dims d, const double *fx, const double 
                          const double *fz, double *bx, double *by, double *bz);
 // 1 / sum of the interior face coefficients of each cell, and (diag non-null) the sum itself
 void launch_invdiag(cudaStream_t s, Dims d, const double *fx, const double *fy, const double *fz,
-                    double *invd64, double *diag);
+                    double *invd64, i64 invd_half, double *diag);
 void launch_coarsen(cudaStream_t s, Dims fine, const double *ffx, const double *ffy,
                     const double *ffz, double *cfx, double *cfy, double *cfz);
 void launch_to_f32(cudaStream_t s, i64 n, const double *src, float *dst);
@@ -366,9 +366,11 @@ void launch_pack_inv_rho(cudaStream_t s, Lay L, const double *sinv, float *st, f
 // FP64 red-black half sweep of one colour, in place
 // FP64 red-only residual + restriction in diagonal form (dg = sum of the cell's face betas)
 void launch_rr_red_diag64(cudaStream_t s, Dims fine, double h2, Coef<double> c, const double *dg,
-                          const double *b, const double *x, double *bc);
-void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const double *b, double *p,
-                        int colour);
+                          const double *b, const double *x, double *bc, bool b_split = false);
+// b_split: h2 b colour by colour as in Lay (only with invd_split, the reciprocal diagonal likewise); from_zero: the red
+// half sweep of x = 0, which need not have been written (b not split)
+void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const double *b, double *p, int colour,
+                        bool b_split = false, bool invd_split = false, bool from_zero = false);
 template <typename T>
 void launch_apply(cudaStream_t s, Dims d, double ih2, Coef<T> c, const T *x, T *y);
 template <typename T>
@@ -392,7 +394,7 @@ struct TailLevel {
     int nx, ny, nz;
     i64 half;              // colour stride of the FP32 arrays in memory (Lay.half)
     double h2, ih2;
-    const void *fx, *fy, *fz, *invd, *diag;  // the level's arrays (FP32 in its Lay, FP64 natural)
+    const void *fx, *fy, *fz, *invd, *diag;  // the level's arrays (FP32 in its Lay; FP64 natural, invd colour by colour)
     void *x, *b;
     // set by tail_layout
     int hx, q4, nit, rs;   // nx / 2, row quads and cells of a colour per CTA, row stride of x
@@ -433,7 +435,7 @@ template <typename T>
 void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, ReduceOut ro, bool squares);
 // b64 = (b - sum[0]/n) * scale, with the sum of squares of b64 into out[0]
 void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, double scale, double *b64,
-                     double *partials, ReduceOut ro);
+                     double *partials, ReduceOut ro, const Dims *split = nullptr);
 // fine FP64 residual in diagonal form, h^2 r = h^2 b - (diag p_c - sum_f beta_f p_nb):
 // out[0] = sum (h^2 r)^2, out[1] = sum p; optional r32 = s32 * h^2 r in the level-0 layout L.
 // On a slab of a decomposed grid (d.zlo or d.zhi, even nx; p with its ghost planes beside the
@@ -441,7 +443,7 @@ void launch_sub_mean(cudaStream_t s, i64 n, const double *b, const double *sum, 
 // and r32 is stored in the slab's layout L (L.half the colour stride)
 void launch_fine_resid2(cudaStream_t s, Dims d, Lay L, double h2, const double *fx, const double *fy,
                         const double *fz, const double *diag, const double *b, bool b_scaled, const double *p,
-                        float *r32, float s32, double *partials, ReduceOut ro);
+                        float *r32, float s32, double *partials, ReduceOut ro, bool b_split = false);
 // r32 = (float)(ih2 scale) * trunc_fp32(b): the scaled FP32 residual of p = 0, as the outer
 // residual kernels would write it (b = h^2 b~ in the mixed modes)
 void launch_zero_resid32(cudaStream_t s, Dims d, Lay L, const double *b, double scale32, float *r32);
