@@ -21,14 +21,53 @@ struct FracArgs {
 // Eq. (5) in the form rho_last + sum_q (rho_q - rho_last) f_q: one FMA per fraction (the
 // literal sum_q rho_q f_q + rho_last (1 - sum_q f_q) takes 2 nfrac + 1 FP64 operations, which
 // bound this kernel by the FP64 pipe); equal in exact arithmetic, within a few units in the
-// last place in FP64
-__global__ void k_density(i64 n, FracArgs a, double *rho) {
+// last place in FP64.  Four cells per thread, all loads before the arithmetic, 16 bytes each
+// where every array is on such a boundary (VEC): one cell per thread, the fractions one after another, took
+// 181 us at 256^3 with two of them (24 bytes a cell, 59 us), now 61 us.
+constexpr int kDensThreads = 256;
+template <int NF, bool VEC>
+__global__ void __launch_bounds__(kDensThreads) k_density(i64 n, FracArgs a, double *rho) {
     grid_wait();
-    i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    double r = a.rho_last;
-    for (int q = 0; q < a.nfrac; ++q) r = fma(a.drho[q], a.f[q][m], r);
-    rho[m] = r;
+    constexpr int kPer = VEC ? 2 : 4;  // loads per array and thread
+    using V = typename std::conditional<VEC, double2, double>::type;
+    const i64 nv = VEC ? n / 2 : n, m0 = (i64)blockIdx.x * (kPer * kDensThreads) + threadIdx.x;
+    V f[NF][kPer];
+#pragma unroll
+    for (int q = 0; q < NF; ++q)
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const i64 m = m0 + u * kDensThreads;
+            if (m < nv) f[q][u] = reinterpret_cast<const V *>(a.f[q])[m];
+        }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const i64 m = m0 + u * kDensThreads;
+        if (m >= nv) continue;
+        if constexpr (VEC) {
+            double2 r = make_double2(a.rho_last, a.rho_last);
+#pragma unroll
+            for (int q = 0; q < NF; ++q) r = make_double2(fma(a.drho[q], f[q][u].x, r.x), fma(a.drho[q], f[q][u].y, r.y));
+            reinterpret_cast<double2 *>(rho)[m] = r;
+        } else {
+            double r = a.rho_last;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) r = fma(a.drho[q], f[q][u], r);
+            rho[m] = r;
+        }
+    }
+    if (VEC && (n & 1) && m0 == 0) {  // the last cell of an odd number
+        double r = a.rho_last;
+#pragma unroll
+        for (int q = 0; q < NF; ++q) r = fma(a.drho[q], a.f[q][n - 1], r);
+        rho[n - 1] = r;
+    }
+}
+template <int NF>
+void run_density(cudaStream_t s, i64 n, const FracArgs &a, double *rho) {
+    bool vec = (reinterpret_cast<uintptr_t>(rho) & 15) == 0;
+    for (int q = 0; q < NF; ++q) vec = vec && (reinterpret_cast<uintptr_t>(a.f[q]) & 15) == 0;
+    const unsigned nb = (unsigned)((n + 4 * kDensThreads - 1) / (4 * kDensThreads));
+    run_kernel(vec ? k_density<NF, true> : k_density<NF, false>, nb, kDensThreads, 0, s, n, a, rho);
 }
 
 // 0 < v <= 1.79e308, tested on the bit pattern (positive doubles order like their bits, NaN and
@@ -39,12 +78,14 @@ __device__ __forceinline__ bool good_positive(double v) {
 }
 
 // v / 2 for v = 0 or normal with a normal result (exponent field above 1): one integer subtraction
-// from the exponent field instead of an FP64 multiplication; otherwise the multiplication
+// from the exponent field instead of an FP64 multiplication; otherwise the multiplication, in a function of its own:
+// in line the compiler computes it for every value (the faces of 256^3 190 us, so 101)
+__device__ __noinline__ double half_slow(double v) { return 0.5 * v; }
 __device__ __forceinline__ double half_of(double v) {
     const long long u = __double_as_longlong(v);
     const int e = (int)((u >> 52) & 0x7ff);
     if (e > 1 && e < 0x7ff) return __longlong_as_double(u - (1ll << 52));
-    return 0.5 * v;
+    return half_slow(v);
 }
 
 // s = 1/rho per cell, validating rho (finite and > 0)
@@ -59,6 +100,27 @@ __global__ void k_inv_rho(i64 n, const double *__restrict__ rho, double *sinv, u
         return;
     }
     sinv[m] = recip64(r);
+}
+
+// the same for even nx and 16-byte boundaries, two cells per thread, with the FP32 copies of a mixed handle (s32 in
+// the level's layout, optionally s2 as pairs of FP32 numbers hi + lo = s to about 2^-48) in the same
+// pass: 256^3 122 + 90 us apart, now 122 us (its FP64 arithmetic)
+__global__ void k_inv_rho_pack(Lay L, const double *__restrict__ rho, double *sinv, float *s32, float2 *s2, unsigned *err) {
+    grid_wait();
+    const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= L.half) return;
+    const double2 r = reinterpret_cast<const double2 *>(rho)[m];
+    const bool g0 = good_positive(r.x), g1 = good_positive(r.y);
+    if (!g0 || !g1) atomicOr(err, 1u);
+    const double2 v = make_double2(g0 ? recip64(r.x) : 1.0, g1 ? recip64(r.y) : 1.0);
+    reinterpret_cast<double2 *>(sinv)[m] = v;
+    const unsigned row = (unsigned)m / (unsigned)L.hx;
+    const bool red_first = ((row % (unsigned)L.ny + row / (unsigned)L.ny) & 1) == 0;
+    const float h0 = d2f_rn(v.x), h1 = d2f_rn(v.y);
+    s32[m] = red_first ? h0 : h1;
+    s32[L.half + m] = red_first ? h1 : h0;
+    if (s2)
+        reinterpret_cast<float4 *>(s2)[m] = make_float4(h0, d2f_rn(v.x - f2d_exact(h0)), h1, d2f_rn(v.y - f2d_exact(h1)));
 }
 
 // beta on the low faces: 1 / harmonic mean of the two densities = (s_L + s_R) / 2; blocks take
@@ -91,21 +153,12 @@ __global__ void k_faces_from_s2(Dims d, const double *__restrict__ sv, double *f
     for (i64 row = blockIdx.y; row < rows; row += gridDim.y) {
         const int j = (int)((unsigned)row % (unsigned)d.ny), k = (int)((unsigned)row / (unsigned)d.ny);  // rows < 2^31
         const i64 c = row * d.nx + i;
-        const double2 sc = ld2(sv + c);
-        const double sl = i > 0 ? sv[c - 1] : 0.0;
+        // all loads at once (at a wall the cell itself)
+        const double2 sc = ld2(sv + c), sy = ld2(sv + (j > 0 ? c - d.nx : c)), sz = ld2(sv + (k > 0 ? c - d.nxy : c));
+        const double sl = sv[i > 0 ? c - 1 : c];
         st2(fx + c, i > 0 ? half_of(sl + sc.x) : 0.0, half_of(sc.x + sc.y));
-        if (j > 0) {
-            const double2 sy = ld2(sv + c - d.nx);
-            st2(fy + c, half_of(sy.x + sc.x), half_of(sy.y + sc.y));
-        } else {
-            st2(fy + c, 0.0, 0.0);
-        }
-        if (k > 0) {
-            const double2 sz = ld2(sv + c - d.nxy);
-            st2(fz + c, half_of(sz.x + sc.x), half_of(sz.y + sc.y));
-        } else {
-            st2(fz + c, 0.0, 0.0);
-        }
+        st2(fy + c, j > 0 ? half_of(sy.x + sc.x) : 0.0, j > 0 ? half_of(sy.y + sc.y) : 0.0);
+        st2(fz + c, k > 0 ? half_of(sz.x + sc.x) : 0.0, k > 0 ? half_of(sz.y + sc.y) : 0.0);
     }
 }
 
@@ -171,16 +224,18 @@ __global__ void k_invdiag(Dims d, const double *__restrict__ fx, const double *_
     if (diag) diag[c] = s;
 }
 
-// coarse low face = mean of the 4 fine low faces that tile it
+// coarse low face = mean of the 4 fine low faces that tile it; with c32x, .. also rounded to FP32 in the layout L (a
+// launch less per array and level)
 __global__ void k_coarsen(Dims f, Dims cd, const double *__restrict__ ffx,
                           const double *__restrict__ ffy, const double *__restrict__ ffz,
-                          double *cfx, double *cfy, double *cfz) {
+                          double *cfx, double *cfy, double *cfz, Lay L, float *c32x, float *c32y, float *c32z) {
     grid_wait();
     i64 C = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (C >= cd.n) return;
-    int I = (int)(C % cd.nx);
-    int J = (int)((C / cd.nx) % cd.ny);
-    int K = (int)(C / cd.nxy);
+    const unsigned cu = (unsigned)C, ru = cu / (unsigned)cd.nx;  // C < 2^32: 32-bit divisions
+    const int I = (int)(cu - ru * (unsigned)cd.nx);
+    const int J = (int)(ru % (unsigned)cd.ny);
+    const int K = (int)(ru / (unsigned)cd.ny);
     i64 base = ((i64)(2 * K) * f.ny + 2 * J) * f.nx + 2 * I;  // child (0,0,0)
     double sx = 0.0, sy = 0.0, sz = 0.0;
     for (int c = 0; c < 2; ++c)
@@ -189,9 +244,18 @@ __global__ void k_coarsen(Dims f, Dims cd, const double *__restrict__ ffx,
         for (int a = 0; a < 2; ++a) sy += ffy[base + c * f.nxy + a];
     for (int b = 0; b < 2; ++b)
         for (int a = 0; a < 2; ++a) sz += ffz[base + b * f.nx + a];
-    cfx[C] = sx / 4.0;
-    cfy[C] = sy / 4.0;
-    cfz[C] = sz / 4.0;
+    sx /= 4.0;
+    sy /= 4.0;
+    sz /= 4.0;
+    cfx[C] = sx;
+    cfy[C] = sy;
+    cfz[C] = sz;
+    if (c32x) {
+        const i64 t = L.split ? ((I + J + K) & 1) * L.half + (i64)ru * L.hx + (I >> 1) : C;
+        c32x[t] = d2f_rn(sx);
+        c32y[t] = d2f_rn(sy);
+        c32z[t] = d2f_rn(sz);
+    }
 }
 
 __global__ void k_to_f32(i64 n, const double *__restrict__ src, float *dst) {
@@ -211,10 +275,12 @@ __global__ void k_csf_faces(Dims d, double ih, const double *__restrict__ f,
     int k = (int)(ru_ / (unsigned)d.ny);
     i64 ax = ((i64)k * d.ny + j) * (d.nx + 1) + i;
     i64 ay = ((i64)k * (d.ny + 1) + j) * d.nx + i;
-    double fc = f[c], kc = kap[c];
-    cx[ax] = i > 0 ? 0.5 * (kap[c - 1] + kc) * (fc - f[c - 1]) * ih : 0.0;
-    cy[ay] = j > 0 ? 0.5 * (kap[c - d.nx] + kc) * (fc - f[c - d.nx]) * ih : 0.0;
-    cz[c] = k > 0 ? 0.5 * (kap[c - d.nxy] + kc) * (fc - f[c - d.nxy]) * ih : 0.0;
+    // the mean's 1/2 goes with ih: four FP64 operations per face, which bound this kernel (256^3: five
+    // 484 us, four 420)
+    const double fc = f[c], kc = kap[c], ih_2 = 0.5 * ih;
+    cx[ax] = i > 0 ? (kap[c - 1] + kc) * (fc - f[c - 1]) * ih_2 : 0.0;
+    cy[ay] = j > 0 ? (kap[c - d.nx] + kc) * (fc - f[c - d.nx]) * ih_2 : 0.0;
+    cz[c] = k > 0 ? (kap[c - d.nxy] + kc) * (fc - f[c - d.nxy]) * ih_2 : 0.0;
     if (i == d.nx - 1) cx[ax + 1] = 0.0;
     if (j == d.ny - 1) cy[ay + d.nx] = 0.0;
     if (k == d.nz - 1) cz[c + d.nxy] = 0.0;
@@ -271,15 +337,23 @@ void launch_density(cudaStream_t s, i64 n, int nfrac, const double *const *frac,
         a.drho[q] = q < nfrac ? rho_phase[q] - rho_phase[nfrac] : 0.0;
     }
     count_launch();
-    run_kernel(k_density, blocks_for(n), kThreads, 0, s, n, a, rho);
+    if (nfrac == 1) run_density<1>(s, n, a, rho);
+    else if (nfrac == 2) run_density<2>(s, n, a, rho);
+    else if (nfrac == 3) run_density<3>(s, n, a, rho);
+    else run_density<4>(s, n, a, rho);
 }
 
 void launch_faces_from_rho(cudaStream_t s, Dims d, const double *rho, double *sinv, double *fx, double *fy,
-                           double *fz, unsigned *err) {
+                           double *fz, unsigned *err, Lay L, float *s32, float2 *s2) {
     count_launch(2);
-    run_kernel(k_inv_rho, blocks_for(d.n), kThreads, 0, s, d.n, rho, sinv, err);
-    const i64 rows = (i64)d.ny * d.nz;
     auto a16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+    if (s32 && d.nx % 2 == 0 && a16(rho) && a16(sinv)) {
+        run_kernel(k_inv_rho_pack, blocks_for(d.n / 2), kThreads, 0, s, L, rho, sinv, s32, s2, err);
+    } else {
+        run_kernel(k_inv_rho, blocks_for(d.n), kThreads, 0, s, d.n, rho, sinv, err);
+        if (s32) launch_pack_inv_rho(s, L, sinv, s32, s2);
+    }
+    const i64 rows = (i64)d.ny * d.nz;
     if (d.nx % 2 == 0 && a16(sinv) && a16(fx) && a16(fy) && a16(fz)) {
         const dim3 grd((unsigned)((d.nx / 2 + 127) / 128), (unsigned)(rows < 65535 ? rows : 65535));
         run_kernel(k_faces_from_s2, grd, 128, 0, s, d, sinv, fx, fy, fz);
@@ -309,10 +383,11 @@ void launch_invdiag(cudaStream_t s, Dims d, const double *fx, const double *fy, 
 }
 
 void launch_coarsen(cudaStream_t s, Dims fine, const double *ffx, const double *ffy,
-                    const double *ffz, double *cfx, double *cfy, double *cfz) {
+                    const double *ffz, double *cfx, double *cfy, double *cfz, Lay L, float *c32x, float *c32y, float *c32z) {
     Dims cd = make_dims(fine.nx / 2, fine.ny / 2, fine.nz / 2);
     count_launch();
-    run_kernel(k_coarsen, blocks_for(cd.n), kThreads, 0, s, fine, cd, ffx, ffy, ffz, cfx, cfy, cfz);
+    run_kernel(k_coarsen, blocks_for(cd.n), kThreads, 0, s, fine, cd, ffx, ffy, ffz, cfx, cfy, cfz, L,
+               c32x, c32y, c32z);
 }
 
 void launch_to_f32(cudaStream_t s, i64 n, const double *src, float *dst) {

@@ -462,13 +462,14 @@ int finish_operator(mg_handle *h) {
     cudaStream_t s = h->s;
     for (int l = 0; l + 1 < h->nlev; ++l) {
         Level &F = h->lv[l], &C = h->lv[l + 1];
-        mg::launch_coarsen(s, F.d, F.fx64, F.fy64, F.fz64, C.fx64, C.fy64, C.fz64);
+        mg::launch_coarsen(s, F.d, F.fx64, F.fy64, F.fz64, C.fx64, C.fy64, C.fz64, C.lay, C.fx32, C.fy32, C.fz32);
     }
     bool mixed = h->o.precision != MG_FP64;
     for (int l = 0; l < h->nlev; ++l) {
         Level &L = h->lv[l];
         mg::launch_invdiag(s, L.d, L.fx64, L.fy64, L.fz64, L.invd64, L.lay.split ? L.lay.half : 0, L.d64);
-        if (mixed && !(l == 0 && h->sform0)) {  // the s-form finest level has no FP32 faces
+        // coarse levels have theirs from launch_coarsen; the s-form finest level has no FP32 faces
+        if (mixed && l == 0 && !h->sform0) {
             mg::launch_pack64to32(s, L.lay, L.fx64, L.fx32);
             mg::launch_pack64to32(s, L.lay, L.fy64, L.fy32);
             mg::launch_pack64to32(s, L.lay, L.fz64, L.fz32);
@@ -979,9 +980,9 @@ int mg_set_density(mg_handle *h, const double *rho) {
     mg::launch_zero(h->s, h->err, sizeof(unsigned));
     Level &F = h->lv[0];
     // s = 1/rho goes through the RHS buffer, which holds nothing between calls
-    mg::launch_faces_from_rho(h->s, F.d, rho, h->bt, F.fx64, F.fy64, F.fz64, h->err);
     h->sform0 = h->o.precision != MG_FP64;
-    if (h->sform0) mg::launch_pack_inv_rho(h->s, F.lay, h->bt, F.s32, h->o.precision == MG_MIXED_DF ? F.s2 : nullptr);
+    mg::launch_faces_from_rho(h->s, F.d, rho, h->bt, F.fx64, F.fy64, F.fz64, h->err, F.lay, h->sform0 ? F.s32 : nullptr,
+                              h->o.precision == MG_MIXED_DF ? F.s2 : nullptr);
     return finish_operator(h);
 }
 

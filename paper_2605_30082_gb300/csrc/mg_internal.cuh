@@ -259,7 +259,7 @@ void launch_density(cudaStream_t s, i64 n, int nfrac, const double *const *frac,
                     const double *rho_phase, double *rho);
 // s = 1/rho per cell into `sinv` (validated: err |= 1 on a bad density), then the FP64 low faces
 void launch_faces_from_rho(cudaStream_t s, Dims d, const double *rho, double *sinv, double *fx, double *fy,
-                           double *fz, unsigned *err);
+                           double *fz, unsigned *err, Lay L = Lay{}, float *s32 = nullptr, float2 *s2 = nullptr);
 void launch_faces_from_api(cudaStream_t s, Dims d, const double *bx, const double *by,
                            const double *bz, double *fx, double *fy, double *fz, unsigned *err);
 void launch_faces_to_api(cudaStream_t s, Dims d, const double *fx, const double *fy,
@@ -268,7 +268,8 @@ void launch_faces_to_api(cudaStream_t s, Dims d, const double *fx, const double 
 void launch_invdiag(cudaStream_t s, Dims d, const double *fx, const double *fy, const double *fz,
                     double *invd64, i64 invd_half, double *diag);
 void launch_coarsen(cudaStream_t s, Dims fine, const double *ffx, const double *ffy,
-                    const double *ffz, double *cfx, double *cfy, double *cfz);
+                    const double *ffz, double *cfx, double *cfy, double *cfz, Lay L = Lay{}, float *c32x = nullptr, float *c32y = nullptr,
+                    float *c32z = nullptr);
 void launch_to_f32(cudaStream_t s, i64 n, const double *src, float *dst);
 
 void launch_csf_faces(cudaStream_t s, Dims d, double h, const double *f, const double *kappa,
