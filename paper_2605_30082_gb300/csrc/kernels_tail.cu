@@ -1,13 +1,13 @@
 // The coarse levels of a V-cycle in one launch: one thread-block cluster holds every level from
 // `first` down in its CTAs' shared memory and runs their smoothing sweeps, transfers and the
-// dense coarse solve with cluster barriers between them.
+// dense coarse solve, CTAs waiting only for what they read.
 //
 // What bounds the levels below about 40^3 is the chain of dependent launches (ten per level and
 // cycle, 2-3 us each, for work of a fraction of a microsecond), so the
-// chain is made of cheaper links: a half sweep here is one shared-memory round trip and a cluster
-// barrier, 0.6 us at 32^3 and 0.5 us at 16^3.  The levels 32^3, 16^3 and 8^3 of a cycle take 28 us
-// (launch by launch 50 us): 4 us to copy the contexts in, 6 us for the dense product of 512
-// cells (its FP64 FMAs on 16 SMs), 3 us for the transfers each way.  A 64^3 projection step went
+// chain is made of cheaper links: a half sweep here is one shared-memory round trip and a wait for
+// the neighbours' ghosts, 0.5 us at 32^3 and 0.4 us at 16^3.  The levels 32^3, 16^3 and 8^3 of a cycle take 26 us
+// (launch by launch 50 us): 2 us to copy the contexts in beside the kernel before, 5.5 us for the dense product of
+// 512 cells (4 us of it the FP64 FMAs on 16 SMs), 5 us for the transfers, 16 half sweeps.  A 64^3 projection step went
 // from 2.50 to 2.18 ms, a 32^3 one in FP64 from 2.16 to 1.67 ms.
 //
 // Layout.  The rows (y, z) of a level are dealt out in quads, the four rows of one coarse row
@@ -23,8 +23,15 @@
 // Threads.  Item e of a colour is the cell k = (e / 4) % hx of row e % 4 of quad e / (4 hx); a
 // thread owns up to kCells items of each colour and keeps their faces, right-hand side and the
 // six neighbours' addresses in registers while a level is smoothed, so that a half sweep is six
-// shared loads, the arithmetic and the stores (about 150 clocks) and a cluster barrier (480 clocks
-// with 512 threads and 16 CTAs, 600 with 1024 threads).  These contexts are laid out in memory once per
+// shared loads, the arithmetic and the stores.
+//
+// Waits.  A CTA sends its ghosts, restricted residuals and coarse results by st.async, which counts their bytes at
+// an mbarrier of the receiver; the receiver knows how many will come.  Stores and a barrier of the
+// cluster instead cost 830 clocks per exchange between 16 CTAs of 512 threads, this 465, and all CTAs then wait for the
+// slowest (64^3 step 1561 -> 1500 us with the shared-memory copies of the parameters and addresses below).  Before a
+// level reads other CTAs' x on the way up the barrier stays.
+//
+// These contexts are laid out in memory once per
 // operator (k_tail_prepare), one image per CTA and level in the order of its shared memory, and
 // copied in at the start of a launch.
 //
@@ -47,25 +54,32 @@ namespace {
 
 constexpr int kTailThreads = 512;
 
-template <typename T>
-__device__ __forceinline__ T ld_cluster(unsigned a);
-template <>
-__device__ __forceinline__ float ld_cluster<float>(unsigned a) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
+__device__ __forceinline__ void ld_cluster_wide(unsigned a, float (&v)[1]) {
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v[0]) : "r"(a) : "memory");
 }
-template <>
-__device__ __forceinline__ double ld_cluster<double>(unsigned a) {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
-    return v;
+__device__ __forceinline__ void ld_cluster_wide(unsigned a, float (&v)[4]) {
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_cluster_wide(unsigned a, double (&v)[1]) {
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[0]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_cluster_wide(unsigned a, double (&v)[2]) {
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a) : "memory");
 }
 __device__ __forceinline__ void st_cluster(unsigned a, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 __device__ __forceinline__ void st_cluster(unsigned a, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+// a remote store that reports its bytes to the mbarrier m of the CTA it goes to
+__device__ __forceinline__ void st_async(unsigned a, float v, unsigned m) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a), "r"(__float_as_uint(v)), "r"(m)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async(unsigned a, double v, unsigned m) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a), "l"(__double_as_longlong(v)), "r"(m)
+                 : "memory");
 }
 __device__ __forceinline__ unsigned map_cluster(unsigned a, int rank) {
     unsigned r;
@@ -76,13 +90,16 @@ __device__ __forceinline__ unsigned map_cluster(unsigned a, int rank) {
 // one cell of a thread: face coefficients in the order x-, x+, y-, y+, z-, z+, the divisor (FP32:
 // their sum; FP64: the reciprocal of it, and the sum for the residual), the right-hand side, and
 // element offsets from the level's x: the cell, its six neighbours, two per word; ghost copies of
-// the cell in other CTAs (cluster addresses, 0: none)
+// the cell in other CTAs (cluster addresses, 0: none) and the mbarriers there
 template <typename T>
 struct Cell {
     T w[6], d, dg, b;
     unsigned ax, ay, az, own;
-    unsigned g0, g1;
+    unsigned g0, g1, m0, m1;
 };
+
+// bound on the polls of one wait for ghosts (each suspends the thread for up to some microseconds)
+constexpr int kTailPolls = 1 << 16;
 
 template <typename T>
 struct Tail {
@@ -91,7 +108,10 @@ struct Tail {
     static constexpr int kReal = f64 ? 8 : 7, kWords = 6;  // context fields: T and unsigned
     static constexpr unsigned kNone = 0xffffffffu;         // Cell::own of a missing cell
     const TailArgs &a;
+    const TailLevel *lv;  // a.lv in shared memory: parameters of a launch come from far away when first read
+    const unsigned *cb;   // where the CTAs' shared memory begins in the cluster's: a mapa per address costs a sweep's worth
     char *sm;
+    unsigned sm0, mbar;   // shared addresses of sm and of the mbarriers
     int rank, ncta, tid;
 
     __device__ T *x(const TailLevel &L) const { return reinterpret_cast<T *>(sm + L.off_x); }
@@ -103,6 +123,15 @@ struct Tail {
     // (their x) and of its own coarse row's b at k = 0, red
     __device__ int *jk(const TailLevel &L) const { return reinterpret_cast<int *>(sm + L.off_q); }
     __device__ unsigned *crow(const TailLevel &L) const { return reinterpret_cast<unsigned *>(jk(L) + L.q4); }
+    // bytes of one colour that other CTAs write into this one's ghosts, and of the right-hand side
+    __device__ unsigned ghost_bytes(const TailLevel &L) const { return (unsigned)jk(L)[L.q4 * 11]; }
+    __device__ unsigned cell_bytes(const TailLevel &L) const { return (unsigned)jk(L)[L.q4 * 11 + 1]; }
+    // the mbarriers: ghosts of colour c and the right-hand side of level l, the coarsest level's r and e.  Each level has
+    // its own because a CTA may be a level ahead of another.
+    __device__ unsigned bar_x(int l, int c) const { return mbar + 8 * (3 * l + c); }
+    __device__ unsigned bar_b(int l) const { return mbar + 8 * (3 * l + 2); }
+    __device__ unsigned bar_r() const { return mbar + 8 * (3 * kTailLevels); }
+    __device__ unsigned bar_e() const { return bar_r() + 8; }
     __device__ double *rc() const { return reinterpret_cast<double *>(sm + a.off_rc); }
     __device__ T *ec() const { return reinterpret_cast<T *>(sm + a.off_ec); }
     __device__ T *cw() const { return reinterpret_cast<T *>(sm + a.off_cw); }
@@ -117,26 +146,35 @@ struct Tail {
 
     // a remote place: CTA and byte offset from the start of shared memory; bit 0 is free
     __device__ static unsigned place(int owner, i64 bytes) { return (unsigned)owner << 24 | (unsigned)bytes; }
-    __device__ unsigned at(unsigned pl) const {
-        return map_cluster(saddr(sm) + (pl & 0xfffffeu), (int)(pl >> 24));
-    }
+    __device__ unsigned at(unsigned pl) const { return cb[pl >> 24] + (pl & 0xfffffeu); }
+    // the address in CTA `owner` of what lies at a in this one
+    __device__ unsigned there(unsigned a, int owner) const { return cb[owner] + (a - sm0); }
 
     // right-hand side (and, in the ascent alone, x with its ghosts) of this CTA's cells from memory
     __device__ void load_b(const TailLevel &L) const {
-        for (int i = tid; i < 2 * L.nit; i += kTailThreads) {
+        T v[2 * kCells];  // all of a thread's loads together
+        bool in[2 * kCells];
+#pragma unroll
+        for (int u = 0; u < 2 * kCells; ++u) {
+            const int e = tid + (u % kCells) * kTailThreads, i = (u / kCells) * L.nit + e;
             int col, k, y, z;
-            if (cell_of(L, i, col, k, y, z)) b(L)[i] = reinterpret_cast<const T *>(L.b)[gidx(L, col, k, y, z)];
+            in[u] = e < L.nit && cell_of(L, i, col, k, y, z);
+            if (in[u]) v[u] = reinterpret_cast<const T *>(L.b)[gidx(L, col, k, y, z)];
         }
+#pragma unroll
+        for (int u = 0; u < 2 * kCells; ++u)
+            if (in[u]) b(L)[(u / kCells) * L.nit + tid + (u % kCells) * kTailThreads] = v[u];
     }
-    __device__ void load_x(const TailLevel &L) const {
+    __device__ void load_x(int l) const {
+        const TailLevel &L = lv[l];
         for (int col = 0; col < 2; ++col) {
             Cell<T> q[kCells];
-            restore(L, col, q);
+            restore(l, col, q);
 #pragma unroll
             for (int c = 0; c < kCells; ++c) {
                 int cc, k, y, z;
                 if (q[c].own == kNone || !cell_of(L, col * L.nit + tid + c * kTailThreads, cc, k, y, z)) continue;
-                put(x(L), q[c], reinterpret_cast<const T *>(L.x)[gidx(L, col, k, y, z)]);
+                put_plain(x(L), q[c], reinterpret_cast<const T *>(L.x)[gidx(L, col, k, y, z)]);
             }
         }
     }
@@ -150,7 +188,8 @@ struct Tail {
         return q >= 0;
     }
     // this thread's cells of one colour, without b
-    __device__ __forceinline__ void restore(const TailLevel &L, int col, Cell<T> (&q)[kCells]) const {
+    __device__ __forceinline__ void restore(int l, int col, Cell<T> (&q)[kCells]) const {
+        const TailLevel &L = lv[l];
 #pragma unroll
         for (int c = 0; c < kCells; ++c) {
             const int e = tid + c * kTailThreads;
@@ -169,6 +208,8 @@ struct Tail {
             q[c].own = w[3 * n2];
             q[c].g0 = w[4 * n2] == kNone ? 0u : at(w[4 * n2]);
             q[c].g1 = w[5 * n2] == kNone ? 0u : at(w[5 * n2]);
+            q[c].m0 = q[c].g0 ? there(bar_x(l, col), (int)(w[4 * n2] >> 24)) : 0u;
+            q[c].m1 = q[c].g1 ? there(bar_x(l, col), (int)(w[5 * n2] >> 24)) : 0u;
         }
     }
     __device__ __forceinline__ void restore_b(const TailLevel &L, int col, Cell<T> (&q)[kCells]) const {
@@ -178,11 +219,13 @@ struct Tail {
     }
     // x of this CTA's cells into memory, and b
     __device__ void store(const TailLevel &L, bool with_b) const {
-        for (int i = tid; i < 2 * L.nit; i += kTailThreads) {
+#pragma unroll
+        for (int u = 0; u < 2 * kCells; ++u) {
+            const int e = tid + (u % kCells) * kTailThreads, i = (u / kCells) * L.nit + e;
             int col, k, y, z;
-            if (!cell_of(L, i, col, k, y, z)) continue;
+            if (e >= L.nit || !cell_of(L, i, col, k, y, z)) continue;
             const i64 g = gidx(L, col, k, y, z);
-            reinterpret_cast<T *>(L.x)[g] = x(L)[(div_by((i - col * L.nit) >> 2, L.magic_hx) * 4 + (i - col * L.nit) % 4) * L.rs + col * L.hx + k];
+            reinterpret_cast<T *>(L.x)[g] = x(L)[ctxw(L)[3 * 2 * L.nit + i]];
             if (with_b) reinterpret_cast<T *>(L.b)[g] = b(L)[i];
         }
     }
@@ -200,13 +243,43 @@ struct Tail {
         v[4] = X[q.az & 0xffffu];
         v[5] = X[q.az >> 16];
     }
-    __device__ __forceinline__ static void put(T *X, const Cell<T> &q, T v) {
+    __device__ __forceinline__ static void put_plain(T *X, const Cell<T> &q, T v) {
         X[q.own] = v;
         if (q.g0) st_cluster(q.g0, v);
         if (q.g1) st_cluster(q.g1, v);
     }
+    __device__ __forceinline__ static void put(T *X, const Cell<T> &q, T v, bool send) {
+        X[q.own] = v;
+        if (send && q.g0) st_async(q.g0, v, q.m0);
+        if (send && q.g1) st_async(q.g1, v, q.m1);
+    }
 
-    __device__ __forceinline__ void half(T *X, T h2, const Cell<T> (&q)[kCells]) const {
+    // until `bytes` have come in for the mbarrier m; its bytes may come before this.  The poll is bounded: past it
+    // the run goes on without waiting and leaves NaN and an error flag.
+    __device__ __forceinline__ void expect(unsigned m, unsigned bytes) const {
+        if (tid == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(m), "r"(bytes) : "memory");
+    }
+    __device__ __forceinline__ void wait(unsigned m, unsigned parity, bool &lost) const {
+        unsigned done = 0;
+        for (int it = 0; it < kTailPolls && !done && !lost; ++it)
+            asm volatile(
+                "{.reg .pred P; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2; selp.u32 %0, 1, 0, P;}"
+                : "=r"(done)
+                : "r"(m), "r"(parity)
+                : "memory");
+        lost = lost || !done;
+    }
+    // after the cells of colour col have been put: until this CTA's are visible to its threads and the ghosts'
+    // have arrived.  A neighbour sends the next values of a ghost only once it has had every cell of
+    // this CTA that reads the present ones, so nothing is overwritten early.
+    __device__ __forceinline__ void exchange(int l, int col, unsigned &parity, bool &lost) const {
+        expect(bar_x(l, col), ghost_bytes(lv[l]));
+        __syncthreads();
+        wait(bar_x(l, col), parity >> (2 * l + col) & 1u, lost);
+        parity ^= 1u << (2 * l + col);
+    }
+
+    __device__ __forceinline__ void half(T *X, T h2, const Cell<T> (&q)[kCells], bool send) const {
 #pragma unroll
         for (int c = 0; c < kCells; ++c) {
             if (q[c].own == kNone) continue;
@@ -215,8 +288,8 @@ struct Tail {
             T num = first_two(q[c].w[0], v[0], q[c].w[1], v[1]);
 #pragma unroll
             for (int u = 2; u < 6; ++u) num = fma(q[c].w[u], v[u], num);
-            if constexpr (f64) put(X, q[c], fma(h2, q[c].b, num) * q[c].d);
-            else put(X, q[c], __fdividef(fmaf(h2, q[c].b, num), q[c].d));
+            if constexpr (f64) put(X, q[c], fma(h2, q[c].b, num) * q[c].d, send);
+            else put(X, q[c], __fdividef(fmaf(h2, q[c].b, num), q[c].d), send);
         }
     }
 
@@ -229,7 +302,8 @@ struct Tail {
     // mean of the children's residuals (black ones 0 after a black half sweep) into the next
     // level's b: its owner's shared memory, every CTA's copy for the coarse solve, or memory.  The four
     // red children of a coarse cell are four neighbouring lanes.
-    __device__ void restrict_red(const TailLevel &L, const TailLevel *C, bool coarse_mem, const Cell<T> (&q)[kCells]) const {
+    __device__ void restrict_red(int l, const TailLevel *C, bool coarse_mem, const Cell<T> (&q)[kCells]) const {
+        const TailLevel &L = lv[l];
         const T *X = x(L);
         const int cnx = L.nx >> 1, cny = L.ny >> 1;
 #pragma unroll
@@ -266,12 +340,14 @@ struct Tail {
             const int lq = div_by(e >> 2, L.magic_hx), k = (e >> 2) - lq * L.hx;
             const int J = jk(L)[lq] & 0xffff, K = jk(L)[lq] >> 16;
             if (C) {
-                st_cluster(at(crow(L)[lq * 10 + 9]) + (unsigned)((((k + J + K) & 1) * C->nit + (k >> 1) * 4) * sizeof(T)), bc);
+                const unsigned pl = crow(L)[lq * 10 + 9];
+                st_async(at(pl) + (unsigned)((((k + J + K) & 1) * C->nit + (k >> 1) * 4) * sizeof(T)), bc,
+                         there(bar_b(l + 1), (int)(pl >> 24)));
             } else if (coarse_mem) {
                 reinterpret_cast<T *>(a.bc)[coarse_idx(k, J, K, cnx, cny)] = bc;
             } else {
                 const unsigned r0 = saddr(rc() + (K * cny + J) * cnx + k);
-                for (int t = ch; t < ncta; t += 4) st_cluster(map_cluster(r0, t), (double)bc);
+                for (int t = ch; t < ncta; t += 4) st_async(there(r0, t), (double)bc, there(bar_r(), t));
             }
         }
     }
@@ -299,9 +375,9 @@ struct Tail {
             for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             const double t0 = __shfl_sync(0xffffffffu, s, 0), t1 = __shfl_sync(0xffffffffu, s, 16);
             if (lane < ncta) {
-                const unsigned e0 = map_cluster(saddr(ec() + row), lane);
-                st_cluster(e0, (T)t0);
-                if (two) st_cluster(e0 + (unsigned)(stride * sizeof(T)), (T)t1);
+                const unsigned e0 = there(saddr(ec() + row), lane), m = there(bar_e(), lane);
+                st_async(e0, (T)t0, m);
+                if (two) st_async(e0 + (unsigned)(stride * sizeof(T)), (T)t1, m);
             }
         }
     }
@@ -309,25 +385,36 @@ struct Tail {
     // the 3 x 3 coarse rows around each quad into this CTA's scratch, in the order of I with its end
     // values repeated beyond the walls: cw[(9 quad + 3 (K' - K + 1) + J' - J + 1) (cnx + 2) + I + 1]
     __device__ void gather(const TailLevel &L, const TailLevel &C) const {
-        const int rows = L.q4 * 9, n = rows * C.nx, st = C.nx + 2;
-        for (int e0 = tid; e0 < n; e0 += 4 * kTailThreads) {
-            T v[4];
-            int d[4], Ic[4];
+        constexpr int kV = 16 / (int)sizeof(T);
+        if (C.hx % kV == 0) gather_wide<kV>(L, C);
+        else gather_wide<1>(L, C);
+    }
+    // kV cells of one colour per load, all of a thread's loads in flight (32^3 from 16^3: 576 loads of 16 bytes)
+    template <int kV>
+    __device__ void gather_wide(const TailLevel &L, const TailLevel &C) const {
+        constexpr int kU = kV > 1 ? 2 : 4;
+        const int per = C.nx / kV, n = L.q4 * 9 * per, st = C.nx + 2;
+        for (int e0 = tid; e0 < n; e0 += kU * kTailThreads) {
+            T v[kU][kV];
+            int d[kU], Ic[kU];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = min(e0 + u * kTailThreads, n - 1), r = div_by(e, C.magic_nx), i = e - r * C.nx;
+            for (int u = 0; u < kU; ++u) {
+                const int e = min(e0 + u * kTailThreads, n - 1), r = div_by(e * kV, C.magic_nx), i = (e - r * per) * kV;
                 const unsigned pl = crow(L)[r + r / 9];  // ten words per quad
                 const int col = i >= C.hx;
                 Ic[u] = 2 * (i - col * C.hx) + ((col + (int)pl) & 1);  // bit 0: parity of J' + K'
                 d[u] = r * st + Ic[u] + 1;
-                v[u] = pl != kNone ? ld_cluster<T>(at(pl) + (unsigned)(i * sizeof(T))) : T(0);
+#pragma unroll
+                for (int w = 0; w < kV; ++w) v[u][w] = T(0);
+                if (pl != kNone) ld_cluster_wide(at(pl) + (unsigned)(i * sizeof(T)), v[u]);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < kU; ++u) {
                 if (e0 + u * kTailThreads >= n) continue;
-                cw()[d[u]] = v[u];
-                if (Ic[u] == 0) cw()[d[u] - 1] = v[u];
-                if (Ic[u] == C.nx - 1) cw()[d[u] + 1] = v[u];
+#pragma unroll
+                for (int w = 0; w < kV; ++w) cw()[d[u] + 2 * w] = v[u][w];
+                if (Ic[u] == 0) cw()[d[u] - 1] = v[u][0];
+                if (Ic[u] + 2 * (kV - 1) == C.nx - 1) cw()[d[u] + 2 * kV - 1] = v[u][kV - 1];
             }
         }
     }
@@ -386,7 +473,7 @@ struct Tail {
                 for (int u = 2; u < 8; ++u) r = fma(w[u & 1] * w[(u >> 1) & 1] * w[u >> 2], c[u], r);
                 v += r;
             }
-            put(X, q[m], v);
+            put(X, q[m], v, true);
         }
     }
 };
@@ -404,9 +491,13 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
     unsigned *ctxw = reinterpret_cast<unsigned *>(img + (L.off_w - L.off_c));
     int *jk = reinterpret_cast<int *>(img + (L.off_q - L.off_c));
     unsigned *crow = reinterpret_cast<unsigned *>(jk + L.q4);
+    __shared__ int ghosts, quads;
+    if (threadIdx.x == 0) ghosts = quads = 0;
+    __syncthreads();
     for (int lq = threadIdx.x; lq < L.q4; lq += 256) {
         const int qd = rank * L.q4 + lq, K = qd / cny, J = qd - K * cny;
         jk[lq] = K < cnz ? J | K << 16 : -1;
+        if (K < cnz) atomicAdd(&quads, 1);
         // the coarse rows around the quad (their x) and the place of its own coarse row's b
         for (int r = 0; r < 10 && C; ++r) {
             unsigned pl = U::kNone;
@@ -456,6 +547,7 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
                 if (owner == rank) {
                     out[d] = sn * L.rs;
                 } else {
+                    if (k == 0 && col == 0) atomicAdd(&ghosts, 1);
                     out[d] = (L.q4 * 4 + s * 2 + d) * L.rs;
                     w[4 + d] = U::place(owner, L.off_x + (i64)((L.q4 * 4 + sn * 2 + d) * L.rs + cell) * sizeof(T));
                 }
@@ -470,6 +562,11 @@ __global__ void __launch_bounds__(256) k_tail_prepare(const __grid_constant__ Ta
         for (int u = 0; u < U::kReal; ++u) ctx[u * 2 * L.nit + i] = f[u];
         for (int u = 0; u < U::kWords; ++u) ctxw[u * 2 * L.nit + i] = w[u];
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        jk[L.q4 * 11] = ghosts * L.hx * (int)sizeof(T);  // one colour's
+        jk[L.q4 * 11 + 1] = quads * 4 * L.nx * (int)sizeof(T);
+    }
 }
 
 // mode: kTailAll the whole descent and ascent; kTailDown / kTailUp one of them, with the
@@ -478,11 +575,26 @@ template <typename T>
 __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs a, int mode) {
     extern __shared__ __align__(16) char tail_smem[];
     cg::cluster_group cl = cg::this_cluster();
-    const Tail<T> t{a, tail_smem, (int)cl.block_rank(), (int)cl.num_blocks(), (int)threadIdx.x};
+    __shared__ __align__(8) unsigned long long mbar[3 * kTailLevels + 2];
+    __shared__ TailLevel lv[kTailLevels];
+    static_assert(sizeof(TailLevel) % 4 == 0 && std::is_trivially_copyable<TailLevel>::value, "copied by words");
+    for (int e = threadIdx.x; e < a.nl * (int)(sizeof(TailLevel) / 4); e += kTailThreads)
+        reinterpret_cast<unsigned *>(lv)[e] = reinterpret_cast<const unsigned *>(a.lv)[e];
+    __shared__ unsigned cb[16];
+    const unsigned sm0 = Tail<T>::saddr(tail_smem);
+    if (threadIdx.x < cl.num_blocks()) cb[threadIdx.x] = map_cluster(sm0, (int)threadIdx.x);
+    const Tail<T> t{a, lv, cb, tail_smem, sm0, Tail<T>::saddr(mbar), (int)cl.block_rank(), (int)cl.num_blocks(), (int)threadIdx.x};
+    if (t.tid == 0) {
+        for (int c = 0; c < 3 * kTailLevels + 2; ++c) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(t.mbar + 8 * c) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    unsigned parity = 0;  // of bar_x, bit 2 l + c
+    bool lost = false;
+    __syncthreads();
     const bool from_mem = mode == kTailUp;
 #pragma unroll 1
     for (int l = 0; l < a.nl; ++l) {
-        const TailLevel &L = a.lv[l];
+        const TailLevel &L = lv[l];
         const char *img = reinterpret_cast<const char *>(a.img) + L.img + (size_t)t.rank * L.img_bytes;
         const float4 *src = reinterpret_cast<const float4 *>(img);
         float4 *dst = reinterpret_cast<float4 *>(tail_smem + L.off_c);
@@ -503,15 +615,15 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
     }
     grid_wait();  // the contexts were written long before (set-up ends with a synchronisation); b was not
     __syncthreads();
-    t.load_b(a.lv[0]);
+    t.load_b(lv[0]);
     if (from_mem) {
         cl.sync();  // every CTA's ghosts are zeroed before others write them
         for (int l = 0; l < a.nl; ++l) {
-            t.load_x(a.lv[l]);
-            if (l > 0) t.load_b(a.lv[l]);
+            t.load_x(l);
+            if (l > 0) t.load_b(lv[l]);
         }
         for (int q = t.tid; q < a.nc; q += kTailThreads) {
-            const int cnx = a.lv[a.nl - 1].nx >> 1, cny = a.lv[a.nl - 1].ny >> 1, row = q / cnx;
+            const int cnx = lv[a.nl - 1].nx >> 1, cny = lv[a.nl - 1].ny >> 1, row = q / cnx;
             t.ec()[q] = reinterpret_cast<const T *>(a.xc)[t.coarse_idx(q - row * cnx, row % cny, row / cny, cnx, cny)];
         }
     }
@@ -521,9 +633,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
     Cell<T> first[Tail<T>::kCells], second[Tail<T>::kCells];
     auto restore = [&](int v) {  // everything but b, which may still be on its way
         const bool up = v >= a.nl;
-        const TailLevel &L = a.lv[up ? 2 * a.nl - 1 - v : v];
-        t.restore(L, up ? 1 : 0, first);
-        t.restore(L, up ? 0 : 1, second);
+        const int l = up ? 2 * a.nl - 1 - v : v;
+        t.restore(l, up ? 1 : 0, first);
+        t.restore(l, up ? 0 : 1, second);
     };
     restore(v0);
     cl.barrier_wait();
@@ -531,39 +643,55 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
     for (int v = v0; v < v1; ++v) {
         const bool up = v >= a.nl;
         const int l = up ? 2 * a.nl - 1 - v : v;
-        const TailLevel &L = a.lv[l];
-        const TailLevel *C = l + 1 < a.nl ? &a.lv[l + 1] : nullptr;
+        const TailLevel &L = lv[l];
+        const TailLevel *C = l + 1 < a.nl ? &lv[l + 1] : nullptr;
         t.restore_b(L, up ? 1 : 0, first);
         t.restore_b(L, up ? 0 : 1, second);
+        const int c0 = up ? 1 : 0;
         if (up) {
             t.prolong_red(L, C, second);
-            cl.sync();
+            // the last remote reads are over here: no CTA leaves before the others have come this far
+            if (v + 1 == v1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+            t.exchange(l, 0, parity, lost);
         }
         T *X = t.x(L);
         const T h2 = (T)L.h2;
 #pragma unroll 1
         for (int sw = up ? a.post : a.pre;;) {
-            t.half(X, h2, first);
-            cl.sync();
-            t.half(X, h2, second);
-            if (--sw == 0) break;
-            cl.sync();
+            t.half(X, h2, first, true);
+            t.exchange(l, c0, parity, lost);
+            --sw;
+            t.half(X, h2, second, !up || sw > 0);  // nothing reads the ghosts of an ascent's last half sweep
+            if (sw == 0) break;
+            t.exchange(l, 1 - c0, parity, lost);
         }
         if (!up) {
-            cl.sync();
-            t.restrict_red(L, C, mode == kTailDown, first);
+            t.exchange(l, 1 - c0, parity, lost);
+            t.restrict_red(l, C, mode == kTailDown, first);
         }
-        // the next level's contexts come in while the barrier completes; after the last one no CTA
-        // leaves while others write its ghosts
-        cl.barrier_arrive();
+        // the next level's contexts come in meanwhile.  On the way down a CTA waits for what it
+        // reads; on the way up the next level reads other CTAs' x
+        if (up && v + 1 < v1) cl.barrier_arrive();
         if (v + 1 < v1) restore(v + 1);
-        cl.barrier_wait();
-        if (!up && mode == kTailAll && l == a.nl - 1) {
+        if (up) {
+            cl.barrier_wait();
+        } else if (C) {
+            t.expect(t.bar_b(l + 1), t.cell_bytes(*C));
+            t.wait(t.bar_b(l + 1), 0, lost);
+        } else if (mode == kTailAll) {
+            t.expect(t.bar_r(), (unsigned)(a.nc * sizeof(double)));
+            t.wait(t.bar_r(), 0, lost);
             t.coarse_solve();
-            cl.sync();
+            t.expect(t.bar_e(), (unsigned)(a.nc * sizeof(T)));
+            t.wait(t.bar_e(), 0, lost);
         }
     }
-    for (int l = 0; l < (mode == kTailDown ? a.nl : 1); ++l) t.store(a.lv[l], l > 0);
+    if (__syncthreads_or(lost)) {  // the level's x without a number fails the solve
+        if (t.tid == 0) atomicOr(a.err, 8u);
+        for (int i = t.tid; i < (lv[0].off_b - lv[0].off_x) / (int)sizeof(T); i += kTailThreads) t.x(lv[0])[i] = (T)NAN;
+        __syncthreads();
+    }
+    for (int l = 0; l < (mode == kTailDown ? a.nl : 1); ++l) t.store(lv[l], l > 0);
 }
 
 template <typename T>
@@ -643,7 +771,7 @@ bool tail_layout(TailArgs &a, bool fp64, int ncta) {
         L.off_b = take((i64)2 * L.nit * es);
         L.off_c = take((i64)real * 2 * L.nit * es);
         L.off_w = take((i64)Tail<float>::kWords * 2 * L.nit * 4);
-        L.off_q = take(4 * (i64)L.q4 * 11);
+        L.off_q = take(4 * ((i64)L.q4 * 11 + 2));
         L.img_bytes = (int)(off - L.off_c);
         L.img = img;
         img += (i64)ncta * L.img_bytes;

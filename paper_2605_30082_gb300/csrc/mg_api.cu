@@ -440,6 +440,7 @@ void bind_tail(mg_handle *h) {
     mg::TailArgs &a = h->tail;
     a.pinv = h->pinv;
     a.img = h->tail_img;
+    a.err = h->err;
     Level &C = h->lv[h->nlev - 1];
     a.bc = f64 ? (void *)C.b64 : (void *)C.b32;
     a.xc = f64 ? (void *)C.x64 : (void *)C.x32;
@@ -721,13 +722,19 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
     MG_CUDA(h, cudaEventSynchronize(h->ev1));
     rc = check_launch(h, "solve");
     if (rc) return rc;
-    if (fused0(h, 0)) {  // a bounded wait of a fused sweep that ran out sets bit 4
+    // a bounded wait that ran out sets bit 4 (a fused sweep) or 8 (the coarse levels' cluster, which then
+    // leaves no numbers)
+    if (fused0(h, 0) || status == MG_ERR_DIVERGED) {
         MG_READBACK_ERR(h, s);
         MG_CUDA(h, cudaStreamSynchronize(s));
         const unsigned herr = *h->herr;
         if (herr & 4u) {
             MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), s));
             return fail(h, MG_ERR_CUDA, "a fused sweep gave up waiting for its shared-memory copies");
+        }
+        if (herr & 8u) {
+            MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), s));
+            return fail(h, MG_ERR_CUDA, "the coarse levels' cluster gave up waiting for its neighbours' cells");
         }
     }
     if (st) {

@@ -389,7 +389,7 @@ void launch_coarse_matvec(cudaStream_t s, int nc, const double *pinv, const T *r
 // ---- the coarse levels of a V-cycle in one cluster launch (kernels_tail.cu) -------------
 constexpr int kTailLevels = 6;
 constexpr int kTailCells32 = 2, kTailCells64 = 1;  // cells of a colour per thread
-constexpr int kTailMaxSmem = 227 * 1024, kTailMinSmem = 118 * 1024;  // per CTA, dynamic
+constexpr int kTailMaxSmem = 225 * 1024, kTailMinSmem = 118 * 1024;  // per CTA, dynamic
 enum { kTailAll = 0, kTailDown = 1, kTailUp = 2 };
 struct TailLevel {
     int nx, ny, nz;
@@ -413,6 +413,7 @@ struct TailArgs {
     i64 half_c;
     void *img;             // img_total bytes, written by launch_tail_prepare
     i64 img_total;
+    unsigned *err;         // |= 8 when a wait for ghosts ran out
     int ncta, smem, off_rc, off_ec, off_cw;
 };
 // lays the levels (nx, ny, nz, nc set) out over ncta CTAs; false if they do not fit
