@@ -64,17 +64,16 @@ __device__ __forceinline__ T flux_sum(const Dims &d, int i, int j, int k, i64 c,
 // Lay (BSPLIT, DSPLIT; even nx; b then times h2): 56 bytes in natural order took 137 us, 122 us in colour order.
 // ZERO (red, x = 0 on entry): x = h2 b invd, no neighbour is read
 template <bool BSPLIT, bool DSPLIT, bool ZERO, typename T>
-__global__ void k_rbgs_half(Dims d, T h2, Coef<T> cf, const T *__restrict__ b, T *x, int colour) {
-    grid_wait();
+__global__ void k_rbgs_half(Dims d, FastDiv by_half, FastDiv by_ny, T h2, Coef<T> cf, const T *__restrict__ b, T *x, int colour) {
     const int half = (d.nx + 1) >> 1;
     // black sweeps run from the last plane down: they begin with what the red one left in L2
-    const i64 t = (i64)(colour ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
-    const i64 rows = (i64)d.ny * d.nz;
-    if (t >= rows * half) return;
-    const unsigned tu = (unsigned)t, rowu = tu / (unsigned)half;  // t < 2^31: 32-bit divisions
+    const unsigned t = (colour ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;  // below 2^31
+    const unsigned rowu = t / by_half;
     const i64 row = rowu;
-    const int m = (int)(tu - rowu * (unsigned)half);
-    const int j = (int)(rowu % (unsigned)d.ny), k = (int)(rowu / (unsigned)d.ny);
+    const int m = (int)(t - rowu * (unsigned)half);
+    const int k = (int)(rowu / by_ny), j = (int)(rowu - (unsigned)k * d.ny);
+    grid_wait();
+    if (rowu >= (unsigned)d.ny * d.nz) return;
     const int i = 2 * m + ((colour + j + k) & 1);
     if (i >= d.nx) return;
     const i64 c = row * d.nx + i;
@@ -305,7 +304,8 @@ void launch_rbgs_half64(cudaStream_t s, Dims d, double h2, Coef<double> c, const
     auto kernel = !invd_split ? (from_zero ? k_rbgs_half<false, false, true, double> : k_rbgs_half<false, false, false, double>)
                   : !b_split  ? (from_zero ? k_rbgs_half<false, true, true, double> : k_rbgs_half<false, true, false, double>)
                               : k_rbgs_half<true, true, false, double>;
-    run_kernel(kernel, blocks_for(work), kThreads, 0, s, d, h2, c, b, p, colour);
+    run_kernel(kernel, blocks_for(work), kThreads, 0, s, d, make_div((unsigned)(d.nx + 1) / 2), make_div((unsigned)d.ny), h2, c, b, p,
+               colour);
 }
 
 template <typename T>

@@ -131,18 +131,16 @@ __device__ __forceinline__ void df_add(float &h, float &l, float t) {
 template <bool SFORM, bool FROM_ZERO, int UPDATE = 0, bool GHOST = false>
 __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            Upd up = Upd{}) {
-    grid_wait();
     const int hx = L.hx, kv = hx >> 2;
     // black sweeps run from the last plane down: they begin with what the red one left in L2
-    const i64 t = (i64)(col ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
-    const i64 rows = (i64)L.ny * L.nz;
-    if (t >= rows * kv) return;
-    // thread and row indices stay below 2^31 (at most 2e9 cells): 32-bit divisions, several
-    // times cheaper than 64-bit ones
-    const unsigned tu = (unsigned)t, rowu = tu / (unsigned)kv;
+    const unsigned t = (col ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
+    // thread and row indices stay below 2^31 (at most 2e9 cells)
+    const unsigned rowu = t / L.by4;
     const i64 row = rowu;
-    const int k0 = (int)(tu - rowu * (unsigned)kv) << 2;
-    const int y = (int)(rowu % (unsigned)L.ny), z = (int)(rowu / (unsigned)L.ny);
+    const int k0 = (int)(t - rowu * (unsigned)kv) << 2;
+    const int z = (int)(rowu / L.by_ny), y = (int)(rowu - (unsigned)z * L.ny);
+    grid_wait();
+    if (rowu >= (unsigned)L.ny * L.nz) return;
     const int p = (col + y + z) & 1;  // x = 2k + p
     const i64 own = col * L.half + row * hx + k0;
     const i64 opp = (1 - col) * L.half + row * hx + k0;
@@ -829,9 +827,9 @@ __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, fl
     if (T >= crows * kv) return;
     // thread and row indices stay below 2^31 (at most 2e9 cells): 32-bit divisions, several
     // times cheaper than 64-bit ones
-    const unsigned Tu = (unsigned)T, crowu = Tu / (unsigned)kv;
+    const unsigned Tu = (unsigned)T, crowu = Tu / L.by4;
     const int k0 = (int)(Tu - crowu * (unsigned)kv) << 2;
-    const int J = (int)(crowu % (unsigned)Lc.ny), K = (int)(crowu / (unsigned)Lc.ny);
+    const int K = (int)(crowu / Lc.by_ny), J = (int)(crowu - (unsigned)K * Lc.ny);
     const i64 dy = hx, dz = (i64)L.ny * hx;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -926,16 +924,16 @@ constexpr int kRrRowThreads = 128;
 template <bool SFORM, bool TAIL>
 __global__ void __launch_bounds__(kRrRowThreads, 6) k_rr_red_row(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                                                                  const float *__restrict__ xv, float *bc) {
-    grid_wait();
-    if (TAIL) trigger_next();
     const int hx = L.hx, kv = hx >> 2;
     const unsigned T = blockIdx.x * blockDim.x + threadIdx.x, lane = T & 31, total = (unsigned)Lc.ny * Lc.nz * kv;
     const unsigned vi = (T >> 5) * 8 + (lane & 7), vc = min(vi, total - 1);  // 4-cell vector of the coarse level
     const int ch = lane >> 3;
-    const unsigned crow = vc / (unsigned)kv;
+    const unsigned crow = vc / L.by4;
     const int k0 = (int)(vc - crow * (unsigned)kv) << 2;
-    const int J = (int)(crow % (unsigned)Lc.ny), K = (int)(crow / (unsigned)Lc.ny);
+    const int K = (int)(crow / Lc.by_ny), J = (int)(crow - (unsigned)K * Lc.ny);
     const i64 dy = hx, dz = (i64)L.ny * hx;
+    grid_wait();
+    if (TAIL) trigger_next();
     const int y = 2 * J + (ch & 1), z = 2 * K + (ch >> 1);
     const int p = (y + z) & 1;  // red cells of this row sit at x = 2k + p
     const i64 row = (i64)z * L.ny + y;
@@ -1027,10 +1025,10 @@ __global__ void k_prolong_red_vec(Lay L, Lay Lc, const float *__restrict__ ec, f
     if (t >= rows * kv) return;
     // thread and row indices stay below 2^31 (at most 2e9 cells): 32-bit divisions, several
     // times cheaper than 64-bit ones
-    const unsigned tu = (unsigned)t, rowu = tu / (unsigned)kv;
+    const unsigned tu = (unsigned)t, rowu = tu / L.by4;
     const i64 row = rowu;
     const int k0 = (int)(tu - rowu * (unsigned)kv) << 2;
-    const int y = (int)(rowu % (unsigned)L.ny), z = (int)(rowu / (unsigned)L.ny);
+    const int z = (int)(rowu / L.by_ny), y = (int)(rowu - (unsigned)z * L.ny);
     const int p = (y + z) & 1;  // red x = 2k + p, coarse I = k
     const int J = y >> 1, K = z >> 1;
     float out[4];
@@ -1101,9 +1099,9 @@ __global__ void __launch_bounds__(kProlThreads, 10) k_prolong_red8(Lay L, Lay Lc
     if (t >= crows * kv) return;
     // thread and row indices stay below 2^31 (at most 2e9 cells): 32-bit divisions, several
     // times cheaper than 64-bit ones
-    const unsigned tu = (unsigned)t, crowu = tu / (unsigned)kv;
+    const unsigned tu = (unsigned)t, crowu = 2 * tu / L.by4;
     const int k0 = (int)(tu - crowu * (unsigned)kv) << 3;
-    const int J = (int)(crowu % (unsigned)Lc.ny), K = (int)(crowu / (unsigned)Lc.ny);
+    const int K = (int)(crowu / Lc.by_ny), J = (int)(crowu - (unsigned)K * Lc.ny);
     const int hxc = Lc.hx, ncx = Lc.nx;
     const int Js[3] = {max(J - 1, 0), J, min(J + 1, Lc.ny - 1)};
     const int Ks[3] = {(GHOST && Lc.zlo) ? K - 1 : max(K - 1, 0), K, (GHOST && Lc.zhi) ? K + 1 : min(K + 1, Lc.nz - 1)};
@@ -1173,12 +1171,12 @@ __global__ void __launch_bounds__(kProlThreads, 10) k_prolong_red8(Lay L, Lay Lc
 constexpr i64 kProlRowCells = 8000000;
 constexpr int kProlRowThreads = 128;
 __global__ void __launch_bounds__(kProlRowThreads, 8) k_prolong_red_row(Lay L, Lay Lc, const float *__restrict__ ec, float *xv) {
-    grid_wait();
     const int hx = L.hx, kv = hx >> 3;  // 8-cell groups per fine row
-    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = t / (unsigned)kv;
-    if (row >= (unsigned)L.ny * L.nz) return;
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = 2 * t / L.by4;
     const int k0 = (int)(t - row * (unsigned)kv) << 3;
-    const int y = (int)(row % (unsigned)L.ny), z = (int)(row / (unsigned)L.ny);
+    const int z = (int)(row / L.by_ny), y = (int)(row - (unsigned)z * L.ny);
+    grid_wait();
+    if (row >= (unsigned)L.ny * L.nz) return;
     const int d = y & 1, e = z & 1, J = y >> 1, K = z >> 1, hxc = Lc.hx;
     const int J2 = d ? min(J + 1, Lc.ny - 1) : max(J - 1, 0), K2 = e ? min(K + 1, Lc.nz - 1) : max(K - 1, 0);
     float *xr = xv + (i64)row * hx + k0;
@@ -1382,6 +1380,8 @@ Lay make_lay(Dims d) {
     L.hx = d.nx / 2;
     L.half = d.n / 2;
     L.zlo = L.zhi = 0;
+    L.by4 = make_div((unsigned)(L.hx / 4));
+    L.by_ny = make_div((unsigned)L.ny);
     return L;
 }
 

@@ -39,6 +39,22 @@ inline Dims make_dims(int nx, int ny, int nz) {
     return d;
 }
 
+// Division of n < 2^31 by a fixed d >= 1 with one multiplication (m = floor(2^32 (2^s - d) / d) + 1, s = ceil(log2 d)):
+// n / d = (umulhi(n, m) + n) >> s.  A 32-bit division by a variable takes some 20 dependent
+// instructions, and the small half sweeps, where a thread has three before its first load, feel them.
+struct FastDiv {
+    unsigned m, s;
+};
+inline FastDiv make_div(unsigned d) {
+    if (d < 1) d = 1;
+    unsigned s = 0;
+    while ((1ull << s) < d) ++s;
+    return FastDiv{(unsigned)(((1ull << 32) * ((1ull << s) - d)) / d + 1), s};
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned operator/(unsigned n, const FastDiv &f) { return (__umulhi(n, f.m) + n) >> f.s; }
+#endif
+
 // Storage layout of an FP32 level: colour-split (all red cells, then all black, each
 // colour row by row, cell x of a row at k = x >> 1) when nx is even, else natural.
 // A z slab of a decomposed level (mg_dd.cu, split layout only) keeps a ghost plane below and
@@ -54,6 +70,7 @@ struct Lay {
     int hx;     // nx / 2
     i64 half;   // n / 2 (a slab: the colour stride)
     int zlo, zhi;
+    FastDiv by4, by_ny;  // by hx / 4, by ny
 };
 Lay make_lay(Dims d);
 
