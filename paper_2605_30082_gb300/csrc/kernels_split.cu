@@ -136,17 +136,19 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
     const unsigned t = (col ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * blockDim.x + threadIdx.x;
     // thread and row indices stay below 2^31 (at most 2e9 cells)
     const unsigned rowu = t / L.by4;
-    const i64 row = rowu;
+    // offsets within a level fit 32 bits (a slab's two ghost planes might not)
+    using Off = typename std::conditional<GHOST, i64, int>::type;
+    const Off row = (Off)rowu;
     const int k0 = (int)(t - rowu * (unsigned)kv) << 2;
     const int z = (int)(rowu / L.by_ny), y = (int)(rowu - (unsigned)z * L.ny);
     grid_wait();
     if (rowu >= (unsigned)L.ny * L.nz) return;
     const int p = (col + y + z) & 1;  // x = 2k + p
-    const i64 own = col * L.half + row * hx + k0;
-    const i64 opp = (1 - col) * L.half + row * hx + k0;
+    const Off own = (col ? (Off)L.half : 0) + row * hx + k0;
+    const Off opp = (col ? 0 : (Off)L.half) + row * hx + k0;
     const bool hy0 = y > 0, hy1 = y < L.ny - 1;
     const bool hz0 = z > 0 || (GHOST && L.zlo), hz1 = z < L.nz - 1 || (GHOST && L.zhi);
-    const i64 dy = hx, dz = (i64)L.ny * hx;
+    const Off dy = hx, dz = (Off)L.ny * hx;
     // same-row other-colour window: xm[v] = O[k0+v+p-1], xp[v] = O[k0+v+p]
     auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
         const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
@@ -160,7 +162,7 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
             q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
         }
     };
-    auto ld4 = [&](const float *A, i64 off, bool ok, float (&v)[4]) {
+    auto ld4 = [&](const float *A, Off off, bool ok, float (&v)[4]) {
         if (ok) {
             const float4 c4 = *reinterpret_cast<const float4 *>(A + off);
             v[0] = c4.x; v[1] = c4.y; v[2] = c4.z; v[3] = c4.w;
@@ -232,7 +234,7 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
         const float4 blk = *reinterpret_cast<const float4 *>(xv + opp);
         const float bk[4] = {blk.x, blk.y, blk.z, blk.w};
         const float al = up.alpha, sh = up.shift;
-        float2 *pr = up.p2 + row * L.nx + 2 * k0;
+        float2 *pr = up.p2 + (i64)row * L.nx + 2 * k0;
         float4 pvs[4];  // all loads before the first store
 #pragma unroll
         for (int v = 0; v < 4; ++v) pvs[v] = *reinterpret_cast<const float4 *>(pr + 2 * v);
@@ -249,7 +251,7 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
         const float4 blk = *reinterpret_cast<const float4 *>(xv + opp);
         const float bk[4] = {blk.x, blk.y, blk.z, blk.w};
         const float al = up.alpha, sh = up.shift;
-        double *pr = up.p + row * L.nx + 2 * k0;
+        double *pr = up.p + (i64)row * L.nx + 2 * k0;
         double2 pvs[4];  // all loads before the first store
 #pragma unroll
         for (int v = 0; v < 4; ++v) pvs[v] = *reinterpret_cast<const double2 *>(pr + 2 * v);
@@ -931,13 +933,13 @@ __global__ void __launch_bounds__(kRrRowThreads, 6) k_rr_red_row(Lay L, Lay Lc, 
     const unsigned crow = vc / L.by4;
     const int k0 = (int)(vc - crow * (unsigned)kv) << 2;
     const int K = (int)(crow / Lc.by_ny), J = (int)(crow - (unsigned)K * Lc.ny);
-    const i64 dy = hx, dz = (i64)L.ny * hx;
+    const int dy = hx, dz = L.ny * hx;
     grid_wait();
     if (TAIL) trigger_next();
     const int y = 2 * J + (ch & 1), z = 2 * K + (ch >> 1);
     const int p = (y + z) & 1;  // red cells of this row sit at x = 2k + p
-    const i64 row = (i64)z * L.ny + y;
-    const i64 own = row * hx + k0, opp = L.half + row * hx + k0;
+    const int row = z * L.ny + y;
+    const int own = row * hx + k0, opp = (int)L.half + own;
     const bool hy0 = y > 0, hy1 = y < L.ny - 1, hz0 = z > 0, hz1 = z < L.nz - 1;
     const bool xw0 = (p == 0 && k0 == 0), xw1 = (p == 1 && k0 + 4 == hx);
     auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
@@ -952,7 +954,7 @@ __global__ void __launch_bounds__(kRrRowThreads, 6) k_rr_red_row(Lay L, Lay Lc, 
             q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
         }
     };
-    auto ld4 = [&](const float *A, i64 off, bool ok, float (&v)[4]) {
+    auto ld4 = [&](const float *A, int off, bool ok, float (&v)[4]) {
         if (ok) {
             const float4 c4 = *reinterpret_cast<const float4 *>(A + off);
             v[0] = c4.x; v[1] = c4.y; v[2] = c4.z; v[3] = c4.w;
