@@ -149,18 +149,15 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
     const bool hy0 = y > 0, hy1 = y < L.ny - 1;
     const bool hz0 = z > 0 || (GHOST && L.zlo), hz1 = z < L.nz - 1 || (GHOST && L.zhi);
     const Off dy = hx, dz = (Off)L.ny * hx;
+    const bool edge = p ? k0 + 4 < hx : k0 > 0;  // the window's fifth cell lies in the row
+    const int eo = p ? 4 : -1;
     // same-row other-colour window: xm[v] = O[k0+v+p-1], xp[v] = O[k0+v+p]
     auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
+        // by selection: the rows of a warp have both parities, and a branch would run both ways
         const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
-        if (p) {
-            const float e = (k0 + 4 < hx) ? O[opp + 4] : 0.f;
-            m[0] = c4.x; m[1] = c4.y; m[2] = c4.z; m[3] = c4.w;
-            q[0] = c4.y; q[1] = c4.z; q[2] = c4.w; q[3] = e;
-        } else {
-            const float e = (k0 > 0) ? O[opp - 1] : 0.f;
-            m[0] = e; m[1] = c4.x; m[2] = c4.y; m[3] = c4.z;
-            q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
-        }
+        const float e = edge ? O[opp + eo] : 0.f;
+        m[0] = p ? c4.x : e; m[1] = p ? c4.y : c4.x; m[2] = p ? c4.z : c4.y; m[3] = p ? c4.w : c4.z;
+        q[0] = m[1]; q[1] = m[2]; q[2] = m[3]; q[3] = p ? e : c4.w;
     };
     auto ld4 = [&](const float *A, Off off, bool ok, float (&v)[4]) {
         if (ok) {
@@ -942,17 +939,13 @@ __global__ void __launch_bounds__(kRrRowThreads, 6) k_rr_red_row(Lay L, Lay Lc, 
     const int own = row * hx + k0, opp = (int)L.half + own;
     const bool hy0 = y > 0, hy1 = y < L.ny - 1, hz0 = z > 0, hz1 = z < L.nz - 1;
     const bool xw0 = (p == 0 && k0 == 0), xw1 = (p == 1 && k0 + 4 == hx);
+    const bool edge = p ? k0 + 4 < hx : k0 > 0;  // the window's fifth cell lies in the row
+    const int eo = p ? 4 : -1;
     auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
         const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
-        if (p) {
-            const float e = (k0 + 4 < hx) ? O[opp + 4] : 0.f;
-            m[0] = c4.x; m[1] = c4.y; m[2] = c4.z; m[3] = c4.w;
-            q[0] = c4.y; q[1] = c4.z; q[2] = c4.w; q[3] = e;
-        } else {
-            const float e = (k0 > 0) ? O[opp - 1] : 0.f;
-            m[0] = e; m[1] = c4.x; m[2] = c4.y; m[3] = c4.z;
-            q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
-        }
+        const float e = edge ? O[opp + eo] : 0.f;
+        m[0] = p ? c4.x : e; m[1] = p ? c4.y : c4.x; m[2] = p ? c4.z : c4.y; m[3] = p ? c4.w : c4.z;
+        q[0] = m[1]; q[1] = m[2]; q[2] = m[3]; q[3] = p ? e : c4.w;
     };
     auto ld4 = [&](const float *A, int off, bool ok, float (&v)[4]) {
         if (ok) {
