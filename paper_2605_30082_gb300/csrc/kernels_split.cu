@@ -121,6 +121,55 @@ __device__ __forceinline__ void df_add(float &h, float &l, float t) {
     l = e - (h - s);
 }
 
+// pairs of FP32 numbers: one instruction for two cells
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// two cells of a half sweep: (hh b + sum w x) / sum w over the faces x-, x+, y-, y+, z-, z+; SFORM: w = c + a, else w = a
+template <bool SFORM, bool FROM_ZERO>
+__device__ __forceinline__ void relax2(float hh, f32x2 b, f32x2 c, f32x2 a0, f32x2 a1, f32x2 a2, f32x2 a3, f32x2 a4, f32x2 a5, f32x2 v0,
+                                       f32x2 v1, f32x2 v2, f32x2 v3, f32x2 v4, f32x2 v5, float &o0, float &o1) {
+    const f32x2 w0 = SFORM ? add2(c, a0) : a0, w1 = SFORM ? add2(c, a1) : a1, w2 = SFORM ? add2(c, a2) : a2;
+    const f32x2 w3 = SFORM ? add2(c, a3) : a3, w4 = SFORM ? add2(c, a4) : a4, w5 = SFORM ? add2(c, a5) : a5;
+    f32x2 num;
+    if (FROM_ZERO) {
+        num = mul2(pack2(hh, hh), b);
+    } else {
+        num = fma2(w0, v0, mul2(w1, v1));
+        num = fma2(w2, v2, num);
+        num = fma2(w3, v3, num);
+        num = fma2(w4, v4, num);
+        num = fma2(w5, v5, num);
+        num = fma2(pack2(hh, hh), b, num);
+    }
+    const f32x2 den = add2(add2(add2(w0, w1), add2(w2, w3)), add2(w4, w5));
+    float n0, n1, d0, d1;
+    unpack2(num, n0, n1);
+    unpack2(den, d0, d1);
+    o0 = __fdividef(n0, d0);
+    o1 = __fdividef(n1, d1);
+}
+
 // ---- vectorised half sweep on split levels (hx % 4 == 0) ---------------------------------
 // one thread updates 4 consecutive cells (k0..k0+3) of colour col in one row.
 // UPDATE (last red half sweep of the finest level): instead of storing the 4 new red values,
@@ -128,8 +177,10 @@ __device__ __forceinline__ void df_add(float &h, float &l, float t) {
 // together the 8 consecutive cells x = 2 k0 .. 2 k0 + 7 -- to the solution: the FP64 one
 // (UPDATE 1) or the double-float one (UPDATE 2).
 // GHOST: a slab of a decomposed level (L.zlo / L.zhi), its ghost planes as z neighbours
+// On levels in L2 the instructions bound it, not the bytes: divisions for the indices, the parity branch of the
+// window, selects at walls that few rows have and scalar arithmetic took 224 x 160 x 96 with its adjoint from 5.6 to 6.6 ms.
 template <bool SFORM, bool FROM_ZERO, int UPDATE = 0, bool GHOST = false>
-__global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
+__global__ void __launch_bounds__(kThreads, 4) k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            Upd up = Upd{}) {
     const int hx = L.hx, kv = hx >> 2;
     // black sweeps run from the last plane down: they begin with what the red one left in L2
@@ -150,81 +201,79 @@ __global__ void k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__
     const bool hz0 = z > 0 || (GHOST && L.zlo), hz1 = z < L.nz - 1 || (GHOST && L.zhi);
     const Off dy = hx, dz = (Off)L.ny * hx;
     const bool edge = p ? k0 + 4 < hx : k0 > 0;  // the window's fifth cell lies in the row
-    const int eo = p ? 4 : -1;
-    // same-row other-colour window: xm[v] = O[k0+v+p-1], xp[v] = O[k0+v+p]
-    auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
-        // by selection: the rows of a warp have both parities, and a branch would run both ways
-        const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
-        const float e = edge ? O[opp + eo] : 0.f;
-        m[0] = p ? c4.x : e; m[1] = p ? c4.y : c4.x; m[2] = p ? c4.z : c4.y; m[3] = p ? c4.w : c4.z;
-        q[0] = m[1]; q[1] = m[2]; q[2] = m[3]; q[3] = p ? e : c4.w;
+    const Off oe = opp + (p ? 4 : -1);
+    const float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto ld = [](const float *A, Off off) { return *reinterpret_cast<const float4 *>(A + off); };
+    // the other colour's cells left (m) and right (q) of the row's: o shifted by one cell or not, e the fifth.  By
+    // selection: the rows of a warp have both parities, and a branch would run both ways
+    auto window = [&](const float4 &o, float e, float4 &m, float4 &q) {
+        m = make_float4(p ? o.x : e, p ? o.y : o.x, p ? o.z : o.y, p ? o.w : o.z);
+        q = make_float4(m.y, m.z, m.w, p ? e : o.w);
     };
-    auto ld4 = [&](const float *A, Off off, bool ok, float (&v)[4]) {
-        if (ok) {
-            const float4 c4 = *reinterpret_cast<const float4 *>(A + off);
-            v[0] = c4.x; v[1] = c4.y; v[2] = c4.z; v[3] = c4.w;
-        } else {
-            v[0] = v[1] = v[2] = v[3] = 0.f;
-        }
-    };
-    // wall masks along x: the first cell of a row has no x-1 when p == 0, the last no x+1 when p == 1
-    const bool xw0 = (p == 0 && k0 == 0), xw1 = (p == 1 && k0 + 4 == hx);
-    float xm[4], xp[4], ym[4], yp[4], zm[4], zp[4];
+    // neighbouring rows, at a wall the row itself: loaded without a branch, put right behind one
+    const Off oy0 = hy0 ? opp - dy : opp, oy1 = hy1 ? opp + dy : opp, oz0 = hz0 ? opp - dz : opp, oz1 = hz1 ? opp + dz : opp;
+    const bool inner = hy0 && hy1 && hz0 && hz1;
+    float4 xm = f0, xp = f0, ym = f0, yp = f0, zm = f0, zp = f0;
     if (!FROM_ZERO) {
-        window(xv, xm, xp);
-        ld4(xv, opp - dy, hy0, ym);
-        ld4(xv, opp + dy, hy1, yp);
-        ld4(xv, opp - dz, hz0, zm);
-        ld4(xv, opp + dz, hz1, zp);
+        ym = ld(xv, oy0);
+        yp = ld(xv, oy1);
+        zm = ld(xv, oz0);
+        zp = ld(xv, oz1);
+        float e = 0.f;
+        if (edge) e = xv[oe];
+        window(ld(xv, opp), e, xm, xp);
     }
-    float w0[4], w1[4], w2[4], w3[4], w4[4], w5[4];
+    const float4 bb = ld(b, own);
+    float4 w0, w1, w2, w3, w4, w5;  // SFORM: s of the neighbours; a weight is the cell's s plus theirs
+    float4 sc = f0;
     if (SFORM) {
-        float sc[4], sm_[4], sp_[4], s2[4], s3[4], s4[4], s5[4];
-        ld4(cf.s, own, true, sc);
-        window(cf.s, sm_, sp_);
-        ld4(cf.s, opp - dy, hy0, s2);
-        ld4(cf.s, opp + dy, hy1, s3);
-        ld4(cf.s, opp - dz, hz0, s4);
-        ld4(cf.s, opp + dz, hz1, s5);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            w0[v] = (v == 0 && xw0) ? 0.f : sc[v] + sm_[v];
-            w1[v] = (v == 3 && xw1) ? 0.f : sc[v] + sp_[v];
-            w2[v] = hy0 ? sc[v] + s2[v] : 0.f;
-            w3[v] = hy1 ? sc[v] + s3[v] : 0.f;
-            w4[v] = hz0 ? sc[v] + s4[v] : 0.f;
-            w5[v] = hz1 ? sc[v] + s5[v] : 0.f;
-        }
+        sc = ld(cf.s, own);
+        w2 = ld(cf.s, oy0);
+        w3 = ld(cf.s, oy1);
+        w4 = ld(cf.s, oz0);
+        w5 = ld(cf.s, oz1);
+        // beyond a wall s = -s of the cell, so that the weight s + s is an exact 0
+        float e = p ? -sc.w : -sc.x;
+        if (edge) e = cf.s[oe];
+        window(ld(cf.s, opp), e, w0, w1);
     } else {
-        float d0[4], d1[4];
-        ld4(cf.fx, own, true, w0);           // low x face (0 at x = 0)
-        window(cf.fx, d0, w1);               // high x face = the x+1 neighbour's low face
-        if (xw1) w1[3] = 0.f;
-        ld4(cf.fy, own, true, w2);
-        ld4(cf.fy, opp + dy, hy1, w3);
-        ld4(cf.fz, own, true, w4);
-        ld4(cf.fz, opp + dz, hz1, w5);
-        (void)d0;
-        (void)d1;
+        w0 = ld(cf.fx, own);  // low x face (0 at x = 0)
+        float e = 0.f;
+        if (edge) e = cf.fx[oe];
+        float4 d;
+        window(ld(cf.fx, opp), e, d, w1);  // high x face = the x+1 neighbour's low face
+        w2 = ld(cf.fy, own);
+        w3 = ld(cf.fy, oy1);
+        w4 = ld(cf.fz, own);
+        w5 = ld(cf.fz, oz1);
     }
-    float bb[4];
-    ld4(b, own, true, bb);
+    if (!inner) {
+        const float4 no = make_float4(-sc.x, -sc.y, -sc.z, -sc.w);  // faces: 0
+        if (!hy0) {
+            ym = f0;
+            if (SFORM) w2 = no;
+        }
+        if (!hy1) {
+            yp = f0;
+            w3 = no;
+        }
+        if (!hz0) {
+            zm = f0;
+            if (SFORM) w4 = no;
+        }
+        if (!hz1) {
+            zp = f0;
+            w5 = no;
+        }
+    }
     const float hh = SFORM ? 2.f * h2 : h2;
     float out[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        float num = 0.f;
-        if (!FROM_ZERO) {
-            num = w0[v] * xm[v];
-            num += w1[v] * xp[v];
-            num += w2[v] * ym[v];
-            num += w3[v] * yp[v];
-            num += w4[v] * zm[v];
-            num += w5[v] * zp[v];
-        }
-        const float den = ((w0[v] + w1[v]) + (w2[v] + w3[v])) + (w4[v] + w5[v]);
-        out[v] = __fdividef(hh * bb[v] + num, den);
-    }
+    auto lo = [](const float4 &q) { return pack2(q.x, q.y); };
+    auto hi = [](const float4 &q) { return pack2(q.z, q.w); };
+    relax2<SFORM, FROM_ZERO>(hh, lo(bb), lo(sc), lo(w0), lo(w1), lo(w2), lo(w3), lo(w4), lo(w5), lo(xm), lo(xp), lo(ym), lo(yp), lo(zm),
+                             lo(zp), out[0], out[1]);
+    relax2<SFORM, FROM_ZERO>(hh, hi(bb), hi(sc), hi(w0), hi(w1), hi(w2), hi(w3), hi(w4), hi(w5), hi(xm), hi(xp), hi(ym), hi(yp), hi(zm),
+                             hi(zp), out[2], out[3]);
     if (UPDATE == 0) {
         *reinterpret_cast<float4 *>(xv + own) = make_float4(out[0], out[1], out[2], out[3]);
     } else if (UPDATE == 2) {
@@ -387,28 +436,6 @@ struct ZrTile {
                     // several tiles) the vectors beside the tile's rows
 };
 
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -545,27 +572,11 @@ __global__ void __launch_bounds__(kZrThreads, kZrBlocks) k_half_zr(Lay L, ZrTile
             sm = make_float4(sl, szc.x, szc.y, szc.z);
         }
         float4 out;
-        auto pair = [&](f32x2 c, f32x2 bq, f32x2 a0, f32x2 a1, f32x2 a2, f32x2 a3, f32x2 a4, f32x2 a5, f32x2 v0, f32x2 v1,
-                        f32x2 v2, f32x2 v3, f32x2 v4, f32x2 v5, float &o0, float &o1) {
-            const f32x2 w0 = add2(c, a0), w1 = add2(c, a1), w2 = add2(c, a2), w3 = add2(c, a3), w4 = add2(c, a4), w5 = add2(c, a5);
-            f32x2 num = fma2(w0, v0, mul2(w1, v1));
-            num = fma2(w2, v2, num);
-            num = fma2(w3, v3, num);
-            num = fma2(w4, v4, num);
-            num = fma2(w5, v5, num);
-            num = fma2(pack2(hh, hh), bq, num);
-            const f32x2 den = add2(add2(add2(w0, w1), add2(w2, w3)), add2(w4, w5));
-            float n0, n1, d0, d1;
-            unpack2(num, n0, n1);
-            unpack2(den, d0, d1);
-            o0 = __fdividef(n0, d0);
-            o1 = __fdividef(n1, d1);
-        };
         auto lo = [](const float4 &q) { return pack2(q.x, q.y); };
         auto up = [](const float4 &q) { return pack2(q.z, q.w); };
-        pair(lo(sc), lo(bv), lo(sm), lo(sp), lo(s2), lo(s3), lo(s4), lo(s5), lo(xm), lo(xp), lo(ym), lo(yp), lo(xzm), lo(xzp),
+        relax2<true, false>(hh, lo(bv), lo(sc), lo(sm), lo(sp), lo(s2), lo(s3), lo(s4), lo(s5), lo(xm), lo(xp), lo(ym), lo(yp), lo(xzm), lo(xzp),
              out.x, out.y);
-        pair(up(sc), up(bv), up(sm), up(sp), up(s2), up(s3), up(s4), up(s5), up(xm), up(xp), up(ym), up(yp), up(xzm), up(xzp),
+        relax2<true, false>(hh, up(bv), up(sc), up(sm), up(sp), up(s2), up(s3), up(s4), up(s5), up(xm), up(xp), up(ym), up(yp), up(xzm), up(xzp),
              out.z, out.w);
         if (act) *reinterpret_cast<float4 *>(xv + own0 + (i64)z * dz) = out;
         xzm = xzc;
