@@ -559,7 +559,7 @@ def run_ours(args):
                "traffic": _traffic("k_half_zr", cells),
                "kernel": "k_half_zr (finest-level FP32 red-black half sweep, z-marching tiles of rows shared "
                          "in shared memory, planes loaded by cp.async two ahead; the one from-zero sweep per "
-                         "outer iteration is k_half_z0)",
+                         "outer iteration is k_half_vec)",
                "launch_ms": round(avg_sm, 4), "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)"}
     n_fr, ms_fr = prof["fine_residual"]
     avg_fr = ms_fr / max(n_fr, 1)

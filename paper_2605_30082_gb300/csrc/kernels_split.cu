@@ -178,9 +178,11 @@ __device__ __forceinline__ void relax2(float hh, f32x2 b, f32x2 c, f32x2 a0, f32
 // (UPDATE 1) or the double-float one (UPDATE 2).
 // GHOST: a slab of a decomposed level (L.zlo / L.zhi), its ghost planes as z neighbours
 // On levels in L2 the instructions bound it, not the bytes: divisions for the indices, the parity branch of the
-// window, selects at walls that few rows have and scalar arithmetic took 224 x 160 x 96 with its adjoint from 5.6 to 6.6 ms.
+// window, selects at walls that few rows have and scalar arithmetic made 224 x 160 x 96 with its adjoint 6.6 ms, not
+// 5.6.  Without them it also beats kernels that march planes (face form at 256^3 staged by cp.async, 532 us a V-cycle against
+// 522; first sweep from zero, 757 against 754 at 512 x 256 x 256) and, up to 60 M cells, the row-sharing one below.
 template <bool SFORM, bool FROM_ZERO, int UPDATE = 0, bool GHOST = false>
-__global__ void __launch_bounds__(kThreads, 4) k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
+__global__ void __launch_bounds__(kThreads, UPDATE == 1 ? 3 : 4) k_half_vec(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            Upd up = Upd{}) {
     const int hx = L.hx, kv = hx >> 2;
     // black sweeps run from the last plane down: they begin with what the red one left in L2
@@ -311,103 +313,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_half_vec(Lay L, float h2, Coef3
     }
 }
 
-// ---- z-marching half sweep from zero (split levels, rows of a multiple of 32 vectors) --------
-// The first half sweep of a V-cycle from x = 0 reads no x: with num = 0 it is h^2 b over the sum of the
-// coefficients.  A warp covers 32 consecutive vectors of one row; a thread walks ZC planes and keeps
-// the other colour's s of planes z - 1, z and z + 1 in registers, so that each plane of it comes from
-// memory once; the window scalars come from the neighbouring lanes.  Lanes past the end of a row,
-// or rows past ny, compute on clamped (in-bounds) indices and store nothing.  512^3 166 us against 185 with
-// k_half_vec, 256^3 23.9 against 25.1, 256 x 128 x 128 5.0 against 5.6, below that the latter is faster.
-template <bool SFORM, int ZC, bool GHOST = false>
-__global__ void __launch_bounds__(64, 12) k_half_z0(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col) {
-    grid_wait();
-    const int hx = L.hx, kv = hx >> 2;
-    const int kvi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int yi = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool active = kvi < kv && yi < L.ny;
-    const int k0 = min(kvi, kv - 1) << 2;
-    const int y = min(yi, L.ny - 1);
-    const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, L.nz);
-    const int lane = threadIdx.x & 31;
-    const i64 dy = hx, dz = (i64)L.ny * hx;
-    const bool hy0 = y > 0, hy1 = y < L.ny - 1;
-    const bool kl = k0 > 0, kr = k0 + 4 < hx;
-    i64 opp = (i64)(1 - col) * L.half + ((i64)z0 * L.ny + y) * hx + k0;
-    i64 own = (i64)col * L.half + ((i64)z0 * L.ny + y) * hx + k0;
-    const float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto ld = [](const float *A, i64 off) { return *reinterpret_cast<const float4 *>(A + off); };
-    const bool glo = GHOST && L.zlo, ghi = GHOST && L.zhi;  // a slab's ghost planes are neighbours
-    float4 szm = f0, szc = f0;
-    if (SFORM) {
-        if (z0 > 0 || glo) szm = ld(cf.s, opp - dz);
-        szc = ld(cf.s, opp);
-    }
-    const float hh = SFORM ? 2.f * h2 : h2;
-    for (int z = z0; z < z1; ++z) {
-        const bool hz0 = z > 0 || glo, hz1 = z < L.nz - 1 || ghi;
-        const int p = (col + y + z) & 1;  // x = 2k + p
-        const bool xw0 = (p == 0 && !kl), xw1 = (p == 1 && !kr);
-        float w0[4], w1[4], w2[4], w3[4], w4[4], w5[4];
-        float4 szp = f0;
-        if (SFORM) {
-            float4 s2 = f0, s3 = f0;
-            if (hz1) szp = ld(cf.s, opp + dz);
-            if (hy0) s2 = ld(cf.s, opp - dy);
-            if (hy1) s3 = ld(cf.s, opp + dy);
-            const float4 sc4 = ld(cf.s, own);
-            float sl = __shfl_up_sync(0xffffffffu, szc.w, 1), sr = __shfl_down_sync(0xffffffffu, szc.x, 1);
-            if (lane == 0) sl = kl ? cf.s[opp - 1] : 0.f;
-            if (lane == 31) sr = kr ? cf.s[opp + 4] : 0.f;
-            const float so[4] = {szc.x, szc.y, szc.z, szc.w}, sc[4] = {sc4.x, sc4.y, sc4.z, sc4.w};
-            const float s2v[4] = {s2.x, s2.y, s2.z, s2.w}, s3v[4] = {s3.x, s3.y, s3.z, s3.w};
-            const float s4v[4] = {szm.x, szm.y, szm.z, szm.w}, s5v[4] = {szp.x, szp.y, szp.z, szp.w};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float sm = p ? so[v] : (v ? so[v - 1] : sl);
-                const float sp = p ? (v < 3 ? so[v + 1] : sr) : so[v];
-                w0[v] = (v == 0 && xw0) ? 0.f : sc[v] + sm;
-                w1[v] = (v == 3 && xw1) ? 0.f : sc[v] + sp;
-                w2[v] = hy0 ? sc[v] + s2v[v] : 0.f;
-                w3[v] = hy1 ? sc[v] + s3v[v] : 0.f;
-                w4[v] = hz0 ? sc[v] + s4v[v] : 0.f;
-                w5[v] = hz1 ? sc[v] + s5v[v] : 0.f;
-            }
-        } else {
-            const float4 fo = ld(cf.fx, opp);  // low x faces of the other colour = high faces of own
-            float fr = __shfl_down_sync(0xffffffffu, fo.x, 1);
-            if (lane == 31) fr = kr ? cf.fx[opp + 4] : 0.f;
-            const float fov[4] = {fo.x, fo.y, fo.z, fo.w};
-            const float4 a0 = ld(cf.fx, own), a2 = ld(cf.fy, own), a4 = ld(cf.fz, own);
-            const float4 a3 = hy1 ? ld(cf.fy, opp + dy) : f0, a5 = hz1 ? ld(cf.fz, opp + dz) : f0;
-            const float a0v[4] = {a0.x, a0.y, a0.z, a0.w}, a2v[4] = {a2.x, a2.y, a2.z, a2.w};
-            const float a3v[4] = {a3.x, a3.y, a3.z, a3.w}, a4v[4] = {a4.x, a4.y, a4.z, a4.w};
-            const float a5v[4] = {a5.x, a5.y, a5.z, a5.w};
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                w0[v] = a0v[v];
-                w1[v] = (v == 3 && xw1) ? 0.f : (p ? (v < 3 ? fov[v + 1] : fr) : fov[v]);
-                w2[v] = a2v[v];
-                w3[v] = a3v[v];
-                w4[v] = a4v[v];
-                w5[v] = a5v[v];
-            }
-        }
-        const float4 b4 = ld(b, own);
-        const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
-        float out[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float den = ((w0[v] + w1[v]) + (w2[v] + w3[v])) + (w4[v] + w5[v]);
-            out[v] = __fdividef(hh * bv[v], den);
-        }
-        if (active) *reinterpret_cast<float4 *>(xv + own) = make_float4(out[0], out[1], out[2], out[3]);
-        szm = szc;
-        szc = szp;
-        own += dz;
-        opp += dz;
-    }
-}
-
+// ---- row-sharing half sweep -----------------------------------------------------------------
 // Row-sharing half sweep for the s-form regular sweep (the finest level's dominant kernel).  A
 // block takes a tile of RY rows of W four-cell vectors (RY W <= kZrThreads, one vector per
 // thread) and marches ZC planes.  The other colour's x and s of the tile's rows and of the rows
@@ -427,8 +333,7 @@ __global__ void __launch_bounds__(64, 12) k_half_z0(Lay L, float h2, Coef32 cf, 
 // k_half_vec: bitwise the same results.
 constexpr int kZrThreads = 128, kZrStages = 4, kZrBlocks = 4;  // blocks per SM
 constexpr int kZrMaxSmem = 56 * 1024;                            // per block
-constexpr int kZrMinVec = 4;                                     // vectors per row
-constexpr i64 kZrFullCells = 3500000, kZrCells = 7000000;        // see run_half_zr
+constexpr i64 kZrCells = 60000000;                               // see run_half_zr
 struct ZrTile {
     int w, ry, zc;  // vectors per row, rows and planes of a tile
     int pitch;      // row stride in shared memory: whole 128 B lines, as cp.async writes them
@@ -621,202 +526,21 @@ ZrTile zr_tile(const Lay &L) {
     return T;
 }
 
-// Whether the s-form regular sweep of L goes to k_half_zr (and its launch).  Below these sizes
-// the whole level sits in L2 and k_half_vec, which loads everything at once, is as fast or faster: rows of
-// 32 vectors (every thread in use) 256 x 128 x 64 4.9 us against 5.0, 256 x 128 x 128 8.1 against 7.6, x 192 11.9 against 11.0; rows of 20 to
-// 28 vectors 160^3 8.8 against 9.5, 192^3 14.6 against 14.4, 224^3 27.7 against 22.5.
+// Whether the s-form regular sweep of L goes to k_half_zr (and its launch): tiles that use all of a block's threads, on
+// levels of 60 M cells and more, where it is the one that HBM alone bounds.  V-cycles with it and with k_half_vec: 512^3
+// 2883 against 2965 us, 512 x 512 x 256 1474 against 1508, 256 x 512 x 512 1462 against 1496, 1024 x 256 x 256 1485 against 1518;
+// 512 x 384 x 256 1136 against 1129, 256^3 411 against 404, 192^3 230 against 193; partial tiles 448^3 2058 against 2005,
+// 576 x 512 x 448 2983 against 2935.
 template <bool GHOST>
 bool run_half_zr(cudaStream_t s, const Lay &L, float h2, const float *sv, const float *b, float *x, int col) {
     const int kv = L.hx / 4;
-    if (!L.split || L.hx % 4 != 0 || kv < kZrMinVec) return false;
+    if (L.n < kZrCells) return false;
     const ZrTile T = zr_tile(L);
-    if (L.n < (T.w * T.ry == kZrThreads ? kZrFullCells : kZrCells)) return false;
+    if (T.w * T.ry != kZrThreads) return false;
     static std::atomic<unsigned long long> opted{0};
     if (!opt_in_smem((const void *)k_half_zr<GHOST>, kZrMaxSmem, opted)) return true;  // the caller checks the error
     run_kernel(k_half_zr<GHOST>, dim3((kv + T.w - 1) / T.w, (L.ny + T.ry - 1) / T.ry, (L.nz + T.zc - 1) / T.zc), kZrThreads,
                (size_t)kZrStages * T.slot * sizeof(float4), s, L, T, h2, sv, b, x, col);
-    return true;
-}
-
-// Staged z-marching half sweep for the face-form regular sweep (the levels below the finest, whose
-// coarsened faces are stored per face, and a finest level loaded from face coefficients).  A
-// thread's nine per-plane vectors -- the other colour's x in rows y -+ 1, the other colour's
-// low x faces (its cells' high x faces), its own low x, y and z faces, the other colour's low
-// y faces in row y + 1 and low z faces in plane z + 1 (its high y and z faces), its own b --
-// travel by cp.async into a ring of kZfStages planes in shared memory, one plane ahead of the
-// plane being computed, as in k_half_zr; the other colour's row y (planes z -+ 1) rolls
-// through registers, the window scalars of the warp's edge lanes are loaded one plane ahead.
-// Every thread reads back only its own copies after cp.async.wait_group (no barrier, no spin).
-// Arithmetic as k_half_vec, in the same order: bitwise the same results.
-constexpr int kZfStages = 2;
-constexpr int kZfFields = 9;  // ym, yp, fo, own fx, fy, fz, fy at y + 1, fz at z + 1, own b
-constexpr size_t kZfSmem = (size_t)kZfStages * kZfFields * 64 * sizeof(float4);
-
-template <int ZC, int MINB>
-__global__ void __launch_bounds__(64, MINB) k_half_zf(Lay L, float h2, Coef32 cf, const float *__restrict__ b,
-                                                       float *xv, int col) {
-    grid_wait();
-    extern __shared__ float4 stg[];  // [kZfStages][kZfFields][64 threads]
-    constexpr int D = kZfStages;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int hx = L.hx, kv = hx >> 2;
-    const int kvi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int yi = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool active = kvi < kv && yi < L.ny;
-    const int k0 = min(kvi, kv - 1) << 2;
-    const int y = min(yi, L.ny - 1);
-    const int z0 = (col ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * ZC, z1 = min(z0 + ZC, L.nz);
-    const int lane = threadIdx.x & 31;
-    const i64 dy = hx, dz = (i64)L.ny * hx;
-    const bool hy0 = y > 0, hy1 = y < L.ny - 1;
-    const bool kl = k0 > 0, kr = k0 + 4 < hx;
-    const i64 row0 = ((i64)z0 * L.ny + y) * hx + k0;
-    const i64 opp0 = (i64)(1 - col) * L.half + row0;
-    const i64 own0 = (i64)col * L.half + row0;
-    const float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto ld = [](const float *A, i64 off) { return *reinterpret_cast<const float4 *>(A + off); };
-    auto slot = [&](int st, int f) { return stg + (st * kZfFields + f) * 64 + tid; };
-    // plane z0 + t into stage t % D (slots whose neighbour is outside the grid are not copied
-    // and never read)
-    auto issue = [&](int t) {
-        const i64 o = opp0 + (i64)t * dz, w = own0 + (i64)t * dz;
-        const int st = t % D;
-        if (hy0) cp_async16(slot(st, 0), xv + o - dy);
-        if (hy1) {
-            cp_async16(slot(st, 1), xv + o + dy);
-            cp_async16(slot(st, 6), cf.fy + o + dy);
-        }
-        cp_async16(slot(st, 2), cf.fx + o);
-        cp_async16(slot(st, 3), cf.fx + w);
-        cp_async16(slot(st, 4), cf.fy + w);
-        cp_async16(slot(st, 5), cf.fz + w);
-        if (z0 + t < L.nz - 1) cp_async16(slot(st, 7), cf.fz + o + dz);
-        cp_async16(slot(st, 8), b + w);
-    };
-    // the window scalars beyond the warp's edge lanes (lane 0: x at k0 - 1; lane 31: x and the
-    // low x face at k0 + 4)
-    auto scalars = [&](i64 o, float &xl, float &xr, float &fr) {
-        xl = xr = fr = 0.f;
-        if (lane == 0 && kl) xl = xv[o - 1];
-        if (lane == 31 && kr) {
-            xr = xv[o + 4];
-            fr = cf.fx[o + 4];
-        }
-    };
-    // other colour, row y: planes z-1, z, z+1 (rolling)
-    float4 xzm = z0 > 0 ? ld(xv, opp0 - dz) : f0, xzc = ld(xv, opp0);
-    float4 xzp = z0 + 1 < L.nz ? ld(xv, opp0 + dz) : f0;
-#pragma unroll
-    for (int t = 0; t < D - 1; ++t) {
-        if (z0 + t < z1) issue(t);
-        cp_async_commit();  // one group per plane, empty past the chunk: the counting stays uniform
-    }
-    float cxl, cxr, cfr;
-    scalars(opp0, cxl, cxr, cfr);
-    for (int z = z0; z < z1; ++z) {
-        const int t = z - z0;
-        if (z + D - 1 < z1) issue(t + D - 1);
-        cp_async_commit();
-        const i64 opp = opp0 + (i64)t * dz, own = own0 + (i64)t * dz;
-        float nxl = 0.f, nxr = 0.f, nfr = 0.f;
-        float4 xzpp = f0;
-        if (z + 1 < z1) {
-            scalars(opp + dz, nxl, nxr, nfr);
-            if (z + 2 < L.nz) xzpp = ld(xv, opp + 2 * dz);
-        }
-        cp_async_wait<D - 1>();  // all but the D - 1 newest groups done: plane z has landed
-        const int st = t % D;
-        const bool hz1 = z < L.nz - 1;
-        const int p = (col + y + z) & 1;  // x = 2k + p
-        const bool xw1 = (p == 1 && !kr);
-        const float4 ym = hy0 ? *slot(st, 0) : f0, yp = hy1 ? *slot(st, 1) : f0;
-        const float4 fo = *slot(st, 2), a0 = *slot(st, 3), a2 = *slot(st, 4), a4 = *slot(st, 5);
-        const float4 a3 = hy1 ? *slot(st, 6) : f0, a5 = hz1 ? *slot(st, 7) : f0;
-        const float4 b4 = *slot(st, 8);
-        float fr = __shfl_down_sync(0xffffffffu, fo.x, 1);
-        if (lane == 31) fr = cfr;
-        float xl = __shfl_up_sync(0xffffffffu, xzc.w, 1), xr = __shfl_down_sync(0xffffffffu, xzc.x, 1);
-        if (lane == 0) xl = cxl;
-        if (lane == 31) xr = cxr;
-        const float fov[4] = {fo.x, fo.y, fo.z, fo.w};
-        const float a0v[4] = {a0.x, a0.y, a0.z, a0.w}, a2v[4] = {a2.x, a2.y, a2.z, a2.w};
-        const float a3v[4] = {a3.x, a3.y, a3.z, a3.w}, a4v[4] = {a4.x, a4.y, a4.z, a4.w};
-        const float a5v[4] = {a5.x, a5.y, a5.z, a5.w};
-        const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
-        const float xo[4] = {xzc.x, xzc.y, xzc.z, xzc.w};
-        const float ymv[4] = {ym.x, ym.y, ym.z, ym.w}, ypv[4] = {yp.x, yp.y, yp.z, yp.w};
-        const float zmv[4] = {xzm.x, xzm.y, xzm.z, xzm.w}, zpv[4] = {xzp.x, xzp.y, xzp.z, xzp.w};
-        float out[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float w0 = a0v[v];
-            const float w1 = (v == 3 && xw1) ? 0.f : (p ? (v < 3 ? fov[v + 1] : fr) : fov[v]);
-            const float w2 = a2v[v], w3 = a3v[v], w4 = a4v[v], w5 = a5v[v];
-            const float xm = p ? xo[v] : (v ? xo[v - 1] : xl);
-            const float xp = (v == 3 && xw1) ? 0.f : (p ? (v < 3 ? xo[v + 1] : xr) : xo[v]);
-            float num = w0 * xm;
-            num += w1 * xp;
-            num += w2 * ymv[v];
-            num += w3 * ypv[v];
-            num += w4 * zmv[v];
-            num += w5 * zpv[v];
-            const float den = ((w0 + w1) + (w2 + w3)) + (w4 + w5);
-            out[v] = __fdividef(h2 * bv[v] + num, den);
-        }
-        if (active) *reinterpret_cast<float4 *>(xv + own) = make_float4(out[0], out[1], out[2], out[3]);
-        xzm = xzc;
-        xzc = xzp;
-        xzp = xzpp;
-        cxl = nxl;
-        cxr = nxr;
-        cfr = nfr;
-    }
-    cp_async_wait<0>();  // only empty groups can remain; leave none behind
-}
-
-// rows of whole warps of vectors
-bool full_rows(const Lay &L) { return L.split && L.hx % 128 == 0; }
-
-// blocks of 64 threads over the vectors (x) and rows (y) of a level with full rows, zc planes each
-void row_grid(const Lay &L, int zc, dim3 &grid, dim3 &block) {
-    const int kv = L.hx / 4, vb = (kv % 64 == 0) ? 64 : 32, ry = 64 / vb;
-    block = dim3(vb, ry);
-    grid = dim3(kv / vb, (L.ny + ry - 1) / ry, (L.nz + zc - 1) / zc);
-}
-
-// The first half sweep from zero of a level with full rows and at least 4 M cells: k_half_z0, 16 planes per thread
-// where that still gives about 4 waves of 64-thread blocks (12 resident per SM), else 4.  False: not one of its levels.
-template <bool SFORM, bool GHOST>
-bool run_half_z0(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col) {
-    if (!full_rows(L) || L.n < 4000000) return false;
-    dim3 grid, block;
-    row_grid(L, 16, grid, block);
-    if ((i64)grid.x * grid.y * grid.z >= (i64)4 * device_sms() * 12) {
-        run_kernel(k_half_z0<SFORM, 16, GHOST>, grid, block, 0, s, L, h2, cf, b, x, col);
-    } else {
-        row_grid(L, 4, grid, block);
-        run_kernel(k_half_z0<SFORM, 4, GHOST>, grid, block, 0, s, L, h2, cf, b, x, col);
-    }
-    return true;
-}
-
-// The face form's regular sweeps, staged, on levels with full rows that give at least four waves of 4-plane
-// blocks (11 blocks x 18 KB of staging per SM): 256^3 43.6 us against 52 with k_half_vec, 384^3 145 against 169;
-// 256 x 128 x 128 has too few blocks (8.6 against 8.8), and rows that leave lanes idle are slower (288^3 103 against 73).
-bool run_half_zf(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col) {
-    if (!full_rows(L)) return false;
-    dim3 grid, block;
-    row_grid(L, 4, grid, block);
-    if ((i64)grid.x * grid.y * grid.z < (i64)4 * device_sms() * 11) return false;
-    static const bool carveout = [] {
-        // a preference only: the launch is valid either way
-        if (cudaFuncSetAttribute(k_half_zf<4, 11>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-            (void)cudaGetLastError();
-        return true;
-    }();
-    (void)carveout;
-    run_kernel(k_half_zf<4, 11>, grid, block, kZfSmem, s, L, h2, cf, b, x, col);
     return true;
 }
 
@@ -1397,12 +1121,10 @@ template <bool SFORM, bool GHOST>
 void half32_vec(cudaStream_t s, const Lay &L, float h2, const Coef32 &cf, const float *b, float *x, int col, bool from_zero) {
     const i64 work = (i64)L.ny * L.nz * (L.hx / 4);
     if (from_zero) {
-        if (!run_half_z0<SFORM, GHOST>(s, L, h2, cf, b, x, col))
-            run_kernel(k_half_vec<SFORM, true, 0, GHOST>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
+        run_kernel(k_half_vec<SFORM, true, 0, GHOST>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
         return;
     }
     if (SFORM && run_half_zr<GHOST>(s, L, h2, cf.s, b, x, col)) return;
-    if (!SFORM && !GHOST && run_half_zf(s, L, h2, cf, b, x, col)) return;
     run_kernel(k_half_vec<SFORM, false, 0, GHOST>, blocks_for(work), kThreads, 0, s, L, h2, cf, b, x, col, Upd{});
 }
 
