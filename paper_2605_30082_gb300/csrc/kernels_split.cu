@@ -48,11 +48,15 @@ struct Coef32 {
 // sum_f beta_f x_nb and sum_f beta_f at cell (x, y, z), SFORM carries a factor 2
 __device__ __forceinline__ void stencil_any(const Lay &L, const Coef32 &cf, const float *__restrict__ xv,
                                             int x, int y, int z, float &num, float &den) {
-    const i64 c = sto(L, x, y, z);
     const bool hx0 = x > 0, hx1 = x < L.nx - 1, hy0 = y > 0, hy1 = y < L.ny - 1, hz0 = z > 0, hz1 = z < L.nz - 1;
-    const i64 n0 = hx0 ? sto(L, x - 1, y, z) : c, n1 = hx1 ? sto(L, x + 1, y, z) : c;
-    const i64 n2 = hy0 ? sto(L, x, y - 1, z) : c, n3 = hy1 ? sto(L, x, y + 1, z) : c;
-    const i64 n4 = hz0 ? sto(L, x, y, z - 1) : c, n5 = hz1 ? sto(L, x, y, z + 1) : c;
+    // offsets fit 32 bits; in split storage all six neighbours are of the other colour, two of them at k + p - 1 and
+    // k + p of the row (x = 2 k + p)
+    const int row = z * L.ny + y, w = L.split ? L.hx : L.nx, c = (int)sto(L, x, y, z);
+    const int o = L.split ? (((x + y + z) & 1) ? 0 : (int)L.half) + row * w + (x >> 1) : c;
+    const int n1o = L.split ? o + (x & 1) : c + 1;
+    const int n0 = hx0 ? n1o - (L.split ? 1 : 2) : c, n1 = hx1 ? n1o : c;
+    const int n2 = hy0 ? o - w : c, n3 = hy1 ? o + w : c;
+    const int n4 = hz0 ? o - L.ny * w : c, n5 = hz1 ? o + L.ny * w : c;
     float w0, w1, w2, w3, w4, w5;
     if (cf.s) {
         const float sc = cf.s[c];
@@ -83,16 +87,12 @@ __device__ __forceinline__ void stencil_any(const Lay &L, const Coef32 &cf, cons
 // half sweep of colour `col`, one thread per cell of that colour, any layout
 __global__ void k_half_any(Lay L, float h2, Coef32 cf, const float *__restrict__ b, float *xv, int col,
                            int from_zero) {
-    grid_wait();
-    const int halfw = (L.nx + 1) >> 1;
-    const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    const i64 rows = (i64)L.ny * L.nz;
-    if (t >= rows * halfw) return;
-    const i64 row = t / halfw;
-    const int m = (int)(t - row * halfw);
-    const int y = (int)(row % L.ny), z = (int)(row / L.ny);
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = t / L.by_half;  // below 2^31
+    const int m = (int)(t - row * (unsigned)((L.nx + 1) >> 1));
+    const int z = (int)(row / L.by_ny), y = (int)(row - (unsigned)z * L.ny);
     const int x = 2 * m + ((col + y + z) & 1);
-    if (x >= L.nx) return;
+    grid_wait();
+    if (row >= (unsigned)L.ny * L.nz || x >= L.nx) return;
     float num, den;
     stencil_any(L, cf, xv, x, y, z, num, den);
     if (from_zero) num = 0.f;
@@ -977,15 +977,16 @@ __global__ void k_residual_any(Lay L, float ih2, Coef32 cf, const float *__restr
 // (exact after a black half sweep, which solves every black row)
 __global__ void k_resid_restrict_any(Lay L, Lay Lc, float ih2, Coef32 cf, const float *__restrict__ b,
                                      const float *__restrict__ xv, float *bc, int red_only) {
+    const unsigned T = blockIdx.x * blockDim.x + threadIdx.x, row = T / Lc.by_nx;
+    const int I = (int)(T - row * (unsigned)Lc.nx), K = (int)(row / Lc.by_ny), J = (int)(row - (unsigned)K * Lc.ny);
     grid_wait();
-    const i64 T = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (T >= Lc.n) return;
-    const int I = (int)(T % Lc.nx);
-    const i64 row = T / Lc.nx;
-    const int J = (int)(row % Lc.ny), K = (int)(row / Lc.ny);
     float s = 0.f;
+#pragma unroll
     for (int cc = 0; cc < 2; ++cc)
+#pragma unroll
         for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
             for (int aa = 0; aa < 2; ++aa) {
                 const int x = 2 * I + aa, y = 2 * J + bb, z = 2 * K + cc;
                 if (red_only && ((x + y + z) & 1)) continue;
@@ -996,12 +997,10 @@ __global__ void k_resid_restrict_any(Lay L, Lay Lc, float ih2, Coef32 cf, const 
 
 // x += P ec on cells of colour `only_col` (0 red, 1 black) or on all cells (-1)
 __global__ void k_prolong_any(Lay L, Lay Lc, const float *__restrict__ ec, float *xv, int kind, int only_col) {
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, row = t / L.by_nx;
+    const int x = (int)(t - row * (unsigned)L.nx), z = (int)(row / L.by_ny), y = (int)(row - (unsigned)z * L.ny);
     grid_wait();
-    const i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.n) return;
-    const int x = (int)(t % L.nx);
-    const i64 row = t / L.nx;
-    const int y = (int)(row % L.ny), z = (int)(row / L.ny);
     if (only_col >= 0 && ((x + y + z) & 1) != only_col) return;
     const int I = x >> 1, J = y >> 1, K = z >> 1;
     float v;
@@ -1112,6 +1111,8 @@ Lay make_lay(Dims d) {
     L.zlo = L.zhi = 0;
     L.by4 = make_div((unsigned)(L.hx / 4));
     L.by_ny = make_div((unsigned)L.ny);
+    L.by_nx = make_div((unsigned)L.nx);
+    L.by_half = make_div((unsigned)(L.nx + 1) / 2);
     return L;
 }
 

@@ -70,7 +70,7 @@ struct Lay {
     int hx;     // nx / 2
     i64 half;   // n / 2 (a slab: the colour stride)
     int zlo, zhi;
-    FastDiv by4, by_ny;  // by hx / 4, by ny
+    FastDiv by4, by_ny, by_nx, by_half;  // by hx / 4, ny, nx, (nx + 1) / 2
 };
 Lay make_lay(Dims d);
 
