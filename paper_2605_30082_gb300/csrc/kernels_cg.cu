@@ -92,11 +92,10 @@ __global__ void k_cg_apply32(Lay L, float ih2, Coef32c cf, const float *__restri
     double acc = 0.0;
     for (i64 t = (i64)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * per_col; t += (i64)gridDim.x * blockDim.x) {
         const int col = t >= per_col;
-        // t < n / 4 < 2^31: 32-bit divisions (64-bit ones cost several times as many instructions)
-        const unsigned tt = (unsigned)(t - col * per_col), rowu = tt / (unsigned)kv;
+        const unsigned tt = (unsigned)(t - col * per_col), rowu = tt / L.by4;  // t < n / 4 < 2^31
         const i64 row = rowu;
         const int k0 = (int)(tt - rowu * (unsigned)kv) << 2;
-        const int y = (int)(rowu % (unsigned)L.ny), z = (int)(rowu / (unsigned)L.ny);
+        const int z = (int)(rowu / L.by_ny), y = (int)(rowu - (unsigned)z * L.ny);
         const int p = (col + y + z) & 1;
         const i64 own = col * L.half + row * hx + k0;
         const i64 opp = (1 - col) * L.half + row * hx + k0;
@@ -110,18 +109,15 @@ __global__ void k_cg_apply32(Lay L, float ih2, Coef32c cf, const float *__restri
                 v[0] = v[1] = v[2] = v[3] = 0.f;
             }
         };
+        const bool edge = p ? k0 + 4 < hx : k0 > 0;
+        const int eo = p ? 4 : -1;
         // same-row window of the other colour: m[v] = O[k0+v+p-1], n[v] = O[k0+v+p]
         auto window = [&](const float *O, float (&m)[4], float (&nn)[4]) {
+            // by selection: a warp's rows have both parities
             const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
-            if (p) {
-                const float e = (k0 + 4 < hx) ? O[opp + 4] : 0.f;
-                m[0] = c4.x; m[1] = c4.y; m[2] = c4.z; m[3] = c4.w;
-                nn[0] = c4.y; nn[1] = c4.z; nn[2] = c4.w; nn[3] = e;
-            } else {
-                const float e = (k0 > 0) ? O[opp - 1] : 0.f;
-                m[0] = e; m[1] = c4.x; m[2] = c4.y; m[3] = c4.z;
-                nn[0] = c4.x; nn[1] = c4.y; nn[2] = c4.z; nn[3] = c4.w;
-            }
+            const float e = edge ? O[opp + eo] : 0.f;
+            m[0] = p ? c4.x : e; m[1] = p ? c4.y : c4.x; m[2] = p ? c4.z : c4.y; m[3] = p ? c4.w : c4.z;
+            nn[0] = m[1]; nn[1] = m[2]; nn[2] = m[3]; nn[3] = p ? e : c4.w;
         };
         float dc[4], dm[4], dp[4], d2[4], d3[4], d4[4], d5[4];
         ld4(d, own, true, dc);
@@ -191,19 +187,24 @@ __global__ void k_cg_dots32(i64 n4, const float4 *__restrict__ r, const float4 *
     block_sum_pair(a, b, partials);
 }
 
-// d = z + beta d with beta = -alpha (z . q_prev) / (r_prev . z_prev); first: d = z
+// d = z + beta d with beta = -alpha (z . q_prev) / (r_prev . z_prev); first: d = z.  One thread of a block forms
+// beta: an FP64 division is some ten instructions of 64 clocks each for a warp, and with one in every thread the
+// divisions bound this kernel and k_cg_update32 (256 x 128 x 192: 24 and 29 us, so 10 and 19)
 __global__ void k_cg_dir32(i64 n4, const float4 *__restrict__ z, float4 *dv, const double *__restrict__ sc,
                            int first, int rz_prev) {
     grid_wait();
-    const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n4) return;
-    const float4 zv = z[m];
+    __shared__ float sbeta;
+    const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x, mc = m < n4 ? m : n4 - 1;
+    const float4 zv = z[mc];
     if (first) {
-        dv[m] = zv;
+        if (m < n4) dv[m] = zv;
         return;
     }
-    const float beta = (float)(-sc[CG_ALPHA] * sc[CG_ZQ] / sc[rz_prev]);
-    float4 v = dv[m];
+    float4 v = dv[mc];
+    if (threadIdx.x == 0) sbeta = (float)(-sc[CG_ALPHA] * sc[CG_ZQ] / sc[rz_prev]);
+    __syncthreads();
+    if (m >= n4) return;
+    const float beta = sbeta;
     v.x = fmaf(beta, v.x, zv.x);
     v.y = fmaf(beta, v.y, zv.y);
     v.z = fmaf(beta, v.z, zv.z);
@@ -215,13 +216,18 @@ __global__ void k_cg_dir32(i64 n4, const float4 *__restrict__ z, float4 *dv, con
 __global__ void k_cg_update32(i64 n4, float4 *x, float4 *r, const float4 *__restrict__ dv,
                               const float4 *__restrict__ q, double *sc, int rz_cur) {
     grid_wait();
-    const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    const double alpha_d = sc[rz_cur] / sc[CG_PQ];
-    if (m == 0) sc[CG_ALPHA] = alpha_d;
+    __shared__ float salpha;
+    const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x, mc = m < n4 ? m : n4 - 1;
+    const float4 dd = dv[mc], qq = q[mc];
+    float4 xv = x[mc], rv = r[mc];
+    if (threadIdx.x == 0) {
+        const double alpha_d = sc[rz_cur] / sc[CG_PQ];
+        if (m == 0) sc[CG_ALPHA] = alpha_d;
+        salpha = (float)alpha_d;
+    }
+    __syncthreads();
     if (m >= n4) return;
-    const float alpha = (float)alpha_d;
-    const float4 dd = dv[m], qq = q[m];
-    float4 xv = x[m], rv = r[m];
+    const float alpha = salpha;
     xv.x = fmaf(alpha, dd.x, xv.x);
     xv.y = fmaf(alpha, dd.y, xv.y);
     xv.z = fmaf(alpha, dd.z, xv.z);
@@ -278,13 +284,14 @@ __global__ void k_cg_dir64(i64 n, const double *__restrict__ z, double *dv, cons
                            int first, int rz_prev) {
     grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
+    __shared__ double sbeta;
     if (first) {
-        dv[m] = z[m];
+        if (m < n) dv[m] = z[m];
         return;
     }
-    const double beta = -sc[CG_ALPHA] * sc[CG_ZQ] / sc[rz_prev];
-    dv[m] = fma(beta, dv[m], z[m]);
+    if (threadIdx.x == 0) sbeta = -sc[CG_ALPHA] * sc[CG_ZQ] / sc[rz_prev];
+    __syncthreads();
+    if (m < n) dv[m] = fma(sbeta, dv[m], z[m]);
 }
 
 // alpha = (r . z) / (d . A d); x += alpha d, r -= alpha A d; partials of |r|^2 (and of sum x)
