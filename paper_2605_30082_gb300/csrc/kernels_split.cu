@@ -564,17 +564,19 @@ __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, fl
     const unsigned Tu = (unsigned)T, crowu = Tu / L.by4;
     const int k0 = (int)(Tu - crowu * (unsigned)kv) << 2;
     const int K = (int)(crowu / Lc.by_ny), J = (int)(crowu - (unsigned)K * Lc.ny);
-    const i64 dy = hx, dz = (i64)L.ny * hx;
+    using Off = typename std::conditional<GHOST, i64, int>::type;  // as in k_half_vec
+    const Off dy = hx, dz = (Off)L.ny * hx;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int ch = 0; ch < 4; ++ch) {
         const int y = 2 * J + (ch & 1), z = 2 * K + (ch >> 1);
-        const int p = (y + z) & 1;  // red cells of this row sit at x = 2k + p
-        const i64 row = (i64)z * L.ny + y;
-        const i64 own = row * hx + k0;               // red half
-        const i64 opp = L.half + row * hx + k0;      // black half
-        const bool hy0 = y > 0, hy1 = y < L.ny - 1;
-        const bool hz0 = z > 0 || (GHOST && L.zlo), hz1 = z < L.nz - 1 || (GHOST && L.zhi);
+        const int p = (ch & 1) ^ (ch >> 1);  // red cells of this row sit at x = 2k + p
+        const Off row = (Off)z * L.ny + y;
+        const Off own = row * hx + k0;                // red half
+        const Off opp = (Off)L.half + row * hx + k0;  // black half
+        // half of the neighbours are siblings
+        const bool hy0 = (ch & 1) || y > 0, hy1 = !(ch & 1) || y < L.ny - 1;
+        const bool hz0 = (ch >> 1) || z > 0 || (GHOST && L.zlo), hz1 = !(ch >> 1) || z < L.nz - 1 || (GHOST && L.zhi);
         const bool xw0 = (p == 0 && k0 == 0), xw1 = (p == 1 && k0 + 4 == hx);
         auto window = [&](const float *O, float (&m)[4], float (&q)[4]) {
             const float4 c4 = *reinterpret_cast<const float4 *>(O + opp);
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(kRrThreads, 12) k_rr_red_vec(Lay L, Lay Lc, fl
                 q[0] = c4.x; q[1] = c4.y; q[2] = c4.z; q[3] = c4.w;
             }
         };
-        auto ld4 = [&](const float *A, i64 off, bool ok, float (&v)[4]) {
+        auto ld4 = [&](const float *A, Off off, bool ok, float (&v)[4]) {
             if (ok) {
                 const float4 c4 = *reinterpret_cast<const float4 *>(A + off);
                 v[0] = c4.x; v[1] = c4.y; v[2] = c4.z; v[3] = c4.w;
