@@ -66,10 +66,10 @@ NCU_DRAM_BYTES_PER_CELL = {"k_half_zr": 10.03, "k_fine_resid_pair": 54.3,
 GATE_ERR = 1e-9
 GATE_RTOL = 1e-11
 # FP64 flops per grid cell of the plain FP64 V-cycle's finest-level kernels (a fused multiply-
-# add counts 2): half sweep 7 FMA + 1 multiply per updated cell (half the cells); red residual +
-# restriction 7 FMA + 1 multiply + 1 add per red child; red prolongation 8 FMA per red cell;
+# add counts 2): half sweep 6 FMA + 1 add + 1 multiply per updated cell (half the cells); red residual +
+# restriction 7 FMA + 1 add per red child; red prolongation 18 FMA per 4 red cells;
 # outer residual 7 FMA per cell
-FP64_FLOPS_PER_CELL = {"smooth": 7.5, "resid_restrict": 8.0, "prolong": 8.0, "fine_residual": 14.0}
+FP64_FLOPS_PER_CELL = {"smooth": 7.0, "resid_restrict": 7.5, "prolong": 4.5, "fine_residual": 14.0}
 
 
 # algorithmic bytes per fine grid cell of one launch of each profiled class (the smoother's
