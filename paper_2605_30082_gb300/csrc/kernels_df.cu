@@ -39,21 +39,23 @@ __device__ __forceinline__ void df_fma(float &ah, float &al, float xh, float xl,
 
 __device__ __forceinline__ float df_value(float h, float l) { return h + l; }
 
-__global__ void k_split(i64 n, const double *__restrict__ src, float2 *dst) {
+// two numbers per thread, 16 bytes each way (n is even: the double-float mode takes even nx; a solution is on a
+// 16-byte boundary, the rest in the handle's own memory).  192^3: 29 us one per thread, 22 so
+__global__ void k_split(i64 n2, const double2 *__restrict__ src, float4 *dst) {
     grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    const double v = src[m];
-    const float hi = d2f_rn(v);
-    dst[m] = make_float2(hi, d2f_rn(v - f2d_exact(hi)));
+    if (m >= n2) return;
+    const double2 v = src[m];
+    const float h0 = d2f_rn(v.x), h1 = d2f_rn(v.y);
+    dst[m] = make_float4(h0, d2f_rn(v.x - f2d_exact(h0)), h1, d2f_rn(v.y - f2d_exact(h1)));
 }
 
-__global__ void k_join(i64 n, const float2 *__restrict__ src, double *dst) {
+__global__ void k_join(i64 n2, const float4 *__restrict__ src, double2 *dst) {
     grid_wait();
     const i64 m = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    const float2 v = src[m];
-    dst[m] = f2d_exact(v.x) + f2d_exact(v.y);
+    if (m >= n2) return;
+    const float4 v = src[m];
+    dst[m] = make_double2(f2d_exact(v.x) + f2d_exact(v.y), f2d_exact(v.z) + f2d_exact(v.w));
 }
 
 // h^2 r = h^2 b + sum_f beta_f p_nb - d p_c in double-float (b already scaled by h^2);
@@ -380,12 +382,12 @@ __global__ void k_update_df(Dims d, Lay L, float2 *p, const float *__restrict__ 
 
 void launch_split(cudaStream_t s, i64 n, const double *src, float2 *dst) {
     count_launch();
-    run_kernel(k_split, blocks_for(n), kThreads, 0, s, n, src, dst);
+    run_kernel(k_split, blocks_for(n / 2), kThreads, 0, s, n / 2, reinterpret_cast<const double2 *>(src), reinterpret_cast<float4 *>(dst));
 }
 
 void launch_join(cudaStream_t s, i64 n, const float2 *src, double *dst) {
     count_launch();
-    run_kernel(k_join, blocks_for(n), kThreads, 0, s, n, src, dst);
+    run_kernel(k_join, blocks_for(n / 2), kThreads, 0, s, n / 2, reinterpret_cast<const float4 *>(src), reinterpret_cast<double2 *>(dst));
 }
 
 void launch_resid_df(cudaStream_t s, Dims d, Lay L, const float2 *fx, const float2 *fy, const float2 *fz,

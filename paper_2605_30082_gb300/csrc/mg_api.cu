@@ -468,7 +468,9 @@ int finish_operator(mg_handle *h) {
     bool mixed = h->o.precision != MG_FP64;
     for (int l = 0; l < h->nlev; ++l) {
         Level &L = h->lv[l];
-        mg::launch_invdiag(s, L.d, L.fx64, L.fy64, L.fz64, L.invd64, L.lay.split ? L.lay.half : 0, L.d64);
+        // the double-float residual of a density takes neither the diagonal nor the faces
+        double *diag = l == 0 && h->o.precision == MG_MIXED_DF && h->sform0 ? nullptr : L.d64;
+        mg::launch_invdiag(s, L.d, L.fx64, L.fy64, L.fz64, L.invd64, L.lay.split ? L.lay.half : 0, diag);
         // coarse levels have theirs from launch_coarsen; the s-form finest level has no FP32 faces
         if (mixed && l == 0 && !h->sform0) {
             mg::launch_pack64to32(s, L.lay, L.fx64, L.fx32);
@@ -476,7 +478,7 @@ int finish_operator(mg_handle *h) {
             mg::launch_pack64to32(s, L.lay, L.fz64, L.fz32);
         }
     }
-    if (h->o.precision == MG_MIXED_DF) {
+    if (h->o.precision == MG_MIXED_DF && !h->sform0) {
         Level &F = h->lv[0];
         mg::launch_split(s, F.d.n, F.fx64, F.fx2);
         mg::launch_split(s, F.d.n, F.fy64, F.fy2);

@@ -47,3 +47,19 @@ def test_density_set_up_does_not_depend_on_alignment(dims, prec):
         s.set_density(r)
         p.append(s.solve(b))
     assert torch.equal(p[0], p[1])
+
+
+def test_double_float_operator_from_density_then_from_faces():
+    """The pairs of the faces and of the diagonal are formed only for an operator from faces: also after one from a density."""
+    dims = (24, 12, 20)
+    b = dev(np.random.default_rng(84).standard_normal(dims[::-1]))
+    faces = [dev(f) for f in O.faces_from_density(random_rho(dims, 85))]
+    p = []
+    for first in (True, False):
+        s = Solver(dims, h=1.0 / 64, precision="mixed_df", coarsest=4, rtol=1e-8)
+        if first:
+            s.set_density(dev(random_rho(dims, 86)))
+            s.solve(b)
+        s.set_face_coeffs(*faces)
+        p.append(s.solve(b))
+    assert torch.equal(p[0], p[1])
