@@ -38,8 +38,8 @@
 // Arithmetic.  Per cell as in the level kernels (kernels_split.cu: k_half_vec, k_rr_red_vec or, where nx / 2
 // is no multiple of 4, k_resid_restrict_any, k_prolong_red8 where the coarse nx is a multiple of 8, else
 // k_prolong_red_vec; FP64:
-// k_rbgs_half, k_rr_red_diag64, k_prolong_col; the coarse product as k_coarse_matvec), in the
-// same order.
+// k_rbgs_half, k_rr_red_diag64, k_prolong_col, from which k_prolong_red64 differs by roundings; the coarse product as
+// k_coarse_matvec), in the same order.
 #include <cooperative_groups.h>
 
 #include <type_traits>
