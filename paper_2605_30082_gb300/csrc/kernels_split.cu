@@ -54,9 +54,12 @@ __device__ __forceinline__ void stencil_any(const Lay &L, const Coef32 &cf, cons
     const int row = z * L.ny + y, w = L.split ? L.hx : L.nx, c = (int)sto(L, x, y, z);
     const int o = L.split ? (((x + y + z) & 1) ? 0 : (int)L.half) + row * w + (x >> 1) : c;
     const int n1o = L.split ? o + (x & 1) : c + 1;
-    const int n0 = hx0 ? n1o - (L.split ? 1 : 2) : c, n1 = hx1 ? n1o : c;
-    const int n2 = hy0 ? o - w : c, n3 = hy1 ? o + w : c;
-    const int n4 = hz0 ? o - L.ny * w : c, n5 = hz1 ? o + L.ny * w : c;
+    // beyond a wall, with weight 0: o, in split storage a cell of the other colour.  Not the cell itself, which a sweep
+    // from zero is the first to write: 0 times a NaN left there by a solve that diverged, or by the memory's last owner,
+    // would go into this solve and every later one
+    const int n0 = hx0 ? n1o - (L.split ? 1 : 2) : o, n1 = hx1 ? n1o : o;
+    const int n2 = hy0 ? o - w : o, n3 = hy1 ? o + w : o;
+    const int n4 = hz0 ? o - L.ny * w : o, n5 = hz1 ? o + L.ny * w : o;
     float w0, w1, w2, w3, w4, w5;
     if (cf.s) {
         const float sc = cf.s[c];
