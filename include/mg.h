@@ -333,8 +333,14 @@ long long mg_kernel_launches(void);
  *   MG_INJECT_DIVERGE     the next outer residual norm the solve reads back (after its first
  *                         V-cycle or outer iteration) is replaced by infinity on the host: the
  *                         solve returns MG_ERR_DIVERGED.
+ *   MG_INJECT_TAIL_WAIT   the next launch of the coarse levels' cluster (hierarchies of at least
+ *                         three levels; pre, post >= 1; trilinear prolongation): its first CTA
+ *                         expects four bytes more of its neighbours' cells than they send, so
+ *                         that its bounded wait runs out (about a second) and then its
+ *                         neighbours'; the cluster sets bit 8 of the device error word and
+ *                         leaves NaN, and the solve returns MG_ERR_CUDA and clears the word.
  * Each fault fires once.  MG_ERR_ARG for unknown bits. */
-enum { MG_INJECT_FUSED_WAIT = 1, MG_INJECT_DIVERGE = 2 };
+enum { MG_INJECT_FUSED_WAIT = 1, MG_INJECT_DIVERGE = 2, MG_INJECT_TAIL_WAIT = 4 };
 int mg_debug_inject(mg_handle *h, int faults);
 
 /* FP64 fused multiply-add rate of the current device, for the roofline of the FP64

@@ -24,7 +24,7 @@ MG_METHOD_VCYCLE, MG_METHOD_FCG = 0, 1
 MG_F64, MG_F32 = 0, 1
 MG_MAX_LEVELS, MG_MAX_COARSE, MG_HIST_LEN = 24, 1024, 256
 MG_NOALLOC_MAX_CELLS = 512
-MG_INJECT_FUSED_WAIT, MG_INJECT_DIVERGE = 1, 2
+MG_INJECT_FUSED_WAIT, MG_INJECT_DIVERGE, MG_INJECT_TAIL_WAIT = 1, 2, 4
 (MG_PROF_SMOOTH, MG_PROF_RESID_RESTRICT, MG_PROF_PROLONG, MG_PROF_COARSE,
  MG_PROF_FINE_RESIDUAL, MG_PROF_UPDATE, MG_PROF_ADJOINT_GRAD, MG_PROF_PROJECT,
  MG_PROF_DENSITY_GRAD, MG_PROF_COARSE_LEVELS, MG_PROF_SETUP, MG_PROF_RHS, MG_PROF_DENSITY,

@@ -404,6 +404,11 @@ __global__ void __launch_bounds__(kReduceThreads, 5)
     fine_resid_pair<true, false, LAST, true>(d, L, h2, fx, fy, fz, dg, b, p, r32, s32, partials, ro);
 }
 
+__global__ void k_add_u32(unsigned *p, int v) {
+    grid_wait();
+    *p += (unsigned)v;
+}
+
 // n4 words, the first 4 nv of them as 16-byte stores
 __global__ void k_zero(float *p, i64 nv, i64 n4) {
     const i64 t0 = (i64)blockIdx.x * blockDim.x + threadIdx.x, nt = (i64)gridDim.x * blockDim.x;
@@ -933,6 +938,11 @@ void launch_readback(cudaStream_t s, const double *src, double *dst_mapped, int 
 void launch_readback_u32(cudaStream_t s, const unsigned *src, unsigned *dst_mapped) {
     count_launch();
     run_kernel(k_readback, 1, 32, 0, s, nullptr, nullptr, 0, src, dst_mapped);
+}
+
+void launch_add_u32(cudaStream_t s, unsigned *p, int v) {
+    count_launch();
+    run_kernel(k_add_u32, 1, 1, 0, s, p, v);
 }
 
 void launch_zero(cudaStream_t s, void *p, size_t bytes) {

@@ -29,7 +29,7 @@
 // an mbarrier of the receiver; the receiver knows how many will come.  Stores and a barrier of the
 // cluster instead cost 830 clocks per exchange between 16 CTAs of 512 threads, this 465, and all CTAs then wait for the
 // slowest (64^3 step 1561 -> 1500 us with the shared-memory copies of the parameters and addresses below).  Before a
-// level reads other CTAs' x on the way up the barrier stays.
+// level reads other CTAs' x on the way up the barrier stays, and one at the end, behind a CTA's last remote store.
 //
 // These contexts are laid out in memory once per
 // operator (k_tail_prepare), one image per CTA and level in the order of its shared memory, and
@@ -98,8 +98,9 @@ struct Cell {
     unsigned g0, g1, m0, m1;
 };
 
-// bound on the polls of one wait for ghosts (each suspends the thread for up to some microseconds)
-constexpr int kTailPolls = 1 << 16;
+// bound on one wait for other CTAs' cells, about a second at the top clock, and how long a CTA that gave up stays
+// after its cluster's last remote store has been issued, far more than one takes to arrive (330 clocks)
+constexpr long long kTailWaitCycles = 1ll << 31, kTailLingerCycles = 1ll << 17;
 
 template <typename T>
 struct Tail {
@@ -254,26 +255,37 @@ struct Tail {
         if (send && q.g1) st_async(q.g1, v, q.m1);
     }
 
-    // until `bytes` have come in for the mbarrier m; its bytes may come before this.  The poll is bounded: past it
-    // the run goes on without waiting and leaves NaN and an error flag.
-    __device__ __forceinline__ void expect(unsigned m, unsigned bytes) const {
-        if (tid == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(m), "r"(bytes) : "memory");
+    // until `bytes` have come in for the mbarrier m; its bytes may come before this.  The wait is bounded: a thread
+    // whose wait runs out is lost.  It then neither waits nor stores into other CTAs any more, so that no mbarrier
+    // gets bytes of a later phase or a second arrival in one phase, and its neighbours' waits run out in turn;
+    // it takes part in every barrier up to the end, and its CTA leaves NaN and an error flag.
+    __device__ __forceinline__ void expect(unsigned m, unsigned bytes, bool lost) const {
+        if (tid == 0 && !lost)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(m), "r"(bytes) : "memory");
+    }
+    __device__ __forceinline__ static bool arrived(unsigned m, unsigned parity) {
+        unsigned done;
+        asm volatile(
+            "{.reg .pred P; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2; selp.u32 %0, 1, 0, P;}"
+            : "=r"(done)
+            : "r"(m), "r"(parity)
+            : "memory");
+        return done != 0;
     }
     __device__ __forceinline__ void wait(unsigned m, unsigned parity, bool &lost) const {
-        unsigned done = 0;
-        for (int it = 0; it < kTailPolls && !done && !lost; ++it)
-            asm volatile(
-                "{.reg .pred P; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2; selp.u32 %0, 1, 0, P;}"
-                : "=r"(done)
-                : "r"(m), "r"(parity)
-                : "memory");
-        lost = lost || !done;
+        if (lost || arrived(m, parity)) return;
+        const long long t0 = clock64();
+        while (!arrived(m, parity))
+            if (clock64() - t0 > kTailWaitCycles) {
+                lost = true;
+                return;
+            }
     }
     // after the cells of colour col have been put: until this CTA's are visible to its threads and the ghosts'
     // have arrived.  A neighbour sends the next values of a ghost only once it has had every cell of
     // this CTA that reads the present ones, so nothing is overwritten early.
     __device__ __forceinline__ void exchange(int l, int col, unsigned &parity, bool &lost) const {
-        expect(bar_x(l, col), ghost_bytes(lv[l]));
+        expect(bar_x(l, col), ghost_bytes(lv[l]), lost);
         __syncthreads();
         wait(bar_x(l, col), parity >> (2 * l + col) & 1u, lost);
         parity ^= 1u << (2 * l + col);
@@ -302,7 +314,7 @@ struct Tail {
     // mean of the children's residuals (black ones 0 after a black half sweep) into the next
     // level's b: its owner's shared memory, every CTA's copy for the coarse solve, or memory.  The four
     // red children of a coarse cell are four neighbouring lanes.
-    __device__ void restrict_red(int l, const TailLevel *C, bool coarse_mem, const Cell<T> (&q)[kCells]) const {
+    __device__ void restrict_red(int l, const TailLevel *C, bool coarse_mem, const Cell<T> (&q)[kCells], bool lost) const {
         const TailLevel &L = lv[l];
         const T *X = x(L);
         const int cnx = L.nx >> 1, cny = L.ny >> 1;
@@ -341,11 +353,11 @@ struct Tail {
             const int J = jk(L)[lq] & 0xffff, K = jk(L)[lq] >> 16;
             if (C) {
                 const unsigned pl = crow(L)[lq * 10 + 9];
-                st_async(at(pl) + (unsigned)((((k + J + K) & 1) * C->nit + (k >> 1) * 4) * sizeof(T)), bc,
+                if (!lost) st_async(at(pl) + (unsigned)((((k + J + K) & 1) * C->nit + (k >> 1) * 4) * sizeof(T)), bc,
                          there(bar_b(l + 1), (int)(pl >> 24)));
             } else if (coarse_mem) {
                 reinterpret_cast<T *>(a.bc)[coarse_idx(k, J, K, cnx, cny)] = bc;
-            } else {
+            } else if (!lost) {
                 const unsigned r0 = saddr(rc() + (K * cny + J) * cnx + k);
                 for (int t = ch; t < ncta; t += 4) st_async(there(r0, t), (double)bc, there(bar_r(), t));
             }
@@ -353,7 +365,7 @@ struct Tail {
     }
 
     // e = A^+ r on the coarsest level, every CTA receiving the whole e
-    __device__ void coarse_solve() const {
+    __device__ void coarse_solve(bool lost) const {
         const int lane = tid & 31, warp = tid >> 5, n = a.nc;
         const double *r = rc();
         // two rows per warp: lanes 0-15 end up with the first row's sum, 16-31 with the second's, each
@@ -374,7 +386,7 @@ struct Tail {
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             const double t0 = __shfl_sync(0xffffffffu, s, 0), t1 = __shfl_sync(0xffffffffu, s, 16);
-            if (lane < ncta) {
+            if (lane < ncta && !lost) {
                 const unsigned e0 = there(saddr(ec() + row), lane), m = there(bar_e(), lane);
                 st_async(e0, (T)t0, m);
                 if (two) st_async(e0 + (unsigned)(stride * sizeof(T)), (T)t1, m);
@@ -419,7 +431,7 @@ struct Tail {
         }
     }
     // x += P e on the red cells q, e the next level's x
-    __device__ void prolong_red(const TailLevel &L, const TailLevel *C, const Cell<T> (&q)[kCells]) const {
+    __device__ void prolong_red(const TailLevel &L, const TailLevel *C, const Cell<T> (&q)[kCells], bool lost) const {
         const int cnx = L.nx >> 1, cny = L.ny >> 1, cnz = L.nz >> 1;
         if (C) {
             gather(L, *C);
@@ -473,7 +485,7 @@ struct Tail {
                 for (int u = 2; u < 8; ++u) r = fma(w[u & 1] * w[(u >> 1) & 1] * w[u >> 2], c[u], r);
                 v += r;
             }
-            put(X, q[m], v, true);
+            put(X, q[m], v, !lost);
         }
     }
 };
@@ -637,6 +649,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
         t.restore(l, up ? 1 : 0, first);
         t.restore(l, up ? 0 : 1, second);
     };
+    // the last of this thread's remote accesses is over: no CTA leaves the kernel before all threads of the cluster have
+    // come this far, whether or not their waits ran out (what was sent before may still be under way)
+    auto leave = [] { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); };
     restore(v0);
     cl.barrier_wait();
 #pragma unroll 1
@@ -649,44 +664,46 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
         t.restore_b(L, up ? 0 : 1, second);
         const int c0 = up ? 1 : 0;
         if (up) {
-            t.prolong_red(L, C, second);
-            // the last remote reads are over here: no CTA leaves before the others have come this far
-            if (v + 1 == v1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+            t.prolong_red(L, C, second, lost);
             t.exchange(l, 0, parity, lost);
         }
         T *X = t.x(L);
         const T h2 = (T)L.h2;
 #pragma unroll 1
         for (int sw = up ? a.post : a.pre;;) {
-            t.half(X, h2, first, true);
+            t.half(X, h2, first, !lost);
             t.exchange(l, c0, parity, lost);
             --sw;
-            t.half(X, h2, second, !up || sw > 0);  // nothing reads the ghosts of an ascent's last half sweep
+            if (up && sw == 0 && v + 1 == v1) leave();
+            t.half(X, h2, second, !lost && (!up || sw > 0));  // nothing reads the ghosts of an ascent's last half sweep
             if (sw == 0) break;
             t.exchange(l, 1 - c0, parity, lost);
         }
         if (!up) {
             t.exchange(l, 1 - c0, parity, lost);
-            t.restrict_red(l, C, mode == kTailDown, first);
+            if (mode == kTailDown && v + 1 == v1) leave();
+            t.restrict_red(l, C, mode == kTailDown, first, lost);
         }
         // the next level's contexts come in meanwhile.  On the way down a CTA waits for what it
         // reads; on the way up the next level reads other CTAs' x
         if (up && v + 1 < v1) cl.barrier_arrive();
         if (v + 1 < v1) restore(v + 1);
-        if (up) {
+        if (up || v + 1 == v1) {
             cl.barrier_wait();
         } else if (C) {
-            t.expect(t.bar_b(l + 1), t.cell_bytes(*C));
+            t.expect(t.bar_b(l + 1), t.cell_bytes(*C), lost);
             t.wait(t.bar_b(l + 1), 0, lost);
-        } else if (mode == kTailAll) {
-            t.expect(t.bar_r(), (unsigned)(a.nc * sizeof(double)));
+        } else {
+            t.expect(t.bar_r(), (unsigned)(a.nc * sizeof(double)), lost);
             t.wait(t.bar_r(), 0, lost);
-            t.coarse_solve();
-            t.expect(t.bar_e(), (unsigned)(a.nc * sizeof(T)));
+            t.coarse_solve(lost);
+            t.expect(t.bar_e(), (unsigned)(a.nc * sizeof(T)), lost);
             t.wait(t.bar_e(), 0, lost);
         }
     }
     if (__syncthreads_or(lost)) {  // the level's x without a number fails the solve
+        // what other CTAs had sent this one, which a CTA that was not lost has waited for, arrives first
+        for (const long long t0 = clock64(); clock64() - t0 < kTailLingerCycles;) {}
         if (t.tid == 0) atomicOr(a.err, 8u);
         for (int i = t.tid; i < (lv[0].off_b - lv[0].off_x) / (int)sizeof(T); i += kTailThreads) t.x(lv[0])[i] = (T)NAN;
         __syncthreads();
@@ -794,6 +811,11 @@ void launch_tail_prepare(cudaStream_t s, const TailArgs &a, bool fp64) {
     const dim3 grd(a.ncta, a.nl);
     if (fp64) run_kernel(k_tail_prepare<double>, grd, 256, 0, s, a);
     else run_kernel(k_tail_prepare<float>, grd, 256, 0, s, a);
+}
+
+unsigned *tail_ghost_bytes(const TailArgs &a) {
+    const TailLevel &L = a.lv[0];
+    return reinterpret_cast<unsigned *>(reinterpret_cast<char *>(a.img) + L.img + (L.off_q - L.off_c) + 4 * (i64)L.q4 * 11);
 }
 
 void launch_tail(cudaStream_t s, const TailArgs &a, bool fp64, int mode) {

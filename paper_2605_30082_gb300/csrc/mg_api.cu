@@ -208,17 +208,28 @@ cudaStream_t swap_handle_stream(mg_handle *h, cudaStream_t s) {
 namespace {
 
 // ---- the coarse levels in one cluster (kernels_tail.cu) ----------------------------------
+void launch_tail(mg_handle *h, int mode) {
+    const bool f64 = h->o.precision == MG_FP64;
+    const bool inject = (h->inject & MG_INJECT_TAIL_WAIT) != 0 && !mg::stream_capturing(h->s);
+    if (inject) {  // a test's fault: bytes that nobody sends
+        h->inject &= ~MG_INJECT_TAIL_WAIT;
+        mg::launch_add_u32(h->s, mg::tail_ghost_bytes(h->tail), 4);
+        cudaStreamSynchronize(h->s);  // the cluster reads its image ahead of its wait for the kernel before it
+    }
+    mg::launch_tail(h->s, h->tail, f64, mode);
+    if (inject) mg::launch_add_u32(h->s, mg::tail_ghost_bytes(h->tail), -4);
+}
 void run_tail(mg_handle *h) {
     const bool f64 = h->o.precision == MG_FP64;
     if (!h->tail_split) {
-        mg::launch_tail(h->s, h->tail, f64, mg::kTailAll);
+        launch_tail(h, mg::kTailAll);
         return;
     }
     Level &C = h->lv[h->nlev - 1];
-    mg::launch_tail(h->s, h->tail, f64, mg::kTailDown);
+    launch_tail(h, mg::kTailDown);
     if (f64) mg::launch_coarse_matvec<double>(h->s, h->nc, h->pinv, C.b64, C.x64);
     else mg::launch_coarse_matvec32(h->s, C.lay, h->pinv, C.b32, C.x32);
-    mg::launch_tail(h->s, h->tail, f64, mg::kTailUp);
+    launch_tail(h, mg::kTailUp);
 }
 
 // ---- FP64 V-cycle: in-place per-colour half sweeps, standalone transfers --------------
@@ -1315,7 +1326,7 @@ int mg_profile_read(mg_handle *h, int cls, long long *launches, double *ms) {
 long long mg_kernel_launches(void) { return (long long)mg::launches_total(); }
 
 int mg_debug_inject(mg_handle *h, int faults) {
-    if (!h || (faults & ~(MG_INJECT_FUSED_WAIT | MG_INJECT_DIVERGE))) return MG_ERR_ARG;
+    if (!h || (faults & ~(MG_INJECT_FUSED_WAIT | MG_INJECT_DIVERGE | MG_INJECT_TAIL_WAIT))) return MG_ERR_ARG;
     h->inject = faults;
     return MG_OK;
 }

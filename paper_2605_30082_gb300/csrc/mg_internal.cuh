@@ -440,6 +440,8 @@ void launch_tail_prepare(cudaStream_t s, const TailArgs &a, bool fp64);
 // one V-cycle of those levels from x = 0 on lv[0].b into lv[0].x (mode kTailAll), or its descent
 // or ascent alone.  pre, post >= 1, trilinear prolongation, every level's nx, ny, nz even.
 void launch_tail(cudaStream_t s, const TailArgs &a, bool fp64, int mode);
+// where the first CTA's image keeps the bytes it expects of its neighbours per colour of the first level
+unsigned *tail_ghost_bytes(const TailArgs &a);
 
 // ---- reductions, fine-level FP64 passes, adjoint -----------------------------------
 // partials: reduce_blocks(n) x 2 doubles; out: 2 doubles (deterministic order)
@@ -449,6 +451,8 @@ void launch_tail(cudaStream_t s, const TailArgs &a, bool fp64, int mode);
 // streams run on the copy engines
 void launch_readback(cudaStream_t s, const double *src, double *dst_mapped, int n);
 void launch_readback_u32(cudaStream_t s, const unsigned *src, unsigned *dst_mapped);
+// *p += v, one thread (test faults)
+void launch_add_u32(cudaStream_t s, unsigned *p, int v);
 // out[0] = sum x, out[1] = sum x^2 (0 unless `squares`)
 template <typename T>
 void launch_sum_sumsq(cudaStream_t s, i64 n, const T *x, double *partials, ReduceOut ro, bool squares);
