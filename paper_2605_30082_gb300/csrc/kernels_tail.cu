@@ -38,8 +38,8 @@
 // Arithmetic.  Per cell as in the level kernels (kernels_split.cu: k_half_vec, k_rr_red_vec or, where nx / 2
 // is no multiple of 4, k_resid_restrict_any, k_prolong_red8 where the coarse nx is a multiple of 8, else
 // k_prolong_red_vec; FP64:
-// k_rbgs_half, k_rr_red_diag64, k_prolong_col, from which k_prolong_red64 differs by roundings; the coarse product as
-// k_coarse_matvec), in the same order.
+// k_rbgs_half, k_rr_red_diag64, k_prolong_red64; the coarse product as k_coarse_matvec), in the same order, so that a
+// cycle is bitwise the one launched level by level.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -461,7 +461,14 @@ struct Tail {
             // c[4 kk + 2 jj + ii]: own (0) or neighbour (1) along z, y, x
             const T c[8] = {o[0], o[si], o[sj], o[sj + si], o[sk], o[sk + si], o[sk + sj], o[sk + sj + si]};
             T v = X[q[m].own];
-            if (!f64 && cnx % 8 == 0) {
+            if constexpr (f64) {
+                // as k_prolong_red64: y, then z, then x, weights 3 and 1, 1/64 at the end
+                T R[2];
+#pragma unroll
+                for (int ii = 0; ii < 2; ++ii)
+                    R[ii] = fma(T(3), fma(T(3), c[ii], c[2 + ii]), fma(T(3), c[4 + ii], c[6 + ii]));
+                v = fma(fma(T(3), R[0], R[1]), T(0.015625), v);
+            } else if (cnx % 8 == 0) {
                 // separable: y and z first, rows in the order J - 1, J, J + 1 and then K - 1, K, K + 1
                 T R[2];
 #pragma unroll
