@@ -480,9 +480,9 @@ int cycle(mg_dd *dd) {
 }
 
 // per slab, by the whole grid's fused residual kernel over the slab's own planes (its ghost
-// planes as neighbours): sum of (h^2 r)^2 and sum of x; one read-back for all slabs, added in
-// slab order (the all-reduce of the two scalars a rank would exchange)
-int slab_residual_norms(mg_dd *dd, double *rn2_h4, double *sp) {
+// planes as neighbours): sum of (h^2 r)^2; one read-back for all slabs, added in slab order (the
+// all-reduce of the scalar a rank would exchange)
+int slab_residual_norms(mg_dd *dd, double *rn2_h4) {
     const int P = dd->P;
     const double h2 = dd->o.h * dd->o.h;
     for (int r = 0; r < P; ++r) {
@@ -493,13 +493,9 @@ int slab_residual_norms(mg_dd *dd, double *rn2_h4, double *sp) {
     std::vector<double> h(2 * (size_t)P);
     DD_CUDA(dd, cudaMemcpyAsync(h.data(), dd->red, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, dd->s));
     DD_CUDA(dd, cudaStreamSynchronize(dd->s));
-    double q = 0.0, x = 0.0;
-    for (int r = 0; r < P; ++r) {
-        q += h[2 * r];
-        x += h[2 * r + 1];
-    }
+    double q = 0.0;
+    for (int r = 0; r < P; ++r) q += h[2 * r];
     *rn2_h4 = q;
-    *sp = x;
     return MG_OK;
 }
 
@@ -1041,11 +1037,9 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     while (status == MG_ERR_NOT_CONVERGED && cycles < dd->o.max_cycles) {
         rc = cycle(dd);
         if (rc) return rc;
-        double rn2, sp;
-        rc = slab_residual_norms(dd, &rn2, &sp);
+        double rn2;
+        rc = slab_residual_norms(dd, &rn2);
         if (rc) return rc;
-        // zero mean, ghosts included (they hold the neighbours' planes, shifted alike)
-        for (Slab &S : dd->lv[0]) mg::launch_add_const(s, S.d.n + 2 * S.d.nxy, S.xe, -sp / n);
         rr = std::sqrt(rn2) * ih2 / nb;
         ++cycles;
         if (hn < MG_HIST_LEN) hist[hn++] = rr;
@@ -1055,7 +1049,7 @@ int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *st) {
         }
         if (rr <= dd->o.rtol) status = MG_OK;
     }
-    // exact zero-mean gauge at exit (the per-cycle shifts use the residual kernel's FP32 sum of x)
+    // zero mean at exit only, as in the whole-grid FP64 solve: a constant in x does not change a cycle
     if (nb > 0.0) {
         double sx;
         rc = slab_sum_x(dd, &sx);
