@@ -415,6 +415,10 @@ int mg_dd_vcycle(mg_dd *dd, const double *b, double *x);
 /* As mg_solve in the solver's precision (MG_FP64 or MG_MIXED): zero-mean p with
  * A p = b - mean(b) to opts.rtol, from p = 0. */
 int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *stats);
+/* Test hook: mg_debug_inject on the whole-grid handle of the levels from the switch level down;
+ * MG_INJECT_TAIL_WAIT hits the next cycle that is launched, not replayed as a graph (mixed: the
+ * last of an outer iteration). */
+int mg_dd_debug_inject(mg_dd *dd, int faults);
 
 /* ---- allocation-free entry point ----------------------------------------------------
  * The paper has no counterpart to this call.  It exists for callers that cannot

@@ -107,6 +107,7 @@ SIGNATURES = {
     "mg_dd_set_density": (_i, [_v, _v]),
     "mg_dd_vcycle": (_i, [_v, _v, _v]),
     "mg_dd_solve": (_i, [_v, _v, _v, C.POINTER(mg_stats)]),
+    "mg_dd_debug_inject": (_i, [_v, _i]),
 }
 
 
@@ -446,6 +447,11 @@ def mg_dd_set_density(dd, rho, dims):
 def mg_dd_vcycle(dd, b, x, dims):
     cs = cell_shape(dims)
     return lib().mg_dd_vcycle(dd, _dev(b, shape=cs, name="b"), _dev(x, shape=cs, name="x"))
+
+
+def mg_dd_debug_inject(dd, faults):
+    """Arm one-shot test faults (MG_INJECT_* bits) on the whole-grid handle inside; returns the status."""
+    return lib().mg_dd_debug_inject(dd, int(faults))
 
 
 def mg_dd_solve(dd, b, p, dims, stats: mg_stats | None = None):

@@ -559,6 +559,18 @@ int next_inner(double rr_prev, double rr, int k, double rtol) {
     return kn < 1 ? 1 : (kn > kMaxAdaptive ? kMaxAdaptive : kn);
 }
 
+// MG_ERR_CUDA if a bounded wait ran out since the last look: bit 4 of the error word (a fused sweep) or 8 (the
+// coarse levels' cluster, which then leaves no numbers).  Clears the word.
+int check_waits(mg_handle *h) {
+    MG_READBACK_ERR(h, h->s);
+    MG_CUDA(h, cudaStreamSynchronize(h->s));
+    const unsigned herr = *h->herr;
+    if (!(herr & 12u)) return MG_OK;
+    MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->s));
+    return fail(h, MG_ERR_CUDA, herr & 4u ? "a fused sweep gave up waiting for its shared-memory copies"
+                                          : "the coarse levels' cluster gave up waiting for its neighbours' cells");
+}
+
 // ---- one solve A x = b - mean(b), zero-mean x -------------------------------------------
 int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st) {
     cudaStream_t s = h->s;
@@ -735,20 +747,9 @@ int solve_impl(mg_handle *h, const double *b, double *p, int warm, mg_stats *st)
     MG_CUDA(h, cudaEventSynchronize(h->ev1));
     rc = check_launch(h, "solve");
     if (rc) return rc;
-    // a bounded wait that ran out sets bit 4 (a fused sweep) or 8 (the coarse levels' cluster, which then
-    // leaves no numbers)
     if (fused0(h, 0) || status == MG_ERR_DIVERGED) {
-        MG_READBACK_ERR(h, s);
-        MG_CUDA(h, cudaStreamSynchronize(s));
-        const unsigned herr = *h->herr;
-        if (herr & 4u) {
-            MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), s));
-            return fail(h, MG_ERR_CUDA, "a fused sweep gave up waiting for its shared-memory copies");
-        }
-        if (herr & 8u) {
-            MG_CUDA(h, cudaMemsetAsync(h->err, 0, sizeof(unsigned), s));
-            return fail(h, MG_ERR_CUDA, "the coarse levels' cluster gave up waiting for its neighbours' cells");
-        }
+        rc = check_waits(h);
+        if (rc) return rc;
     }
     if (st) {
         st->status = status;
@@ -791,6 +792,7 @@ namespace mg {
 Lay handle_lay32(mg_handle *h, int l) { return h->lv[l].lay; }
 float *handle_b32(mg_handle *h, int l) { return h->lv[l].b32; }
 float *handle_x32(mg_handle *h, int l) { return h->lv[l].x32; }
+int handle_check_waits(mg_handle *h) { return check_waits(h); }
 void handle_vcycle32(mg_handle *h, int l) { vcycle32(h, l, h->lv[l].b32, h->lv[l].x32); }
 int handle_first_inner() { return kFirstAdaptive; }
 int handle_next_inner(double rr_prev, double rr, int k, double rtol) { return next_inner(rr_prev, rr, k, rtol); }

@@ -643,6 +643,7 @@ int solve_mixed(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ev.e[0], ev.e[1]);
     DD_CUDA(dd, cudaGetLastError());
+    if (status == MG_ERR_DIVERGED && (rc = mg::handle_check_waits(dd->ch))) return dd_fail(dd, rc, "%s", mg_last_error(dd->ch));
     if (st) {
         st->status = status;
         st->cycles = cycles;
@@ -997,6 +998,8 @@ int mg_dd_vcycle(mg_dd *dd, const double *b, double *x) {
     DD_CUDA(dd, cudaStreamSynchronize(s));
     return MG_OK;
 }
+
+int mg_dd_debug_inject(mg_dd *dd, int faults) { return dd ? mg_debug_inject(dd->ch, faults) : MG_ERR_ARG; }
 
 int mg_dd_solve(mg_dd *dd, const double *b, double *p, mg_stats *st) {
     mg::NvtxRange nvtx_("mg_dd_solve");

@@ -219,6 +219,8 @@ Lay handle_lay32(mg_handle *h, int l);
 float *handle_b32(mg_handle *h, int l);
 float *handle_x32(mg_handle *h, int l);
 void handle_vcycle32(mg_handle *h, int l);
+// MG_ERR_CUDA, with the handle's message, if a bounded wait of its kernels ran out
+int handle_check_waits(mg_handle *h);
 // the adaptive inner-cycle count of the mixed outer loop: the first, and the next from the
 // contraction of the last outer iteration (k cycles from relres rr_prev to rr)
 int handle_first_inner();
