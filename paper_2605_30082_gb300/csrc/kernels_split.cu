@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, UPDATE == 1 ? 3 : 4) k_half_vec(Lay 
 
 // ---- row-sharing half sweep -----------------------------------------------------------------
 // Row-sharing half sweep for the s-form regular sweep (the finest level's dominant kernel).  A
-// block takes a tile of RY rows of W four-cell vectors (RY W <= kZrThreads, one vector per
+// block takes a tile of RY rows of W four-cell vectors (RY W = kZrThreads, one vector per
 // thread) and marches ZC planes.  The other colour's x and s of the tile's rows and of the rows
 // above and below travel by cp.async into a ring of kZrStages planes in shared memory, two planes
 // ahead, with the cells' own s and b; every row is fetched once per block and read three times
@@ -338,10 +338,11 @@ constexpr int kZrThreads = 128, kZrStages = 4, kZrBlocks = 4;  // blocks per SM
 constexpr int kZrMaxSmem = 56 * 1024;                            // per block
 constexpr i64 kZrCells = 60000000;                               // see run_half_zr
 struct ZrTile {
-    int w, ry, zc;  // vectors per row, rows and planes of a tile
+    int w, ry, zc;  // vectors per row, rows and planes of a tile, w ry = kZrThreads
     int pitch;      // row stride in shared memory: whole 128 B lines, as cp.async writes them
     int slot;       // float4 of one plane's slot: ry + 2 rows of x and of s, own s and b, and (rows in
                     // several tiles) the vectors beside the tile's rows
+    int used;       // threads with a vector, per mille
 };
 
 
@@ -495,51 +496,41 @@ __global__ void __launch_bounds__(kZrThreads, kZrBlocks) k_half_zr(Lay L, ZrTile
     cp_async_wait<0>();  // only copies that nothing reads can remain; leave none behind
 }
 
-// Tiles of k_half_zr.  A tile that uses all of a block's threads comes first, then one that holds whole
-// rows (no vectors beside it), then a wide one; widths other than the whole row are multiples of 128 B.
-// 384^3 (48 vectors per row) takes 89.8 us in tiles of 16 x 8, 94 in 24 x 5, 99 in 48 x 2; 576 x 512 x 448 (72) 213 us in
-// 24 x 5, 221 in 16 x 8, 228 in 36 x 3; 448^3 (56) 143 us in 32 x 4, 147 in 56 x 2, 155 in 16 x 8.
-// Planes: the most up to 16 (fewer re-read boundary planes) that still give 1.6 waves of blocks, at least 4.
+// Tiles of k_half_zr: rows of 64, 32 or 16 vectors (or whole rows of 8), whole 128 B lines each, the widest of those that
+// leave the fewest threads beyond the end of a row.
 ZrTile zr_tile(const Lay &L) {
     ZrTile T;
     const int kv = L.hx / 4;
-    int best = 0, parts = 1;
-    T.w = 1;
-    for (int w = 64; w >= 8; w -= 8) {
-        for (int q = 0; q < 2; ++q) {  // whole rows of up to 64 vectors (tried once, at w = 64), then w
-            const int cand = q == 0 ? kv : w;
-            if (q == 0 ? (w != 64 || kv > 64) : (cand >= kv || cand < 16)) continue;
-            const int n = (kv + cand - 1) / cand;
-            // per mille of the threads in use, times 1.1 for whole rows
-            const int score = (q == 0 ? 1100 : 1000) * (kv * (kZrThreads / cand)) / (n * kZrThreads);
-            if (score > best) {
-                best = score;
-                T.w = cand;
-                parts = n;
-            }
+    T.w = T.used = 0;
+    for (int w = 64; w >= 8; w /= 2) {
+        if (w > kv || (w == 8 && kv != 8)) continue;
+        const int n = (kv + w - 1) / w, used = 1000 * kv / (n * w);
+        if (used > T.used) {
+            T.used = used;
+            T.w = w;
         }
     }
+    if (!T.w) return T;
     T.ry = kZrThreads / T.w;
-    const i64 xy = (i64)parts * ((L.ny + T.ry - 1) / T.ry);
-    const i64 want = (i64)device_sms() * kZrBlocks * 8 / 5;
     T.zc = 16;
-    while (T.zc > 4 && xy * ((L.nz + T.zc - 1) / T.zc) < want) T.zc /= 2;
-    T.pitch = (T.w + 7) & ~7;
-    T.slot = 2 * (T.ry + 2) * T.pitch + 2 * kZrThreads + (parts > 1 ? 4 * T.ry : 0);
+    T.pitch = T.w;
+    T.slot = 2 * (T.ry + 2) * T.w + 2 * kZrThreads + (kv > T.w ? 4 * T.ry : 0);
     return T;
 }
 
-// Whether the s-form regular sweep of L goes to k_half_zr (and its launch): tiles that use all of a block's threads, on
-// levels of 60 M cells and more, where it is the one that HBM alone bounds.  V-cycles with it and with k_half_vec: 512^3
-// 2883 against 2965 us, 512 x 512 x 256 1474 against 1508, 256 x 512 x 512 1462 against 1496, 1024 x 256 x 256 1485 against 1518;
-// 512 x 384 x 256 1136 against 1129, 256^3 411 against 404, 192^3 230 against 193; partial tiles 448^3 2058 against 2005,
-// 576 x 512 x 448 2983 against 2935.
+// Whether the s-form regular sweep of L goes to k_half_zr (and its launch): tiles that leave at most a tenth of the threads
+// idle, on levels of 60 M cells and more, where it is the one that HBM alone bounds.  (A whole grid of that size has sides
+// that are multiples of 64, or its coarsest level would be too large; only a slab's last planes can be part of a tile.)
+// V-cycles with it and with k_half_vec: 512^3 2883 against 2965 us, 512 x 512 x 256 1474 against 1508, 256 x 512 x 512
+// 1462 against 1496, 1024 x 256 x 256 1485 against 1518;
+// 512 x 384 x 256 1136 against 1129, 256^3 411 against 404, 192^3 230 against 193; tiles with more idle threads 448^3 2058 against
+// 2005, 576 x 512 x 448 2983 against 2935.
 template <bool GHOST>
 bool run_half_zr(cudaStream_t s, const Lay &L, float h2, const float *sv, const float *b, float *x, int col) {
     const int kv = L.hx / 4;
     if (L.n < kZrCells) return false;
     const ZrTile T = zr_tile(L);
-    if (T.w * T.ry != kZrThreads) return false;
+    if (T.used <= 900) return false;
     static std::atomic<unsigned long long> opted{0};
     if (!opt_in_smem((const void *)k_half_zr<GHOST>, kZrMaxSmem, opted)) return true;  // the caller checks the error
     run_kernel(k_half_zr<GHOST>, dim3((kv + T.w - 1) / T.w, (L.ny + T.ry - 1) / T.ry, (L.nz + T.zc - 1) / T.zc), kZrThreads,
