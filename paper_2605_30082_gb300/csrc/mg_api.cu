@@ -407,7 +407,7 @@ void vcycle32(mg_handle *h, int l, const float *b, float *x, const OuterUpdate *
 }
 
 // Which levels run as one cluster launch: from the first level (below the finest) that fits the
-// threads and shared memory of 16 CTAs (8 where the device refuses 16): 32768 cells in FP32 and
+// threads and shared memory of 16 CTAs: 32768 cells in FP32 and
 // 16384 in FP64, where 16 SMs update one colour in about 1 us, half of what a launch over the
 // whole device costs.  With more than 512 coarse cells the dense product (n^2 FP64 FMAs, 4 us
 // on 16 SMs at 512) goes to the whole device between two cluster launches.
@@ -436,7 +436,7 @@ void plan_tail(mg_handle *h) {
             t.h2 = L.h2;
             t.ih2 = L.ih2;
         }
-        if (mg::tail_layout(a, f64, 16) || mg::tail_layout(a, f64, 8)) {
+        if (mg::tail_layout(a, f64, 16)) {
             h->tail_l = l;
             h->tail_split = h->nc > kTailCoarse;
             return;
