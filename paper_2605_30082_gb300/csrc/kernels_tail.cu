@@ -691,11 +691,12 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
             if (mode == kTailDown && v + 1 == v1) leave();
             t.restrict_red(l, C, mode == kTailDown, first, lost);
         }
+        if (v + 1 == v1) break;
         // the next level's contexts come in meanwhile.  On the way down a CTA waits for what it
         // reads; on the way up the next level reads other CTAs' x
-        if (up && v + 1 < v1) cl.barrier_arrive();
-        if (v + 1 < v1) restore(v + 1);
-        if (up || v + 1 == v1) {
+        if (up) cl.barrier_arrive();
+        restore(v + 1);
+        if (up) {
             cl.barrier_wait();
         } else if (C) {
             t.expect(t.bar_b(l + 1), t.cell_bytes(*C), lost);
@@ -708,14 +709,17 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
             t.wait(t.bar_e(), 0, lost);
         }
     }
-    if (__syncthreads_or(lost)) {  // the level's x without a number fails the solve
-        // what other CTAs had sent this one, which a CTA that was not lost has waited for, arrives first
-        for (const long long t0 = clock64(); clock64() - t0 < kTailLingerCycles;) {}
+    const bool gave_up = __syncthreads_or(lost);
+    if (gave_up) {  // the level's x without a number fails the solve
         if (t.tid == 0) atomicOr(a.err, 8u);
         for (int i = t.tid; i < (lv[0].off_b - lv[0].off_x) / (int)sizeof(T); i += kTailThreads) t.x(lv[0])[i] = (T)NAN;
         __syncthreads();
     }
     for (int l = 0; l < (mode == kTailDown ? a.nl : 1); ++l) t.store(lv[l], l > 0);
+    cl.barrier_wait();  // that of leave(), over by now where no wait ran out
+    // what other CTAs had sent this one, which a CTA that did not give up has waited for, arrives before it goes
+    if (gave_up)
+        for (const long long t0 = clock64(); clock64() - t0 < kTailLingerCycles;) {}
 }
 
 template <typename T>
