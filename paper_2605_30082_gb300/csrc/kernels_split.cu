@@ -324,11 +324,12 @@ __global__ void __launch_bounds__(kThreads, UPDATE == 1 ? 3 : 4) k_half_vec(Lay 
 // ahead, with the cells' own s and b; every row is fetched once per block and read three times
 // (as y - 1, y and y + 1) from there.  A slot is refilled behind the block barrier that ends its plane.
 //
-// What bounded its predecessor (each thread fetching its own six vectors per plane) was the traffic between L2 and the SMs, 36 B per updated cell, and 87 instructions per cell: 215 us per 512^3
-// half sweep (6.24 TB/s of its 10 B per cell, 0.92 of the copy bandwidth) and, on grids that fit L2, no
+// What bounded its predecessor (each thread fetching its own six vectors per plane) was the traffic between L2 and the
+// SMs, 36 B per updated cell, and 87 instructions per cell: 215 us per 512^3 half sweep (6.24 TB/s of its 10 B per cell, 0.92 of the copy bandwidth) and, on grids that fit L2, no
 // more than 5.3 TB/s.  Sharing rows (28 B at W = 64, RY = 2; 24 B at W = 32, RY = 4), walls folded into
 // s (a missing neighbour's s is taken as -s, so that its weight is an exact 0) and packed FP32
-// pairs (f32x2) leave it bound by HBM: 194 us, 6.92 TB/s; 512 x 512 x 64 38.4 -> 28 us, x 32 19.8 -> 12.7 us.  More rows per block
+// pairs (f32x2) leave it bound by HBM: 194 us by itself, 202 us inside a solve (6.63 TB/s, 0.975 of the copy bandwidth);
+// by itself 512 x 512 x 64 38.4 -> 28 us, x 32 19.8 -> 12.7 us.  More rows per block
 // (4 of 64 vectors) gave 202 us, one 206 us, three stages 219 us, five 197 us.
 //
 // Blocks of black sweeps take the planes from above, so that a sweep begins with the planes the one

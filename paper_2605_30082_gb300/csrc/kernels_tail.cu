@@ -1,14 +1,15 @@
 // The coarse levels of a V-cycle in one launch: one thread-block cluster holds every level from
-// `first` down in its CTAs' shared memory and runs their smoothing sweeps, transfers and the
+// a given one (TailArgs::lv[0]) down in its CTAs' shared memory and runs their smoothing sweeps, transfers and the
 // dense coarse solve, CTAs waiting only for what they read.
 //
 // What bounds the levels below about 40^3 is the chain of dependent launches (ten per level and
-// cycle, 2-3 us each, for work of a fraction of a microsecond), so the
+// cycle, 1.5-2 us each with programmatic serialisation, for work of a fraction of a microsecond), so the
 // chain is made of cheaper links: a half sweep here is one shared-memory round trip and a wait for
-// the neighbours' ghosts, 0.5 us at 32^3 and 0.4 us at 16^3.  The levels 32^3, 16^3 and 8^3 of a cycle take 26 us
-// (launch by launch 50 us): 2 us to copy the contexts in beside the kernel before, 5.5 us for the dense product of
-// 512 cells (4 us of it the FP64 FMAs on 16 SMs), 5 us for the transfers, 16 half sweeps.  A 64^3 projection step went
-// from 2.50 to 2.18 ms, a 32^3 one in FP64 from 2.16 to 1.67 ms.
+// the neighbours' ghosts, 0.5 us at 32^3 and 0.4 us at 16^3.  The levels 32^3, 16^3 and 8^3 of a cycle take about 25 us:
+// 2 us to copy the contexts in beside the kernel before, 5.5 us for the dense product of
+// 512 cells (4 us of it the FP64 FMAs on 16 SMs), 5 us for the transfers, 16 half sweeps.  A whole cycle and its share
+// of a residual, launch by launch and with the cluster: 64^3 mixed 56.7 and 43.5 us, down to 4^3 73.5 and 44.2; 64^3 in
+// FP64 124 and 102, 32^3 82.9 and 58.3; 128^3 94.7 and 85.8; 72 x 80 x 88 with 990 coarse cells (two launches) 67.5 and 64.6.
 //
 // Layout.  The rows (y, z) of a level are dealt out in quads, the four rows of one coarse row
 // (J, K), so that the eight children of a coarse cell sit in one CTA; CTA r holds the quads

@@ -408,8 +408,8 @@ void vcycle32(mg_handle *h, int l, const float *b, float *x, const OuterUpdate *
 
 // Which levels run as one cluster launch: from the first level (below the finest) that fits the
 // threads and shared memory of 16 CTAs: 32768 cells in FP32 and
-// 16384 in FP64, where 16 SMs update one colour in about 1 us, half of what a launch over the
-// whole device costs.  With more than 512 coarse cells the dense product (n^2 FP64 FMAs, 4 us
+// 16384 in FP64, where 16 SMs update one colour in about 0.5 us and a launch over the whole device
+// takes 1.5-2 us (whole cycles with both stand in kernels_tail.cu).  With more than 512 coarse cells the dense product (n^2 FP64 FMAs, 4 us
 // on 16 SMs at 512) goes to the whole device between two cluster launches.
 constexpr int kTailCoarse = 512;
 
